@@ -6,11 +6,24 @@ namespace mixkvq {
 // Partials live at ws[slot * kPartialFloats + h * 130 + {0: m (log2 domain), 1: l, 2..129: o}].
 // mode 0: stream s owns slots [s*n, s*n + n).  mode 1: the attention grid of `n` CTAs split the
 // S*units_per_stream work units evenly; CTA c wrote its part of stream s to slot c + s.
-__global__ void __launch_bounds__(128)
+//
+// One CTA per (stream, head).  What bounds it is latency: a stream has between 1 partial (many streams) and 74 (four
+// streams, 296 CTAs), 0.5 KB each.  The warps of the CTA take the partials in turn (warp w: w, w + W, ...), kChunk of
+// them in flight per warp, so that up to W * kChunk partials cost one round trip to memory; the warps' results meet in
+// shared memory.  B200, attention + merge per layer from a graph: one sequence of 4000 tokens (74 partials) 17.2 us with
+// one thread per channel walking chunks of 12, 9.6 us so; 8 sequences of 32768 tokens (9 partials) 41.7 and
+// 40.4 us.
+constexpr int kCombineChunk = 8;
+constexpr int kCombineMaxWarps = 8;
+
+__global__ void __launch_bounds__(kCombineMaxWarps * 32)
 combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int Hkv, int Hq, int mode, int n,
                long long units_per_stream, int S, const int4* __restrict__ seq, const int* __restrict__ seq_prefix,
                float* __restrict__ lse_out) {
-  const int s = blockIdx.x / g, h = blockIdx.x % g, c = threadIdx.x;
+  __shared__ float mlS[kCombineMaxWarps][2];
+  __shared__ __align__(16) float oS[kCombineMaxWarps][kD];
+  const int s = blockIdx.x / g, h = blockIdx.x % g;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = blockDim.x >> 5;
   int first, count;
   // started early (programmatic dependent launch): wait here for the kernel that wrote the partials
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -33,49 +46,74 @@ combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int
     first = c0 + s;
     count = c1 - c0 + 1;
   }
-  const int b = s / Hkv, hk = s % Hkv;
+  // ---- this warp's partials: one pass with a running maximum; a lane has channels 2 lane, 2 lane + 1 and 64 more
   const float* base = ws + (size_t)first * kPartialFloats + h * 130;
-  // one pass with a running maximum; the loads of a chunk of partials are independent of one another, so a stream with
-  // up to kChunk partials costs one round trip to memory
-  constexpr int kChunk = 12;
-  float M = -INFINITY, l = 0.f, o = 0.f;
-  for (int i0 = 0; i0 < count; i0 += kChunk) {
-    float m[kChunk], ll[kChunk], oo[kChunk];
+  float M = -INFINITY, l = 0.f;
+  float2 oa = make_float2(0.f, 0.f), ob = make_float2(0.f, 0.f);
+  for (int i0 = warp; i0 < count; i0 += W * kCombineChunk) {
+    float2 ml[kCombineChunk], xa[kCombineChunk], xb[kCombineChunk];
 #pragma unroll
-    for (int j = 0; j < kChunk; ++j) {
-      const bool in = i0 + j < count;
-      const float* p = base + (size_t)(in ? i0 + j : i0) * kPartialFloats;
-      m[j] = in ? p[0] : -INFINITY;
-      ll[j] = p[1];
-      oo[j] = p[2 + c];
+    for (int j = 0; j < kCombineChunk; ++j) {
+      const int i = i0 + j * W;
+      ml[j] = make_float2(-INFINITY, 0.f);
+      xa[j] = xb[j] = make_float2(0.f, 0.f);
+      if (i < count) {
+        const float2* p = reinterpret_cast<const float2*>(base + (size_t)i * kPartialFloats);
+        ml[j] = p[0];
+        xa[j] = p[1 + lane];
+        xb[j] = p[33 + lane];
+      }
     }
     float Mn = M;
 #pragma unroll
-    for (int j = 0; j < kChunk; ++j) Mn = fmaxf(Mn, m[j]);
+    for (int j = 0; j < kCombineChunk; ++j) Mn = fmaxf(Mn, ml[j].x);
     const float f0 = (M == -INFINITY) ? 0.f : exp2f(M - Mn);
     l *= f0;
-    o *= f0;
+    oa.x *= f0; oa.y *= f0; ob.x *= f0; ob.y *= f0;
 #pragma unroll
-    for (int j = 0; j < kChunk; ++j) {
-      const float f = (m[j] == -INFINITY) ? 0.f : exp2f(m[j] - Mn);
-      l += f * ll[j];
-      o += f * oo[j];
+    for (int j = 0; j < kCombineChunk; ++j) {
+      const float f = (ml[j].x == -INFINITY) ? 0.f : exp2f(ml[j].x - Mn);
+      l += f * ml[j].y;
+      oa.x += f * xa[j].x; oa.y += f * xa[j].y;
+      ob.x += f * xb[j].x; ob.y += f * xb[j].y;
     }
     M = Mn;
   }
-  // l == 0 only when every split gave up (its partial is then m = -inf, l = 0, o = 0 and the status word says so) or
+  // ---- the warps' results
+  if (lane == 0) {
+    mlS[warp][0] = M;
+    mlS[warp][1] = l;
+  }
+  *reinterpret_cast<float2*>(&oS[warp][2 * lane]) = oa;
+  *reinterpret_cast<float2*>(&oS[warp][64 + 2 * lane]) = ob;
+  __syncthreads();
+  const int c = threadIdx.x;
+  if (c >= kD) return;
+  float Mt = -INFINITY, lt = 0.f, ot = 0.f;
+  for (int w = 0; w < W; ++w) Mt = fmaxf(Mt, mlS[w][0]);
+  for (int w = 0; w < W; ++w) {
+    const float mw = mlS[w][0], f = (mw == -INFINITY) ? 0.f : exp2f(mw - Mt);
+    lt += f * mlS[w][1];
+    ot += f * oS[w][c];
+  }
+  // lt == 0 only when every split gave up (its partial is then m = -inf, l = 0, o = 0 and the status word says so) or
   // when the sequence of a ragged batch holds no token
-  out[((size_t)b * Hq + hk * g + h) * kD + c] = l > 0.f ? o / l : 0.f;
-  // natural logarithm of the softmax denominator (the maximum M is kept in the base-2 domain)
-  if (lse_out != nullptr && c == 0) lse_out[(size_t)b * Hq + hk * g + h] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
+  const int b = s / Hkv, hk = s % Hkv;
+  out[((size_t)b * Hq + hk * g + h) * kD + c] = lt > 0.f ? ot / lt : 0.f;
+  // natural logarithm of the softmax denominator (the maximum is kept in the base-2 domain)
+  if (lse_out != nullptr && c == 0)
+    lse_out[(size_t)b * Hq + hk * g + h] = lt > 0.f ? (Mt + log2f(lt)) * 0.6931471805599453f : -INFINITY;
 }
 
 cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, int mode, int n,
                            long long units_per_stream, int S, cudaStream_t stream, const int4* seq, const int* seq_prefix,
                            float* lse_out) {
+  // eight warps when four with a chunk each do not cover a stream's partials in one round trip (a ragged batch may give
+  // nearly all CTAs to one sequence), four otherwise: more warps only lengthen the last step
+  const int partials = mode == 0 ? n : (seq != nullptr ? n : n / S + 1);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(S * g));
-  cfg.blockDim = dim3(128);
+  cfg.blockDim = dim3(partials > 4 * kCombineChunk ? kCombineMaxWarps * 32 : 128);
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
