@@ -262,12 +262,14 @@ int append_run_first(mixkvq_cache* cache, int layer, int b0, int nb, const void*
     if (r0 == 0 && n_tokens - t > cache->R) {
       int nblk = (n_tokens - t - 1) / cache->R;
       if (nblk > 32768) nblk = 32768;                  // grid.y limit
+      const int left = n_tokens - t - nblk * cache->R, tail = left <= cache->R ? left : 0;
       LayerView lv = view(cache, layer, b0, nb);
-      if (launch_flush_bulk(lv, k, v, q, n_stride, t, nblk, st) != cudaSuccess) return MIXKVQ_E_CUDA;
-      cache->launches += cache->cfg.importance_mode == 1 ? 4 : 3;
+      if (launch_flush_bulk(lv, k, v, q, n_stride, t, nblk, tail, st) != cudaSuccess) return MIXKVQ_E_CUDA;
+      cache->launches += cache->cfg.importance_mode == 1 ? 3 : 2;
       cache->last_packed_writer = layer;
       nb0 += nblk;
-      t += nblk * cache->R;
+      r0 = tail;
+      t += nblk * cache->R + tail;
       continue;
     }
     const int m = (n_tokens - t < cache->R - r0) ? n_tokens - t : cache->R - r0;
@@ -334,7 +336,8 @@ int mixkvq_cache_init(const mixkvq_config* cfg, void* cache_dev, size_t bytes, v
   if (cudaMemsetAsync(h->mem, 0, kHeaderBytes, st) != cudaSuccess) { delete h; return MIXKVQ_E_CUDA; }
   for (int l = 0; l < cfg->n_layers; ++l)
     if (zero_layer_state(h, l, st) != MIXKVQ_OK) { delete h; return MIXKVQ_E_CUDA; }
-  if (attention_ws_setup() != cudaSuccess || attention_tc_setup() != cudaSuccess || prefill_attention_setup() != cudaSuccess) { delete h; return MIXKVQ_E_CUDA; }
+  if (attention_ws_setup() != cudaSuccess || attention_tc_setup() != cudaSuccess || prefill_attention_setup() != cudaSuccess ||
+      flush_setup() != cudaSuccess) { delete h; return MIXKVQ_E_CUDA; }
   *out = h;
   return MIXKVQ_OK;
 }

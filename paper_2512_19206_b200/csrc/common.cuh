@@ -118,18 +118,6 @@ __device__ inline int quant_code(float x, float z, float s, int max_code) {
   return min(max(c, 0), max_code);
 }
 
-// The same code by a shortcut, bit-identical to quant_code for every input: with r = RN(1 / s) the product (x - z) * r is
-// within 2e-6 of the IEEE quotient (codes are at most 15), so it rounds to the same integer unless it lies within 1e-4
-// of a half-integer; only then is the IEEE division carried out.  r is computed once per group.
-__device__ inline int quant_code_fast(float x, float z, float s, float r, int max_code) {
-  if (s == 0.0f) return 0;
-  const float y = __fmul_rn(__fsub_rn(x, z), r);
-  const float frac = y - floorf(y);
-  if (fabsf(frac - 0.5f) < 1e-4f) return quant_code(x, z, s, max_code);
-  int c = __float2int_rn(y);
-  return min(max(c, 0), max_code);
-}
-
 // Section 4.2: A_d = (acc / cnt) * (range / (2^B - 1)) in fp64; tier by the two thresholds.
 // error_only (the ablation without the query term): I_d = 1, so A_d = S_d.
 __device__ inline uint8_t salience_tier(double acc, uint32_t cnt, float mx, float mn, int score_bits,
@@ -209,7 +197,8 @@ cudaError_t launch_rope(void* k, void* q, const float* cos_t, const float* sin_t
                         int pos0, cudaStream_t stream);
 cudaError_t launch_flush(const LayerView& lv, cudaStream_t stream);
 cudaError_t launch_flush_bulk(const LayerView& lv, const void* k, const void* v, const void* q, int n_tokens, int t0,
-                              int nb, cudaStream_t stream);
+                              int nb, int tail, cudaStream_t stream);
+cudaError_t flush_setup();
 cudaError_t launch_select_window(const LayerView& lv, uint8_t* tiers, double* salience, cudaStream_t stream);
 cudaError_t launch_select_raw(const void* q, const void* k, int B, int Hq, int Hkv, int lq, int lk, int score_bits,
                               float tau_bf16, float tau_u4, uint8_t* tiers, double* salience, cudaStream_t stream);
