@@ -1,233 +1,92 @@
 // Fused split-K GQA decode attention over the mixed-precision cache (Eq. 1 with Eq. 3 applied on the fly),
 // warp-specialised form.
 //
-// Work unit = 32 tokens of one stream.  All units of all streams are split evenly over the CTAs; inside a CTA they
-// are split over PAIRS of warps.  A pair shares one ring of staged units (1-D bulk copies signalled on mbarriers):
+// Work unit = 32 tokens of one stream, taken two at a time (a step of 64 tokens; blocks hold an even number of units).  All
+// units of all streams are split evenly over the CTAs; inside a CTA they are split over PAIRS of warps.  A pair shares one
+// ring of staged steps (1-D bulk copies signalled on mbarriers):
 //
-//   the logits warp   expands the unit's 2-bit key codes into tensor-core A fragments (one logic op and one fp16 FMA
+//   the logits warp   expands the step's 2-bit key codes into tensor-core A fragments (one logic op and one fp16 FMA
 //                     per pair of codes: A = c*s, exact in fp16) and runs q.K^T on mma.sync m16n8k16 tiles with the g
-//                     query heads of the KV head as the N dimension.  The zero-point term q.z of the key group (one
-//                     extra tile chain per group) is the initial value of the accumulators; the promoted (BF16)
-//                     channels and the UINT4 high plane are further tiles.  The unit's 32 x 8 logits go to the
-//                     partner through shared memory.
-//   the values warp   keeps the online softmax (lazily raised reference maximum), builds the unit's value-scale tables,
+//                     query heads of the KV head as the N dimension.  The zero-point term q.z of the key groups is one
+//                     more tile chain per step (rows 0..7 the first unit's group, rows 8..15 the second's); the promoted
+//                     (BF16) channels and the UINT4 high plane are further tiles.  The step's 64 x 8 logits go to the
+//                     partner through shared memory, in the place of the key codes and scales they were made from.
+//   the values warp   keeps the online softmax (lazily raised reference maximum), builds the value-scale tables,
 //                     folds the value scales into the probabilities and runs P.V with the raw value codes as fp16
 //                     subnormals in the A operand (one logic op per pair of codes); value zero-points and the softmax
 //                     denominator ride on one extra tile.  It owns the output accumulators and refills the ring.
 //
 // Neither warp holds the other's state, so both need far fewer registers than a warp that does everything, more warps
-// fit an SM, and the logits of unit n+1 overlap the values of unit n.  The packed layout stores the codes in A-fragment
-// order: a lane's 16-byte shared-memory load is exactly its registers; nothing dequantized is ever written back to
-// shared memory.  Unquantized units (residual window, sink) are read straight from global memory in bf16 and are taken
+// fit an SM, and the logits of one step overlap the values of the one before.  The packed layout stores the codes in
+// A-fragment order: a lane's 16-byte shared-memory load is exactly its registers; nothing dequantized is ever written back
+// to shared memory.  Unquantized units (residual window, sink) are read straight from global memory in bf16 and are taken
 // first, while the first staged copies are in flight.
-#include "common.cuh"
+//
+// What bounds it: instruction issue and the latency of each warp's chain of dependent work, with three or four warps per
+// scheduler.  Two units per step instead of one (attention_single.cu) give every chain an independent twin, halve the
+// waits, hand-overs and zero-point tiles per unit (690 -> 598 warp instructions per unit) and need no hand-over buffers; the
+// promoted channels and the UINT4 plane, read from global memory a unit ahead there, come through shared memory two steps ahead
+// (without that the longer steps were slower than single units: 39.0 us at the 7b shape).  us per launch, one unit / two:
+// 7b shape (B = 8, T = 32768) 36.7 / 35.3; three tiers 54.4 / 48.7; 4-bit base (8b shape, B = 16, T = 16384) 110.7 / 109.5;
+// 4-bit values 88.4 / 81.4; 32b shape (B = 64, T = 32768, G = 128) 463 / 438 = 3.1 TB/s.
+#include "warp_ops.cuh"
 
 namespace mixkvq {
 
 cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, int mode, int n,
                            long long units_per_stream, int S, cudaStream_t stream, const int4* seq = nullptr,
                            const int* seq_prefix = nullptr, float* lse_out = nullptr);
+// the same split, one unit at a time (attention_single.cu)
+cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, cudaStream_t stream);
+cudaError_t attention_single_setup();
 
 namespace {
 
-#ifndef MIXKVQ_WS_PAIRS
-#define MIXKVQ_WS_PAIRS 4
-#define MIXKVQ_WS_CTAS 2
-#endif
-constexpr int kPairs = MIXKVQ_WS_PAIRS;      // warp pairs per CTA
-constexpr int kThreads = kPairs * 64;
-constexpr int kCtasPerSm = MIXKVQ_WS_CTAS;
-constexpr int kStages = 4;                   // ring stages per pair (a power of two)
-// one ring stage: a key-meta group (512 B) followed by the unit (<= 2560 B; <= 3584 B with 4-bit values), as in the block
-__host__ __device__ constexpr int stage_bytes(bool v4) { return v4 ? 4096 : 3072; }
-constexpr int kKeyMetaOff = 0;
-constexpr int kUnitOff = 512;
-// per-pair tables: key scales {s, -4s} (576) | key zero-point tiles (576) | value scales (320) | value zero-point tile (1088)
-constexpr int kKprepOff = 0, kZprepOff = 576, kSvpOff = 1152, kZvpOff = 1472, kPrepBytes = 2560;
-// hand-over of a unit's logits: 32 bytes per lane, then 8 bytes per lane with the zero-point term of the unit's key
-// group; one buffer per ring stage and one for unquantized units
-constexpr int kLBufBytes = 1280, kLBufZeroOff = 1024;
-__host__ __device__ constexpr int pair_bytes(bool v4) {
-  return kStages * stage_bytes(v4) + kPrepBytes + (kStages + 1) * kLBufBytes;
+// Warp pairs per CTA (two CTAs per SM): four at 128 registers per thread, or three at 168 where the logits warp needs more
+// (UINT4 tiles or a second key plane) or the shared memory does not hold four.
+__host__ __device__ constexpr int pairs_of(int u4, bool v4) { return u4 != 0 || v4 ? 3 : 4; }
+constexpr int kCtasPerSm = 2;
+constexpr int kStages = 3;                   // ring stages per pair
+__host__ __device__ constexpr int unit_bytes_of(int G, bool v4) { return 2048 + 128 * (kD / G) + (v4 ? 1024 : 0); }
+// one ring stage: the two units of a step with their key-meta groups (512 B each) in the block's own order: a group before
+// each unit (G = 32), or one group before both
+__host__ __device__ constexpr int stage_bytes(int G, bool v4) { return (G == 32 ? 1024 : 512) + 2 * unit_bytes_of(G, v4); }
+// per-pair tables: key scales {s, -4s} of two groups (2 x 576) | key zero-point tiles (576) | value scales of two units
+// (2 x 320) | value zero-point tiles of two units (2 x 544)
+constexpr int kKprepOff = 0, kZprepOff = 1152, kSvpOff = 1728, kZvpOff = 2368, kPrepBytes = 3456;
+constexpr int kKprepGroup = 576, kSvpUnit = 320, kZvpUnit = 544;
+constexpr int kRBufBytes = 1024;             // hand-over of an unquantized unit's logits: 32 bytes per lane
+// A step's extras (the promoted channels and the UINT4 high plane), copied by the logits warp kSlots - 1 steps ahead:
+// the head of the block's channel lists (64 B, in a step that begins a block) | rows of the first kRowPairs pairs of
+// promoted channels of both units (128 B each) | three tiers: the first kPlanePairs pairs of UINT4 channels of both units
+// (16 B each); 4-bit base: both units' dense planes.  What does not fit is read from global memory (rare).
+constexpr int kSlots = 3, kRowPairs = 4, kPlanePairs = 16;
+constexpr int kRowsOff = 128, kPlaneOff = kRowsOff + 2 * kRowPairs * 128;
+__host__ __device__ constexpr int slot_bytes(int u4) { return kPlaneOff + (u4 == 1 ? 2 * kPlanePairs * 16 : u4 == 2 ? 2048 : 0); }
+__host__ __device__ constexpr int slots_of(int u4, bool v4) { return u4 == 2 && v4 ? 2 : kSlots; }
+__host__ __device__ constexpr int pair_bytes(int G, int u4, bool v4) {
+  return kStages * stage_bytes(G, v4) + slots_of(u4, v4) * slot_bytes(u4) + kPrepBytes + kRBufBytes;
 }
-// mbarriers of a pair: staged copy landed [kStages], logits ready [kStages], then for unquantized units: ready, taken
+// mbarriers of a pair: staged copy landed [stages], logits ready [stages], then for unquantized units: ready, taken
 constexpr int kBarsPerPair = 2 * kStages + 2;
 constexpr int kQS = 136;                     // halves per row of the query tables (272 bytes: rows fall on different banks)
-constexpr int kBarBytes = ((kPairs * kBarsPerPair * 8 + 127) / 128) * 128;
 constexpr int kPrefixBytes = ((kMaxRaggedBatch + 1) * 4 + 15) / 16 * 16;     // a ragged batch's prefix sums
-constexpr int kSharedTail = kBarBytes + 2 * 8 * kQS * 2 + 2 * kPairs * 32 + kPrefixBytes;
-__host__ __device__ constexpr int smem_bytes(bool v4) { return kPairs * pair_bytes(v4) + kSharedTail; }
+__host__ __device__ constexpr int bar_bytes(int pairs) { return (pairs * kBarsPerPair * 8 + 127) / 128 * 128; }
+__host__ __device__ constexpr int smem_bytes(int G, int u4, bool v4) {
+  return pairs_of(u4, v4) * (pair_bytes(G, u4, v4) + 64) + bar_bytes(pairs_of(u4, v4)) + (u4 == 1 ? 2 : 1) * 8 * kQS * 2 + kPrefixBytes;
+}
 constexpr int kResidualWeight = 3;           // an unquantized 32-token unit counts as this many packed units in the split
 constexpr int kMergeStride = 132;            // floats per head row of a pair's output in the merge
-// With three tiers and with a 4-bit base the logits warp is by far the longer role (further tiles for the UINT4 high
-// plane, or a second key pass): the promoted channels' tile is then the values warp's work.  With two tiers it stays with
-// the logits warp: a stall of the values warp on global loads delays the ring's refill, which costs more there than the
-// tile does.  (The gathered UINT4 tiles stay with the logits warp in every case: moved, they made the values warp the
-// longer role and the kernel slower.)
-__host__ __device__ constexpr bool promoted_in_values(int u4) { return u4 != 0; }
 constexpr float kMaxSlack = 3.0f;            // a packed unit's probabilities are at most 2^kMaxSlack (log2 domain)
 // A wait on a barrier polls at most this many times; a poll suspends the thread for up to about a microsecond, so
 // the wait gives up after about two seconds at the latest (a few milliseconds if the polls return at once).
 constexpr uint32_t kWaitPolls = 1u << 21;
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-// Polls a phase of a barrier up to max_polls times; false if it never completed.
-__device__ __forceinline__ bool mbar_wait_polls(uint32_t bar, uint32_t parity, uint32_t max_polls) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t"
-      ".reg .pred p, q;\n\t"
-      ".reg .u32 n;\n\t"
-      "mov.u32 n, 0;\n"
-      "MIXKVQ_WAIT:\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n\t"
-      "@p bra MIXKVQ_DONE;\n\t"
-      "add.u32 n, n, 1;\n\t"
-      "setp.lt.u32 q, n, %3;\n\t"
-      "@q bra MIXKVQ_WAIT;\n"
-      "MIXKVQ_DONE:\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t"
-      "}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(max_polls)
-      : "memory");
-  return ok != 0;
-}
-// one lane of the (converged) warp arrives on the barrier
-__device__ __forceinline__ void mbar_arrive_one(uint32_t bar) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar)
-      : "memory");
-}
-// one lane of the (converged) warp stages `bytes` from global memory at shared address dst and arms the barrier for
-// bytes + extra (extra > 0 only in the test of the give-up path); nothing happens when `enabled` is 0
-__device__ __forceinline__ void stage_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, uint32_t extra,
-                                           uint32_t enabled) {
-  asm volatile(
-      "{\n\t.reg .pred p, e;\n\t.reg .u32 tx;\n\t"
-      "setp.ne.u32 e, %5, 0;\n\t"
-      "elect.sync _|p, 0xffffffff;\n\t"
-      "and.pred p, p, e;\n\t"
-      "add.u32 tx, %2, %4;\n\t"
-      "@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%3], tx;\n\t"
-      "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t"
-      "}" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar), "r"(extra), "r"(enabled)
-      : "memory");
-}
-// the same for a unit whose key-group scales do not lie directly before it: two copies on one barrier
-__device__ __forceinline__ void stage_copy2(uint32_t dst_a, const void* src_a, uint32_t bytes_a, uint32_t dst_b,
-                                            const void* src_b, uint32_t bytes_b, uint32_t bar, uint32_t extra) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .u32 tx;\n\t"
-      "elect.sync _|p, 0xffffffff;\n\t"
-      "add.u32 tx, %2, %5;\n\t"
-      "add.u32 tx, tx, %7;\n\t"
-      "@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%6], tx;\n\t"
-      "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%6];\n\t"
-      "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%3], [%4], %5, [%6];\n\t"
-      "}" ::"r"(dst_a),
-      "l"(src_a), "r"(bytes_a), "r"(dst_b), "l"(src_b), "r"(bytes_b), "r"(bar), "r"(extra)
-      : "memory");
-}
-// shared-memory accesses by 32-bit shared address (the offsets added at the call sites fold into the instruction)
-__device__ __forceinline__ uint4 lds128(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint2 lds64(uint32_t a) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t lds32(uint32_t a) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t lds16(uint32_t a) {
-  uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
-  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
-}
-__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
-  asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(a), "r"(x), "r"(y) : "memory");
-}
-__device__ __forceinline__ void sts32(uint32_t a, uint32_t x) {
-  asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
-}
-__device__ __forceinline__ void sts16(uint32_t a, uint32_t x) {
-  asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)x) : "memory");
-}
-
-__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                        uint32_t b0, uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-// d = a * b + c with the accumulator input in other registers than the result
-__device__ __forceinline__ void mma_f16_to(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                           uint32_t b1, float c0, float c1, float c2, float c3) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
-               : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
-}
-__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1) {
-  asm(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
-  uint32_t y;
-  asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t hfma2_u(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-  return d;
-}
-__device__ __forceinline__ uint32_t hmul2_u(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-// 2^x by the special-function unit alone (no range fix-up): inputs here are <= kMaxSlack or -inf
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
-  __half2 h = __floats2half2_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-__device__ __forceinline__ uint32_t pack_bf162(float lo, float hi) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
-// two bf16 in one word -> two fp16 in one word (exact inside the fp16 range)
-__device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t w) { return pack_half2(bf_lo(w), bf_hi(w)); }
-
 // Byte offset of (k-tile kt, lane column t) in the key-scale table: 16 bytes {s_a, -4 s_a, s_b, -4 s_b} (half2 each: the
 // lane's channel pairs 16kt + 2t, +1 and 16kt + 8 + 2t, +1); 16 bytes of padding after every second k-tile keep the
-// preparation's stores free of bank conflicts.
+// preparation's stores free of bank conflicts.  The zero-point table has the same shape: {z_a of unit 0, of unit 1, z_b of
+// unit 0, of unit 1}, times 2^(pos - 8): the A fragment of a tile whose rows 0..7 are unit 0's group, rows 8..15 unit 1's.
 __device__ __forceinline__ constexpr int kprep_off(int kt, int t) { return 144 * (kt >> 1) + 64 * (kt & 1) + 16 * t; }
-// First 32-bit word of k-tile kt in the zero-point tile table (16 words per k-tile, four extra every second k-tile).
-__device__ __forceinline__ constexpr int zprep_word(int kt) { return 16 * kt + 4 * (kt >> 1); }
 // Bit position (inside each 16-bit half, after the shift below) of k-tile kt's 2-bit field.
 __device__ __forceinline__ constexpr int key_pos(int kt) { return (0x86486464u >> (4 * kt)) & 0xF; }
 // k-tiles 0,1 are read from (w << 4), 2..4 from w, 5..7 from (w >> 6)
@@ -240,20 +99,24 @@ __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp
 // per channel pair, gathered), 2 = 4-bit base (dense high plane)
 // kV4: 4-bit values (a second plane of 2-bit value codes per unit, scale 4 s_v)
 template <int G, int kU4, bool kV4>
-#ifdef MIXKVQ_WS_MAXNREG
-__global__ void __maxnreg__(MIXKVQ_WS_MAXNREG)
-#else
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
-#endif
+__global__ void __launch_bounds__(pairs_of(kU4, kV4) * 64, kCtasPerSm)
 attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float scale_log2e, float* __restrict__ ws,
                     uint32_t four2) {
   constexpr int VG = kD / G;              // value groups per token
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group
-  constexpr int kStageBytes = stage_bytes(kV4);
-  constexpr int kPairBytes = pair_bytes(kV4);
-  constexpr int kPrepBase = kStages * kStageBytes;             // offsets inside a pair's shared memory
-  constexpr int kLBufBase = kPrepBase + kPrepBytes;
-  constexpr int kRBufBase = kLBufBase + kStages * kLBufBytes;
+  constexpr int UPG = G / 32;             // units per key group
+  constexpr int kGroups = UPG == 1 ? 2 : 1;                    // key groups of a step
+  constexpr int kPairs = pairs_of(kU4, kV4), kThreads = kPairs * 64;
+  constexpr int kSlotCount = slots_of(kU4, kV4), kSlotBytes = slot_bytes(kU4);
+  constexpr int kStageBytes = stage_bytes(G, kV4);
+  constexpr int kPairBytes = pair_bytes(G, kU4, kV4);
+  // a unit: key codes 1024, value codes 1024, value scales (and the values' high plane 1024)
+  constexpr uint32_t kUnitBytes = unit_bytes_of(G, kV4);
+  constexpr uint32_t kUnitStep = kUnitBytes + (UPG == 1 ? 512u : 0u);      // from a step's first unit to its second, staged
+  constexpr int kSlotBase = kStages * kStageBytes;             // offsets inside a pair's shared memory
+  constexpr int kPrepBase = kSlotBase + kSlotCount * kSlotBytes;
+  constexpr int kQBytes = (kU4 == 1 ? 2 : 1) * 8 * kQS * 2;
+  constexpr int kRBufBase = kPrepBase + kPrepBytes;
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, t = lane & 3;
   const int pair = warp >> 1;
@@ -265,9 +128,9 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   const uint32_t bar_u32 = tail_u32 + pair * (kBarsPerPair * 8);            // staged copy landed [kStages]
   const uint32_t lfull_u32 = bar_u32 + kStages * 8;                         // logits ready [kStages]
   const uint32_t rfull_u32 = bar_u32 + 2 * kStages * 8, rempty_u32 = rfull_u32 + 8;
-  const uint32_t qb16_u32 = tail_u32 + kBarBytes;                           // [8][kQS] q, bf16 bits (0 for heads >= g)
-  const uint32_t qf16_u32 = qb16_u32 + 8 * kQS * 2;                         // [8][kQS] q, fp16
-  float* mS = reinterpret_cast<float*>(smem + kPairs * kPairBytes + kBarBytes + 2 * 8 * kQS * 2);    // [kPairs][8]
+  const uint32_t qb16_u32 = tail_u32 + bar_bytes(kPairs);                           // [8][kQS] q, bf16 bits (0 for heads >= g)
+  const uint32_t qf16_u32 = qb16_u32 + 8 * kQS * 2;                         // [8][kQS] q, fp16 (three tiers)
+  float* mS = reinterpret_cast<float*>(smem + kPairs * kPairBytes + bar_bytes(kPairs) + kQBytes);    // [kPairs][8]
   float* lS = mS + kPairs * 8;                                                                       // [kPairs][8]
   int* prefS = reinterpret_cast<int*>(lS + kPairs * 8);                     // ragged batch: seq_prefix[0 .. B]
 
@@ -276,18 +139,12 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (!logits_role) {
-    // constant rows of the zero-point / denominator tile: row 4 is all ones, the other rows >= VG stay zero
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const int idx = lane + 32 * i, rem = idx % 144, row = rem >> 4;      // [2 ks: 144 words][8 rows][4 t][4]
-      if (idx < 272) sts32(ring_u32 + kPrepBase + kZvpOff + 4 * idx, (row == 4 && (idx & 1) == 0) ? 0x3C003C00u : 0u);
-    }
+    // constant rows of the zero-point / denominator tiles ([2 units][2 ks: 68 words][8 rows][4 t]{k 2t.., k 8 + 2t..}):
+    // row 4 is all ones, the other rows >= VG stay zero
+    for (int i = lane; i < 2 * kZvpUnit / 4; i += 32)
+      sts32(ring_u32 + kPrepBase + kZvpOff + 4 * i, ((i % 68) >> 3) == 4 ? 0x3C003C00u : 0u);
   }
   __syncthreads();
-
-  // codes of 32 tokens: keys 1024, values 1024, value scales (and the values' high plane 1024)
-  constexpr uint32_t kUnitBytes = 2048u + 128u * (kD / G) + (kV4 ? 1024u : 0u);
-  constexpr int UPG = G / 32;                                 // units per key group
 
   const int S = lv.B * lv.Hkv, U = lv.U, g = lv.g;
   // Fill of the stream at hand: the same for every stream, or (ragged batch) taken per sequence from the table in
@@ -321,18 +178,19 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   const long long total = lv.seq != nullptr ? (long long)prefS[lv.B] : (long long)Us * S;
   const long long cb = split_begin(total, gridDim.x, blockIdx.x), ce = split_begin(total, gridDim.x, blockIdx.x + 1);
 
-  uint32_t ring_stage = 0;        // ring stage of the next packed unit this pair consumes
+  uint32_t ring_stage = 0;        // ring stage of the next step this pair consumes
   uint32_t ring_parity = 0;       // phase parity of that stage's barriers
   uint32_t rit = 0;               // unquantized units handed over by this pair so far (both warps count them alike)
   bool gave_up = false;
   // A wait that runs out sets gave_up; the warp carries on with whatever the shared memory holds (every address it
   // forms stays inside the CTA's shared memory and the stream's arrays), its later waits are skipped, and the pair's
-  // result is replaced by zeros at the end.  Straight-line code: no exit in the middle of a unit.
+  // result is replaced by zeros at the end.  Straight-line code: no exit in the middle of a step.
   auto wait_or_give_up = [&](uint32_t bar, uint32_t parity) {
     if (!gave_up && !mbar_wait_polls(bar, parity, lv.wait_polls ? lv.wait_polls : kWaitPolls)) gave_up = true;
   };
+  auto next_stage = [&](uint32_t sg) { return sg + 1u == (uint32_t)kStages ? 0u : sg + 1u; };
   auto advance_stage = [&]() {
-    ring_stage = (ring_stage + 1u) & (kStages - 1);
+    ring_stage = next_stage(ring_stage);
     ring_parity ^= (ring_stage == 0u) ? 1u : 0u;
   };
 
@@ -359,93 +217,125 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     }
     seg += ue - ub;
     // ---- this pair's share of the segment.  The unquantized units of the segment go to different pairs (unit i to
-    // pair kPairs - 1 - i % kPairs); the packed units are split in order so that every pair carries about the same weight.
-    const int pk_b = min(ub, packed_units), pk_e = min(ue, packed_units);
+    // pair kPairs - 1 - i % kPairs); the packed units are split in order, in steps of two, so that every pair carries about
+    // the same weight.  (A stream's packed units are even in number; a boundary at an odd one moves up, on both sides.)
+    const int pk_b = (min(ub, packed_units) + 1) & ~1, pk_e = (min(ue, packed_units) + 1) & ~1;
     const int res_b = (max(ub, packed_units) - packed_units + kResidualWeight - 1) / kResidualWeight;
     const int res_e = ue > packed_units ? (ue - packed_units + kResidualWeight - 1) / kResidualWeight : res_b;
     const int n_res = res_e - res_b;
     int wb = pk_b, we = pk_b;
     {
-      const int weight = (pk_e - pk_b) + kResidualWeight * n_res;
-      int remaining = pk_e - pk_b;
+      const int n_packed = pk_e - pk_b, weight = n_packed + kResidualWeight * n_res;
+      int given = 0, res_given = 0;              // packed and unquantized units of the pairs before
 #pragma unroll
       for (int w = 0; w < kPairs; ++w) {
-        const int share = weight * (w + 1) / kPairs - weight * w / kPairs;       // weight < 2^24: 32-bit arithmetic
-        const int first_i = kPairs - 1 - w;                                   // unquantized units first_i, first_i + kPairs, ...
-        const int res_w = n_res > first_i ? (n_res - first_i + kPairs - 1) / kPairs : 0;
-        int p = min(remaining, max(0, share - kResidualWeight * res_w));
-        if (w == kPairs - 1) p = remaining;
+        const int first_i = kPairs - 1 - w;      // unquantized units first_i, first_i + kPairs, ...
+        res_given += n_res > first_i ? (n_res - first_i + kPairs - 1) / kPairs : 0;
+        // everything up to this pair against its exact share (weight < 2^24: 32-bit arithmetic)
+        const int upto = w == kPairs - 1
+                             ? n_packed
+                             : min(n_packed, max(given, (weight * (w + 1) / kPairs - kResidualWeight * res_given + 1) & ~1));
         if (w == pair) {
-          wb = pk_e - remaining;
-          we = wb + p;
+          wb = pk_b + given;
+          we = pk_b + upto;
         }
-        remaining -= p;
+        given = upto;
       }
     }
-    const int n_pack = we - wb;
+    const int n_steps = (we - wb) >> 1;
 
     // ---- the first copies of this segment go out before anything else (values warp): they do not depend on the query.
     // The packed units of a stream are one uniform sequence (a group's scales, then its units), whatever the block size,
-    // so the copy source only ever moves forward: `isrc` is the next unit to stage, `ig` its index inside its key group.
+    // so the copy source only ever moves forward: `isrc` is the next step to stage.
     int issued = 0;
-    const char* isrc = lv.base + (size_t)s * lv.base_stride + (size_t)wb * kUnitBytes + 512u * (size_t)(wb / UPG + 1);
-    int ig = wb & (UPG - 1);
-    // stages the next unit (if there is one left) in ring stage sg; all lanes keep the position
+    const char* isrc = lv.base + (size_t)s * lv.base_stride + (size_t)wb * kUnitBytes + 512u * (size_t)((wb + UPG - 1) / UPG);
+    uint32_t ihalf = UPG == 4 ? (uint32_t)(wb >> 1) & 1u : 0u;      // G = 128: the step is its group's second half
+    // stages the next step (if there is one left) in ring stage sg; all lanes keep the position
     auto issue = [&](uint32_t sg, bool first) {
       const uint32_t dst = ring_u32 + sg * kStageBytes, bar = bar_u32 + sg * 8u;
-      const uint32_t enabled = issued < n_pack ? 1u : 0u;
-      if (UPG == 1) {
-        // the group's scales lie directly before the unit: one copy
-        stage_copy(dst + kKeyMetaOff, isrc - 512, 512u + kUnitBytes, bar, first ? lv.debug_extra_tx : 0u, enabled);
-        isrc += kUnitBytes + 512;
+      const uint32_t enabled = issued < n_steps ? 1u : 0u;
+      if (UPG != 4 || ihalf == 0u) {
+        stage_copy(dst, isrc, (uint32_t)kStageBytes, bar, first ? lv.debug_extra_tx : 0u, enabled);
+        isrc += kStageBytes;
       } else {
+        // the group's scales lie before its first half: they are in the tables already, unless this is the first step
         if (enabled) {
-          if (ig == 0) stage_copy(dst + kKeyMetaOff, isrc - 512, 512u + kUnitBytes, bar, first ? lv.debug_extra_tx : 0u, 1u);
-          else if (first)
-            stage_copy2(dst + kUnitOff, isrc, kUnitBytes, dst + kKeyMetaOff, isrc - (size_t)ig * kUnitBytes - 512, 512u, bar,
-                        lv.debug_extra_tx);
-          else stage_copy(dst + kUnitOff, isrc, kUnitBytes, bar, 0u, 1u);
+          if (first) stage_copy2(dst + 512, isrc, 2 * kUnitBytes, dst, isrc - 2 * kUnitBytes - 512, 512u, bar, lv.debug_extra_tx);
+          else stage_copy(dst + 512, isrc, 2 * kUnitBytes, bar, 0u, 1u);
         }
-        isrc += kUnitBytes;
-        ig = (ig + 1) & (UPG - 1);
-        if (ig == 0) isrc += 512;
+        isrc += 2 * kUnitBytes;
       }
+      if (UPG == 4) ihalf ^= 1u;
       issued += (int)enabled;
     };
     const uint32_t stage0 = ring_stage, parity0 = ring_parity;
-    // the logits warp's first block: its table entry and the head of its extras (the lists of promoted channels) are a
-    // chain of two dependent loads; they go out here, with the first copies
+    // The extras of a step are copied kSlotCount - 1 steps ahead (logits warp).  The copies' cursor: block cbi and unit cu in
+    // it, the block's table entry and the next one's, requested a block ahead.
     const char* extras = lv.extras + (size_t)s * lv.extras_stride;
     const uint2* table = reinterpret_cast<const uint2*>(lv.table + (size_t)s * lv.table_stride);
-    uint2 pf_entry = make_uint2(0u, 0u), pf_entry_next = make_uint2(0u, 0u);
-    uint4 pf_head = make_uint4(~0u, ~0u, ~0u, ~0u);
-    uint32_t pf_ids[4] = {0xFFFFu, 0xFFFFu, 0xFFFFu, 0xFFFFu};   // three tiers: the lane's four pairs of UINT4 channel numbers
-    // the channel lists of the block with table entry e: the head of its extras and (three tiers) the UINT4 channel
-    // numbers of the lane's pairs t, t + 4, t + 8, t + 12
-    auto request_lists = [&](const uint2& e) {
-      if (e.y & 0xFFFFu) {
-        const char* ex = extras + (size_t)e.x * 16;
-        pf_head = *reinterpret_cast<const uint4*>(ex);
+    const uint32_t slot0_u32 = ring_u32 + kSlotBase;
+    int cbi = 0, cu = 0, requested = 0;
+    uint2 c_entry = make_uint2(0u, 0u), c_next = make_uint2(0u, 0u);
+    // requests the next step's extras (nothing past the last step); returns its block's counts: pairs of promoted channels,
+    // UINT4 channels << 8, and bit 16 in a step that begins a block (or is the first one)
+    auto request_extras = [&](uint32_t slot) -> uint32_t {
+      uint32_t counts = 0u;
+      if (requested < n_steps) {
+        const int n16 = c_entry.y & 0xFF, n4 = (c_entry.y >> 8) & 0xFF, n16p = (n16 + 1) >> 1;
+        const bool begins = requested == 0 || cu == 0;
+        counts = (uint32_t)n16p | ((uint32_t)n4 << 8) | (begins ? 0x10000u : 0u);
+        const uint32_t hdr = extras_header_bytes(n16, n4), unit = extras_unit_bytes(n16, n4, kU4 == 2);
+        const char* ex = extras + (size_t)c_entry.x * 16;
+        const char* exu = ex + hdr + (size_t)cu * unit;
+        const uint32_t dst = slot0_u32 + slot * kSlotBytes;
+        if (begins && 16u * lane < min(hdr, 64u)) cp_async16(dst + 16 * lane, ex + 16 * lane);
+        // rows: lane = (pair, 16-byte piece); the pieces of a row are swizzled by the pair so that the tile's reads fall on
+        // different banks
+        if ((lane >> 3) < n16p) {
+          const uint32_t rd = dst + kRowsOff + (lane >> 3) * 128 + (((lane & 7) ^ (2 * (lane >> 3))) << 4);
+          cp_async16(rd, exu + 16 * lane);
+          cp_async16(rd + kRowPairs * 128, exu + unit + 16 * lane);
+        }
         if constexpr (kU4 == 1) {
-          const int n16p = ((e.y & 0xFF) + 1) >> 1, n4pairs = (((e.y >> 8) & 0xFF) + 1) >> 1;
+          if ((lane & 15) < (n4 + 1) >> 1) cp_async16(dst + kPlaneOff + 16 * lane, exu + (lane >> 4) * unit + 128 * n16p + 16 * (lane & 15));
+        }
+        if constexpr (kU4 == 2) {
+          if (n16 + n4 > 0) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int p = 4 * i + (lane & 3);
-            pf_ids[i] = p < n4pairs ? (uint32_t)*reinterpret_cast<const uint16_t*>(ex + 2 * n16p + 2 * p) : 0xFFFFu;
+            for (int k = 0; k < 4; ++k)
+              cp_async16(dst + kPlaneOff + 512 * k + 16 * lane, exu + (k >> 1) * unit + 128 * n16p + 512 * (k & 1) + 16 * lane);
           }
         }
+        ++requested;
+        cu += 2;
+        if (cu == U) {
+          cu = 0;
+          ++cbi;
+          c_entry = c_next;
+          if (cbi + 1 < f_nb) c_next = table[cbi + 1];
+        }
       }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      return counts;
+    };
+    uint32_t counts[kSlotCount];              // of the current step and those ahead
+#pragma unroll
+    for (int i = 0; i < kSlotCount; ++i) counts[i] = 0u;
+    auto request_first = [&]() {
+      cbi = wb / U;
+      cu = wb - cbi * U;
+      c_entry = table[cbi];
+      if (cbi + 1 < f_nb) c_next = table[cbi + 1];
+#pragma unroll
+      for (int i = 0; i < kSlotCount - 1; ++i) counts[i] = request_extras(i);
     };
     if (!logits_role) {
 #pragma unroll 1
-      for (int i = 0; i < kStages; ++i) issue((ring_stage + i) & (kStages - 1), i == 0);
+      for (uint32_t i = 0, sg = ring_stage; i < (uint32_t)kStages; ++i, sg = next_stage(sg)) issue(sg, i == 0);
     }
-    if (n_pack > 0 && lv.stage_early && (logits_role || promoted_in_values(kU4))) {
-      pf_entry = table[wb / U];
-      if (wb / U + 1 < f_nb) pf_entry_next = table[wb / U + 1];
-      if (logits_role ? kU4 != 2 : promoted_in_values(kU4)) request_lists(pf_entry);     // whoever needs the lists
-    }
+    if (logits_role && n_steps > 0 && lv.stage_early) request_first();
     dep_wait();
+    if (logits_role && n_steps > 0 && !lv.stage_early) request_first();
 
     // ---- query of this stream: bf16 and fp16 tables (heads >= g are zero rows)
     {
@@ -468,11 +358,12 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     // takes its rows from the step's tensors, stores them and updates the importance accumulator
     const int jn = f_r - 1;
 
+    const uint32_t qrow_u32 = qb16_u32 + r * (kQS * 2), qfrow_u32 = qf16_u32 + r * (kQS * 2);
+
     if (logits_role) {
       // =====================================================================================================
       // logits warp
       // =====================================================================================================
-      const uint32_t qrow_u32 = qb16_u32 + r * (kQS * 2), qfrow_u32 = qf16_u32 + r * (kQS * 2);
       // ---- unquantized units: bf16 keys straight from global memory.  The channel a k-slot stands for is free as long as
       // both operands agree: lane column t of k-tile 2j (2j+1) takes channels 32j + 8t + 0..3 (4..7), so that a lane's
       // four k-tiles' worth of a token row is one 16-byte load.
@@ -531,16 +422,6 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       }
 
       // ---- packed units
-      int bi = 0, u = 0;                     // block and unit inside it of the next unit to consume
-      if (n_pack > 0) {
-        bi = wb / U;
-        u = wb - bi * U;
-        if (!lv.stage_early) {
-          pf_entry = table[bi];
-          if (bi + 1 < f_nb) pf_entry_next = table[bi + 1];
-          if constexpr (kU4 != 2) request_lists(pf_entry);
-        }
-      }
       // B fragments of q for the base key tiles: head r, channels 16kt + {2t, 2t+1} and {2t+8, 2t+9}, times mult(kt)
       uint32_t bq[8][2];
 #pragma unroll
@@ -554,232 +435,139 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       }
       // per-lane constants of the key-group preparation: the lane converts channels 4*lane .. 4*lane+3 (k-tile lane / 4)
       const float pk_zs = __uint_as_float((119u + (uint32_t)key_pos(lane >> 2)) << 23);        // 2^(pos - 8)
-      // zero-point tiles: [8 kt][4 t]{z ch0, z ch0, z ch1, z ch1} half2 z / mult; the lane's first pair
-      const uint32_t zp_wr = ring_u32 + kPrepBase + kZprepOff + 4 * (zprep_word(lane >> 2) + 8 * (lane & 1) + ((lane & 3) >> 1) * 2);
       const uint32_t kp_wr = ring_u32 + kPrepBase + kKprepOff + kprep_off(lane >> 2, 2 * (lane & 1)) + 8 * ((lane >> 1) & 1);
+      const uint32_t zp_wr = kp_wr + (kZprepOff - kKprepOff);
       const uint32_t kp_rd = ring_u32 + kPrepBase + kKprepOff + 16 * t;
       const uint32_t zp_rd = ring_u32 + kPrepBase + kZprepOff + 16 * t;
-      const uint32_t lane16 = ring_u32 + lane * 16, lane32 = ring_u32 + kLBufBase + lane * 32;
-      const uint32_t lane8 = ring_u32 + kLBufBase + kLBufZeroOff + lane * 8;
+      const uint32_t lane16 = ring_u32 + lane * 16;
       // byte offset inside the scale table of channel c's scale (half)
       auto scale_byte = [&](uint32_t c) -> uint32_t {
         const int kt = c >> 4, col = c & 15;
         return c < 128 ? (uint32_t)(kprep_off(kt, (col & 7) >> 1) + 8 * (col >> 3) + 2 * (col & 1)) : 0xFFFFu;
       };
-      float zc[4] = {0.f, 0.f, 0.f, 0.f};   // zero-point term q . z of the current key group (every row the same)
-
-      int done = 0;
-      while (done < n_pack) {
-        // ---- a block: its table entry, its promoted channels' query entries
-        const uint2 entry = pf_entry;
-        const uint4 head = pf_head;              // the first 16 bytes of the block's extras: up to 8 pairs of promoted channels
-        const uint32_t ids[4] = {pf_ids[0], pf_ids[1], pf_ids[2], pf_ids[3]};
-        // Everything a block needs from global memory before its first unit was requested a whole block earlier: here
-        // go out the lists of block bi + 1 (its table entry arrived during the block before) and the entry of bi + 2.
-        pf_entry = pf_entry_next;
-        if constexpr (kU4 != 2) {          // the UINT4 channel numbers (three tiers) or the promoted channels' (two tiers)
-          if (bi + 1 < f_nb) request_lists(pf_entry);
-        }
-        if (bi + 2 < f_nb) pf_entry_next = table[bi + 2];
-        const int n16 = entry.y & 0xFF, n4 = (entry.y >> 8) & 0xFF, n16p = (n16 + 1) >> 1;
-        const char* ex = extras + (size_t)entry.x * 16;                       // the block's extras
-        const uint32_t ex_unit = extras_unit_bytes(n16, n4, kU4 == 2);
-        const char* exu = ex + extras_header_bytes(n16, n4) + (size_t)u * ex_unit;   // ... of the current unit
-        const int nu = min(U - u, n_pack - done);                                 // units of this block for this warp
-        // B fragments of the block's first 16 promoted channels (gathered query entries; 0 past the block's count)
-        uint32_t xb0 = 0u, xb1 = 0u;
-        // A fragments of the first 16 promoted channels of a unit: lane (r, t) holds channel pairs t and t + 4 for tokens
-        // r, r + 8 of both m-tiles.  Pairs past the block's count read an existing pair instead (their query entries are 0).
-        uint32_t xa[2][4] = {{0u, 0u, 0u, 0u}, {0u, 0u, 0u, 0u}};
-        const int xa_lo = (min(t, n16p - 1) * 32 + r) * 4, xa_hi = (min(t + 4, n16p - 1) * 32 + r) * 4;
-        auto load_xa = [&](const char* e) {
-#pragma unroll
-          for (int mt = 0; mt < 2; ++mt) {
-            xa[mt][0] = *reinterpret_cast<const uint32_t*>(e + xa_lo + mt * 64);
-            xa[mt][1] = *reinterpret_cast<const uint32_t*>(e + xa_lo + mt * 64 + 32);
-            xa[mt][2] = *reinterpret_cast<const uint32_t*>(e + xa_hi + mt * 64);
-            xa[mt][3] = *reinterpret_cast<const uint32_t*>(e + xa_hi + mt * 64 + 32);
-          }
-        };
-        if (!promoted_in_values(kU4) && n16 > 0) {
-          load_xa(exu);
-          auto gather_q = [&](int p, uint32_t word) -> uint32_t {       // pair p < 8: its two channel numbers are in `word`
-            if (p >= n16p) return 0u;
-            const uint32_t ids = word >> (16 * (p & 1));
-            const uint32_t c0 = ids & 0xFF, c1 = (ids >> 8) & 0xFF;
-            const uint32_t lo = (c0 < 128) ? lds16(qrow_u32 + 2 * c0) : 0u, hi = (c1 < 128) ? lds16(qrow_u32 + 2 * c1) : 0u;
-            return lo | (hi << 16);
-          };
-          xb0 = gather_q(t, (t & 2) ? head.y : head.x);
-          xb1 = gather_q(t + 4, (t & 2) ? head.w : head.z);
-        }
-        // the block's first 32 UINT4 channels (two tiles of eight pairs): B fragments (gathered fp16 query pairs) and, per
-        // pair, where the two channels' scales sit in the scale table (byte offset of the half, 0xFFFF: no channel)
-        uint32_t u4q[2][2] = {{0u, 0u}, {0u, 0u}}, u4s[2][2] = {{~0u, ~0u}, {~0u, ~0u}};
-        if (kU4 == 1 && n4 > 0) {
-#pragma unroll
-          for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-            for (int hp = 0; hp < 2; ++hp) {
-              // pair 8 kk + 4 hp + t: its channel numbers were requested a block ahead (0xFF: no channel)
-              const uint32_t c0 = ids[2 * kk + hp] & 0xFFu, c1 = ids[2 * kk + hp] >> 8;
-              const uint32_t q0 = c0 < 128 ? lds16(qfrow_u32 + 2 * c0) : 0u;
-              const uint32_t q1 = c1 < 128 ? lds16(qfrow_u32 + 2 * c1) : 0u;
-              u4q[kk][hp] = q0 | (q1 << 16);
-              u4s[kk][hp] = scale_byte(c0) | (scale_byte(c1) << 16);
-            }
-        }
-
-        // The UINT4 high-plane words of a unit's first two tiles (three tiers) are requested one unit ahead inside a block.
-        uint32_t u4n[2][2] = {{0u, 0u}, {0u, 0u}};
-        auto request_plane = [&](const char* e) {
-          if constexpr (kU4 == 1) {
-            if (n4 > 0) {
-              const int n4pairs = (n4 + 1) >> 1;
-              const uint32_t* hw = reinterpret_cast<const uint32_t*>(e + 128 * n16p);
-#pragma unroll
-              for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-                for (int hp = 0; hp < 2; ++hp) {
-                  const int pp = 8 * kk + 4 * hp + t;
-                  u4n[kk][hp] = pp < n4pairs ? hw[pp * 4 + (r & 3)] : 0u;
-                }
-            }
-          }
-        };
-        if constexpr (kU4 == 1) request_plane(exu);
-
+      float zc[4] = {0.f, 0.f, 0.f, 0.f};   // zero-point terms q . z: [0..1] of unit 0's key group, [2..3] of unit 1's
+      // B fragment of the block's first 2 kRowPairs promoted channels (gathered query entries; 0 past the count)
+      uint32_t xb = 0u;
+      // three tiers: the block's first 2 kPlanePairs UINT4 channels (two tiles of eight pairs): B fragments (gathered fp16
+      // query pairs) and, per pair, where the two channels' scales sit in the scale table (0xFFFF: no channel)
+      uint32_t u4q[2][2] = {{0u, 0u}, {0u, 0u}}, u4s[2][2] = {{~0u, ~0u}, {~0u, ~0u}};
+      // query entries of a pair of channel numbers (0xFF: no channel)
+      auto query_pair = [&](uint32_t row, uint32_t two) -> uint32_t {
+        const uint32_t c0 = two & 0xFFu, c1 = (two >> 8) & 0xFFu;
+        return (c0 < 128 ? lds16(row + 2 * c0) : 0u) | ((c1 < 128 ? lds16(row + 2 * c1) : 0u) << 16);
+      };
+      uint32_t slot = 0;                    // of the current step
 #pragma unroll 1
-        for (int iu = 0; iu < nu; ++iu) {
-          wait_or_give_up(bar_u32 + ring_stage * 8u, ring_parity);
-          const uint32_t stg = lane16 + ring_stage * kStageBytes;         // this lane's 16 bytes of the stage's first section
-          const bool has_meta = (UPG == 1) || (done + iu == 0) || (((u + iu) & (UPG - 1)) == 0);
-          // this unit's UINT4 high-plane words (requested a unit ago); the next unit's are requested right away
-          const uint32_t u4w[2][2] = {{u4n[0][0], u4n[0][1]}, {u4n[1][0], u4n[1][1]}};
-          if constexpr (kU4 == 1) {
-            if (iu + 1 < nu) request_plane(exu + ex_unit);
-          }
-          // the key codes: two 16-byte loads per lane are the A fragments of all sixteen key tiles (with a 4-bit base the
-          // first plane to run is the high plane, which lies with the block's extras in global memory)
-          uint4 hw0, hw1;
-          if constexpr (kU4 == 2) {
-            const uint4* kplane = reinterpret_cast<const uint4*>(exu + 128 * n16p);
-            hw0 = kplane[lane];
-            hw1 = kplane[32 + lane];
-          } else {
-            hw0 = lds128(stg + kUnitOff);
-            hw1 = lds128(stg + kUnitOff + 512);
-          }
-
-          // ---- key-group preparation: fp16 scale pairs {s, -4s} in fragment order, zero-point tile.  The tables of the
-          // previous group were last read by this warp alone.
-          if (has_meta) {
-            __syncwarp();
-            const uint4 mz = lds128(stg + kKeyMetaOff);   // channels 4*lane .. 4*lane+3
+      for (int i = 0; i < n_steps; ++i) {
+        wait_or_give_up(bar_u32 + ring_stage * 8u, ring_parity);
+        const uint32_t stg = lane16 + ring_stage * kStageBytes;         // this lane's 16 bytes of the stage's first section
+        // G = 128: the group's second half finds the tables as the first left them
+        const bool has_meta = UPG != 4 || i == 0 || (((wb >> 1) + i) & 1) == 0;
+        // the extras of a later step are requested into the slot that was read in the step before; this step's have arrived
+        const uint32_t later = request_extras(slot == 0 ? kSlotCount - 1 : slot - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSlotCount - 1) : "memory");
+        // the key codes: two 16-byte loads per lane and unit are the A fragments of all its sixteen key tiles
+        uint4 kw[2][2];
+#pragma unroll
+        for (int un = 0; un < 2; ++un) {
+          kw[un][0] = lds128(stg + 512 + un * kUnitStep);
+          kw[un][1] = lds128(stg + 512 + un * kUnitStep + 512);
+        }
+        // ---- key-group preparation: fp16 scale pairs {s, -4s} in fragment order, zero-point tile.  The tables of the
+        // previous step were last read by this warp alone.
+        if (has_meta) {
+          __syncwarp();
+          uint32_t za[2], zb[2];
+#pragma unroll
+          for (int gi = 0; gi < kGroups; ++gi) {
+            const uint4 mz = lds128(stg + gi * (512 + kUnitBytes));   // channels 4*lane .. 4*lane+3
             const uint32_t neg4 = 0xC400C400u;   // half2(-4, -4)
             const uint32_t ma = pack_half2(bf_lo(mz.x), bf_lo(mz.y)), mb = pack_half2(bf_lo(mz.z), bf_lo(mz.w));
-            sts64(kp_wr, ma, hmul2_u(ma, neg4));
-            sts64(kp_wr + 16, mb, hmul2_u(mb, neg4));
-            const uint32_t za = pack_half2(bf_hi(mz.x) * pk_zs, bf_hi(mz.y) * pk_zs);
-            const uint32_t zb = pack_half2(bf_hi(mz.z) * pk_zs, bf_hi(mz.w) * pk_zs);
-            sts64(zp_wr, za, za);
-            sts64(zp_wr + 16, zb, zb);
-            __syncwarp();      // the tables written above are read by other lanes below
-            // the zero-point term q . z of the group: a tile chain of its own (the tile's rows are equal, so are the rows
-            // of the result), independent of the key tiles below; the partner adds it to the logits
-#pragma unroll
-            for (int kt2 = 0; kt2 < 8; ++kt2) {
-              const uint4 zz = lds128(zp_rd + 4 * zprep_word(kt2));
-              if (kt2 == 0) mma_f16_to(zc, zz.x, zz.y, zz.z, zz.w, bq[0][0], bq[0][1], 0.f, 0.f, 0.f, 0.f);
-              else mma_f16(zc, zz.x, zz.y, zz.z, zz.w, bq[kt2][0], bq[kt2][1]);
-            }
+            sts64(kp_wr + kKprepGroup * gi, ma, hmul2_u(ma, neg4));
+            sts64(kp_wr + kKprepGroup * gi + 16, mb, hmul2_u(mb, neg4));
+            za[gi] = pack_half2(bf_hi(mz.x) * pk_zs, bf_hi(mz.y) * pk_zs);
+            zb[gi] = pack_half2(bf_hi(mz.z) * pk_zs, bf_hi(mz.w) * pk_zs);
           }
+          sts64(zp_wr, za[0], za[kGroups - 1]);
+          sts64(zp_wr + 16, zb[0], zb[kGroups - 1]);
+        }
+        __syncwarp();      // tables and extras are read by other lanes below, and the key codes' place is written at the end
 
-          // ---- q.K^T on the key tiles.  One pass over a plane of 2-bit codes: the base (low) plane with the scales s, and,
-          // with a 4-bit base, first the dense high plane (codes c >> 2, laid out like the low plane) with the scales 4s.
-          float Sx[2][4];
-          auto key_pass = [&](const uint4& w0, const uint4& w1, bool first, bool high) {
-            const uint32_t kw[2][4] = {{w0.x, w0.y, w0.z, w0.w}, {w1.x, w1.y, w1.z, w1.w}};
+        float Sx[2][2][4];
 #pragma unroll
-            for (int kt = 0; kt < 8; ++kt) {
-              // scales of the lane's channel pairs (16kt + 2t, +1) and (16kt + 8 + 2t, +1); code bias 4 -> offset -4 s
-              uint4 kp = lds128(kp_rd + kprep_off(kt, 0));
-              if (high) kp = make_uint4(hmul2_u(kp.x, four2), hmul2_u(kp.y, four2), hmul2_u(kp.z, four2), hmul2_u(kp.w, four2));
-              const uint32_t mask = 0x00030003u << key_pos(kt);
+        for (int un = 0; un < 2; ++un)
 #pragma unroll
-              for (int mt = 0; mt < 2; ++mt) {
-                uint32_t a[4];
+          for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  const uint32_t code = (key_shift(kw[mt][j], kt) & mask) | four2;           // 4 + c * 2^(pos-8)
-                  a[j] = hfma2_u(code, j < 2 ? kp.x : kp.z, j < 2 ? kp.y : kp.w);            // c * s * 2^(pos-8)
-                }
-                if (first && kt == 0) mma_f16_to(Sx[mt], a[0], a[1], a[2], a[3], bq[0][0], bq[0][1], 0.f, 0.f, 0.f, 0.f);
-                else mma_f16(Sx[mt], a[0], a[1], a[2], a[3], bq[kt][0], bq[kt][1]);
+            for (int k = 0; k < 4; ++k) Sx[un][mt][k] = 0.f;
+        const uint32_t slot_u32 = slot0_u32 + slot * kSlotBytes;
+        const int n16p = counts[0] & 0xFF, n4pairs = (((counts[0] >> 8) & 0xFF) + 1) >> 1;
+        if (counts[0] & 0x10000u) {
+          // a block begins: its channel lists
+          xb = t < n16p ? query_pair(qrow_u32, lds16(slot_u32 + 2 * t)) : 0u;
+          if constexpr (kU4 == 1) {
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+              for (int hp = 0; hp < 2; ++hp) {
+                const int p = 8 * kk + 4 * hp + t;
+                const uint32_t two = p < n4pairs && n16p <= kRowPairs ? lds16(slot_u32 + 2 * n16p + 2 * p) : 0xFFFFu;
+                u4q[kk][hp] = query_pair(qfrow_u32, two);
+                u4s[kk][hp] = scale_byte(two & 0xFFu) | (scale_byte(two >> 8) << 16);
               }
-            }
-          };
-          if constexpr (kU4 == 2) {
-            key_pass(hw0, hw1, true, true);
-            const uint4 kw0 = lds128(stg + kUnitOff);
-            const uint4 kw1 = lds128(stg + kUnitOff + 512);
-            key_pass(kw0, kw1, false, false);
-          } else {
-            key_pass(hw0, hw1, true, false);
           }
-          // ---- promoted channels (raw bf16 keys) with a gathered q
-          if (!promoted_in_values(kU4) && n16 > 0) {
+        }
+        // where the step's extras lie in global memory, for what the slot does not hold
+        const bool spill16 = n16p > kRowPairs, spill4 = kU4 == 1 && (n4pairs > kPlanePairs || (n4pairs > 0 && spill16));
+        const char* ex = nullptr;
+        const char* exu = nullptr;
+        uint32_t ex_unit = 0u;
+        if (spill16 || spill4) {
+          const int bi = (wb + 2 * i) / U;
+          const uint2 e = table[bi];
+          const int n16 = e.y & 0xFF, n4 = (e.y >> 8) & 0xFF;
+          ex = extras + (size_t)e.x * 16;
+          ex_unit = extras_unit_bytes(n16, n4, kU4 == 2);
+          exu = ex + extras_header_bytes(n16, n4) + (size_t)(wb + 2 * i - bi * U) * ex_unit;
+        }
+        // ---- promoted channels: raw bf16 keys (A fragments with k = 8: lane (r, t) holds channel pair t for tokens r, r + 8 of
+        // both m-tiles), a gathered q.  Pairs past the count read the last pair (their query entries are 0).
+        if (n16p > 0) {
+          const uint32_t row = slot_u32 + kRowsOff + 128 * min(t, n16p - 1) + 4 * r, sw = 32 * min(t, n16p - 1);
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) mma_bf16(Sx[mt], xa[mt][0], xa[mt][1], xa[mt][2], xa[mt][3], xb0, xb1);
-            // the registers are free again: request the next unit's pairs now, most of an iteration ahead of their use
-            if (iu + 1 < nu) load_xa(exu + ex_unit);
-            for (int kk = 1; kk * 8 < n16p; ++kk) {       // more than 16 promoted channels
-              uint32_t a[2][4], id0 = 0xFFFFFFFFu, id1 = 0xFFFFFFFFu;
-              const uint32_t* xw = reinterpret_cast<const uint32_t*>(exu);
-              const int p0 = 8 * kk + t, p1 = p0 + 4;
+          for (int un = 0; un < 2; ++un)
 #pragma unroll
-              for (int mt = 0; mt < 2; ++mt) a[mt][0] = a[mt][1] = a[mt][2] = a[mt][3] = 0;
-              if (p0 < n16p) {
-                id0 = *reinterpret_cast<const uint16_t*>(ex + 2 * p0);
+            for (int mt = 0; mt < 2; ++mt)
+              mma_bf16_k8(Sx[un][mt], lds32(row + un * (kRowPairs * 128) + (sw ^ (64 * mt))), lds32(row + un * (kRowPairs * 128) + (sw ^ (64 * mt + 32))), xb);
+          if (spill16) {
+#pragma unroll 2
+            for (int p0 = kRowPairs; p0 < n16p; p0 += 4) {
+              const int p = min(p0 + t, n16p - 1);
+              const uint32_t b = p0 + t < n16p ? query_pair(qrow_u32, *reinterpret_cast<const uint16_t*>(ex + 2 * p)) : 0u;
+              const char* e = exu + (p * 32 + r) * 4;
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
-                  a[mt][0] = xw[p0 * 32 + mt * 16 + r];
-                  a[mt][1] = xw[p0 * 32 + mt * 16 + 8 + r];
-                }
-              }
-              if (p1 < n16p) {
-                id1 = *reinterpret_cast<const uint16_t*>(ex + 2 * p1);
+              for (int un = 0; un < 2; ++un)
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
-                  a[mt][2] = xw[p1 * 32 + mt * 16 + r];
-                  a[mt][3] = xw[p1 * 32 + mt * 16 + 8 + r];
-                }
-              }
-              auto gather_bf16 = [&](uint32_t ids) -> uint32_t {
-                const uint32_t c0 = ids & 0xFF, c1 = (ids >> 8) & 0xFF;
-                const uint32_t lo = (c0 < 128) ? lds16(qrow_u32 + 2 * c0) : 0u, hi = (c1 < 128) ? lds16(qrow_u32 + 2 * c1) : 0u;
-                return lo | (hi << 16);
-              };
-              const uint32_t b0 = gather_bf16(id0), b1 = gather_bf16(id1);
-#pragma unroll
-              for (int mt = 0; mt < 2; ++mt) mma_bf16(Sx[mt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
+                for (int mt = 0; mt < 2; ++mt)
+                  mma_bf16_k8(Sx[un][mt], *reinterpret_cast<const uint32_t*>(e + un * ex_unit + 64 * mt),
+                              *reinterpret_cast<const uint32_t*>(e + un * ex_unit + 64 * mt + 32), b);
             }
           }
-          // ---- UINT4 high plane: c_hi * 4s, gathered q in fp16.  The first two tiles (32 channels) use the block's gathered
-          // query pairs and scale positions; further tiles look their channels up per unit.
-          if (kU4 == 1 && n4 > 0) {
-            const int n4pairs = (n4 + 1) >> 1;
-            const uint32_t* hw = reinterpret_cast<const uint32_t*>(exu + 128 * n16p);
-            const unsigned char* ids4 = reinterpret_cast<const unsigned char*>(ex) + 2 * n16p;
+        }
+        // ---- UINT4 high plane (three tiers): c_hi * 4s, gathered q in fp16.  The first two tiles (32 channels) use the
+        // block's gathered query pairs and scale positions; further tiles look their channels up per step.
+        if constexpr (kU4 == 1) {
+          if (n4pairs > 0) {
             const uint32_t kpb = ring_u32 + kPrepBase + kKprepOff;
-            auto plane_tile = [&](const uint32_t (&words)[2], const uint32_t (&sidx)[2], const uint32_t (&qb)[2]) {
+            auto plane_tile = [&](int un, const uint32_t (&words)[2], const uint32_t (&sidx)[2], const uint32_t (&qb)[2]) {
               uint32_t a[2][4];
 #pragma unroll
               for (int hp = 0; hp < 2; ++hp) {
                 const uint32_t w = words[hp] >> (8 * (r >> 2));
                 const uint32_t i0 = sidx[hp] & 0xFFFFu, i1 = sidx[hp] >> 16;
-                const uint32_t s0 = i0 != 0xFFFFu ? lds16(kpb + i0) : 0u;
-                const uint32_t s1 = i1 != 0xFFFFu ? lds16(kpb + i1) : 0u;
+                const uint32_t tb = kpb + (UPG == 1 ? kKprepGroup * un : 0);
+                const uint32_t s0 = i0 != 0xFFFFu ? lds16(tb + i0) : 0u;
+                const uint32_t s1 = i1 != 0xFFFFu ? lds16(tb + i1) : 0u;
                 const uint32_t sc = s0 | (s1 << 16);
                 const uint32_t m4 = hmul2_u(sc, four2);                // 4s
                 const uint32_t o4 = hmul2_u(sc, 0xCC00CC00u);          // -16s
@@ -793,46 +581,111 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
                   }
               }
 #pragma unroll
-              for (int mt = 0; mt < 2; ++mt) mma_f16(Sx[mt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], qb[0], qb[1]);
+              for (int mt = 0; mt < 2; ++mt) mma_f16(Sx[un][mt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], qb[0], qb[1]);
             };
-            plane_tile(u4w[0], u4s[0], u4q[0]);
-            if (n4pairs > 8) plane_tile(u4w[1], u4s[1], u4q[1]);
-            for (int kk = 2; kk * 8 < n4pairs; ++kk) {
-              uint32_t sidx[2], qb[2], words[2] = {0u, 0u};
+            if (!spill16) {
+              const uint32_t pl = slot_u32 + kPlaneOff + 16 * t + 4 * (r & 3);
 #pragma unroll
-              for (int hp = 0; hp < 2; ++hp) {
-                const int p = 8 * kk + 4 * hp + t;
-                uint32_t c0 = 255u, c1 = 255u;
-                if (p < n4pairs) {
-                  c0 = ids4[2 * p];
-                  c1 = ids4[2 * p + 1];
-                  words[hp] = hw[p * 4 + (r & 3)];
+              for (int kk = 0; kk < 2; ++kk) {
+                if (kk * 8 < n4pairs) {
+#pragma unroll
+                  for (int un = 0; un < 2; ++un) {
+                    // (pairs past the count have zero scales and query entries)
+                    const uint32_t words[2] = {lds32(pl + un * (16 * kPlanePairs) + 128 * kk), lds32(pl + un * (16 * kPlanePairs) + 128 * kk + 64)};
+                    plane_tile(un, words, u4s[kk], u4q[kk]);
+                  }
                 }
-                const uint32_t q0 = c0 < 128 ? lds16(qfrow_u32 + 2 * c0) : 0u;
-                const uint32_t q1 = c1 < 128 ? lds16(qfrow_u32 + 2 * c1) : 0u;
-                qb[hp] = q0 | (q1 << 16);
-                sidx[hp] = scale_byte(c0) | (scale_byte(c1) << 16);
               }
-              plane_tile(words, sidx, qb);
+            }
+            if (spill4) {
+              for (int p0 = spill16 ? 0 : kPlanePairs; p0 < n4pairs; p0 += 8) {
+                uint32_t sidx[2], qb[2], words[2][2] = {{0u, 0u}, {0u, 0u}};
+#pragma unroll
+                for (int hp = 0; hp < 2; ++hp) {
+                  const int p = p0 + 4 * hp + t;
+                  uint32_t two = 0xFFFFu;
+                  if (p < n4pairs) {
+                    two = *reinterpret_cast<const uint16_t*>(ex + 2 * n16p + 2 * p);
+#pragma unroll
+                    for (int un = 0; un < 2; ++un)
+                      words[un][hp] = reinterpret_cast<const uint32_t*>(exu + un * ex_unit + 128 * n16p)[p * 4 + (r & 3)];
+                  }
+                  qb[hp] = query_pair(qfrow_u32, two);
+                  sidx[hp] = scale_byte(two & 0xFFu) | (scale_byte(two >> 8) << 16);
+                }
+#pragma unroll
+                for (int un = 0; un < 2; ++un) plane_tile(un, words[un], sidx, qb);
+              }
             }
           }
-
-          // ---- hand the logits over: [m-tile][tokens r / r + 8] x heads 2t, 2t+1.  The buffer of this stage is free: the
-          // partner took its last contents before it refilled the stage.
-          {
-            const uint32_t lb = lane32 + ring_stage * kLBufBytes;
-            sts128(lb, __float_as_uint(Sx[0][0]), __float_as_uint(Sx[0][1]), __float_as_uint(Sx[0][2]), __float_as_uint(Sx[0][3]));
-            sts128(lb + 16, __float_as_uint(Sx[1][0]), __float_as_uint(Sx[1][1]), __float_as_uint(Sx[1][2]), __float_as_uint(Sx[1][3]));
-            sts64(lane8 + ring_stage * kLBufBytes, __float_as_uint(zc[0]), __float_as_uint(zc[1]));
-            __syncwarp();
-            mbar_arrive_one(lfull_u32 + ring_stage * 8u);
-          }
-          advance_stage();
-          exu += ex_unit;
         }
-        done += nu;
-        u = 0;
-        ++bi;
+        // ---- q.K^T on the key tiles.  One pass over a plane of 2-bit codes: the base (low) plane with the scales s, and,
+        // with a 4-bit base, first the dense high plane (codes c >> 2, laid out like the low plane) with the scales 4s.
+        auto key_pass = [&](const uint4 (&w)[2][2], bool high) {
+#pragma unroll
+          for (int kt = 0; kt < 8; ++kt) {
+            // scales of the lane's channel pairs (16kt + 2t, +1) and (16kt + 8 + 2t, +1); code bias 4 -> offset -4 s
+            uint4 kp[2];
+#pragma unroll
+            for (int gi = 0; gi < kGroups; ++gi) {
+              kp[gi] = lds128(kp_rd + kKprepGroup * gi + kprep_off(kt, 0));
+              if (high) kp[gi] = make_uint4(hmul2_u(kp[gi].x, four2), hmul2_u(kp[gi].y, four2), hmul2_u(kp[gi].z, four2), hmul2_u(kp[gi].w, four2));
+            }
+            const uint32_t mask = 0x00030003u << key_pos(kt);
+#pragma unroll
+            for (int un = 0; un < 2; ++un) {
+              const uint4& k4 = kp[un & (kGroups - 1)];
+#pragma unroll
+              for (int mt = 0; mt < 2; ++mt) {
+                const uint32_t kwd[4] = {w[un][mt].x, w[un][mt].y, w[un][mt].z, w[un][mt].w};
+                uint32_t a[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                  const uint32_t code = (key_shift(kwd[j], kt) & mask) | four2;              // 4 + c * 2^(pos-8)
+                  a[j] = hfma2_u(code, j < 2 ? k4.x : k4.z, j < 2 ? k4.y : k4.w);            // c * s * 2^(pos-8)
+                }
+                mma_f16(Sx[un][mt], a[0], a[1], a[2], a[3], bq[kt][0], bq[kt][1]);
+              }
+            }
+          }
+        };
+        if constexpr (kU4 == 2) {
+          if (n16p + n4pairs > 0) {          // (a block whose extras did not fit the arena has no high plane)
+            const uint32_t pl = slot_u32 + kPlaneOff + 16 * lane;
+            const uint4 hw[2][2] = {{lds128(pl), lds128(pl + 512)}, {lds128(pl + 1024), lds128(pl + 1536)}};
+            key_pass(hw, true);
+          }
+        }
+        if (has_meta) {
+          // the zero-point terms q . z: a tile chain of its own; the partner adds them to the logits
+#pragma unroll
+          for (int kt = 0; kt < 8; ++kt) {
+            const uint4 zz = lds128(zp_rd + kprep_off(kt, 0));
+            if (kt == 0) mma_f16_to(zc, zz.x, zz.y, zz.z, zz.w, bq[0][0], bq[0][1], 0.f, 0.f, 0.f, 0.f);
+            else mma_f16(zc, zz.x, zz.y, zz.z, zz.w, bq[kt][0], bq[kt][1]);
+          }
+        }
+        key_pass(kw, false);
+
+        // ---- hand the logits over: [m-tile][tokens r / r + 8] x heads 2t, 2t+1, where the units' key codes were, and the
+        // zero-point terms where the first group's scales were (every lane has read both, see the barrier above)
+        {
+          const uint32_t lb = stg + 512 + lane * 16;
+#pragma unroll
+          for (int un = 0; un < 2; ++un)
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+              sts128(lb + un * kUnitStep + 16 * mt, __float_as_uint(Sx[un][mt][0]), __float_as_uint(Sx[un][mt][1]),
+                     __float_as_uint(Sx[un][mt][2]), __float_as_uint(Sx[un][mt][3]));
+          sts128(stg, __float_as_uint(zc[0]), __float_as_uint(zc[1]), __float_as_uint(zc[2]), __float_as_uint(zc[3]));
+          __syncwarp();
+          mbar_arrive_one(lfull_u32 + ring_stage * 8u);
+        }
+#pragma unroll
+        for (int k = 0; k + 2 < kSlotCount; ++k) counts[k] = counts[k + 1];
+        counts[kSlotCount - 2] = later;
+        slot = slot + 1 == kSlotCount ? 0u : slot + 1;
+        advance_stage();
       }
       if (gave_up && lane == 0) atomicOr(lv.status, (uint32_t)MIXKVQ_DEV_COPY_TIMEOUT);
     } else {
@@ -964,229 +817,154 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       }
 
       // ---- packed units
-      // per-lane constants of the value-group preparation: the lane converts the scales and zero-points of token `lane`
-      // value scales: [4 t: 20 words][4 vg][2 ks][2 ch] half2 s_v'; zero-point tile: [2 ks][8 rows][4 t]{ch0, 0, ch1, 0} half2
+      // per-lane constants of the value-group preparation: the lane converts the scales and zero-points of tokens 2 pi,
+      // 2 pi + 1 of a unit, VG / 2 groups of them (VG = 1: of unit lane / 16)
+      // value scales: [4 t: 20 words][4 vg][2 ks][2 ch] half2 s_v'; zero-point tile: [2 ks: 68 words][8 rows][4 t][2 ch] half2
       // (rows < VG z_v, row 4 ones)
-      const float pv_up = __uint_as_float((131u - 2u * (uint32_t)(lane >> 3)) << 23);          // 2^(4 - 2 * (2 ks + ch))
-      const uint32_t sv_wr = ring_u32 + kPrepBase + kSvpOff + 2 * (((((lane & 7) >> 1) * 20 + (lane >> 3)) * 2) + (lane & 1));
-      const uint32_t zv_wr = ring_u32 + kPrepBase + kZvpOff +
-                             2 * ((((lane >> 4) * 144 + ((lane & 7) >> 1) * 4 + 2 * ((lane >> 3) & 1)) * 2) + (lane & 1));
+      const int pi = VG == 1 ? lane & 15 : lane >> 1, vg0 = VG == 1 ? 0 : (lane & 1) * (VG / 2);
+      const int p_ks = pi >> 3, p_ch = (pi >> 2) & 1, p_t = pi & 3;
+      const float pv_up = __uint_as_float((131u - 2u * (uint32_t)(2 * p_ks + p_ch)) << 23);          // 2^(4 - 2 * (2 ks + ch))
+      const uint32_t sv_wr = ring_u32 + kPrepBase + kSvpOff + (VG == 1 ? (uint32_t)(lane >> 4) * kSvpUnit : 0u) +
+                             4 * (p_t * 20 + vg0 * 4 + p_ks * 2 + p_ch);
+      const uint32_t zv_wr = ring_u32 + kPrepBase + kZvpOff + (VG == 1 ? (uint32_t)(lane >> 4) * kZvpUnit : 0u) +
+                             4 * (p_ks * 68 + vg0 * 8 + p_t * 2 + p_ch);
       const uint32_t sv_rd = ring_u32 + kPrepBase + kSvpOff + t * 80;
-      const uint32_t lane16 = ring_u32 + lane * 16, lane32 = ring_u32 + kLBufBase + lane * 32;
-      const uint32_t lane8 = ring_u32 + kLBufBase + kLBufZeroOff + lane * 8;
-      const uint32_t vm_rd = ring_u32 + kUnitOff + 2048 + lane * (4 * VG);
-      // ---- three tiers, 4-bit base: the promoted channels' tile (raw bf16 keys from the blocks' extras, a gathered q) is added here
-      // to the logits the partner hands over.  Requested ahead like everything from global memory: table entries two
-      // blocks, channel lists one block, a unit's rows one unit.
-      const uint32_t qrow_v = qb16_u32 + r * (kQS * 2);
-      int vbi = 0, vcur = 0, vleft = 0;           // block, unit inside it, units of the block left for this warp
-      int n16 = 0, n16p = 0;
-      const char* ex = extras;                    // the block's extras, and those of the current unit
-      const char* exu = extras;
-      uint32_t ex_unit = 0;
-      uint32_t xb0 = 0u, xb1 = 0u, xa[2][4] = {{0u, 0u, 0u, 0u}, {0u, 0u, 0u, 0u}};     // as in the logits warp
-      auto load_xa = [&](const char* e) {
-        const int xa_lo = (min(t, n16p - 1) * 32 + r) * 4, xa_hi = (min(t + 4, n16p - 1) * 32 + r) * 4;
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          xa[mt][0] = *reinterpret_cast<const uint32_t*>(e + xa_lo + mt * 64);
-          xa[mt][1] = *reinterpret_cast<const uint32_t*>(e + xa_lo + mt * 64 + 32);
-          xa[mt][2] = *reinterpret_cast<const uint32_t*>(e + xa_hi + mt * 64);
-          xa[mt][3] = *reinterpret_cast<const uint32_t*>(e + xa_hi + mt * 64 + 32);
-        }
-      };
-      if constexpr (promoted_in_values(kU4)) {
-        if (n_pack > 0) {
-          vbi = wb / U;
-          vcur = wb - vbi * U;
-          if (!lv.stage_early) {
-            pf_entry = table[vbi];
-            if (vbi + 1 < f_nb) pf_entry_next = table[vbi + 1];
-            request_lists(pf_entry);
-          }
-        }
-      }
+      const uint32_t zv_rd = ring_u32 + kPrepBase + kZvpOff + lane * 8;
+      const uint32_t lane16 = ring_u32 + lane * 16;
+      const uint32_t vm_rd = ring_u32 + 512 + 2048 + (2 * pi) * (4 * VG) + 4 * vg0 + (VG == 1 ? (uint32_t)(lane >> 4) * kUnitStep : 0u);
 #pragma unroll 1
-      for (int done = 0; done < n_pack; ++done) {
-        if constexpr (promoted_in_values(kU4)) {
-          if (vleft == 0) {
-            // a block: its table entry and lists arrived a block ago; the next block's lists and the entry after that go out now
-            const uint2 entry = pf_entry;
-            const uint4 head = pf_head;          // the first 16 bytes of the block's extras: up to 8 pairs of promoted channels
-            pf_entry = pf_entry_next;
-            if (vbi + 1 < f_nb) request_lists(pf_entry);
-            if (vbi + 2 < f_nb) pf_entry_next = table[vbi + 2];
-            n16 = entry.y & 0xFF;
-            n16p = (n16 + 1) >> 1;
-            const int n4 = (entry.y >> 8) & 0xFF;
-            ex = extras + (size_t)entry.x * 16;
-            ex_unit = extras_unit_bytes(n16, n4, kU4 == 2);
-            exu = ex + extras_header_bytes(n16, n4) + (size_t)vcur * ex_unit;
-            vleft = min(U - vcur, n_pack - done);
-            xb0 = xb1 = 0u;
-            if (n16 > 0) {
-              load_xa(exu);
-              auto gather_q = [&](int p, uint32_t word) -> uint32_t {     // pair p < 8: its two channel numbers are in `word`
-                if (p >= n16p) return 0u;
-                const uint32_t cc = word >> (16 * (p & 1));
-                const uint32_t c0 = cc & 0xFF, c1 = (cc >> 8) & 0xFF;
-                const uint32_t lo = (c0 < 128) ? lds16(qrow_v + 2 * c0) : 0u, hi = (c1 < 128) ? lds16(qrow_v + 2 * c1) : 0u;
-                return lo | (hi << 16);
-              };
-              xb0 = gather_q(t, (t & 2) ? head.y : head.x);
-              xb1 = gather_q(t + 4, (t & 2) ? head.w : head.z);
-            }
-          }
-        }
+      for (int i = 0; i < n_steps; ++i) {
         wait_or_give_up(bar_u32 + ring_stage * 8u, ring_parity);
-        const uint32_t st = lane16 + ring_stage * kStageBytes + kUnitOff;      // this lane's 16 bytes of the unit's first section
-        // ---- value-group preparation (lane = token).  The tables of the previous unit were last read before the
-        // warp barrier that closed it.
+        const uint32_t st = lane16 + ring_stage * kStageBytes + 512;      // this lane's 16 bytes of the first unit's first section
+        // ---- value-group preparation.  The tables of the previous step were last read before the warp barrier that closed
+        // it.
         {
-          uint32_t mzv[4] = {0u, 0u, 0u, 0u};
           const uint32_t vm = vm_rd + ring_stage * kStageBytes;
+          auto convert = [&](uint32_t m0, uint32_t m1, int un, int k) {          // {s, z} of the pair's two tokens, group vg0 + k
+            sts32(sv_wr + un * kSvpUnit + 16 * k, pack_half2(bf_lo(m0) * pv_up, bf_lo(m1) * pv_up));
+            sts32(zv_wr + un * kZvpUnit + 32 * k, pack_half2(bf_hi(m0), bf_hi(m1)));
+          };
           if constexpr (VG == 4) {
-            const uint4 m = lds128(vm);
-            mzv[0] = m.x; mzv[1] = m.y; mzv[2] = m.z; mzv[3] = m.w;
-          } else if constexpr (VG == 2) {
-            const uint2 m = lds64(vm);
-            mzv[0] = m.x; mzv[1] = m.y;
-          } else {
-            mzv[0] = lds32(vm);
-          }
 #pragma unroll
-          for (int vg = 0; vg < VG; ++vg) {
-            sts16(sv_wr + 16 * vg, __half_as_ushort(__float2half_rn(bf_lo(mzv[vg]) * pv_up)));
-            sts16(zv_wr + 64 * vg, __half_as_ushort(__float2half_rn(bf_hi(mzv[vg]))));
+            for (int un = 0; un < 2; ++un) {
+              const uint2 a = lds64(vm + un * kUnitStep), b = lds64(vm + un * kUnitStep + 16);
+              convert(a.x, b.x, un, 0);
+              convert(a.y, b.y, un, 1);
+            }
+          } else if constexpr (VG == 2) {
+#pragma unroll
+            for (int un = 0; un < 2; ++un) convert(lds32(vm + un * kUnitStep), lds32(vm + un * kUnitStep + 8), un, 0);
+          } else {
+            const uint2 a = lds64(vm);
+            convert(a.x, a.y, 0, 0);
           }
         }
-        const uint4 vw0 = lds128(st + 1024);
-        const uint4 vw1 = lds128(st + 1536);
+        uint4 vw[2][2];
+#pragma unroll
+        for (int un = 0; un < 2; ++un) {
+          vw[un][0] = lds128(st + un * kUnitStep + 1024);
+          vw[un][1] = lds128(st + un * kUnitStep + 1536);
+        }
         __syncwarp();      // the tables written above are read by other lanes below
         wait_or_give_up(lfull_u32 + ring_stage * 8u, ring_parity);
-        const uint32_t lb = lane32 + ring_stage * kLBufBytes;
-        const uint4 s0 = lds128(lb), s1 = lds128(lb + 16);
-        const uint2 zq = lds64(lane8 + ring_stage * kLBufBytes);
-        float sx[2][4] = {{__uint_as_float(s0.x), __uint_as_float(s0.y), __uint_as_float(s0.z), __uint_as_float(s0.w)},
-                          {__uint_as_float(s1.x), __uint_as_float(s1.y), __uint_as_float(s1.z), __uint_as_float(s1.w)}};
-        if constexpr (promoted_in_values(kU4)) {
-          // ---- promoted channels (raw bf16 keys) with a gathered q
-          if (n16 > 0) {
+        float sx[2][2][4];
+        {
+          const uint32_t lb = st + lane * 16;
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) mma_bf16(sx[mt], xa[mt][0], xa[mt][1], xa[mt][2], xa[mt][3], xb0, xb1);
-            // the registers are free again: request the next unit's pairs now, a whole iteration ahead of their use
-            if (vleft > 1) load_xa(exu + ex_unit);
-            for (int kk = 1; kk * 8 < n16p; ++kk) {       // more than 16 promoted channels
-              uint32_t a[2][4], id0 = 0xFFFFFFFFu, id1 = 0xFFFFFFFFu;
-              const uint32_t* xw = reinterpret_cast<const uint32_t*>(exu);
-              const int p0 = 8 * kk + t, p1 = p0 + 4;
+          for (int un = 0; un < 2; ++un)
 #pragma unroll
-              for (int mt = 0; mt < 2; ++mt) a[mt][0] = a[mt][1] = a[mt][2] = a[mt][3] = 0;
-              if (p0 < n16p) {
-                id0 = *reinterpret_cast<const uint16_t*>(ex + 2 * p0);
-#pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
-                  a[mt][0] = xw[p0 * 32 + mt * 16 + r];
-                  a[mt][1] = xw[p0 * 32 + mt * 16 + 8 + r];
-                }
-              }
-              if (p1 < n16p) {
-                id1 = *reinterpret_cast<const uint16_t*>(ex + 2 * p1);
-#pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
-                  a[mt][2] = xw[p1 * 32 + mt * 16 + r];
-                  a[mt][3] = xw[p1 * 32 + mt * 16 + 8 + r];
-                }
-              }
-              auto gather_bf16 = [&](uint32_t cc) -> uint32_t {
-                const uint32_t c0 = cc & 0xFF, c1 = (cc >> 8) & 0xFF;
-                const uint32_t lo = (c0 < 128) ? lds16(qrow_v + 2 * c0) : 0u, hi = (c1 < 128) ? lds16(qrow_v + 2 * c1) : 0u;
-                return lo | (hi << 16);
-              };
-              const uint32_t b0 = gather_bf16(id0), b1 = gather_bf16(id1);
-#pragma unroll
-              for (int mt = 0; mt < 2; ++mt) mma_bf16(sx[mt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
+            for (int mt = 0; mt < 2; ++mt) {
+              const uint4 x = lds128(lb + un * kUnitStep + 16 * mt);
+              sx[un][mt][0] = __uint_as_float(x.x); sx[un][mt][1] = __uint_as_float(x.y);
+              sx[un][mt][2] = __uint_as_float(x.z); sx[un][mt][3] = __uint_as_float(x.w);
             }
-          }
         }
+        const uint4 zq = lds128(st - 512);
         // logit = (sx + q . z) * scale: the zero-point term of the key group is the same for every token of the unit
-        const float zl0 = __uint_as_float(zq.x) * scale_log2e, zl1 = __uint_as_float(zq.y) * scale_log2e;
+        const float zl[2][2] = {{__uint_as_float(zq.x) * scale_log2e, __uint_as_float(zq.y) * scale_log2e},
+                                {__uint_as_float(UPG == 1 ? zq.z : zq.x) * scale_log2e, __uint_as_float(UPG == 1 ? zq.w : zq.y) * scale_log2e}};
         // ---- online softmax (log2 domain); heads 2t, 2t+1; tokens r, r+8 of each m-tile.
         // The reference maximum only has to keep the probabilities inside the fp16 range: it is raised (to the true
-        // maximum so far, with the accumulators rescaled) when a logit of this unit exceeds it by more than kMaxSlack.
+        // maximum so far, with the accumulators rescaled) when a logit of this step exceeds it by more than kMaxSlack.
         {
-          const float u0 = fmaf(fmaxf(fmaxf(sx[0][0], sx[0][2]), fmaxf(sx[1][0], sx[1][2])), scale_log2e, zl0);
-          const float u1 = fmaf(fmaxf(fmaxf(sx[0][1], sx[0][3]), fmaxf(sx[1][1], sx[1][3])), scale_log2e, zl1);
-          if (__any_sync(0xffffffffu, (u0 > m0 + kMaxSlack) || (u1 > m1 + kMaxSlack))) raise_reference(u0, u1);
-        }
-        const float c0 = zl0 - m0, c1 = zl1 - m1;
-        // P^T B fragments: [k-step][tokens 2t.. / 2t+8..], head r
-        uint32_t Pt[2][2];
+          float uu[2];
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          Pt[mt][0] = movmatrix_trans(pack_half2(ex2_approx(fmaf(sx[mt][0], scale_log2e, c0)), ex2_approx(fmaf(sx[mt][1], scale_log2e, c1))));
-          Pt[mt][1] = movmatrix_trans(pack_half2(ex2_approx(fmaf(sx[mt][2], scale_log2e, c0)), ex2_approx(fmaf(sx[mt][3], scale_log2e, c1))));
+          for (int h = 0; h < 2; ++h) {
+            const float a = fmaf(fmaxf(fmaxf(sx[0][0][h], sx[0][0][2 + h]), fmaxf(sx[0][1][h], sx[0][1][2 + h])), scale_log2e, zl[0][h]);
+            const float b = fmaf(fmaxf(fmaxf(sx[1][0][h], sx[1][0][2 + h]), fmaxf(sx[1][1][h], sx[1][1][2 + h])), scale_log2e, zl[1][h]);
+            uu[h] = fmaxf(a, b);
+          }
+          if (__any_sync(0xffffffffu, (uu[0] > m0 + kMaxSlack) || (uu[1] > m1 + kMaxSlack))) raise_reference(uu[0], uu[1]);
+        }
+        // P^T B fragments: [unit][k-step][tokens 2t.. / 2t+8..], head r
+        uint32_t Pt[2][2][2];
+#pragma unroll
+        for (int un = 0; un < 2; ++un) {
+          const float c0 = zl[un][0] - m0, c1 = zl[un][1] - m1;
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh)
+              Pt[un][mt][hh] = movmatrix_trans(pack_half2(ex2_approx(fmaf(sx[un][mt][2 * hh], scale_log2e, c0)),
+                                                          ex2_approx(fmaf(sx[un][mt][2 * hh + 1], scale_log2e, c1))));
         }
         // ---- zero-point and denominator tile: rows 0..VG-1 = z_v of the group, row 4 = ones, the rest zero
 #pragma unroll
-        for (int ks = 0; ks < 2; ++ks) {
-          const uint4 zz = lds128(lane16 + kPrepBase + kZvpOff + ks * 576);
-          mma_f16(Zc, zz.x, zz.y, zz.z, zz.w, Pt[ks][0], Pt[ks][1]);
-        }
-        // ---- P.V: codes as fp16 subnormals, scales folded into P
-        {
-          const uint32_t vw[8] = {vw0.x, vw0.y, vw0.z, vw0.w, vw1.x, vw1.y, vw1.z, vw1.w};
+        for (int un = 0; un < 2; ++un)
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks) {
+            const uint2 zz = lds64(zv_rd + un * kZvpUnit + ks * 272);
+            mma_f16(Zc, zz.x, 0u, zz.y, 0u, Pt[un][ks][0], Pt[un][ks][1]);
+          }
+        // ---- P.V: codes as fp16 subnormals, scales folded into P; with 4-bit values then the high plane (codes >> 2, the
+        // low plane's bit order) with four times the scale
+        auto value_pass = [&](const uint4 (&w)[2][2], bool high) {
 #pragma unroll
           for (int vg = 0; vg < VG; ++vg) {
-            const uint4 sv = lds128(sv_rd + vg * 16);
-            const uint32_t Bp[2][2] = {{hmul2_u(Pt[0][0], sv.x), hmul2_u(Pt[0][1], sv.y)},
-                                       {hmul2_u(Pt[1][0], sv.z), hmul2_u(Pt[1][1], sv.w)}};
+            uint32_t Bp[2][2][2];
 #pragma unroll
-            for (int c = 0; c < TPG; ++c) {
-              const int ct = vg * TPG + c;
-              const uint32_t x0 = vw[ct], x1 = vw[ct] >> 8;
+            for (int un = 0; un < 2; ++un) {
+              const uint4 sv = lds128(sv_rd + un * kSvpUnit + vg * 16);
+              Bp[un][0][0] = hmul2_u(Pt[un][0][0], sv.x); Bp[un][0][1] = hmul2_u(Pt[un][0][1], sv.y);
+              Bp[un][1][0] = hmul2_u(Pt[un][1][0], sv.z); Bp[un][1][1] = hmul2_u(Pt[un][1][1], sv.w);
+              if (high) {
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                  Bp[un][ks][0] = hmul2_u(Bp[un][ks][0], four2);
+                  Bp[un][ks][1] = hmul2_u(Bp[un][ks][1], four2);
+                }
+              }
+            }
+#pragma unroll
+            for (int un = 0; un < 2; ++un) {
+              const uint32_t vwd[8] = {w[un][0].x, w[un][0].y, w[un][0].z, w[un][0].w, w[un][1].x, w[un][1].y, w[un][1].z, w[un][1].w};
 #pragma unroll
               for (int ks = 0; ks < 2; ++ks) {
                 const uint32_t mk0 = 0x00030003u << (4 * ks), mk1 = 0x00030003u << (4 * ks + 2);
-                mma_f16(O[ct], x0 & mk0, x1 & mk0, x0 & mk1, x1 & mk1, Bp[ks][0], Bp[ks][1]);
+#pragma unroll
+                for (int c = 0; c < TPG; ++c) {
+                  const int ct = vg * TPG + c;
+                  const uint32_t x0 = vwd[ct], x1 = vwd[ct] >> 8;
+                  mma_f16(O[ct], x0 & mk0, x1 & mk0, x0 & mk1, x1 & mk1, Bp[un][ks][0], Bp[un][ks][1]);
+                }
               }
             }
           }
-        }
-        // ---- 4-bit values: the high plane (codes >> 2, the low plane's bit order) with four times the scale
+        };
+        value_pass(vw, false);
         if constexpr (kV4) {
-          const uint4 xw0 = lds128(st + 2048 + 128 * VG);
-          const uint4 xw1 = lds128(st + 2048 + 128 * VG + 512);
-          const uint32_t vw[8] = {xw0.x, xw0.y, xw0.z, xw0.w, xw1.x, xw1.y, xw1.z, xw1.w};
 #pragma unroll
-          for (int vg = 0; vg < VG; ++vg) {
-            const uint4 sv = lds128(sv_rd + vg * 16);
-            const uint32_t Bp[2][2] = {{hmul2_u(hmul2_u(Pt[0][0], sv.x), four2), hmul2_u(hmul2_u(Pt[0][1], sv.y), four2)},
-                                       {hmul2_u(hmul2_u(Pt[1][0], sv.z), four2), hmul2_u(hmul2_u(Pt[1][1], sv.w), four2)}};
-#pragma unroll
-            for (int c = 0; c < TPG; ++c) {
-              const int ct = vg * TPG + c;
-              const uint32_t x0 = vw[ct], x1 = vw[ct] >> 8;
-#pragma unroll
-              for (int ks = 0; ks < 2; ++ks) {
-                const uint32_t mk0 = 0x00030003u << (4 * ks), mk1 = 0x00030003u << (4 * ks + 2);
-                mma_f16(O[ct], x0 & mk0, x1 & mk0, x0 & mk1, x1 & mk1, Bp[ks][0], Bp[ks][1]);
-              }
-            }
+          for (int un = 0; un < 2; ++un) {
+            vw[un][0] = lds128(st + un * kUnitStep + 2048 + 128 * VG);
+            vw[un][1] = lds128(st + un * kUnitStep + 2048 + 128 * VG + 512);
           }
+          value_pass(vw, true);
         }
-        // ---- both warps are done with the unit: refill the stage
+        // ---- both warps are done with the step: refill the stage (the logits were written to it by ordinary stores)
         __syncwarp();
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         issue(ring_stage, false);
         advance_stage();
-        if constexpr (promoted_in_values(kU4)) {
-          exu += ex_unit;
-          ++vcur;
-          if (--vleft == 0) {
-            ++vbi;
-            vcur = 0;
-          }
-        }
       }
       if (gave_up) {
         if (lane == 0) atomicOr(lv.status, (uint32_t)MIXKVQ_DEV_COPY_TIMEOUT);
@@ -1194,7 +972,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         // the ring: wait for them (bounded) before the ring is reused below or the CTA ends
         for (int i = max(0, issued - kStages); i < issued; ++i) {
           const uint32_t pos = stage0 + (uint32_t)i;
-          mbar_wait_polls(bar_u32 + (pos % kStages) * 8u, parity0 ^ ((pos / kStages) & 1u), lv.wait_polls ? lv.wait_polls : kWaitPolls);
+          mbar_wait_polls(bar_u32 + (pos % (uint32_t)kStages) * 8u, parity0 ^ ((pos / (uint32_t)kStages) & 1u), lv.wait_polls ? lv.wait_polls : kWaitPolls);
         }
         // what this warp accumulated is not a result: the pair contributes nothing
 #pragma unroll
@@ -1268,8 +1046,8 @@ cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, flo
   // launched with programmatic stream serialization: the kernel itself waits for its predecessor (griddepcontrol.wait)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem_bytes(kV4);
+  cfg.blockDim = dim3(pairs_of(kU4, kV4) * 64);
+  cfg.dynamicSmemBytes = smem_bytes(G, kU4, kV4);
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1299,7 +1077,7 @@ cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws,
 template <int G, int kU4, bool kV4>
 static cudaError_t setup_v() {
   cudaError_t e = cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem_bytes(kV4));
+                                       smem_bytes(G, kU4, kV4));
   if (e != cudaSuccess) return e;
   // the CTAs of an SM only fit with the largest shared-memory carve-out; ask for it explicitly
   return cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4>, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1323,7 +1101,8 @@ cudaError_t attention_ws_setup() {
   if (e != cudaSuccess) return e;
   e = setup_g<64>();
   if (e != cudaSuccess) return e;
-  return setup_g<128>();
+  e = setup_g<128>();
+  return e != cudaSuccess ? e : attention_single_setup();
 }
 
 // Split positions per stream: packed units plus the weighted units of the residual window and the sink.
@@ -1353,8 +1132,15 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   const int S = lv.B * lv.Hkv;
   const long long Us = attention_ws_positions(lv);
   const int grid = attention_ws_grid(lv, n_sms);
+  // Steps of two units need blocks with an even number of them, and pay from about ten steps per warp pair on: with fewer
+  // the coarser split and the longer first step cost more (7b shape, batch 8, us per launch, one unit / two units per step:
+  // 8000 tokens, 27 units per CTA, 12.7 / 13.3; 16000: 21.4 / 20.7; 32768: 36.7 / 35.3).  The gathered UINT4 tiles of three tiers
+  // gain at every length (2000 tokens 9.3 / 8.6, 32768 54.4 / 48.7).
+  const bool three_tiers = !lv.dense_hi && ((lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16);
+  const bool by_two = !(lv.U & 1) && (three_tiers || (lv.seq != nullptr ? lv.seq_total : Us * S) >= 40ll * grid);
   cudaError_t e;
-  if (lv.G == 32) e = launch_g<32>(lv, q, scale, ws, grid, stream);
+  if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, stream);
+  else if (lv.G == 32) e = launch_g<32>(lv, q, scale, ws, grid, stream);
   else if (lv.G == 64) e = launch_g<64>(lv, q, scale, ws, grid, stream);
   else e = launch_g<128>(lv, q, scale, ws, grid, stream);
   *launches = 1;
