@@ -2,10 +2,10 @@
 // warp-specialised form.
 //
 // Work unit = 32 tokens of one stream, taken two at a time (a step of 64 tokens; blocks hold an even number of units).  All
-// units of all streams are split evenly over the CTAs; inside a CTA they are split over PAIRS of warps.  A pair shares one
+// units of all streams are split evenly over the CTAs; inside a CTA they are split over TEAMS of warps.  A team shares one
 // ring of staged steps (1-D bulk copies signalled on mbarriers):
 //
-//   the logits warp   expands the step's 2-bit key codes into tensor-core A fragments (one logic op and one fp16 FMA
+//   a logits warp     expands the step's 2-bit key codes into tensor-core A fragments (one logic op and one fp16 FMA
 //                     per pair of codes: A = c*s, exact in fp16) and runs q.K^T on mma.sync m16n8k16 tiles with the g
 //                     query heads of the KV head as the N dimension.  The zero-point term q.z of the key groups is one
 //                     more tile chain per step (rows 0..7 the first unit's group, rows 8..15 the second's); the promoted
@@ -25,10 +25,12 @@
 // What bounds it: instruction issue and the latency of each warp's chain of dependent work, with three or four warps per
 // scheduler.  Two units per step instead of one (attention_single.cu) give every chain an independent twin, halve the
 // waits, hand-overs and zero-point tiles per unit (690 -> 598 warp instructions per unit) and need no hand-over buffers; the
-// promoted channels and the UINT4 plane, read from global memory a unit ahead there, come through shared memory two steps ahead
-// (without that the longer steps were slower than single units: 39.0 us at the 7b shape).  us per launch, one unit / two:
-// 7b shape (B = 8, T = 32768) 36.7 / 35.3; three tiers 54.4 / 48.7; 4-bit base (8b shape, B = 16, T = 16384) 110.7 / 109.5;
-// 4-bit values 88.4 / 81.4; 32b shape (B = 64, T = 32768, G = 128) 463 / 438 = 3.1 TB/s.
+// promoted channels and the UINT4 plane, read from global memory a unit ahead there, come through shared memory ahead of time
+// (without that the longer steps were slower than single units: 39.0 us at the 7b shape).  Clocks around the waits: with
+// two tiers the logits warp is the longer role by a quarter, with a 4-bit base by a factor of two, hence two logits warps
+// per values warp there.  us per launch, one unit / two units per step / with two logits warps: 7b shape (B = 8, T = 32768) 36.7 /
+// 35.3; three tiers 54.4 / 48.7 / 46.2; 4-bit base (8b shape, B = 16, T = 16384) 110.7 / 109.5 / 101.7; 4-bit values 88.4 / 82;
+// 32b shape (B = 64, T = 32768, G = 128) 463 / 433 = 3.1 TB/s.
 #include "warp_ops.cuh"
 
 namespace mixkvq {
@@ -42,38 +44,47 @@ cudaError_t attention_single_setup();
 
 namespace {
 
-// Warp pairs per CTA (two CTAs per SM): four at 128 registers per thread, or three at 168 where the logits warp needs more
-// (UINT4 tiles or a second key plane) or the shared memory does not hold four.
-__host__ __device__ constexpr int pairs_of(int u4, bool v4) { return u4 != 0 || v4 ? 3 : 4; }
+// A team: one values warp and its logits warps, which take the steps in turn.  Two tiers: one logits warp, four teams per CTA
+// (three where 4-bit values need the shared memory); a UINT4 tier or a 4-bit base makes the logits about twice the values'
+// work, so two logits warps, two teams per CTA.  Two CTAs per SM: 16 warps at 128 registers or 12 at 168.
+__host__ __device__ constexpr int logits_warps_of(int u4) { return u4 != 0 ? 2 : 1; }
+__host__ __device__ constexpr int teams_of(int u4, bool v4) { return u4 != 0 ? 2 : (v4 ? 3 : 4); }
+__host__ __device__ constexpr int threads_of(int u4, bool v4) { return teams_of(u4, v4) * (logits_warps_of(u4) + 1) * 32; }
 constexpr int kCtasPerSm = 2;
-constexpr int kStages = 3;                   // ring stages per pair
+__host__ __device__ constexpr int stages_of(int u4) { return u4 != 0 ? 4 : 3; }            // ring stages per team
+constexpr int kMaxStages = 4;
 __host__ __device__ constexpr int unit_bytes_of(int G, bool v4) { return 2048 + 128 * (kD / G) + (v4 ? 1024 : 0); }
 // one ring stage: the two units of a step with their key-meta groups (512 B each) in the block's own order: a group before
 // each unit (G = 32), or one group before both
 __host__ __device__ constexpr int stage_bytes(int G, bool v4) { return (G == 32 ? 1024 : 512) + 2 * unit_bytes_of(G, v4); }
-// per-pair tables: key scales {s, -4s} of two groups (2 x 576) | key zero-point tiles (576) | value scales of two units
-// (2 x 320) | value zero-point tiles of two units (2 x 544)
-constexpr int kKprepOff = 0, kZprepOff = 1152, kSvpOff = 1728, kZvpOff = 2368, kPrepBytes = 3456;
+// Tables of a team: per logits warp the key scales {s, -4s} of two groups (2 x 576) and the key zero-point tiles (576), then
+// the value scales of two units (2 x 320) and the value zero-point tiles of two units (2 x 544).
+constexpr int kZprepOff = 1152, kKeyPrepBytes = 1728;
+__host__ __device__ constexpr int svp_off(int u4) { return logits_warps_of(u4) * kKeyPrepBytes; }
+__host__ __device__ constexpr int zvp_off(int u4) { return svp_off(u4) + 640; }
+__host__ __device__ constexpr int prep_bytes(int u4) { return zvp_off(u4) + 1088; }
 constexpr int kKprepGroup = 576, kSvpUnit = 320, kZvpUnit = 544;
 constexpr int kRBufBytes = 1024;             // hand-over of an unquantized unit's logits: 32 bytes per lane
-// A step's extras (the promoted channels and the UINT4 high plane), copied by the logits warp kSlots - 1 steps ahead:
+// A step's extras (the promoted channels and the UINT4 high plane), copied a step or two ahead by each logits warp for its own steps
+// (three slots, two where two logits warps take turns; the values warp is no place for this although it has more time: it
+// refills the ring, and with the extras its wait for the copies made the 7b shape 38.9 us instead of 35.3):
 // the head of the block's channel lists (64 B, in a step that begins a block) | rows of the first kRowPairs pairs of
 // promoted channels of both units (128 B each) | three tiers: the first kPlanePairs pairs of UINT4 channels of both units
 // (16 B each); 4-bit base: both units' dense planes.  What does not fit is read from global memory (rare).
-constexpr int kSlots = 3, kRowPairs = 4, kPlanePairs = 16;
+constexpr int kRowPairs = 4, kPlanePairs = 16;
+__host__ __device__ constexpr int slots_of(int u4) { return u4 != 0 ? 2 : 3; }
 constexpr int kRowsOff = 128, kPlaneOff = kRowsOff + 2 * kRowPairs * 128;
 __host__ __device__ constexpr int slot_bytes(int u4) { return kPlaneOff + (u4 == 1 ? 2 * kPlanePairs * 16 : u4 == 2 ? 2048 : 0); }
-__host__ __device__ constexpr int slots_of(int u4, bool v4) { return u4 == 2 && v4 ? 2 : kSlots; }
-__host__ __device__ constexpr int pair_bytes(int G, int u4, bool v4) {
-  return kStages * stage_bytes(G, v4) + slots_of(u4, v4) * slot_bytes(u4) + kPrepBytes + kRBufBytes;
+__host__ __device__ constexpr int team_bytes(int G, int u4, bool v4) {
+  return stages_of(u4) * stage_bytes(G, v4) + logits_warps_of(u4) * (slots_of(u4) * slot_bytes(u4) + kRBufBytes) + prep_bytes(u4);
 }
-// mbarriers of a pair: staged copy landed [stages], logits ready [stages], then for unquantized units: ready, taken
-constexpr int kBarsPerPair = 2 * kStages + 2;
+// mbarriers of a team: staged copy landed [stages], logits ready [stages], then per logits warp for unquantized units: ready, taken
+constexpr int kBarsPerTeam = 2 * kMaxStages + 4;
 constexpr int kQS = 136;                     // halves per row of the query tables (272 bytes: rows fall on different banks)
 constexpr int kPrefixBytes = ((kMaxRaggedBatch + 1) * 4 + 15) / 16 * 16;     // a ragged batch's prefix sums
-__host__ __device__ constexpr int bar_bytes(int pairs) { return (pairs * kBarsPerPair * 8 + 127) / 128 * 128; }
+__host__ __device__ constexpr int bar_bytes(int teams) { return (teams * kBarsPerTeam * 8 + 127) / 128 * 128; }
 __host__ __device__ constexpr int smem_bytes(int G, int u4, bool v4) {
-  return pairs_of(u4, v4) * (pair_bytes(G, u4, v4) + 64) + bar_bytes(pairs_of(u4, v4)) + (u4 == 1 ? 2 : 1) * 8 * kQS * 2 + kPrefixBytes;
+  return teams_of(u4, v4) * (team_bytes(G, u4, v4) + 64) + bar_bytes(teams_of(u4, v4)) + (u4 == 1 ? 2 : 1) * 8 * kQS * 2 + kPrefixBytes;
 }
 constexpr int kResidualWeight = 3;           // an unquantized 32-token unit counts as this many packed units in the split
 constexpr int kMergeStride = 132;            // floats per head row of a pair's output in the merge
@@ -92,49 +103,51 @@ __device__ __forceinline__ constexpr int key_pos(int kt) { return (0x86486464u >
 // k-tiles 0,1 are read from (w << 4), 2..4 from w, 5..7 from (w >> 6)
 __device__ __forceinline__ uint32_t key_shift(uint32_t w, int kt) { return kt < 2 ? (w << 4) : (kt < 5 ? w : (w >> 6)); }
 
-// warp w of the CTA: pair w / 2; the logits warps are spread evenly over the four schedulers of the SM (w mod 4)
+// warp w of the CTA with one logits warp per team: team w / 2; the logits warps are spread evenly over the four schedulers of
+// the SM (w mod 4)
 __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp >> 2)) & 1) == 0; }
 
 // kU4: how the configuration can use the UINT4 tier: 0 = never (tau_u4 >= tau_bf16), 1 = some channels (high plane stored
 // per channel pair, gathered), 2 = 4-bit base (dense high plane)
 // kV4: 4-bit values (a second plane of 2-bit value codes per unit, scale 4 s_v)
 template <int G, int kU4, bool kV4>
-__global__ void __launch_bounds__(pairs_of(kU4, kV4) * 64, kCtasPerSm)
+__global__ void __launch_bounds__(threads_of(kU4, kV4), kCtasPerSm)
 attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float scale_log2e, float* __restrict__ ws,
                     uint32_t four2) {
   constexpr int VG = kD / G;              // value groups per token
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group
   constexpr int UPG = G / 32;             // units per key group
   constexpr int kGroups = UPG == 1 ? 2 : 1;                    // key groups of a step
-  constexpr int kPairs = pairs_of(kU4, kV4), kThreads = kPairs * 64;
-  constexpr int kSlotCount = slots_of(kU4, kV4), kSlotBytes = slot_bytes(kU4);
+  constexpr int kTeams = teams_of(kU4, kV4), kL = logits_warps_of(kU4), kThreads = threads_of(kU4, kV4);
+  constexpr int kStages = stages_of(kU4), kSlotCount = slots_of(kU4), kSlotBytes = slot_bytes(kU4);
   constexpr int kStageBytes = stage_bytes(G, kV4);
-  constexpr int kPairBytes = pair_bytes(G, kU4, kV4);
+  constexpr int kTeamBytes = team_bytes(G, kU4, kV4);
   // a unit: key codes 1024, value codes 1024, value scales (and the values' high plane 1024)
   constexpr uint32_t kUnitBytes = unit_bytes_of(G, kV4);
   constexpr uint32_t kUnitStep = kUnitBytes + (UPG == 1 ? 512u : 0u);      // from a step's first unit to its second, staged
-  constexpr int kSlotBase = kStages * kStageBytes;             // offsets inside a pair's shared memory
-  constexpr int kPrepBase = kSlotBase + kSlotCount * kSlotBytes;
+  constexpr int kSlotBase = kStages * kStageBytes;             // offsets inside a team's shared memory
+  constexpr int kPrepBase = kSlotBase + kL * kSlotCount * kSlotBytes;
+  constexpr int kRBufBase = kPrepBase + prep_bytes(kU4);
   constexpr int kQBytes = (kU4 == 1 ? 2 : 1) * 8 * kQS * 2;
-  constexpr int kRBufBase = kPrepBase + kPrepBytes;
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, t = lane & 3;
-  const int pair = warp >> 1;
-  const bool logits_role = is_logits_warp(warp);
+  const int team = kL == 1 ? warp >> 1 : warp / 3;
+  const bool logits_role = kL == 1 ? is_logits_warp(warp) : warp % 3 != 2;
+  const uint32_t lsub = kL == 1 || !logits_role ? 0u : (uint32_t)(warp % 3);      // which of the team's logits warps
 
   const uint32_t smem_base = smem_u32(smem);
-  const uint32_t ring_u32 = smem_base + pair * kPairBytes;                  // the pair's shared memory starts with its ring
-  const uint32_t tail_u32 = smem_base + kPairs * kPairBytes;
-  const uint32_t bar_u32 = tail_u32 + pair * (kBarsPerPair * 8);            // staged copy landed [kStages]
+  const uint32_t ring_u32 = smem_base + team * kTeamBytes;                  // the team's shared memory starts with its ring
+  const uint32_t tail_u32 = smem_base + kTeams * kTeamBytes;
+  const uint32_t bar_u32 = tail_u32 + team * (kBarsPerTeam * 8);            // staged copy landed [kStages]
   const uint32_t lfull_u32 = bar_u32 + kStages * 8;                         // logits ready [kStages]
-  const uint32_t rfull_u32 = bar_u32 + 2 * kStages * 8, rempty_u32 = rfull_u32 + 8;
-  const uint32_t qb16_u32 = tail_u32 + bar_bytes(kPairs);                           // [8][kQS] q, bf16 bits (0 for heads >= g)
+  const uint32_t rfull_u32 = bar_u32 + 2 * kStages * 8, rempty_u32 = rfull_u32 + 8 * kL;    // [kL] each
+  const uint32_t qb16_u32 = tail_u32 + bar_bytes(kTeams);                           // [8][kQS] q, bf16 bits (0 for heads >= g)
   const uint32_t qf16_u32 = qb16_u32 + 8 * kQS * 2;                         // [8][kQS] q, fp16 (three tiers)
-  float* mS = reinterpret_cast<float*>(smem + kPairs * kPairBytes + bar_bytes(kPairs) + kQBytes);    // [kPairs][8]
-  float* lS = mS + kPairs * 8;                                                                       // [kPairs][8]
-  int* prefS = reinterpret_cast<int*>(lS + kPairs * 8);                     // ragged batch: seq_prefix[0 .. B]
+  float* mS = reinterpret_cast<float*>(smem + kTeams * kTeamBytes + bar_bytes(kTeams) + kQBytes);    // [kTeams][8]
+  float* lS = mS + kTeams * 8;                                                                       // [kTeams][8]
+  int* prefS = reinterpret_cast<int*>(lS + kTeams * 8);                     // ragged batch: seq_prefix[0 .. B]
 
-  if (threadIdx.x < kPairs * kBarsPerPair) {
+  if (threadIdx.x < kTeams * kBarsPerTeam) {
     mbar_init(tail_u32 + 8 * threadIdx.x, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -142,7 +155,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     // constant rows of the zero-point / denominator tiles ([2 units][2 ks: 68 words][8 rows][4 t]{k 2t.., k 8 + 2t..}):
     // row 4 is all ones, the other rows >= VG stay zero
     for (int i = lane; i < 2 * kZvpUnit / 4; i += 32)
-      sts32(ring_u32 + kPrepBase + kZvpOff + 4 * i, ((i % 68) >> 3) == 4 ? 0x3C003C00u : 0u);
+      sts32(ring_u32 + kPrepBase + zvp_off(kU4) + 4 * i, ((i % 68) >> 3) == 4 ? 0x3C003C00u : 0u);
   }
   __syncthreads();
 
@@ -178,12 +191,12 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   const long long total = lv.seq != nullptr ? (long long)prefS[lv.B] : (long long)Us * S;
   const long long cb = split_begin(total, gridDim.x, blockIdx.x), ce = split_begin(total, gridDim.x, blockIdx.x + 1);
 
-  uint32_t ring_stage = 0;        // ring stage of the next step this pair consumes
+  uint32_t ring_stage = 0;        // ring stage of the next step of this warp
   uint32_t ring_parity = 0;       // phase parity of that stage's barriers
-  uint32_t rit = 0;               // unquantized units handed over by this pair so far (both warps count them alike)
+  uint32_t rit[kL] = {};          // unquantized units handed over so far, per logits warp of the team
   bool gave_up = false;
   // A wait that runs out sets gave_up; the warp carries on with whatever the shared memory holds (every address it
-  // forms stays inside the CTA's shared memory and the stream's arrays), its later waits are skipped, and the pair's
+  // forms stays inside the CTA's shared memory and the stream's arrays), its later waits are skipped, and the team's
   // result is replaced by zeros at the end.  Straight-line code: no exit in the middle of a step.
   auto wait_or_give_up = [&](uint32_t bar, uint32_t parity) {
     if (!gave_up && !mbar_wait_polls(bar, parity, lv.wait_polls ? lv.wait_polls : kWaitPolls)) gave_up = true;
@@ -216,8 +229,8 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       ue = (int)min((long long)Us, ce - (long long)s * Us);
     }
     seg += ue - ub;
-    // ---- this pair's share of the segment.  The unquantized units of the segment go to different pairs (unit i to
-    // pair kPairs - 1 - i % kPairs); the packed units are split in order, in steps of two, so that every pair carries about
+    // ---- this team's share of the segment.  The unquantized units of the segment go to different teams (unit i to
+    // team kTeams - 1 - i % kTeams); the packed units are split in order, in steps of two, so that every team carries about
     // the same weight.  (A stream's packed units are even in number; a boundary at an odd one moves up, on both sides.)
     const int pk_b = (min(ub, packed_units) + 1) & ~1, pk_e = (min(ue, packed_units) + 1) & ~1;
     const int res_b = (max(ub, packed_units) - packed_units + kResidualWeight - 1) / kResidualWeight;
@@ -226,16 +239,16 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     int wb = pk_b, we = pk_b;
     {
       const int n_packed = pk_e - pk_b, weight = n_packed + kResidualWeight * n_res;
-      int given = 0, res_given = 0;              // packed and unquantized units of the pairs before
+      int given = 0, res_given = 0;              // packed and unquantized units of the teams before
 #pragma unroll
-      for (int w = 0; w < kPairs; ++w) {
-        const int first_i = kPairs - 1 - w;      // unquantized units first_i, first_i + kPairs, ...
-        res_given += n_res > first_i ? (n_res - first_i + kPairs - 1) / kPairs : 0;
-        // everything up to this pair against its exact share (weight < 2^24: 32-bit arithmetic)
-        const int upto = w == kPairs - 1
+      for (int w = 0; w < kTeams; ++w) {
+        const int first_i = kTeams - 1 - w;      // unquantized units first_i, first_i + kTeams, ...
+        res_given += n_res > first_i ? (n_res - first_i + kTeams - 1) / kTeams : 0;
+        // everything up to this team against its exact share (weight < 2^24: 32-bit arithmetic)
+        const int upto = w == kTeams - 1
                              ? n_packed
-                             : min(n_packed, max(given, (weight * (w + 1) / kPairs - kResidualWeight * res_given + 1) & ~1));
-        if (w == pair) {
+                             : min(n_packed, max(given, (weight * (w + 1) / kTeams - kResidualWeight * res_given + 1) & ~1));
+        if (w == team) {
           wb = pk_b + given;
           we = pk_b + upto;
         }
@@ -249,6 +262,9 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     // so the copy source only ever moves forward: `isrc` is the next step to stage.
     int issued = 0;
     const char* isrc = lv.base + (size_t)s * lv.base_stride + (size_t)wb * kUnitBytes + 512u * (size_t)((wb + UPG - 1) / UPG);
+    // G = 128: a group's scales lie before its first half; a step that is the second half brings them along where its logits
+    // warp did not have the first half
+    constexpr bool kMetaAlways = kL > 1;
     uint32_t ihalf = UPG == 4 ? (uint32_t)(wb >> 1) & 1u : 0u;      // G = 128: the step is its group's second half
     // stages the next step (if there is one left) in ring stage sg; all lanes keep the position
     auto issue = [&](uint32_t sg, bool first) {
@@ -258,9 +274,8 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         stage_copy(dst, isrc, (uint32_t)kStageBytes, bar, first ? lv.debug_extra_tx : 0u, enabled);
         isrc += kStageBytes;
       } else {
-        // the group's scales lie before its first half: they are in the tables already, unless this is the first step
         if (enabled) {
-          if (first) stage_copy2(dst + 512, isrc, 2 * kUnitBytes, dst, isrc - 2 * kUnitBytes - 512, 512u, bar, lv.debug_extra_tx);
+          if (first || kMetaAlways) stage_copy2(dst + 512, isrc, 2 * kUnitBytes, dst, isrc - 2 * kUnitBytes - 512, 512u, bar, first ? lv.debug_extra_tx : 0u);
           else stage_copy(dst + 512, isrc, 2 * kUnitBytes, bar, 0u, 1u);
         }
         isrc += 2 * kUnitBytes;
@@ -269,20 +284,44 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       issued += (int)enabled;
     };
     const uint32_t stage0 = ring_stage, parity0 = ring_parity;
-    // The extras of a step are copied kSlotCount - 1 steps ahead (logits warp).  The copies' cursor: block cbi and unit cu in
-    // it, the block's table entry and the next one's, requested a block ahead.
+    // The extras of a step are copied kSlotCount - 1 of the warp's own steps ahead.  The copies' cursor: block cbi and unit cu
+    // in it, the block's table entry and the entry of the next block or (two logits warps) of the next copy, under way.
     const char* extras = lv.extras + (size_t)s * lv.extras_stride;
     const uint2* table = reinterpret_cast<const uint2*>(lv.table + (size_t)s * lv.table_stride);
-    const uint32_t slot0_u32 = ring_u32 + kSlotBase;
-    int cbi = 0, cu = 0, requested = 0;
+    constexpr int kOwnUnits = 2 * kL;                             // from a warp's step to its next one
+    const uint32_t slot0_u32 = ring_u32 + kSlotBase + lsub * (kSlotCount * kSlotBytes);
+    int cbi = 0, cu = 0, last_bi = -1, to_request = logits_role ? (n_steps - (int)lsub + kL - 1) / kL : 0;
     uint2 c_entry = make_uint2(0u, 0u), c_next = make_uint2(0u, 0u);
-    // requests the next step's extras (nothing past the last step); returns its block's counts: pairs of promoted channels,
+    auto next_position = [&](int& b, int& v) {
+      v += kOwnUnits;
+      if constexpr (kL == 1) {
+        if (v == U) {
+          v = 0;
+          ++b;
+        }
+      } else {
+        while (v >= U) {
+          v -= U;
+          ++b;
+        }
+      }
+    };
+    auto request_entry = [&]() {
+      int b = cbi + 1, v = 0;
+      if constexpr (kL != 1) {
+        b = cbi;
+        v = cu;
+        next_position(b, v);
+      }
+      if (b < f_nb) c_next = table[b];
+    };
+    // requests the next own step's extras (nothing past the last step); returns its block's counts: pairs of promoted channels,
     // UINT4 channels << 8, and bit 16 in a step that begins a block (or is the first one)
     auto request_extras = [&](uint32_t slot) -> uint32_t {
       uint32_t counts = 0u;
-      if (requested < n_steps) {
+      if (to_request > 0) {
         const int n16 = c_entry.y & 0xFF, n4 = (c_entry.y >> 8) & 0xFF, n16p = (n16 + 1) >> 1;
-        const bool begins = requested == 0 || cu == 0;
+        const bool begins = kL == 1 ? last_bi < 0 || cu == 0 : cbi != last_bi;
         counts = (uint32_t)n16p | ((uint32_t)n4 << 8) | (begins ? 0x10000u : 0u);
         const uint32_t hdr = extras_header_bytes(n16, n4), unit = extras_unit_bytes(n16, n4, kU4 == 2);
         const char* ex = extras + (size_t)c_entry.x * 16;
@@ -306,36 +345,36 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
               cp_async16(dst + kPlaneOff + 512 * k + 16 * lane, exu + (k >> 1) * unit + 128 * n16p + 512 * (k & 1) + 16 * lane);
           }
         }
-        ++requested;
-        cu += 2;
-        if (cu == U) {
-          cu = 0;
-          ++cbi;
+        --to_request;
+        last_bi = cbi;
+        next_position(cbi, cu);
+        if (kL != 1 || cbi != last_bi) {
           c_entry = c_next;
-          if (cbi + 1 < f_nb) c_next = table[cbi + 1];
+          request_entry();
         }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
       return counts;
     };
-    uint32_t counts[kSlotCount];              // of the current step and those ahead
+    uint32_t counts[kSlotCount];              // of the current own step and those ahead
 #pragma unroll
     for (int i = 0; i < kSlotCount; ++i) counts[i] = 0u;
     auto request_first = [&]() {
-      cbi = wb / U;
-      cu = wb - cbi * U;
+      cbi = (wb + 2 * (int)lsub) / U;
+      cu = wb + 2 * (int)lsub - cbi * U;
       c_entry = table[cbi];
-      if (cbi + 1 < f_nb) c_next = table[cbi + 1];
+      request_entry();
 #pragma unroll
       for (int i = 0; i < kSlotCount - 1; ++i) counts[i] = request_extras(i);
     };
+    uint32_t slot = 0;                        // of the current own step
     if (!logits_role) {
 #pragma unroll 1
       for (uint32_t i = 0, sg = ring_stage; i < (uint32_t)kStages; ++i, sg = next_stage(sg)) issue(sg, i == 0);
     }
-    if (logits_role && n_steps > 0 && lv.stage_early) request_first();
+    if (to_request > 0 && lv.stage_early) request_first();
     dep_wait();
-    if (logits_role && n_steps > 0 && !lv.stage_early) request_first();
+    if (to_request > 0 && !lv.stage_early) request_first();
 
     // ---- query of this stream: bf16 and fp16 tables (heads >= g are zero rows)
     {
@@ -352,9 +391,9 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       __syncthreads();
     }
 
-    // unquantized units of this pair: first_res, first_res + kPairs, ... < n_res
-    const int first_res = kPairs - 1 - pair;
-    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the pair whose unit holds it
+    // unquantized units of this team: first_res, first_res + kTeams, ... < n_res
+    const int first_res = kTeams - 1 - team;
+    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the team whose unit holds it
     // takes its rows from the step's tensors, stores them and updates the importance accumulator
     const int jn = f_r - 1;
 
@@ -367,7 +406,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       // ---- unquantized units: bf16 keys straight from global memory.  The channel a k-slot stands for is free as long as
       // both operands agree: lane column t of k-tile 2j (2j+1) takes channels 32j + 8t + 0..3 (4..7), so that a lane's
       // four k-tiles' worth of a token row is one 16-byte load.
-      for (int ri = first_res; ri < n_res; ri += kPairs) {
+      for (int ri = first_res + (int)lsub * kTeams; ri < n_res; ri += kL * kTeams) {
         const int bu = res_b + ri;                        // unquantized unit: residual window first, then the sink
         const bool in_sink = bu >= res_units;
         const int wu = in_sink ? bu - res_units : bu;     // unit inside its window
@@ -412,13 +451,13 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
           if (lane == 0) *reinterpret_cast<uint32_t*>(lv.state + (size_t)s * lv.state_stride + 1024) += (uint32_t)g;
         }
         // hand over (the buffer is free once the partner has taken the previous unquantized unit)
-        wait_or_give_up(rempty_u32, (rit & 1u) ^ 1u);
-        const uint32_t rb = ring_u32 + kRBufBase + lane * 32;
+        wait_or_give_up(rempty_u32 + 8 * lsub, (rit[0] & 1u) ^ 1u);
+        const uint32_t rb = ring_u32 + kRBufBase + kRBufBytes * lsub + lane * 32;
         sts128(rb, __float_as_uint(Sx[0][0]), __float_as_uint(Sx[0][1]), __float_as_uint(Sx[0][2]), __float_as_uint(Sx[0][3]));
         sts128(rb + 16, __float_as_uint(Sx[1][0]), __float_as_uint(Sx[1][1]), __float_as_uint(Sx[1][2]), __float_as_uint(Sx[1][3]));
         __syncwarp();
-        mbar_arrive_one(rfull_u32);
-        ++rit;
+        mbar_arrive_one(rfull_u32 + 8 * lsub);
+        ++rit[0];
       }
 
       // ---- packed units
@@ -435,10 +474,11 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       }
       // per-lane constants of the key-group preparation: the lane converts channels 4*lane .. 4*lane+3 (k-tile lane / 4)
       const float pk_zs = __uint_as_float((119u + (uint32_t)key_pos(lane >> 2)) << 23);        // 2^(pos - 8)
-      const uint32_t kp_wr = ring_u32 + kPrepBase + kKprepOff + kprep_off(lane >> 2, 2 * (lane & 1)) + 8 * ((lane >> 1) & 1);
-      const uint32_t zp_wr = kp_wr + (kZprepOff - kKprepOff);
-      const uint32_t kp_rd = ring_u32 + kPrepBase + kKprepOff + 16 * t;
-      const uint32_t zp_rd = ring_u32 + kPrepBase + kZprepOff + 16 * t;
+      const uint32_t kprep_u32 = ring_u32 + kPrepBase + lsub * kKeyPrepBytes;
+      const uint32_t kp_wr = kprep_u32 + kprep_off(lane >> 2, 2 * (lane & 1)) + 8 * ((lane >> 1) & 1);
+      const uint32_t zp_wr = kp_wr + kZprepOff;
+      const uint32_t kp_rd = kprep_u32 + 16 * t;
+      const uint32_t zp_rd = kprep_u32 + kZprepOff + 16 * t;
       const uint32_t lane16 = ring_u32 + lane * 16;
       // byte offset inside the scale table of channel c's scale (half)
       auto scale_byte = [&](uint32_t c) -> uint32_t {
@@ -446,23 +486,23 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         return c < 128 ? (uint32_t)(kprep_off(kt, (col & 7) >> 1) + 8 * (col >> 3) + 2 * (col & 1)) : 0xFFFFu;
       };
       float zc[4] = {0.f, 0.f, 0.f, 0.f};   // zero-point terms q . z: [0..1] of unit 0's key group, [2..3] of unit 1's
-      // B fragment of the block's first 2 kRowPairs promoted channels (gathered query entries; 0 past the count)
-      uint32_t xb = 0u;
       // three tiers: the block's first 2 kPlanePairs UINT4 channels (two tiles of eight pairs): B fragments (gathered fp16
       // query pairs) and, per pair, where the two channels' scales sit in the scale table (0xFFFF: no channel)
       uint32_t u4q[2][2] = {{0u, 0u}, {0u, 0u}}, u4s[2][2] = {{~0u, ~0u}, {~0u, ~0u}};
+      // B fragment of the block's first 2 kRowPairs promoted channels (gathered query entries; 0 past the count)
+      uint32_t xb = 0u;
       // query entries of a pair of channel numbers (0xFF: no channel)
       auto query_pair = [&](uint32_t row, uint32_t two) -> uint32_t {
         const uint32_t c0 = two & 0xFFu, c1 = (two >> 8) & 0xFFu;
         return (c0 < 128 ? lds16(row + 2 * c0) : 0u) | ((c1 < 128 ? lds16(row + 2 * c1) : 0u) << 16);
       };
-      uint32_t slot = 0;                    // of the current step
+      if (lsub == 1u) advance_stage();
 #pragma unroll 1
-      for (int i = 0; i < n_steps; ++i) {
+      for (int i = (int)lsub; i < n_steps; i += kL) {
         wait_or_give_up(bar_u32 + ring_stage * 8u, ring_parity);
         const uint32_t stg = lane16 + ring_stage * kStageBytes;         // this lane's 16 bytes of the stage's first section
         // G = 128: the group's second half finds the tables as the first left them
-        const bool has_meta = UPG != 4 || i == 0 || (((wb >> 1) + i) & 1) == 0;
+        const bool has_meta = UPG != 4 || kMetaAlways || i == 0 || (((wb >> 1) + i) & 1) == 0;
         // the extras of a later step are requested into the slot that was read in the step before; this step's have arrived
         const uint32_t later = request_extras(slot == 0 ? kSlotCount - 1 : slot - 1);
         asm volatile("cp.async.wait_group %0;" ::"n"(kSlotCount - 1) : "memory");
@@ -558,7 +598,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         // block's gathered query pairs and scale positions; further tiles look their channels up per step.
         if constexpr (kU4 == 1) {
           if (n4pairs > 0) {
-            const uint32_t kpb = ring_u32 + kPrepBase + kKprepOff;
+            const uint32_t kpb = kprep_u32;
             auto plane_tile = [&](int un, const uint32_t (&words)[2], const uint32_t (&sidx)[2], const uint32_t (&qb)[2]) {
               uint32_t a[2][4];
 #pragma unroll
@@ -685,6 +725,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         for (int k = 0; k + 2 < kSlotCount; ++k) counts[k] = counts[k + 1];
         counts[kSlotCount - 2] = later;
         slot = slot + 1 == kSlotCount ? 0u : slot + 1;
+        if constexpr (kL == 2) advance_stage();
         advance_stage();
       }
       if (gave_up && lane == 0) atomicOr(lv.status, (uint32_t)MIXKVQ_DEV_COPY_TIMEOUT);
@@ -718,7 +759,8 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       };
 
       // ---- unquantized units: bf16 values straight from global memory, 8x8 tiles transposed in registers
-      for (int ri = first_res; ri < n_res; ri += kPairs) {
+      uint32_t rsub = 0;                    // the logits warp that has the unit
+      for (int ri = first_res; ri < n_res; ri += kTeams) {
         const int bu = res_b + ri;
         const bool in_sink = bu >= res_units;
         const int wu = in_sink ? bu - res_units : bu;
@@ -753,12 +795,14 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
             }
         };
         load_tile(0);
-        wait_or_give_up(rfull_u32, rit & 1u);
-        const uint32_t rb = ring_u32 + kRBufBase + lane * 32;
+        wait_or_give_up(rfull_u32 + 8 * rsub, (rsub ? rit[kL - 1] : rit[0]) & 1u);
+        const uint32_t rb = ring_u32 + kRBufBase + kRBufBytes * rsub + lane * 32;
         const uint4 s0 = lds128(rb), s1 = lds128(rb + 16);
         __syncwarp();
-        mbar_arrive_one(rempty_u32);
-        ++rit;
+        mbar_arrive_one(rempty_u32 + 8 * rsub);
+        if (rsub) ++rit[kL - 1];
+        else ++rit[0];
+        if constexpr (kL == 2) rsub ^= 1u;
         // logits (log2 domain) of tokens j0 + 16 mt + r (+ 8), heads 2t, 2t+1; tokens past the window count for nothing
         float xl[2][4];
         {
@@ -824,12 +868,12 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       const int pi = VG == 1 ? lane & 15 : lane >> 1, vg0 = VG == 1 ? 0 : (lane & 1) * (VG / 2);
       const int p_ks = pi >> 3, p_ch = (pi >> 2) & 1, p_t = pi & 3;
       const float pv_up = __uint_as_float((131u - 2u * (uint32_t)(2 * p_ks + p_ch)) << 23);          // 2^(4 - 2 * (2 ks + ch))
-      const uint32_t sv_wr = ring_u32 + kPrepBase + kSvpOff + (VG == 1 ? (uint32_t)(lane >> 4) * kSvpUnit : 0u) +
+      const uint32_t sv_wr = ring_u32 + kPrepBase + svp_off(kU4) + (VG == 1 ? (uint32_t)(lane >> 4) * kSvpUnit : 0u) +
                              4 * (p_t * 20 + vg0 * 4 + p_ks * 2 + p_ch);
-      const uint32_t zv_wr = ring_u32 + kPrepBase + kZvpOff + (VG == 1 ? (uint32_t)(lane >> 4) * kZvpUnit : 0u) +
+      const uint32_t zv_wr = ring_u32 + kPrepBase + zvp_off(kU4) + (VG == 1 ? (uint32_t)(lane >> 4) * kZvpUnit : 0u) +
                              4 * (p_ks * 68 + vg0 * 8 + p_t * 2 + p_ch);
-      const uint32_t sv_rd = ring_u32 + kPrepBase + kSvpOff + t * 80;
-      const uint32_t zv_rd = ring_u32 + kPrepBase + kZvpOff + lane * 8;
+      const uint32_t sv_rd = ring_u32 + kPrepBase + svp_off(kU4) + t * 80;
+      const uint32_t zv_rd = ring_u32 + kPrepBase + zvp_off(kU4) + lane * 8;
       const uint32_t lane16 = ring_u32 + lane * 16;
       const uint32_t vm_rd = ring_u32 + 512 + 2048 + (2 * pi) * (4 * VG) + 4 * vg0 + (VG == 1 ? (uint32_t)(lane >> 4) * kUnitStep : 0u);
 #pragma unroll 1
@@ -974,7 +1018,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
           const uint32_t pos = stage0 + (uint32_t)i;
           mbar_wait_polls(bar_u32 + (pos % (uint32_t)kStages) * 8u, parity0 ^ ((pos / (uint32_t)kStages) & 1u), lv.wait_polls ? lv.wait_polls : kWaitPolls);
         }
-        // what this warp accumulated is not a result: the pair contributes nothing
+        // what this warp accumulated is not a result: the team contributes nothing
 #pragma unroll
         for (int ct = 0; ct < 8; ++ct)
 #pragma unroll
@@ -983,7 +1027,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         m0 = m1 = -INFINITY;
       }
 
-      // ---- finish this pair's split: true scale, zero-point terms, denominator
+      // ---- finish this team's split: true scale, zero-point terms, denominator
 #pragma unroll
       for (int ct = 0; ct < 8; ++ct) {
         const int vg = ct / TPG;
@@ -995,13 +1039,13 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       }
       const float l0 = __shfl_sync(0xffffffffu, Zc[0], 16 + t), l1 = __shfl_sync(0xffffffffu, Zc[1], 16 + t);
       if (r == 0) {
-        mS[pair * 8 + 2 * t] = m0;
-        mS[pair * 8 + 2 * t + 1] = m1;
-        lS[pair * 8 + 2 * t] = l0;
-        lS[pair * 8 + 2 * t + 1] = l1;
+        mS[team * 8 + 2 * t] = m0;
+        mS[team * 8 + 2 * t + 1] = m1;
+        lS[team * 8 + 2 * t] = l0;
+        lS[team * 8 + 2 * t + 1] = l1;
       }
-      // the pair's unnormalized output goes to its own, now idle, ring as [8 heads][132] floats
-      float* mine = reinterpret_cast<float*>(smem + pair * kPairBytes);
+      // the team's unnormalized output goes to its own, now idle, ring as [8 heads][132] floats
+      float* mine = reinterpret_cast<float*>(smem + team * kTeamBytes);
 #pragma unroll
       for (int ct = 0; ct < 8; ++ct) {
         mine[(2 * t) * kMergeStride + 16 * ct + r] = O[ct][0];
@@ -1011,21 +1055,27 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       }
     }
 
-    // ---- merge the pairs of the CTA, write the partial of (CTA, stream): the 16 threads that own a head add the pairs'
+    // the next segment goes on where this one's steps end
+    {
+      const uint32_t pos = stage0 + (uint32_t)n_steps;
+      ring_stage = pos % (uint32_t)kStages;
+      ring_parity = (parity0 ^ (pos / (uint32_t)kStages)) & 1u;
+    }
+    // ---- merge the teams of the CTA, write the partial of (CTA, stream): the 16 threads that own a head add the teams'
     // rows with the factors 2^(m_p - M).
     __syncthreads();
     for (int idx = threadIdx.x; idx < 256; idx += kThreads) {
       const int h = idx >> 5, c = 4 * (idx & 31);          // head, first of the thread's four channels
-      float M = -INFINITY, L = 0.f, f[kPairs];
+      float M = -INFINITY, L = 0.f, f[kTeams];
 #pragma unroll
-      for (int w = 0; w < kPairs; ++w) M = fmaxf(M, mS[w * 8 + h]);
+      for (int w = 0; w < kTeams; ++w) M = fmaxf(M, mS[w * 8 + h]);
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int w = 0; w < kPairs; ++w) {
+      for (int w = 0; w < kTeams; ++w) {
         const float mw = mS[w * 8 + h];
         f[w] = (mw == -INFINITY) ? 0.f : ex2_approx(mw - M);
         L += f[w] * lS[w * 8 + h];
-        const float4 o = *reinterpret_cast<const float4*>(smem + w * kPairBytes + (h * kMergeStride + c) * 4);
+        const float4 o = *reinterpret_cast<const float4*>(smem + w * kTeamBytes + (h * kMergeStride + c) * 4);
         acc.x += f[w] * o.x; acc.y += f[w] * o.y; acc.z += f[w] * o.z; acc.w += f[w] * o.w;
       }
       float* part = ws + (size_t)(blockIdx.x + s) * kPartialFloats + h * 130;
@@ -1046,7 +1096,7 @@ cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, flo
   // launched with programmatic stream serialization: the kernel itself waits for its predecessor (griddepcontrol.wait)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(pairs_of(kU4, kV4) * 64);
+  cfg.blockDim = dim3(threads_of(kU4, kV4));
   cfg.dynamicSmemBytes = smem_bytes(G, kU4, kV4);
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -1132,12 +1182,14 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   const int S = lv.B * lv.Hkv;
   const long long Us = attention_ws_positions(lv);
   const int grid = attention_ws_grid(lv, n_sms);
-  // Steps of two units need blocks with an even number of them, and pay from about ten steps per warp pair on: with fewer
-  // the coarser split and the longer first step cost more (7b shape, batch 8, us per launch, one unit / two units per step:
-  // 8000 tokens, 27 units per CTA, 12.7 / 13.3; 16000: 21.4 / 20.7; 32768: 36.7 / 35.3).  The gathered UINT4 tiles of three tiers
-  // gain at every length (2000 tokens 9.3 / 8.6, 32768 54.4 / 48.7).
+  // Steps of two units need blocks with an even number of them, and pay from a number of units per CTA on: with fewer the
+  // coarser split and the longer first step cost more.  us per launch, one unit / two units per step: two tiers, G = 32 (7b
+  // shape, batch 8) 8000 tokens, 27 units per CTA, 12.6 / 13.1, 16000 21.5 / 20.5; G = 128 (32b shape, batch 16) 2000 tokens,
+  // 31 units, 13.5 / 13.0, 600 tokens, 10 units, 8.3 / 8.15; three tiers (7b shape) 600 tokens, 3 units, 6.4 / 6.7, 2000 tokens,
+  // 7 units, 9.3 / 7.8; 4-bit base (8b shape, batch 16) 600 tokens, 12 units, 8.9 / 9.3, 2000 tokens, 31 units, 18.7 / 17.7.
   const bool three_tiers = !lv.dense_hi && ((lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16);
-  const bool by_two = !(lv.U & 1) && (three_tiers || (lv.seq != nullptr ? lv.seq_total : Us * S) >= 40ll * grid);
+  const int from_units = three_tiers ? 6 : lv.dense_hi ? 20 : lv.G == 128 ? 10 : 40;
+  const bool by_two = !(lv.U & 1) && (lv.seq != nullptr ? lv.seq_total : Us * S) >= (long long)from_units * grid;
   cudaError_t e;
   if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, stream);
   else if (lv.G == 32) e = launch_g<32>(lv, q, scale, ws, grid, stream);
