@@ -9,14 +9,19 @@
 //   warp 9           one thread issues the bulk copies of the K and V tiles into two-stage rings.
 // Per key tile j and row group g:
 //   S_g = Q_g K_j^T   bf16 operands from shared memory, fp32 accumulator in tensor memory;
-//   softmax           the thread reads its row of S (tcgen05.ld), applies scale and causal mask, keeps the running
-//                     maximum and sum, and writes its row of P as fp16 over the columns S occupied (tcgen05.st);
-//   T_g = P_g V_j     A operand from tensor memory, V from shared memory (MN-major), into a second accumulator that
-//                     the thread folds into its fp32 output row in registers: o = o * alpha + T.
+//   softmax           the thread reads its row of S (tcgen05.ld), applies scale and causal mask, and writes its row of P as
+//                     fp16 over columns that S occupied (tcgen05.st).  When the maximum of a row of the warp rises, the warp
+//                     rescales its rows of O (after the first tiles that is rare: a third of the 256 tiles at L = 32768);
+//   O_g += P_g V_j    A operand from tensor memory, V from shared memory (MN-major), accumulated in tensor memory.
 // The issue order S_A(j+1) behind P_A V(j), S_B(j+1) behind P_B V(j) keeps the tensor core busy on one row group while
-// the other one is in its softmax.  P and V are fp16 (11 significant bits): bf16 probabilities alone would cost up to
+// the other one is in its softmax; the softmax threads never wait for a P V product (products complete in issue order, so S(j)
+// being there means that P V(j-1) is done).  P and V are fp16 (11 significant bits): bf16 probabilities alone would cost up to
 // 2^-9 of the value range.  Every wait on a barrier is bounded; a wait that runs out sets the status word and the
 // role that saw it stops, after which the others run out too and the CTA finishes.
+// B200, whole call per layer, against the form whose threads kept O in registers and folded every P V into it (us): prompt of
+// 32768 tokens (7b shape) 7990 -> 7206, 8192: 690 -> 566, 333: 102 -> 48; 4 x 777 tokens (8b shape) 176 -> 121.  What went: the
+// wait for P V and the fold (1.6 of 3.9 thousand cycles per tile), 5 of 7 thousand cycles per masked diagonal tile, the Q load
+// one piece after the other (4 of 9 thousand cycles per CTA), the wait for the first K and V behind it.
 #include "common.cuh"
 
 namespace mixkvq {
@@ -27,9 +32,9 @@ constexpr int kTile = 128;                       // query rows and key rows per 
 constexpr int kTileBytes = kTile * kD * 2;       // one 128 x 128 tile of 16-bit elements
 constexpr int kQRows = 2 * kTile;                // query rows per CTA
 constexpr int kThreads = 384;
-constexpr int kBars = 17;
+constexpr int kBars = 13;
 constexpr int kSmem = 6 * kTileBytes + 256;      // two Q tiles, two K and two V stages; barriers and tensor-memory slot
-enum Bar { kKFull = 0, kVFull = 2, kKEmpty = 4, kVEmpty = 6, kSFull = 8, kPReady = 10, kTFull = 12, kTFree = 14, kDone = 16 };
+enum Bar { kKFull = 0, kVFull = 2, kKEmpty = 4, kVEmpty = 6, kSFull = 8, kPReady = 10, kDone = 12 };
 constexpr uint32_t kPolls = 1u << 21;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -102,25 +107,19 @@ __device__ __forceinline__ void tmem_wait_ld32(uint32_t (&u)[32]) {
                :
                : "memory");
 }
-__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&u)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]),
-        "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld16(uint32_t (&u)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]), "+r"(u[7]), "+r"(u[8]),
-                 "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]), "+r"(u[15])
-               :
-               : "memory");
-}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&w)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(w[0]), "r"(w[1]),
                "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
                : "memory");
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&u)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+      "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]), "r"(u[8]), "r"(u[9]), "r"(u[10]),
+      "r"(u[11]), "r"(u[12]), "r"(u[13]), "r"(u[14]), "r"(u[15]), "r"(u[16]), "r"(u[17]), "r"(u[18]), "r"(u[19]), "r"(u[20]),
+      "r"(u[21]), "r"(u[22]), "r"(u[23]), "r"(u[24]), "r"(u[25]), "r"(u[26]), "r"(u[27]), "r"(u[28]), "r"(u[29]), "r"(u[30]), "r"(u[31])
+      : "memory");
 }
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -184,74 +183,163 @@ prefill_pack_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __
   }
 }
 
-// One 128-key tile of one row group's softmax.  The thread owns one row of S (128 fp32 columns of its tensor-memory
-// lane at s_addr); columns >= n_valid are masked.  Writes P (fp16 pairs) over columns [0, 64) of the same range.
-template <bool kMask>
-__device__ __forceinline__ void softmax_tile(uint32_t s_addr, int n_valid, float scale_log2e, float& m_run, float& l_run,
-                                             float& alpha) {
-  // ---- pass 1: the row maximum; chunk c + 1 is in flight while chunk c is reduced
+// Two fp32 values in one 64-bit register: the FMA pipe does both halves of these with one instruction.
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t pack2u(uint32_t a, uint32_t b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// One 128-key tile of one row group's softmax.  The thread owns one row of S (128 fp32 columns of its tensor-memory lane at
+// s_addr) and of O (at o_addr).  Writes P (fp16 pairs) over columns [0, 64) of S.  kDiag: the tile on the diagonal, where row i
+// of the group sees columns <= i: warp w (rows 32 w ..) needs the columns of 32-chunks <= w, and a comparison only in chunk w.
+template <bool kDiag>
+__device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, int w, int lane, bool first, float scale_log2e,
+                                             float& m_ref, float& l_run) {
+  // ---- the row's maximum
   float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // four independent chains
-  {
-    uint32_t a[32], b[32];
-    auto reduce = [&](const uint32_t (&u)[32], int cc) {
+  auto reduce = [&](const uint32_t (&u)[32], int last) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i)
-        mx4[i & 3] = fmaxf(mx4[i & 3], (!kMask || 32 * cc + i < n_valid) ? __uint_as_float(u[i]) : -INFINITY);
-    };
+    for (int i = 0; i < 32; i += 2) {
+      const float x0 = kDiag && i > last ? -INFINITY : __uint_as_float(u[i]);
+      const float x1 = kDiag && i + 1 > last ? -INFINITY : __uint_as_float(u[i + 1]);
+      mx4[(i >> 1) & 3] = fmaxf(fmaxf(mx4[(i >> 1) & 3], x0), x1);
+    }
+  };
+  if constexpr (kDiag) {
+#pragma unroll 1
+    for (int c = 0; c <= w; ++c) {
+      uint32_t a[32];
+      tmem_ld32_issue(s_addr + 32 * c, a);
+      tmem_wait_ld32(a);
+      reduce(a, c == w ? lane : 31);
+    }
+  } else {
+    uint32_t a[32], b[32];                          // chunk c + 1 is in flight while chunk c is reduced
     tmem_ld32_issue(s_addr, a);
     tmem_wait_ld32(a);
     tmem_ld32_issue(s_addr + 32, b);
-    reduce(a, 0);
+    reduce(a, 31);
     tmem_wait_ld32(b);
     tmem_ld32_issue(s_addr + 64, a);
-    reduce(b, 1);
+    reduce(b, 31);
     tmem_wait_ld32(a);
     tmem_ld32_issue(s_addr + 96, b);
-    reduce(a, 2);
+    reduce(a, 31);
     tmem_wait_ld32(b);
-    reduce(b, 3);
+    reduce(b, 31);
   }
-  const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-  const float m_new = fmaxf(m_run, mx * scale_log2e);
-  alpha = ex2(m_run - m_new);                       // 0 on the first tile
-  // ---- pass 2: probabilities in chunks of 16 columns, the next chunk in flight; P chunk c (8 columns of fp16 pairs)
-  // lies inside the S columns of chunks <= c, which are already in registers
-  float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
-  {
-    uint32_t a[16], b[16];
-    auto probs = [&](const uint32_t (&u)[16], int cc) {
-      uint32_t w[8];
+  const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale_log2e;
+  if (first) {
+    m_ref = mx;
+  } else if (__any_sync(0xffffffffu, mx > m_ref)) {
+    // raise the reference and rescale what has been accumulated (all products before this S have completed)
+    const float m_new = fmaxf(m_ref, mx), alpha = ex2(m_ref - m_new);
+    const uint64_t alpha2 = pack2(alpha, alpha);
+    uint32_t x[32], y[32];                          // chunk c + 1 is in flight while chunk c is scaled
+    auto rescale = [&](uint32_t (&z)[32], int c) {
+#pragma unroll
+      for (int k = 0; k < 32; k += 2) {
+        float a, b;
+        unpack2(mul2(pack2u(z[k], z[k + 1]), alpha2), a, b);
+        z[k] = __float_as_uint(a);
+        z[k + 1] = __float_as_uint(b);
+      }
+      tmem_st32(o_addr + 32 * c, z);
+    };
+    tmem_ld32_issue(o_addr, x);
+    tmem_wait_ld32(x);
+    tmem_ld32_issue(o_addr + 32, y);
+    rescale(x, 0);
+    tmem_wait_ld32(y);
+    tmem_ld32_issue(o_addr + 64, x);
+    rescale(y, 1);
+    tmem_wait_ld32(x);
+    tmem_ld32_issue(o_addr + 96, y);
+    rescale(x, 2);
+    tmem_wait_ld32(y);
+    rescale(y, 3);
+    l_run *= alpha;
+    m_ref = m_new;
+  }
+  // ---- probabilities in chunks of 32 columns; P chunk c (16 columns of fp16 pairs) lies inside the S columns of chunks
+  // <= c, which are already in registers
+  const uint64_t scale2 = pack2(scale_log2e, scale_log2e), ref2 = pack2(-m_ref, -m_ref);
+  uint64_t sum[2] = {0ull, 0ull};
+  auto probs = [&](const uint32_t (&u)[32], int c, int last) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      uint32_t wd[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const int c0 = 16 * cc + 2 * i;
-        const float p0 = (!kMask || c0 < n_valid) ? ex2(fmaf(__uint_as_float(u[2 * i]), scale_log2e, -m_new)) : 0.f;
-        const float p1 = (!kMask || c0 + 1 < n_valid) ? ex2(fmaf(__uint_as_float(u[2 * i + 1]), scale_log2e, -m_new)) : 0.f;
-        if (i & 1) {
-          sum2 += p0;
-          sum3 += p1;
-        } else {
-          sum0 += p0;
-          sum1 += p1;
+        const int k = 16 * half + 2 * i;
+        float x0, x1;
+        unpack2(fma2(pack2u(u[k], u[k + 1]), scale2, ref2), x0, x1);
+        float p0 = ex2(x0), p1 = ex2(x1);
+        if constexpr (kDiag) {
+          p0 = k <= last ? p0 : 0.f;
+          p1 = k + 1 <= last ? p1 : 0.f;
         }
-        w[i] = pack_half2(p0, p1);
+        sum[i & 1] = add2(sum[i & 1], pack2(p0, p1));
+        wd[i] = pack_half2(p0, p1);
       }
-      tmem_st8(s_addr + 8 * cc, w);
-    };
-    tmem_ld16_issue(s_addr, a);
-    tmem_wait_ld16(a);
-#pragma unroll
-    for (int cc = 0; cc < 8; cc += 2) {
-      tmem_ld16_issue(s_addr + 16 * (cc + 1), b);
-      probs(a, cc);                                // writes columns [8 cc, 8 cc + 8): all inside chunks <= cc
-      tmem_wait_ld16(b);
-      if (cc + 2 < 8) tmem_ld16_issue(s_addr + 16 * (cc + 2), a);
-      probs(b, cc + 1);
-      if (cc + 2 < 8) tmem_wait_ld16(a);
+      tmem_st8(s_addr + 16 * c + 8 * half, wd);
     }
+  };
+  if constexpr (kDiag) {
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+      if (c <= w) {
+        uint32_t a[32];
+        tmem_ld32_issue(s_addr + 32 * c, a);
+        tmem_wait_ld32(a);
+        probs(a, c, c == w ? lane : 31);
+      } else {
+        const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+        tmem_st8(s_addr + 16 * c, zero);
+        tmem_st8(s_addr + 16 * c + 8, zero);
+      }
+    }
+  } else {
+    uint32_t a[32], b[32];                          // the next chunk in flight
+    tmem_ld32_issue(s_addr, a);
+    tmem_wait_ld32(a);
+    tmem_ld32_issue(s_addr + 32, b);
+    probs(a, 0, 31);
+    tmem_wait_ld32(b);
+    tmem_ld32_issue(s_addr + 64, a);
+    probs(b, 1, 31);
+    tmem_wait_ld32(a);
+    tmem_ld32_issue(s_addr + 96, b);
+    probs(a, 2, 31);
+    tmem_wait_ld32(b);
+    probs(b, 3, 31);
   }
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-  l_run = l_run * alpha + ((sum0 + sum1) + (sum2 + sum3));
-  m_run = m_new;
+  float s0, s1;
+  unpack2(add2(sum[0], sum[1]), s0, s1);
+  l_run += s0 + s1;
 }
 
 // q [B, Hq, L, 128] bf16; kt, vt the tile images of prefill_pack_kernel; out [B, Hq, L, 128] fp32.  blockIdx.x / BH
@@ -282,23 +370,44 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  int issued = 0;                  // K and V tiles requested (the copying thread)
+  auto copy_tile = [&](int j, bool keys) {
+    const int st = j & 1, full = (keys ? kKFull : kVFull) + st;
+    // (test hook: the first copy's barrier can be armed for more bytes than arrive, so that it never completes)
+    mbar_expect_tx(bar(full), kTileBytes + (keys && j == 0 ? debug_extra_tx : 0u));
+    bulk_copy(smem_u32((keys ? Ks : Vs) + st * kTileBytes), (keys ? ktg : vtg) + (size_t)j * kTileBytes, kTileBytes, bar(full));
+  };
   if (tid == 9 * 32) {
-    for (int i = 0; i < kBars; ++i) mbar_init(bar(i), (i >= kPReady && i < kTFull) || (i >= kTFree && i < kDone) ? kTile : 1);
+    for (int i = 0; i < kBars; ++i) mbar_init(bar(i), i >= kPReady && i < kDone ? kTile : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // the first tiles are under way while Q is loaded
+    for (; issued < min(2, n_b); ++issued) {
+      copy_tile(issued, true);
+      copy_tile(issued, false);
+    }
   }
-  // both Q tiles: piece i of a tile is 16 bytes at byte 16 i of its image (rows past L are zero)
-  for (int i = tid; i < 2 * kTile * 16; i += kThreads) {
-    const int ii = i & 2047, r = (i >> 11) * kTile + 8 * (ii >> 7) + (ii & 7), c = (ii >> 3) & 15;
-    uint4 x = make_uint4(0u, 0u, 0u, 0u);
-    if (qt * kQRows + r < L) x = *reinterpret_cast<const uint4*>(qg + (size_t)(qt * kQRows + r) * kD + 8 * c);
-    reinterpret_cast<uint4*>(Qs)[i] = x;
+  // both Q tiles: piece i of a tile is 16 bytes at byte 16 i of its image (rows past L are zero).  All of a thread's loads are
+  // in flight at once (one after the other they took 8000 to 12000 cycles of a CTA that needs 3900 per key tile).
+  {
+    constexpr int kPieces = 2 * kTile * 16, kEach = (kPieces + kThreads - 1) / kThreads;
+    uint4 x[kEach];
+#pragma unroll
+    for (int k = 0; k < kEach; ++k) {
+      const int i = tid + k * kThreads, ii = i & 2047, r = (i >> 11) * kTile + 8 * (ii >> 7) + (ii & 7), c = (ii >> 3) & 15;
+      x[k] = make_uint4(0u, 0u, 0u, 0u);
+      if (i < kPieces && qt * kQRows + r < L) x[k] = *reinterpret_cast<const uint4*>(qg + (size_t)(qt * kQRows + r) * kD + 8 * c);
+    }
+#pragma unroll
+    for (int k = 0; k < kEach; ++k)
+      if (tid + k * kThreads < kPieces) reinterpret_cast<uint4*>(Qs)[tid + k * kThreads] = x[k];
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // Q is read by the tensor core
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = *tmem_slot;
-  // tensor-memory columns: S_A / P_A at 0, S_B / P_B at 128, T_A at 256, T_B at 384
+  // tensor-memory columns: S_A / P_A at 0, S_B / P_B at 128, O_A at 256, O_B at 384
   bool dead = false;
   auto wait = [&](int i, uint32_t parity) {
     if (!dead && !mbar_wait_polls(bar(i), parity, max_polls)) {
@@ -320,11 +429,10 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
         for (int ks = 0; ks < 8; ++ks) tc_mma_ss(tbase + 128 * g, qd + (uint64_t)(ks * 16), kd + (uint64_t)(ks * 16), idesc_qk, ks > 0);
         tc_commit(bar(kSFull + g));
       };
-      auto issue_t = [&](int g, int j) {                 // T_g = P_g V_j
+      auto issue_o = [&](int g, int j) {                 // O_g += P_g V_j
         const uint64_t vd = make_desc(smem_u32(Vs + (j & 1) * kTileBytes), 128, 2048);
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) tc_mma_ts(tbase + 256 + 128 * g, tbase + 128 * g + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, ks > 0);
-        tc_commit(bar(kTFull + g));
+        for (int ks = 0; ks < 8; ++ks) tc_mma_ts(tbase + 256 + 128 * g, tbase + 128 * g + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, j > 0 || ks > 0);
       };
       if (wait(kKFull, 0)) {
         tc_fence_after();
@@ -338,9 +446,8 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
         if (!wait(kVFull + st, ph)) break;
         if (j < n_a) {
           if (!wait(kPReady, (uint32_t)j & 1u)) break;
-          if (j > 0 && !wait(kTFree, (uint32_t)(j - 1) & 1u)) break;
           tc_fence_after();
-          issue_t(0, j);
+          issue_o(0, j);
           if (j + 1 < n_a) {
             if (!wait(kKFull + nx, ph_nx)) break;
             tc_fence_after();
@@ -348,9 +455,8 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
           }
         }
         if (!wait(kPReady + 1, (uint32_t)j & 1u)) break;
-        if (j > 0 && !wait(kTFree + 1, (uint32_t)(j - 1) & 1u)) break;
         tc_fence_after();
-        issue_t(1, j);
+        issue_o(1, j);
         tc_commit(bar(kVEmpty + st));
         if (j + 1 < n_b) {
           if (!wait(kKFull + nx, ph_nx)) break;
@@ -364,22 +470,17 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
       wait(kDone, 0);
     } else if (warp == 9 && lane == 0) {
       // ---------------------------------------------------------------- bulk copies of the K and V tiles
-      int issued = 0;
-      for (int j = 0; j < n_b; ++j) {
+      for (int j = 2; j < n_b; ++j) {
         const int st = j & 1;
         const uint32_t ph_prev = (uint32_t)((j >> 1) - 1) & 1u;
-        if (j >= 2 && !wait(kKEmpty + st, ph_prev)) break;
-        // (test hook: the first copy's barrier can be armed for more bytes than arrive, so that it never completes)
-        mbar_expect_tx(bar(kKFull + st), kTileBytes + (j == 0 ? debug_extra_tx : 0u));
-        bulk_copy(smem_u32(Ks + st * kTileBytes), ktg + (size_t)j * kTileBytes, kTileBytes, bar(kKFull + st));
-        if (j >= 2 && !wait(kVEmpty + st, ph_prev)) {   // the K copy above is awaited below like the others
-          issued = j + 1;
+        if (!wait(kKEmpty + st, ph_prev)) break;
+        copy_tile(j, true);
+        issued = j + 1;
+        if (!wait(kVEmpty + st, ph_prev)) {               // the K copy above is awaited below like the others
           mbar_expect_tx(bar(kVFull + st), 0);
           break;
         }
-        mbar_expect_tx(bar(kVFull + st), kTileBytes);
-        bulk_copy(smem_u32(Vs + st * kTileBytes), vtg + (size_t)j * kTileBytes, kTileBytes, bar(kVFull + st));
-        issued = j + 1;
+        copy_tile(j, false);
       }
       // no copy may be in flight when the CTA ends: the last copy into each stage has landed once its barrier's phase is over
       for (int j = max(0, issued - 2); j < issued; ++j) {
@@ -394,53 +495,50 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     // ------------------------------------------------------------------ softmax and output rows
     const int g = warp >> 2, row = tid & 127;
     const uint32_t lane_base = tbase + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t s_addr = lane_base + 128 * g, t_addr = lane_base + 256 + 128 * g;
+    const uint32_t s_addr = lane_base + 128 * g, o_addr = lane_base + 256 + 128 * g;
     const int n = g == 0 ? n_a : n_b;
     const int pos = qt * kQRows + g * kTile + row;     // this thread's query position
-    float o[kD];
-#pragma unroll
-    for (int d = 0; d < kD; ++d) o[d] = 0.f;
-    float m_run = -INFINITY, l_run = 0.f, alpha = 0.f;
+    float m_ref = -INFINITY, l_run = 0.f;
 #pragma unroll 1
     for (int j = 0; j < n; ++j) {
       if (!wait(kSFull + g, (uint32_t)j & 1u)) break;
       tc_fence_after();
-      if ((j + 1) * kTile - 1 > qt * kQRows + g * kTile)      // the tile reaches past the group's first row
-        softmax_tile<true>(s_addr, pos - j * kTile + 1, scale_log2e, m_run, l_run, alpha);
+      if (j == 2 * qt + g)      // the tile on the diagonal
+        softmax_tile<true>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run);
       else
-        softmax_tile<false>(s_addr, kTile, scale_log2e, m_run, l_run, alpha);
+        softmax_tile<false>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run);
       tc_fence_before();
       mbar_arrive(bar(kPReady + g));
-      if (!wait(kTFull + g, (uint32_t)j & 1u)) break;
-      tc_fence_after();
-      {
-        uint32_t xa[32], xb[32];
-        tmem_ld32_issue(t_addr, xa);
-        tmem_wait_ld32(xa);
-        tmem_ld32_issue(t_addr + 32, xb);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] = fmaf(o[i], alpha, __uint_as_float(xa[i]));
-        tmem_wait_ld32(xb);
-        tmem_ld32_issue(t_addr + 64, xa);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) o[32 + i] = fmaf(o[32 + i], alpha, __uint_as_float(xb[i]));
-        tmem_wait_ld32(xa);
-        tmem_ld32_issue(t_addr + 96, xb);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) o[64 + i] = fmaf(o[64 + i], alpha, __uint_as_float(xa[i]));
-        tmem_wait_ld32(xb);
-        // T is in registers: the tensor core may overwrite it while the last chunk is folded in
-        tc_fence_before();
-        mbar_arrive(bar(kTFree + g));
-#pragma unroll
-        for (int i = 0; i < 32; ++i) o[96 + i] = fmaf(o[96 + i], alpha, __uint_as_float(xb[i]));
-      }
     }
-    if (pos < L && !dead) {
+    if (wait(kDone, 0)) {
+      tc_fence_after();
       const float inv = 1.f / l_run;
-      float4* dst = reinterpret_cast<float4*>(out + ((size_t)(b * Hq + h) * L + pos) * kD);
+      // the thread's row in 32-byte stores where the caller's buffer allows (whole sectors: the rows of a warp are 512 bytes
+      // apart), else in 16-byte stores
+      float* dst = out + ((size_t)(b * Hq + h) * L + pos) * kD;
+      const bool wide = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
 #pragma unroll
-      for (int d = 0; d < kD; d += 4) dst[d >> 2] = make_float4(o[d] * inv, o[d + 1] * inv, o[d + 2] * inv, o[d + 3] * inv);
+      for (int c = 0; c < 4; ++c) {
+        uint32_t x[32];
+        tmem_ld32_issue(o_addr + 32 * c, x);
+        tmem_wait_ld32(x);
+        if (pos < L) {
+#pragma unroll
+          for (int d = 0; d < 32; d += 8) {
+            float y[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) y[k] = __uint_as_float(x[d + k]) * inv;
+            if (wide) {
+              asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 32 * c + d), "f"(y[0]), "f"(y[1]),
+                           "f"(y[2]), "f"(y[3]), "f"(y[4]), "f"(y[5]), "f"(y[6]), "f"(y[7])
+                           : "memory");
+            } else {
+              reinterpret_cast<float4*>(dst + 32 * c + d)[0] = make_float4(y[0], y[1], y[2], y[3]);
+              reinterpret_cast<float4*>(dst + 32 * c + d)[1] = make_float4(y[4], y[5], y[6], y[7]);
+            }
+          }
+        }
+      }
     }
   }
   tc_fence_before();
