@@ -32,9 +32,9 @@ constexpr int kTile = 128;                       // query rows and key rows per 
 constexpr int kTileBytes = kTile * kD * 2;       // one 128 x 128 tile of 16-bit elements
 constexpr int kQRows = 2 * kTile;                // query rows per CTA
 constexpr int kThreads = 384;
-constexpr int kBars = 13;
+constexpr int kBars = 16;
 constexpr int kSmem = 6 * kTileBytes + 256;      // two Q tiles, two K and two V stages; barriers and tensor-memory slot
-enum Bar { kKFull = 0, kVFull = 2, kKEmpty = 4, kVEmpty = 6, kSFull = 8, kPReady = 10, kDone = 12 };
+enum Bar { kKFull = 0, kVFull = 2, kKEmpty = 4, kVEmpty = 6, kSFull = 8, kPHalf = 10, kPReady = 12, kDoneA = 14, kDone = 15 };
 constexpr uint32_t kPolls = 1u << 21;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -216,7 +216,7 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 // of the group sees columns <= i: warp w (rows 32 w ..) needs the columns of 32-chunks <= w, and a comparison only in chunk w.
 template <bool kDiag>
 __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, int w, int lane, bool first, float scale_log2e,
-                                             float& m_ref, float& l_run) {
+                                             float& m_ref, float& l_run, uint32_t half_bar) {
   // ---- the row's maximum
   float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // four independent chains
   auto reduce = [&](const uint32_t (&u)[32], int last) {
@@ -283,6 +283,12 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, i
     l_run *= alpha;
     m_ref = m_new;
   }
+  // P of the first 64 keys is handed over on its own: its products run while the other half is computed
+  auto half_ready = [&]() {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    tc_fence_before();
+    mbar_arrive(half_bar);
+  };
   // ---- probabilities in chunks of 32 columns; P chunk c (16 columns of fp16 pairs) lies inside the S columns of chunks
   // <= c, which are already in registers
   const uint64_t scale2 = pack2(scale_log2e, scale_log2e), ref2 = pack2(-m_ref, -m_ref);
@@ -320,6 +326,7 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, i
         tmem_st8(s_addr + 16 * c, zero);
         tmem_st8(s_addr + 16 * c + 8, zero);
       }
+      if (c == 1) half_ready();
     }
   } else {
     uint32_t a[32], b[32];                          // the next chunk in flight
@@ -330,6 +337,7 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, i
     tmem_wait_ld32(b);
     tmem_ld32_issue(s_addr + 64, a);
     probs(b, 1, 31);
+    half_ready();
     tmem_wait_ld32(a);
     tmem_ld32_issue(s_addr + 96, b);
     probs(a, 2, 31);
@@ -378,7 +386,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     bulk_copy(smem_u32((keys ? Ks : Vs) + st * kTileBytes), (keys ? ktg : vtg) + (size_t)j * kTileBytes, kTileBytes, bar(full));
   };
   if (tid == 9 * 32) {
-    for (int i = 0; i < kBars; ++i) mbar_init(bar(i), i >= kPReady && i < kDone ? kTile : 1);
+    for (int i = 0; i < kBars; ++i) mbar_init(bar(i), i >= kPHalf && i < kDoneA ? kTile : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     // the first tiles are under way while Q is loaded
@@ -429,10 +437,22 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
         for (int ks = 0; ks < 8; ++ks) tc_mma_ss(tbase + 128 * g, qd + (uint64_t)(ks * 16), kd + (uint64_t)(ks * 16), idesc_qk, ks > 0);
         tc_commit(bar(kSFull + g));
       };
-      auto issue_o = [&](int g, int j) {                 // O_g += P_g V_j
+      auto issue_o = [&](int g, int j, int half) {       // O_g += P_g V_j over 64 of the tile's keys
         const uint64_t vd = make_desc(smem_u32(Vs + (j & 1) * kTileBytes), 128, 2048);
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) tc_mma_ts(tbase + 256 + 128 * g, tbase + 128 * g + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, j > 0 || ks > 0);
+        for (int k = 0; k < 4; ++k) {
+          const int ks = 4 * half + k;
+          tc_mma_ts(tbase + 256 + 128 * g, tbase + 128 * g + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, j > 0 || ks > 0);
+        }
+      };
+      auto both_halves = [&](int g, int j) {             // as soon as each half of P_g is there
+        if (!wait(kPHalf + g, (uint32_t)j & 1u)) return false;
+        tc_fence_after();
+        issue_o(g, j, 0);
+        if (!wait(kPReady + g, (uint32_t)j & 1u)) return false;
+        tc_fence_after();
+        issue_o(g, j, 1);
+        return true;
       };
       if (wait(kKFull, 0)) {
         tc_fence_after();
@@ -445,18 +465,15 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
         const uint32_t ph = (uint32_t)(j >> 1) & 1u, ph_nx = (uint32_t)((j + 1) >> 1) & 1u;
         if (!wait(kVFull + st, ph)) break;
         if (j < n_a) {
-          if (!wait(kPReady, (uint32_t)j & 1u)) break;
-          tc_fence_after();
-          issue_o(0, j);
+          if (!both_halves(0, j)) break;
+          if (j + 1 == n_a) tc_commit(bar(kDoneA));
           if (j + 1 < n_a) {
             if (!wait(kKFull + nx, ph_nx)) break;
             tc_fence_after();
             issue_s(0, j + 1);
           }
         }
-        if (!wait(kPReady + 1, (uint32_t)j & 1u)) break;
-        tc_fence_after();
-        issue_o(1, j);
+        if (!both_halves(1, j)) break;
         tc_commit(bar(kVEmpty + st));
         if (j + 1 < n_b) {
           if (!wait(kKFull + nx, ph_nx)) break;
@@ -504,40 +521,55 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
       if (!wait(kSFull + g, (uint32_t)j & 1u)) break;
       tc_fence_after();
       if (j == 2 * qt + g)      // the tile on the diagonal
-        softmax_tile<true>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run);
+        softmax_tile<true>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g));
       else
-        softmax_tile<false>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run);
+        softmax_tile<false>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g));
       tc_fence_before();
       mbar_arrive(bar(kPReady + g));
     }
-    if (wait(kDone, 0)) {
+    // Output rows.  The rows of a warp are 512 bytes apart, so direct stores cost a wavefront per lane (10 thousand cycles for
+    // 256 rows at once, about half for 128).  Group A is done a tile earlier than group B and stores directly, in 32-byte
+    // pieces where the caller's buffer allows, under B's last tile; B's rows go through the shared memory, which nobody needs
+    // any more, and leave as one bulk copy each.
+    if (wait(g == 0 ? kDoneA : kDone, 0)) {
       tc_fence_after();
       const float inv = 1.f / l_run;
-      // the thread's row in 32-byte stores where the caller's buffer allows (whole sectors: the rows of a warp are 512 bytes
-      // apart), else in 16-byte stores
       float* dst = out + ((size_t)(b * Hq + h) * L + pos) * kD;
       const bool wide = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
+      const uint32_t staged = smem_u32(smem) + (uint32_t)row * 528u;      // (a row's 16-byte pieces on the banks of no other lane)
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         uint32_t x[32];
         tmem_ld32_issue(o_addr + 32 * c, x);
         tmem_wait_ld32(x);
-        if (pos < L) {
+        float y[32];
+#pragma unroll
+        for (int d = 0; d < 32; ++d) y[d] = __uint_as_float(x[d]) * inv;
+        if (g == 1) {
+#pragma unroll
+          for (int d = 0; d < 32; d += 4)
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(staged + 4 * (32 * c + d)), "f"(y[d]), "f"(y[d + 1]),
+                         "f"(y[d + 2]), "f"(y[d + 3])
+                         : "memory");
+        } else if (pos < L) {
 #pragma unroll
           for (int d = 0; d < 32; d += 8) {
-            float y[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) y[k] = __uint_as_float(x[d + k]) * inv;
             if (wide) {
-              asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 32 * c + d), "f"(y[0]), "f"(y[1]),
-                           "f"(y[2]), "f"(y[3]), "f"(y[4]), "f"(y[5]), "f"(y[6]), "f"(y[7])
+              asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 32 * c + d), "f"(y[d]), "f"(y[d + 1]),
+                           "f"(y[d + 2]), "f"(y[d + 3]), "f"(y[d + 4]), "f"(y[d + 5]), "f"(y[d + 6]), "f"(y[d + 7])
                            : "memory");
             } else {
-              reinterpret_cast<float4*>(dst + 32 * c + d)[0] = make_float4(y[0], y[1], y[2], y[3]);
-              reinterpret_cast<float4*>(dst + 32 * c + d)[1] = make_float4(y[4], y[5], y[6], y[7]);
+              reinterpret_cast<float4*>(dst + 32 * c + d)[0] = make_float4(y[d], y[d + 1], y[d + 2], y[d + 3]);
+              reinterpret_cast<float4*>(dst + 32 * c + d)[1] = make_float4(y[d + 4], y[d + 5], y[d + 6], y[d + 7]);
             }
           }
         }
+      }
+      if (g == 1 && pos < L) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(staged), "r"(kD * 4) : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       }
     }
   }
