@@ -167,6 +167,22 @@ int zero_layer_state(mixkvq_cache* h, int layer, cudaStream_t st) {
   return MIXKVQ_OK;
 }
 
+// all layers at once: one strided fill instead of one per layer
+int zero_all_layers(mixkvq_cache* h, cudaStream_t st) {
+  if (h->layer_stride > 0x7FFFFFFFull) {          // beyond the pitch that a strided fill takes
+    for (int l = 0; l < h->cfg.n_layers; ++l)
+      if (zero_layer_state(h, l, st) != MIXKVQ_OK) return MIXKVQ_E_CUDA;
+    return MIXKVQ_OK;
+  }
+  if (cudaMemset2DAsync(h->mem + kHeaderBytes + h->state_off, h->layer_stride, 0, h->state_stride * h->S, h->cfg.n_layers, st) != cudaSuccess)
+    return MIXKVQ_E_CUDA;
+  std::fill(h->n_blocks.begin(), h->n_blocks.end(), 0);
+  std::fill(h->r.begin(), h->r.end(), 0);
+  std::fill(h->n_sink.begin(), h->n_sink.end(), 0);
+  h->last_packed_writer = kAllPacked;
+  return MIXKVQ_OK;
+}
+
 // Ragged batch: writes the fills of the layer's sequences to its table in device memory (as kernel arguments: ordered
 // in the stream, no copy) and points the view at it.
 int upload_seq_table(mixkvq_cache* h, int layer, cudaStream_t st, LayerView* lv) {
@@ -227,7 +243,7 @@ int run_attention(mixkvq_cache* h, int layer, const void* q, float* out, float s
 // Appends tokens 0 .. n_tokens - 1 of the tensors (whose token dimension is n_stride long) to sequences b0 .. b0 + nb - 1,
 // which share one fill: sink rows first, then flush / bulk blocks / residual rows as the fill demands.
 int append_run_first(mixkvq_cache* cache, int layer, int b0, int nb, const void* k_dev, const void* v_dev, const void* q_dev,
-                     int n_stride, int n_tokens, cudaStream_t st) {
+                     int n_stride, int n_tokens, bool behind_prefill, cudaStream_t st) {
   const char* k = static_cast<const char*>(k_dev) + (size_t)b0 * cache->cfg.n_kv_heads * n_stride * kD * 2;
   const char* v = static_cast<const char*>(v_dev) + (size_t)b0 * cache->cfg.n_kv_heads * n_stride * kD * 2;
   const char* q = static_cast<const char*>(q_dev) + (size_t)b0 * cache->cfg.n_q_heads * n_stride * kD * 2;
@@ -264,7 +280,7 @@ int append_run_first(mixkvq_cache* cache, int layer, int b0, int nb, const void*
       if (nblk > 32768) nblk = 32768;                  // grid.y limit
       const int left = n_tokens - t - nblk * cache->R, tail = left <= cache->R ? left : 0;
       LayerView lv = view(cache, layer, b0, nb);
-      if (launch_flush_bulk(lv, k, v, q, n_stride, t, nblk, tail, st) != cudaSuccess) return MIXKVQ_E_CUDA;
+      if (launch_flush_bulk(lv, k, v, q, n_stride, t, nblk, tail, behind_prefill && t == 0, st) != cudaSuccess) return MIXKVQ_E_CUDA;
       cache->launches += cache->cfg.importance_mode == 1 ? 3 : 2;
       cache->last_packed_writer = layer;
       nb0 += nblk;
@@ -284,8 +300,8 @@ int append_run_first(mixkvq_cache* cache, int layer, int b0, int nb, const void*
 }
 
 int append_run(mixkvq_cache* cache, int layer, int b0, int nb, const void* k_dev, const void* v_dev, const void* q_dev,
-               int n_stride, int n_tokens, cudaStream_t st) {
-  const int rc = append_run_first(cache, layer, b0, nb, k_dev, v_dev, q_dev, n_stride, n_tokens, st);
+               int n_stride, int n_tokens, bool behind_prefill, cudaStream_t st) {
+  const int rc = append_run_first(cache, layer, b0, nb, k_dev, v_dev, q_dev, n_stride, n_tokens, behind_prefill, st);
   for (int b = b0 + 1; b < b0 + nb; ++b) {
     cache->n_sink[fi(cache, layer, b)] = cache->n_sink[fi(cache, layer, b0)];
     cache->r[fi(cache, layer, b)] = cache->r[fi(cache, layer, b0)];
@@ -334,8 +350,7 @@ int mixkvq_cache_init(const mixkvq_config* cfg, void* cache_dev, size_t bytes, v
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(h->mem, 0, kHeaderBytes, st) != cudaSuccess) { delete h; return MIXKVQ_E_CUDA; }
-  for (int l = 0; l < cfg->n_layers; ++l)
-    if (zero_layer_state(h, l, st) != MIXKVQ_OK) { delete h; return MIXKVQ_E_CUDA; }
+  if (zero_all_layers(h, st) != MIXKVQ_OK) { delete h; return MIXKVQ_E_CUDA; }
   if (attention_ws_setup() != cudaSuccess || attention_tc_setup() != cudaSuccess || prefill_attention_setup() != cudaSuccess ||
       flush_setup() != cudaSuccess) { delete h; return MIXKVQ_E_CUDA; }
   *out = h;
@@ -351,11 +366,8 @@ int mixkvq_cache_reset(mixkvq_cache* cache, int layer, void* stream) {
   if (!cache || layer >= cache->cfg.n_layers) return MIXKVQ_E_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (layer >= 0) return zero_layer_state(cache, layer, st);
-  cache->last_packed_writer = kAllPacked;
   if (cudaMemsetAsync(cache->mem, 0, kHeaderBytes, st) != cudaSuccess) return MIXKVQ_E_CUDA;
-  for (int l = 0; l < cache->cfg.n_layers; ++l)
-    if (zero_layer_state(cache, l, st) != MIXKVQ_OK) return MIXKVQ_E_CUDA;
-  return MIXKVQ_OK;
+  return zero_all_layers(cache, st);
 }
 
 int mixkvq_select_channels(mixkvq_cache* cache, int layer, uint8_t* tiers_dev, double* salience_dev, void* stream) {
@@ -418,7 +430,7 @@ int mixkvq_quantize_append_ragged(mixkvq_cache* cache, int layer, const void* k_
     int b1 = b0 + 1;
     while (b1 < B && n_tokens_host[b1] == n_tokens_host[b0] && same_fill(cache, layer, b0, b1)) ++b1;
     if (n_tokens_host[b0] > 0) {
-      const int rc = append_run(cache, layer, b0, b1 - b0, k_dev, v_dev, q_dev, n_tokens_max, n_tokens_host[b0], st);
+      const int rc = append_run(cache, layer, b0, b1 - b0, k_dev, v_dev, q_dev, n_tokens_max, n_tokens_host[b0], false, st);
       if (rc != MIXKVQ_OK) return rc;
     }
     b0 = b1;
@@ -533,7 +545,7 @@ int mixkvq_prefill(mixkvq_cache* cache, int layer, const void* k_dev, const void
     return MIXKVQ_E_CUDA;
   cache->launches += 2;
   cache->last_packed_writer = kNoPackedWrite;
-  return mixkvq_quantize_append(cache, layer, k_dev, v_dev, q_dev, n_tokens, stream);
+  return append_run(cache, layer, 0, cache->cfg.batch, k_dev, v_dev, q_dev, n_tokens, n_tokens, true, static_cast<cudaStream_t>(stream));
 }
 
 int mixkvq_rope_append(mixkvq_cache* cache, int layer, void* k_dev, const void* v_dev, void* q_dev, const float* cos_dev,

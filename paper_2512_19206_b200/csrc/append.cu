@@ -9,6 +9,7 @@ __global__ void __launch_bounds__(256)
 append_tokens_kernel(LayerView lv, const uint16_t* __restrict__ k, const uint16_t* __restrict__ v,
                      const uint16_t* __restrict__ q, int n_tokens, int t0, int m, int r0) {
   __shared__ __align__(16) unsigned char smem[kAbsSumSmem];
+  dependency_wait();
   append_rows(lv, k, v, q, n_tokens, t0, m, r0, blockIdx.x, smem);
 }
 
@@ -16,6 +17,7 @@ append_tokens_kernel(LayerView lv, const uint16_t* __restrict__ k, const uint16_
 __global__ void __launch_bounds__(256)
 sink_append_kernel(LayerView lv, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, int n_tokens,
                    int t0, int m) {
+  dependency_wait();
   const int s = blockIdx.x, tid = threadIdx.x;
   const uint4* ksrc = reinterpret_cast<const uint4*>(k + ((size_t)s * n_tokens + t0) * kD);
   const uint4* vsrc = reinterpret_cast<const uint4*>(v + ((size_t)s * n_tokens + t0) * kD);
@@ -29,16 +31,14 @@ sink_append_kernel(LayerView lv, const __nv_bfloat16* __restrict__ k, const __nv
 
 cudaError_t launch_sink_append(const LayerView& lv, const void* k, const void* v, int n_tokens, int t0, int m,
                                cudaStream_t stream) {
-  sink_append_kernel<<<lv.B * lv.Hkv, 256, 0, stream>>>(lv, static_cast<const __nv_bfloat16*>(k),
-                                                        static_cast<const __nv_bfloat16*>(v), n_tokens, t0, m);
-  return cudaGetLastError();
+  return launch_dependent(sink_append_kernel, dim3(lv.B * lv.Hkv), 256, 0, stream, lv, static_cast<const __nv_bfloat16*>(k),
+                          static_cast<const __nv_bfloat16*>(v), n_tokens, t0, m);
 }
 
 cudaError_t launch_append(const LayerView& lv, const void* k, const void* v, const void* q, int n_tokens, int t0,
                           int m, cudaStream_t stream) {
-  append_tokens_kernel<<<lv.B * lv.Hkv, 256, 0, stream>>>(
-      lv, static_cast<const uint16_t*>(k), static_cast<const uint16_t*>(v), static_cast<const uint16_t*>(q), n_tokens, t0, m, lv.r);
-  return cudaGetLastError();
+  return launch_dependent(append_tokens_kernel, dim3(lv.B * lv.Hkv), 256, 0, stream, lv, static_cast<const uint16_t*>(k),
+                          static_cast<const uint16_t*>(v), static_cast<const uint16_t*>(q), n_tokens, t0, m, lv.r);
 }
 
 }  // namespace mixkvq

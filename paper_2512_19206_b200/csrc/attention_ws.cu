@@ -1093,18 +1093,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
 
 template <int G, int kU4, bool kV4>
 cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, cudaStream_t stream) {
-  // launched with programmatic stream serialization: the kernel itself waits for its predecessor (griddepcontrol.wait)
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(threads_of(kU4, kV4));
-  cfg.dynamicSmemBytes = smem_bytes(G, kU4, kV4);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, attention_ws_kernel<G, kU4, kV4>, lv, qb, sl, ws, 0x44004400u);
+  return launch_dependent(attention_ws_kernel<G, kU4, kV4>, dim3((unsigned)grid), threads_of(kU4, kV4), smem_bytes(G, kU4, kV4), stream, lv, qb, sl, ws, 0x44004400u);
 }
 template <int G, int kU4>
 cudaError_t launch_one(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, cudaStream_t stream) {

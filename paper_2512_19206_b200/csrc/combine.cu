@@ -26,8 +26,7 @@ combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = blockDim.x >> 5;
   int first, count;
   // started early (programmatic dependent launch): wait here for the kernel that wrote the partials
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  dependency_wait();
   if (mode == 0) {
     first = s * n;
     count = n;
@@ -111,24 +110,15 @@ cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, 
   // eight warps when four with a chunk each do not cover a stream's partials in one round trip (a ragged batch may give
   // nearly all CTAs to one sequence), four otherwise: more warps only lengthen the last step
   const int partials = mode == 0 ? n : (seq != nullptr ? n : n / S + 1);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(S * g));
-  cfg.blockDim = dim3(partials > 4 * kCombineChunk ? kCombineMaxWarps * 32 : 128);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, combine_kernel, ws, out, g, Hkv, Hq, mode, n, units_per_stream, S, seq, seq_prefix, lse_out);
+  return launch_dependent(combine_kernel, dim3((unsigned)(S * g)), partials > 4 * kCombineChunk ? kCombineMaxWarps * 32 : 128, 0, stream,
+                          ws, out, g, Hkv, Hq, mode, n, units_per_stream, S, seq, seq_prefix, lse_out);
 }
 
 // The table of a ragged batch, from the host's per-sequence fill (kernel arguments: no copy, ordered in the stream).
 __global__ void seq_table_kernel(SeqTableArgs a, int4* __restrict__ seq, int* __restrict__ seq_prefix) {
   // a link of the chain of dependent launches: started early, waits for everything before it (a kernel that still
   // reads the table's previous contents included), and only then lets the attention kernel behind it start
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  dependency_wait();
   const int b = threadIdx.x;
   if (b < a.n) seq[b] = make_int4(a.fill[3 * b], a.fill[3 * b + 1], a.fill[3 * b + 2], a.w[b]);
   if (b == 0) {
@@ -142,16 +132,7 @@ __global__ void seq_table_kernel(SeqTableArgs a, int4* __restrict__ seq, int* __
 }
 
 cudaError_t launch_seq_table(const SeqTableArgs& a, int4* seq, int* seq_prefix, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(1);
-  cfg.blockDim = dim3(kMaxRaggedBatch);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, seq_table_kernel, a, seq, seq_prefix);
+  return launch_dependent(seq_table_kernel, dim3(1), kMaxRaggedBatch, 0, stream, a, seq, seq_prefix);
 }
 
 // Softmax attention over the union of disjoint token sets from the per-set results: o = sum_r w_r o_r / sum_r w_r with

@@ -167,6 +167,30 @@ __host__ __device__ inline void hi_plane_pos(int jj, int e, int* word, int* bit)
   *bit = 16 * e + 8 * (r >> 2) + 2 * (2 * mt + rh);
 }
 
+// ---- Programmatic dependent launch.  A kernel launched with launch_dependent may be started while the kernel before it in
+// the stream is still running: its launch and set-up overlap that kernel's tail.  It calls dependency_wait() before it touches
+// anything an earlier kernel may write or still read, and that call also lets the kernel behind it be started early.  Since no
+// kernel of this library lets its successor start before its own wait, everything two launches back is complete when a
+// kernel starts.
+__device__ __forceinline__ void dependency_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Even split of `total` work units over `parts`: [begin(i), begin(i+1)).
 __host__ __device__ inline long long split_begin(long long total, int parts, int i) {
   return (total * (long long)i) / parts;
@@ -197,7 +221,7 @@ cudaError_t launch_rope(void* k, void* q, const float* cos_t, const float* sin_t
                         int pos0, cudaStream_t stream);
 cudaError_t launch_flush(const LayerView& lv, cudaStream_t stream);
 cudaError_t launch_flush_bulk(const LayerView& lv, const void* k, const void* v, const void* q, int n_tokens, int t0,
-                              int nb, int tail, cudaStream_t stream);
+                              int nb, int tail, bool behind_prefill, cudaStream_t stream);
 cudaError_t flush_setup();
 cudaError_t launch_select_window(const LayerView& lv, uint8_t* tiers, double* salience, cudaStream_t stream);
 cudaError_t launch_select_raw(const void* q, const void* k, int B, int Hq, int Hkv, int lq, int lk, int score_bits,

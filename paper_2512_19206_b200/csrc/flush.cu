@@ -28,6 +28,7 @@ struct BulkSrc {
   int n_tokens, t0;       // tokens per stream in the tensors, first token of block 0 of this call
   int nb;                 // blocks of this call
   int tail;               // tokens behind them that go to the residual window
+  int behind_prefill;     // the kernel before the first launch is the prefill attention of the same tensors
 };
 
 constexpr int kKeyRow = 68;      // 32-bit words per staged key row: rows r = 0..7 start 4 banks apart
@@ -728,6 +729,7 @@ __device__ inline void values_role(const LayerView& lv, unsigned char* smem, con
 template <int G, bool kTile>
 __global__ void __launch_bounds__(256, 2) flush_kernel(LayerView lv) {
   extern __shared__ __align__(16) unsigned char smem[];
+  dependency_wait();
   const int s = blockIdx.x;
   int block_index = lv.n_blocks;
   if (lv.seq != nullptr) {
@@ -747,18 +749,24 @@ template <int G, bool kTile>
 __global__ void __launch_bounds__(256, 4) bulk_tiers_values_kernel(LayerView lv, BulkSrc src) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int s = blockIdx.x, w = blockIdx.y;
+  // Behind the prefill attention, which neither writes what is read here nor touches the cache, the work starts as soon as an
+  // SM is free of it, and only the end waits.  (With importance mode 1 the kernel before this one is another.)
+  const bool early = src.behind_prefill != 0 && lv.importance_mode != 1;
+  if (!early) dependency_wait();
   if (blockIdx.z == 0) {
     tiers_role(lv, src, smem, s, w);
   } else {
     const uint16_t* rows = src.v + ((size_t)s * src.n_tokens + src.t0 + (size_t)w * lv.R) * kD;
     values_role<G, kTile>(lv, smem, reinterpret_cast<const uint4*>(rows), s, lv.n_blocks + w);
   }
+  if (early) dependency_wait();
 }
 
 // Bulk append, second launch: blockIdx.y < nb: keys of that window, blockIdx.y == nb: the stream's tail.
 template <int G, bool kTile>
 __global__ void __launch_bounds__(256, 4) bulk_keys_tail_kernel(LayerView lv, BulkSrc src) {
   extern __shared__ __align__(16) unsigned char smem[];
+  dependency_wait();
   const int s = blockIdx.x, w = blockIdx.y;
   if (w < src.nb) {
     const uint16_t* rows = src.k + ((size_t)s * src.n_tokens + src.t0 + (size_t)w * lv.R) * kD;
@@ -777,6 +785,7 @@ __global__ void __launch_bounds__(256, 4) bulk_keys_tail_kernel(LayerView lv, Bu
 __global__ void __launch_bounds__(256, 4) bulk_importance_kernel(LayerView lv, BulkSrc src) {
   __shared__ __align__(16) unsigned char smem[kAbsSumSmem];
   __shared__ int lastS;
+  dependency_wait();
   const int s = blockIdx.x, w = blockIdx.y, tid = threadIdx.x, g = lv.g, R = lv.R;
   const int b = s / lv.Hkv, hk = s % lv.Hkv;
   char* state = lv.state + (size_t)s * lv.state_stride;
@@ -864,16 +873,17 @@ cudaError_t setup_one() {
 template <int G, bool kTile>
 cudaError_t single(const LayerView& lv, cudaStream_t stream) {
   const int a = key_smem(lv), b = value_smem(lv);
-  flush_kernel<G, kTile><<<dim3(lv.B * lv.Hkv, 2), 256, a > b ? a : b, stream>>>(lv);
-  return cudaGetLastError();
+  return launch_dependent(flush_kernel<G, kTile>, dim3(lv.B * lv.Hkv, 2), 256, a > b ? a : b, stream, lv);
 }
 template <int G, bool kTile>
 cudaError_t bulk(const LayerView& lv, const BulkSrc& src, cudaStream_t stream) {
   const int S = lv.B * lv.Hkv, b = value_smem(lv), t = tiers_smem_bytes();
-  if (lv.importance_mode == 1) bulk_importance_kernel<<<dim3(S, src.nb), 256, 0, stream>>>(lv, src);
-  bulk_tiers_values_kernel<G, kTile><<<dim3(S, src.nb, 2), 256, t > b ? t : b, stream>>>(lv, src);
-  bulk_keys_tail_kernel<G, kTile><<<dim3(S, src.nb + 1), 256, key_smem(lv), stream>>>(lv, src);
-  return cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (lv.importance_mode == 1) e = launch_dependent(bulk_importance_kernel, dim3(S, src.nb), 256, 0, stream, lv, src);
+  if (e == cudaSuccess)
+    e = launch_dependent(bulk_tiers_values_kernel<G, kTile>, dim3(S, src.nb, 2), 256, t > b ? t : b, stream, lv, src);
+  if (e == cudaSuccess) e = launch_dependent(bulk_keys_tail_kernel<G, kTile>, dim3(S, src.nb + 1), 256, key_smem(lv), stream, lv, src);
+  return e;
 }
 
 }  // namespace
@@ -901,9 +911,9 @@ cudaError_t launch_flush(const LayerView& lv, cudaStream_t stream) {
 // append of the tail.  The first launch is bound by instruction issue (67 % of the slots, the magnitude sums first among
 // them) and its loads, the second by its second wave of CTAs (1024 on 592 places).
 cudaError_t launch_flush_bulk(const LayerView& lv, const void* k, const void* v, const void* q, int n_tokens, int t0,
-                              int nb, int tail, cudaStream_t stream) {
+                              int nb, int tail, bool behind_prefill, cudaStream_t stream) {
   const BulkSrc src{static_cast<const uint16_t*>(k), static_cast<const uint16_t*>(v), static_cast<const uint16_t*>(q), n_tokens,
-                    t0, nb, tail};
+                    t0, nb, tail, behind_prefill ? 1 : 0};
   if (lv.tile) return lv.G == 32 ? bulk<32, true>(lv, src, stream) : lv.G == 64 ? bulk<64, true>(lv, src, stream) : bulk<128, true>(lv, src, stream);
   return lv.G == 32 ? bulk<32, false>(lv, src, stream) : lv.G == 64 ? bulk<64, false>(lv, src, stream) : bulk<128, false>(lv, src, stream);
 }

@@ -160,6 +160,7 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
 __global__ void __launch_bounds__(256)
 prefill_pack_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, unsigned char* __restrict__ kt,
                     unsigned char* __restrict__ vt, int L, int n_tiles) {
+  dependency_wait();
   const int t = blockIdx.x, s = blockIdx.y;
   const __nv_bfloat16* kg = k + ((size_t)s * L + (size_t)t * kTile) * kD;
   const __nv_bfloat16* vg = v + ((size_t)s * L + (size_t)t * kTile) * kD;
@@ -389,7 +390,9 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     for (int i = 0; i < kBars; ++i) mbar_init(bar(i), i >= kPHalf && i < kDoneA ? kTile : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    // the first tiles are under way while Q is loaded
+    // the first tiles are under way while Q is loaded (Q was written before the kernel that packs the tiles: only the tiles
+    // wait for that kernel)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (; issued < min(2, n_b); ++issued) {
       copy_tile(issued, true);
       copy_tile(issued, false);
@@ -410,6 +413,8 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     for (int k = 0; k < kEach; ++k)
       if (tid + k * kThreads < kPieces) reinterpret_cast<uint4*>(Qs)[tid + k * kThreads] = x[k];
   }
+  // Every thread waits for the kernel before: nothing below runs, and no successor starts, before that is complete.
+  dependency_wait();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // Q is read by the tensor core
   tc_fence_before();
   __syncthreads();
@@ -594,12 +599,12 @@ cudaError_t launch_prefill_attention(const void* q, const void* k, const void* v
   const int n_tiles = (L + kTile - 1) / kTile, n_qtiles = (L + kQRows - 1) / kQRows;
   unsigned char* kt = static_cast<unsigned char*>(scratch);
   unsigned char* vt = kt + (size_t)B * Hkv * n_tiles * kTileBytes;
-  prefill_pack_kernel<<<dim3((unsigned)n_tiles, (unsigned)(B * Hkv)), 256, 0, stream>>>(
-      static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), kt, vt, L, n_tiles);
-  prefill_attention_kernel<<<(unsigned)(n_qtiles * B * Hq), kThreads, kSmem, stream>>>(
-      static_cast<const __nv_bfloat16*>(q), kt, vt, out, B * Hq, Hq, Hkv, L, n_tiles, n_qtiles,
-      scale * 1.4426950408889634f, status, max_polls ? max_polls : kPolls, debug_extra_tx);
-  return cudaGetLastError();
+  const cudaError_t e = launch_dependent(prefill_pack_kernel, dim3((unsigned)n_tiles, (unsigned)(B * Hkv)), 256, 0, stream,
+                                         static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), kt, vt, L, n_tiles);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(prefill_attention_kernel, dim3((unsigned)(n_qtiles * B * Hq)), kThreads, kSmem, stream,
+                          static_cast<const __nv_bfloat16*>(q), kt, vt, out, B * Hq, Hq, Hkv, L, n_tiles, n_qtiles,
+                          scale * 1.4426950408889634f, status, max_polls ? max_polls : kPolls, debug_extra_tx);
 }
 
 }  // namespace mixkvq

@@ -16,6 +16,7 @@ namespace {
 __global__ void __launch_bounds__(256)
 rope_kernel(__nv_bfloat16* __restrict__ k, __nv_bfloat16* __restrict__ q, const float* __restrict__ cos_t,
             const float* __restrict__ sin_t, long long k_rows, long long rows, int n_tokens, int pos0) {
+  dependency_wait();
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long row = idx >> 3;
   const int c = (int)(idx & 7);
@@ -55,10 +56,8 @@ cudaError_t launch_rope(void* k, void* q, const float* cos_t, const float* sin_t
                         int pos0, cudaStream_t stream) {
   const long long k_rows = (long long)B * Hkv * n_tokens, rows = k_rows + (long long)B * Hq * n_tokens;
   const long long threads = rows * 8;
-  rope_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(static_cast<__nv_bfloat16*>(k),
-                                                                   static_cast<__nv_bfloat16*>(q), cos_t, sin_t, k_rows,
-                                                                   rows, n_tokens, pos0);
-  return cudaGetLastError();
+  return launch_dependent(rope_kernel, dim3((unsigned)((threads + 255) / 256)), 256, 0, stream, static_cast<__nv_bfloat16*>(k),
+                          static_cast<__nv_bfloat16*>(q), cos_t, sin_t, k_rows, rows, n_tokens, pos0);
 }
 
 }  // namespace mixkvq
