@@ -80,10 +80,11 @@ __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp
 // kU4: how the configuration can use the UINT4 tier: 0 = never (tau_u4 >= tau_bf16), 1 = some channels (high plane stored
 // per channel pair, gathered), 2 = 4-bit base (dense high plane)
 // kV4: 4-bit values (a second plane of 2-bit value codes per unit, scale 4 s_v)
-template <int G, int kU4, bool kV4>
+// kDirect: one CTA per stream, which writes the output (and the log-denominators) instead of a partial
+template <int G, int kU4, bool kV4, bool kDirect>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float scale_log2e, float* __restrict__ ws,
-                    uint32_t four2) {
+                    uint32_t four2, float* __restrict__ out, float* __restrict__ lse_out) {
   constexpr int VG = kD / G;              // value groups per token
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group
   constexpr int kStageBytes = stage_bytes(kV4);
@@ -1087,10 +1088,21 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
         const float4 o = *reinterpret_cast<const float4*>(smem + w * kPairBytes + (h * kMergeStride + c) * 4);
         acc.x += f[w] * o.x; acc.y += f[w] * o.y; acc.z += f[w] * o.z; acc.w += f[w] * o.w;
       }
-      float* part = ws + (size_t)(blockIdx.x + s) * kPartialFloats + h * 130;
-      *reinterpret_cast<float2*>(part + 2 + c) = make_float2(acc.x, acc.y);
-      *reinterpret_cast<float2*>(part + 4 + c) = make_float2(acc.z, acc.w);
-      if (c == 0) *reinterpret_cast<float2*>(part) = make_float2(M, L);
+      if constexpr (kDirect) {
+        // (l == 0: the teams gave up, the status word says so)
+        if (h < g) {
+          const float inv = L > 0.f ? 1.f / L : 0.f;
+          const size_t row = (size_t)s * g + h;           // (b Hkv + hk) g + h = b Hq + hk g + h
+          *reinterpret_cast<float4*>(out + row * kD + c) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+          // natural logarithm of the softmax denominator (the maximum is kept in the base-2 domain)
+          if (lse_out != nullptr && c == 0) lse_out[row] = L > 0.f ? (M + log2f(L)) * 0.6931471805599453f : -INFINITY;
+        }
+      } else {
+        float* part = ws + (size_t)(blockIdx.x + s) * kPartialFloats + h * 130;
+        *reinterpret_cast<float2*>(part + 2 + c) = make_float2(acc.x, acc.y);
+        *reinterpret_cast<float2*>(part + 4 + c) = make_float2(acc.z, acc.w);
+        if (c == 0) *reinterpret_cast<float2*>(part) = make_float2(M, L);
+      }
     }
     if (seg < ce) {
       // another segment follows: its copies are staged into the rings that were just read
@@ -1100,36 +1112,47 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
   }
 }
 
+template <int G, int kU4, bool kV4, bool kDirect>
+cudaError_t launch_d(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
+  return launch_dependent(attention_single_kernel<G, kU4, kV4, kDirect>, dim3((unsigned)grid), kThreads, smem_bytes(kV4), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
+}
 template <int G, int kU4, bool kV4>
-cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, cudaStream_t stream) {
-  return launch_dependent(attention_single_kernel<G, kU4, kV4>, dim3((unsigned)grid), kThreads, smem_bytes(kV4), stream, lv, qb, sl, ws, 0x44004400u);
+cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
+  return out != nullptr ? launch_d<G, kU4, kV4, true>(lv, qb, sl, ws, grid, out, lse, stream)
+                        : launch_d<G, kU4, kV4, false>(lv, qb, sl, ws, grid, out, lse, stream);
 }
 template <int G, int kU4>
-cudaError_t launch_one(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, cudaStream_t stream) {
-  return lv.v_bits == 4 ? launch_v<G, kU4, true>(lv, qb, sl, ws, grid, stream)
-                        : launch_v<G, kU4, false>(lv, qb, sl, ws, grid, stream);
+cudaError_t launch_one(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
+  return lv.v_bits == 4 ? launch_v<G, kU4, true>(lv, qb, sl, ws, grid, out, lse, stream)
+                        : launch_v<G, kU4, false>(lv, qb, sl, ws, grid, out, lse, stream);
 }
 
 template <int G>
-cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws, int grid, cudaStream_t stream) {
+cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse,
+                     cudaStream_t stream) {
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   const float sl = scale * 1.4426950408889634f;
-  if (lv.dense_hi) return launch_one<G, 2>(lv, qb, sl, ws, grid, stream);
+  if (lv.dense_hi) return launch_one<G, 2>(lv, qb, sl, ws, grid, out, lse, stream);
   const bool uses_u4 = (lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16;
-  if (uses_u4) return launch_one<G, 1>(lv, qb, sl, ws, grid, stream);
-  return launch_one<G, 0>(lv, qb, sl, ws, grid, stream);
+  if (uses_u4) return launch_one<G, 1>(lv, qb, sl, ws, grid, out, lse, stream);
+  return launch_one<G, 0>(lv, qb, sl, ws, grid, out, lse, stream);
 }
 
 }  // namespace
 
-template <int G, int kU4, bool kV4>
-static cudaError_t setup_v() {
-  cudaError_t e = cudaFuncSetAttribute(attention_single_kernel<G, kU4, kV4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+template <int G, int kU4, bool kV4, bool kDirect>
+static cudaError_t setup_d() {
+  cudaError_t e = cudaFuncSetAttribute(attention_single_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        smem_bytes(kV4));
   if (e != cudaSuccess) return e;
   // the CTAs of an SM only fit with the largest shared-memory carve-out; ask for it explicitly
-  return cudaFuncSetAttribute(attention_single_kernel<G, kU4, kV4>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  return cudaFuncSetAttribute(attention_single_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               (int)cudaSharedmemCarveoutMaxShared);
+}
+template <int G, int kU4, bool kV4>
+static cudaError_t setup_v() {
+  cudaError_t e = setup_d<G, kU4, kV4, false>();
+  return e != cudaSuccess ? e : setup_d<G, kU4, kV4, true>();
 }
 template <int G, int kU4>
 static cudaError_t setup_one() {
@@ -1152,10 +1175,11 @@ cudaError_t attention_single_setup() {
   return setup_g<128>();
 }
 
-cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, cudaStream_t stream) {
-  if (lv.G == 32) return launch_g<32>(lv, q, scale, ws, grid, stream);
-  if (lv.G == 64) return launch_g<64>(lv, q, scale, ws, grid, stream);
-  return launch_g<128>(lv, q, scale, ws, grid, stream);
+cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse,
+                                    cudaStream_t stream) {
+  if (lv.G == 32) return launch_g<32>(lv, q, scale, ws, grid, out, lse, stream);
+  if (lv.G == 64) return launch_g<64>(lv, q, scale, ws, grid, out, lse, stream);
+  return launch_g<128>(lv, q, scale, ws, grid, out, lse, stream);
 }
 
 }  // namespace mixkvq

@@ -39,7 +39,8 @@ cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, 
                            long long units_per_stream, int S, cudaStream_t stream, const int4* seq = nullptr,
                            const int* seq_prefix = nullptr, float* lse_out = nullptr);
 // the same split, one unit at a time (attention_single.cu)
-cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, cudaStream_t stream);
+cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse,
+                                    cudaStream_t stream);
 cudaError_t attention_single_setup();
 
 namespace {
@@ -110,10 +111,11 @@ __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp
 // kU4: how the configuration can use the UINT4 tier: 0 = never (tau_u4 >= tau_bf16), 1 = some channels (high plane stored
 // per channel pair, gathered), 2 = 4-bit base (dense high plane)
 // kV4: 4-bit values (a second plane of 2-bit value codes per unit, scale 4 s_v)
-template <int G, int kU4, bool kV4>
+// kDirect: one CTA per stream, which writes the output (and the log-denominators) instead of a partial
+template <int G, int kU4, bool kV4, bool kDirect>
 __global__ void __launch_bounds__(threads_of(kU4, kV4), kCtasPerSm)
 attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float scale_log2e, float* __restrict__ ws,
-                    uint32_t four2) {
+                    uint32_t four2, float* __restrict__ out, float* __restrict__ lse_out) {
   constexpr int VG = kD / G;              // value groups per token
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group
   constexpr int UPG = G / 32;             // units per key group
@@ -1078,10 +1080,21 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         const float4 o = *reinterpret_cast<const float4*>(smem + w * kTeamBytes + (h * kMergeStride + c) * 4);
         acc.x += f[w] * o.x; acc.y += f[w] * o.y; acc.z += f[w] * o.z; acc.w += f[w] * o.w;
       }
-      float* part = ws + (size_t)(blockIdx.x + s) * kPartialFloats + h * 130;
-      *reinterpret_cast<float2*>(part + 2 + c) = make_float2(acc.x, acc.y);
-      *reinterpret_cast<float2*>(part + 4 + c) = make_float2(acc.z, acc.w);
-      if (c == 0) *reinterpret_cast<float2*>(part) = make_float2(M, L);
+      if constexpr (kDirect) {
+        // (l == 0: the teams gave up, the status word says so)
+        if (h < g) {
+          const float inv = L > 0.f ? 1.f / L : 0.f;
+          const size_t row = (size_t)s * g + h;           // (b Hkv + hk) g + h = b Hq + hk g + h
+          *reinterpret_cast<float4*>(out + row * kD + c) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+          // natural logarithm of the softmax denominator (the maximum is kept in the base-2 domain)
+          if (lse_out != nullptr && c == 0) lse_out[row] = L > 0.f ? (M + log2f(L)) * 0.6931471805599453f : -INFINITY;
+        }
+      } else {
+        float* part = ws + (size_t)(blockIdx.x + s) * kPartialFloats + h * 130;
+        *reinterpret_cast<float2*>(part + 2 + c) = make_float2(acc.x, acc.y);
+        *reinterpret_cast<float2*>(part + 4 + c) = make_float2(acc.z, acc.w);
+        if (c == 0) *reinterpret_cast<float2*>(part) = make_float2(M, L);
+      }
     }
     if (seg < ce) {
       // another segment follows: its copies are staged into the rings that were just read
@@ -1091,36 +1104,47 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   }
 }
 
+template <int G, int kU4, bool kV4, bool kDirect>
+cudaError_t launch_d(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
+  return launch_dependent(attention_ws_kernel<G, kU4, kV4, kDirect>, dim3((unsigned)grid), threads_of(kU4, kV4), smem_bytes(G, kU4, kV4), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
+}
 template <int G, int kU4, bool kV4>
-cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, cudaStream_t stream) {
-  return launch_dependent(attention_ws_kernel<G, kU4, kV4>, dim3((unsigned)grid), threads_of(kU4, kV4), smem_bytes(G, kU4, kV4), stream, lv, qb, sl, ws, 0x44004400u);
+cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
+  return out != nullptr ? launch_d<G, kU4, kV4, true>(lv, qb, sl, ws, grid, out, lse, stream)
+                        : launch_d<G, kU4, kV4, false>(lv, qb, sl, ws, grid, out, lse, stream);
 }
 template <int G, int kU4>
-cudaError_t launch_one(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, cudaStream_t stream) {
-  return lv.v_bits == 4 ? launch_v<G, kU4, true>(lv, qb, sl, ws, grid, stream)
-                        : launch_v<G, kU4, false>(lv, qb, sl, ws, grid, stream);
+cudaError_t launch_one(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
+  return lv.v_bits == 4 ? launch_v<G, kU4, true>(lv, qb, sl, ws, grid, out, lse, stream)
+                        : launch_v<G, kU4, false>(lv, qb, sl, ws, grid, out, lse, stream);
 }
 
 template <int G>
-cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws, int grid, cudaStream_t stream) {
+cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse,
+                     cudaStream_t stream) {
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   const float sl = scale * 1.4426950408889634f;
-  if (lv.dense_hi) return launch_one<G, 2>(lv, qb, sl, ws, grid, stream);
+  if (lv.dense_hi) return launch_one<G, 2>(lv, qb, sl, ws, grid, out, lse, stream);
   const bool uses_u4 = (lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16;
-  if (uses_u4) return launch_one<G, 1>(lv, qb, sl, ws, grid, stream);
-  return launch_one<G, 0>(lv, qb, sl, ws, grid, stream);
+  if (uses_u4) return launch_one<G, 1>(lv, qb, sl, ws, grid, out, lse, stream);
+  return launch_one<G, 0>(lv, qb, sl, ws, grid, out, lse, stream);
 }
 
 }  // namespace
 
-template <int G, int kU4, bool kV4>
-static cudaError_t setup_v() {
-  cudaError_t e = cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+template <int G, int kU4, bool kV4, bool kDirect>
+static cudaError_t setup_d() {
+  cudaError_t e = cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        smem_bytes(G, kU4, kV4));
   if (e != cudaSuccess) return e;
   // the CTAs of an SM only fit with the largest shared-memory carve-out; ask for it explicitly
-  return cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  return cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               (int)cudaSharedmemCarveoutMaxShared);
+}
+template <int G, int kU4, bool kV4>
+static cudaError_t setup_v() {
+  cudaError_t e = setup_d<G, kU4, kV4, false>();
+  return e != cudaSuccess ? e : setup_d<G, kU4, kV4, true>();
 }
 template <int G, int kU4>
 static cudaError_t setup_one() {
@@ -1154,6 +1178,10 @@ int attention_ws_positions_of(int n_blocks, int r, int n_sink, int U) {
   return n_blocks * U + kResidualWeight * ((r + 31) / 32 + (n_sink + 31) / 32);
 }
 
+static bool three_tiers(const LayerView& lv) {
+  return !lv.dense_hi && ((lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16);
+}
+
 // Number of CTAs the split kernel runs for this layer state (also the number of partial-slot owners).  When there are
 // fewer streams than CTA slots the grid is a multiple of the stream count, so that no CTA straddles two streams
 // (a second segment costs a pipeline drain, a query load and a second partial).  Ragged batch: the positions of all
@@ -1161,7 +1189,14 @@ int attention_ws_positions_of(int n_blocks, int r, int n_sink, int U) {
 int attention_ws_grid(const LayerView& lv, int n_sms) {
   const int S = lv.B * lv.Hkv;
   const long long total = lv.seq != nullptr ? lv.seq_total : attention_ws_positions(lv) * S;
-  int grid = (int)min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), total);
+  // Small caches: two positions per CTA while that leaves one CTA per SM, then more (up to four) before a second CTA per SM:
+  // a CTA has four teams, and every CTA of a stream is a partial to merge (one position per CTA / two / four, us per layer with the
+  // merge: one sequence of 400 tokens 5.6 / 5.5 / 6.0, 4000 tokens 9.6 / 7.1 / 6.3, eight of 333 8.2 / 7.9 / 6.6).
+  const long long wanted = min((total + 1) / 2, max((long long)n_sms, (total + 3) / 4));
+  int grid = (int)min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), wanted);
+  // a few positions per team: one CTA per stream, which needs no merge (eight sequences of 333 tokens, 20 positions: 6.6 -> 5.6 us
+  // per layer and a launch less; 40 positions 9.2 -> 9.9; three tiers, 26 positions, 6.7 -> 9.4)
+  if (lv.seq == nullptr && attention_ws_positions(lv) <= (three_tiers(lv) ? 16 : 28)) grid = min(grid, S);
   if (grid > S && lv.seq == nullptr) grid = grid / S * S;
   return grid < 1 ? 1 : grid;
 }
@@ -1176,16 +1211,21 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // shape, batch 8) 8000 tokens, 27 units per CTA, 12.6 / 13.1, 16000 21.5 / 20.5; G = 128 (32b shape, batch 16) 2000 tokens,
   // 31 units, 13.5 / 13.0, 600 tokens, 10 units, 8.3 / 8.15; three tiers (7b shape) 600 tokens, 3 units, 6.4 / 6.7, 2000 tokens,
   // 7 units, 9.3 / 7.8; 4-bit base (8b shape, batch 16) 600 tokens, 12 units, 8.9 / 9.3, 2000 tokens, 31 units, 18.7 / 17.7.
-  const bool three_tiers = !lv.dense_hi && ((lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16);
-  const int from_units = three_tiers ? 6 : lv.dense_hi ? 20 : lv.G == 128 ? 10 : 40;
+  const int from_units = three_tiers(lv) ? 6 : lv.dense_hi ? 20 : lv.G == 128 ? 10 : 40;
   const bool by_two = !(lv.U & 1) && (lv.seq != nullptr ? lv.seq_total : Us * S) >= (long long)from_units * grid;
+  // With one CTA per stream the split kernel writes the output itself (32b shape, 32 sequences of 900 tokens: 17.9 -> 12.4 us per
+  // layer).  Merging several partials in the kernel, by the CTA that finds all of a stream's written, was slower than a merge
+  // kernel: a fence, a look at the other CTAs' marks and a serial merge against a dependent launch (one sequence of 400
+  // tokens 7.3 us against 5.6; 7b shape 41.1 against 40.7).
+  const bool whole = out != nullptr && lv.seq == nullptr && grid == S;
+  float* const kernel_out = whole ? out : nullptr;
   cudaError_t e;
-  if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, stream);
-  else if (lv.G == 32) e = launch_g<32>(lv, q, scale, ws, grid, stream);
-  else if (lv.G == 64) e = launch_g<64>(lv, q, scale, ws, grid, stream);
-  else e = launch_g<128>(lv, q, scale, ws, grid, stream);
+  if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
+  else if (lv.G == 32) e = launch_g<32>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
+  else if (lv.G == 64) e = launch_g<64>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
+  else e = launch_g<128>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
   *launches = 1;
-  if (e != cudaSuccess || out == nullptr) return e;     // out == nullptr: split kernel only (timing)
+  if (e != cudaSuccess || out == nullptr || whole) return e;     // out == nullptr: split kernel only (timing)
   e = launch_combine(ws, out, lv.g, lv.Hkv, lv.Hq, 1, grid, Us, S, stream, lv.seq, lv.seq_prefix, lse_out);
   *launches = 2;
   return e;

@@ -1,0 +1,42 @@
+"""The decode-attention kernel that writes its output itself (one CTA per stream: small caches, and batches whose streams fill
+the GPU) and the split grids on either side of that choice, against the library's plain-ALU fp32 kernel; the partial form
+gives the same rows and the log-denominator of the merged call."""
+import pytest
+import torch
+
+import gpu_util as U
+from paper_2512_19206_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+TOL = 4e-3          # both kernels are within 2e-3 of the exact result (tests/test_gpu_parity.py)
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2512_19206_b200 import build
+    build.build()
+    from paper_2512_19206_b200 import binding as b
+    b.lib()
+    return b
+
+
+@pytest.mark.parametrize("name,batch,tokens,R,preset", [
+    ("qwen7b", 1, 1, 128, "P24"), ("qwen7b", 1, 128, 128, "P24"), ("qwen7b", 2, 640, 128, "P24"), ("qwen7b", 2, 900, 128, "P24"),
+    ("qwen7b", 2, 300, 128, "P27"), ("qwen7b", 2, 500, 128, "P27"), ("llama8b", 3, 97, 32, "P24"), ("llama8b", 2, 401, 128, "P4BASE"),
+    ("qwen32b", 32, 777, 128, "P24"), ("qwen32b", 32, 1500, 256, "P27"), ("qwen32b", 37, 600, 128, "P24"),
+])
+def test_direct_output(binding, name, batch, tokens, R, preset):
+    w = W.small(W.CONFIGS[name], n_layers=1, batch=batch, tokens=tokens, residual_len=R, group_size=32 if R == 32 else W.CONFIGS[name].group_size,
+                **getattr(W, preset))
+    cache = U.make_cache(binding, w, extras_budget_bytes=(tokens // R + 3) * R * 128)
+    cache.quantize_append(0, *W.tokens(w, 0, 0, tokens, device="cuda"))
+    q = W.decode_query(w, 0, 0, device="cuda")
+    out = cache.decode_attention(0, q, W.softmax_scale())
+    part, lse = cache.decode_attention_partial(0, q, W.softmax_scale())
+    assert torch.equal(out, part) and bool(torch.isfinite(lse).all())
+    merged = binding.merge_partials(torch.stack([part, part]), torch.stack([lse, lse]))      # twice the same set: the same rows
+    assert float((merged - out).abs().max()) <= 1e-6 * float(out.abs().max())
+    cache.set_attention_kernel(1)
+    ref = cache.decode_attention(0, q, W.softmax_scale())
+    assert cache.status() == 0
+    assert float((out - ref).abs().max()) <= TOL
