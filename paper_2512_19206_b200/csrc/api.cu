@@ -201,6 +201,7 @@ int upload_seq_table(mixkvq_cache* h, int layer, cudaStream_t st, LayerView* lv)
     total += (long long)a.Hkv * a.w[b];
   }
   if (total >= (1ll << 31)) return MIXKVQ_E_UNSUPPORTED;
+  lv->seq_ctas = attention_ws_ragged_split(a.w, B, a.Hkv, h->n_sms, a.ctas);
   char* L = h->mem + kHeaderBytes + h->layer_stride * (uint64_t)layer + h->seq_off;
   int4* seq = reinterpret_cast<int4*>(L);
   int* prefix = reinterpret_cast<int*>(L + (size_t)B * 16);

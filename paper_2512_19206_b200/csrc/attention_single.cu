@@ -156,8 +156,10 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
     for (int i = threadIdx.x; i <= lv.B; i += kThreads) prefS[i] = lv.seq_prefix[i];
     __syncthreads();
   }
-  const long long total = lv.seq != nullptr ? (long long)prefS[lv.B] : (long long)Us * S;
-  const long long cb = split_begin(total, gridDim.x, blockIdx.x), ce = split_begin(total, gridDim.x, blockIdx.x + 1);
+  // the CTA's share of all streams' positions; in a ragged batch it is a part of one stream (below)
+  const long long total = (long long)Us * S;
+  const long long cb = lv.seq != nullptr ? 0 : split_begin(total, gridDim.x, blockIdx.x);
+  const long long ce = lv.seq != nullptr ? 1 : split_begin(total, gridDim.x, blockIdx.x + 1);
 
   uint32_t ring_stage = 0;        // ring stage of the next packed unit this pair consumes
   uint32_t ring_parity = 0;       // phase parity of that stage's barriers
@@ -177,25 +179,25 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
   for (long long seg = cb; seg < ce;) {
     int s, ub, ue;
     if (lv.seq != nullptr) {
-      // ragged batch: the sequence whose positions hold seg (sequences without positions are stepped over)
+      // ragged batch: the sequence whose CTAs this one is among (empty sequences have none), the stream and the part of it
       int b = 0;
-      while (b + 1 < lv.B && (long long)prefS[b + 1] <= seg) ++b;
+      while (b + 1 < lv.B && prefS[b + 1] <= (int)blockIdx.x) ++b;
       const int4 f = lv.seq[b];
       f_nb = f.x; f_r = f.y; f_ns = f.z; Us = f.w;
       packed_units = f_nb * U;
       res_units = (f_r + 31) / 32;
       bf16_units = res_units + (f_ns + 31) / 32;
-      const long long rel = seg - (long long)prefS[b];
-      const int hk = (int)(rel / Us);
+      const int parts = (prefS[b + 1] - prefS[b]) / lv.Hkv, rel = (int)blockIdx.x - prefS[b], hk = rel / parts;
       s = b * lv.Hkv + hk;
-      ub = (int)(rel - (long long)hk * Us);
-      ue = (int)min((long long)Us, ce - (long long)prefS[b] - (long long)hk * Us);
+      ub = (int)split_begin(Us, parts, rel - hk * parts);
+      ue = (int)split_begin(Us, parts, rel - hk * parts + 1);
+      seg = ce;
     } else {
       s = (int)(seg / Us);
       ub = (int)(seg - (long long)s * Us);
       ue = (int)min((long long)Us, ce - (long long)s * Us);
+      seg += ue - ub;
     }
-    seg += ue - ub;
     // ---- this pair's share of the segment.  The unquantized units of the segment go to different pairs (unit i to
     // pair kPairs - 1 - i % kPairs); the packed units are split in order so that every pair carries about the same weight.
     const int pk_b = min(ub, packed_units), pk_e = min(ue, packed_units);

@@ -190,8 +190,10 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     for (int i = threadIdx.x; i <= lv.B; i += kThreads) prefS[i] = lv.seq_prefix[i];
     __syncthreads();
   }
-  const long long total = lv.seq != nullptr ? (long long)prefS[lv.B] : (long long)Us * S;
-  const long long cb = split_begin(total, gridDim.x, blockIdx.x), ce = split_begin(total, gridDim.x, blockIdx.x + 1);
+  // the CTA's share of all streams' positions; in a ragged batch it is a part of one stream (below)
+  const long long total = (long long)Us * S;
+  const long long cb = lv.seq != nullptr ? 0 : split_begin(total, gridDim.x, blockIdx.x);
+  const long long ce = lv.seq != nullptr ? 1 : split_begin(total, gridDim.x, blockIdx.x + 1);
 
   uint32_t ring_stage = 0;        // ring stage of the next step of this warp
   uint32_t ring_parity = 0;       // phase parity of that stage's barriers
@@ -212,25 +214,25 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   for (long long seg = cb; seg < ce;) {
     int s, ub, ue;
     if (lv.seq != nullptr) {
-      // ragged batch: the sequence whose positions hold seg (sequences without positions are stepped over)
+      // ragged batch: the sequence whose CTAs this one is among (empty sequences have none), the stream and the part of it
       int b = 0;
-      while (b + 1 < lv.B && (long long)prefS[b + 1] <= seg) ++b;
+      while (b + 1 < lv.B && prefS[b + 1] <= (int)blockIdx.x) ++b;
       const int4 f = lv.seq[b];
       f_nb = f.x; f_r = f.y; f_ns = f.z; Us = f.w;
       packed_units = f_nb * U;
       res_units = (f_r + 31) / 32;
       bf16_units = res_units + (f_ns + 31) / 32;
-      const long long rel = seg - (long long)prefS[b];
-      const int hk = (int)(rel / Us);
+      const int parts = (prefS[b + 1] - prefS[b]) / lv.Hkv, rel = (int)blockIdx.x - prefS[b], hk = rel / parts;
       s = b * lv.Hkv + hk;
-      ub = (int)(rel - (long long)hk * Us);
-      ue = (int)min((long long)Us, ce - (long long)prefS[b] - (long long)hk * Us);
+      ub = (int)split_begin(Us, parts, rel - hk * parts);
+      ue = (int)split_begin(Us, parts, rel - hk * parts + 1);
+      seg = ce;
     } else {
       s = (int)(seg / Us);
       ub = (int)(seg - (long long)s * Us);
       ue = (int)min((long long)Us, ce - (long long)s * Us);
+      seg += ue - ub;
     }
-    seg += ue - ub;
     // ---- this team's share of the segment.  The unquantized units of the segment go to different teams (unit i to
     // team kTeams - 1 - i % kTeams); the packed units are split in order, in steps of two, so that every team carries about
     // the same weight.  (A stream's packed units are even in number; a boundary at an odd one moves up, on both sides.)
@@ -1178,17 +1180,46 @@ int attention_ws_positions_of(int n_blocks, int r, int n_sink, int U) {
   return n_blocks * U + kResidualWeight * ((r + 31) / 32 + (n_sink + 31) / 32);
 }
 
+// Ragged batch: every stream gets CTAs of its own, as many as make the longest share as short as it can be with about two CTAs
+// per SM.  (An even split of all positions, wherever the boundaries fall, gave CTAs that straddle two or three streams and
+// drain, reload and merge for each: eight sequences of 640 to 32768 tokens, 31.6 us for the split kernel, 24.8 us so.)
+int attention_ws_ragged_split(const int* w, int B, int Hkv, int n_sms, int* ctas) {
+  long long total = 0, streams = 0;
+  int longest = 1;
+  for (int b = 0; b < B; ++b) {
+    total += (long long)Hkv * w[b];
+    streams += w[b] > 0 ? Hkv : 0;
+    longest = max(longest, w[b]);
+  }
+  const long long even = min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), min((total + 1) / 2, max((long long)n_sms, (total + 3) / 4)));
+  // with more streams than that, room to split the longest ones
+  const long long cap = min(max(even, streams > even / 2 ? streams + even / 2 : even), (long long)kMaxCtas + streams);
+  auto count = [&](int share) {
+    long long n = 0;
+    for (int b = 0; b < B; ++b) n += (long long)Hkv * ((w[b] + share - 1) / share);
+    return n;
+  };
+  int lo = 1, hi = longest;                 // the smallest share per CTA with which the CTAs stay within the cap
+  while (lo < hi) {
+    const int mid = (lo + hi) / 2;
+    if (count(mid) <= cap) hi = mid;
+    else lo = mid + 1;
+  }
+  for (int b = 0; b < B; ++b) ctas[b] = (w[b] + lo - 1) / lo;
+  return (int)count(lo);
+}
+
 static bool three_tiers(const LayerView& lv) {
   return !lv.dense_hi && ((lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16);
 }
 
 // Number of CTAs the split kernel runs for this layer state (also the number of partial-slot owners).  When there are
 // fewer streams than CTA slots the grid is a multiple of the stream count, so that no CTA straddles two streams
-// (a second segment costs a pipeline drain, a query load and a second partial).  Ragged batch: the positions of all
-// streams are split evenly, wherever the boundaries fall.
+// (a second segment costs a pipeline drain, a query load and a second partial).
 int attention_ws_grid(const LayerView& lv, int n_sms) {
   const int S = lv.B * lv.Hkv;
-  const long long total = lv.seq != nullptr ? lv.seq_total : attention_ws_positions(lv) * S;
+  if (lv.seq != nullptr) return lv.seq_ctas;
+  const long long total = attention_ws_positions(lv) * S;
   // Small caches: two positions per CTA while that leaves one CTA per SM, then more (up to four) before a second CTA per SM:
   // a CTA has four teams, and every CTA of a stream is a partial to merge (one position per CTA / two / four, us per layer with the
   // merge: one sequence of 400 tokens 5.6 / 5.5 / 6.0, 4000 tokens 9.6 / 7.1 / 6.3, eight of 333 8.2 / 7.9 / 6.6).
@@ -1196,8 +1227,8 @@ int attention_ws_grid(const LayerView& lv, int n_sms) {
   int grid = (int)min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), wanted);
   // a few positions per team: one CTA per stream, which needs no merge (eight sequences of 333 tokens, 20 positions: 6.6 -> 5.6 us
   // per layer and a launch less; 40 positions 9.2 -> 9.9; three tiers, 26 positions, 6.7 -> 9.4)
-  if (lv.seq == nullptr && attention_ws_positions(lv) <= (three_tiers(lv) ? 16 : 28)) grid = min(grid, S);
-  if (grid > S && lv.seq == nullptr) grid = grid / S * S;
+  if (attention_ws_positions(lv) <= (three_tiers(lv) ? 16 : 28)) grid = min(grid, S);
+  if (grid > S) grid = grid / S * S;
   return grid < 1 ? 1 : grid;
 }
 

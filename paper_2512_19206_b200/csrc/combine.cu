@@ -32,13 +32,10 @@ combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int
     first = s * n;
     count = n;
   } else if (seq != nullptr) {
-    // ragged batch: sequence b's streams own positions [prefix[b] + hk * w, + w), w = seq[b].w (none when w == 0)
-    const int bq = s / Hkv, w = seq[bq].w;
-    const long long total = seq_prefix[S / Hkv];
-    const long long x0 = (long long)seq_prefix[bq] + (long long)(s % Hkv) * w, x1 = x0 + w - 1;
-    const int c0 = w ? (int)(((x0 + 1) * n - 1) / total) : 0, c1 = w ? (int)(((x1 + 1) * n - 1) / total) : -1;
-    first = c0 + s;
-    count = c1 - c0 + 1;
+    // ragged batch: each of sequence b's streams has (prefix[b + 1] - prefix[b]) / Hkv CTAs of its own (none if it is empty)
+    const int bq = s / Hkv, p0 = seq_prefix[bq];
+    count = (seq_prefix[bq + 1] - p0) / Hkv;
+    first = p0 + (s % Hkv) * count + s;
   } else {
     const long long total = units_per_stream * S;
     const long long x0 = units_per_stream * s, x1 = units_per_stream * (s + 1) - 1;
@@ -180,7 +177,7 @@ __global__ void seq_table_kernel(SeqTableArgs a, int4* __restrict__ seq, int* __
     int acc = 0;
     for (int i = 0; i < a.n; ++i) {
       seq_prefix[i] = acc;
-      acc += a.Hkv * a.w[i];
+      acc += a.Hkv * a.ctas[i];
     }
     seq_prefix[a.n] = acc;
   }

@@ -59,11 +59,12 @@ struct LayerView {
   // more than are copied, so that it never completes (0 in normal use)
   uint32_t debug_extra_tx;
   // Ragged batch (sequences of different fill): per sequence (n_blocks, r, n_sink, split positions of one of its
-  // streams) and the prefix sums over the sequences of Hkv * positions ([B + 1], the last one = seq_total), both in
-  // device memory; null when every sequence has the fill n_blocks, r, n_sink above.
+  // streams) and the prefix sums over the sequences of Hkv * CTAs per stream ([B + 1], the last one = seq_ctas), both in
+  // device memory; null when every sequence has the fill n_blocks, r, n_sink above.  seq_total: positions of all streams.
   const int4* seq;
   const int* seq_prefix;
   long long seq_total;
+  int seq_ctas;
 };
 
 __host__ __device__ inline uint32_t extras_header_bytes(int n16, int n4) {
@@ -211,8 +212,11 @@ cudaError_t launch_prefill_attention(const void* q, const void* k, const void* v
 size_t prefill_scratch_bytes(int B, int Hkv, int L);
 cudaError_t prefill_attention_setup();
 int attention_ws_positions_of(int n_blocks, int r, int n_sink, int U);
-// writes a ragged batch's table: fill[3 b + {0, 1, 2}] = (n_blocks, r, n_sink) of sequence b, positions w[b] per stream
-struct SeqTableArgs { int n, Hkv; int fill[3 * kMaxRaggedBatch]; int w[kMaxRaggedBatch]; };
+// writes a ragged batch's table: fill[3 b + {0, 1, 2}] = (n_blocks, r, n_sink) of sequence b, positions w[b] and CTAs
+// ctas[b] per stream
+struct SeqTableArgs { int n, Hkv; int fill[3 * kMaxRaggedBatch]; int w[kMaxRaggedBatch]; int ctas[kMaxRaggedBatch]; };
+// CTAs per stream of every sequence (ctas[b], 0 for an empty one); returns the CTAs of all streams
+int attention_ws_ragged_split(const int* w, int B, int Hkv, int n_sms, int* ctas);
 cudaError_t launch_seq_table(const SeqTableArgs& a, int4* seq, int* seq_prefix, cudaStream_t stream);
 cudaError_t launch_empty_partial(float* out, float* lse, int rows, cudaStream_t stream);
 cudaError_t launch_merge_partials(const float* o_parts, const float* lse_parts, int n_parts, int rows, float* out,
