@@ -728,18 +728,21 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
           const uint2 vn = reinterpret_cast<const uint2*>(lv.new_v + (size_t)s * kD)[lane];
           reinterpret_cast<uint2*>(lv.resv + (size_t)s * lv.resv_stride + (size_t)jn * 256)[lane] = vn;
         }
-        // the first tile's loads go out before the wait for the logits
-        uint32_t x[2][4];      // [ks][{tokens r, channels lo}, {tokens r, channels hi}, {tokens r + 8, lo}, {tokens r + 8, hi}]
+        // The loads of all eight tiles are in flight at once, before the wait for the logits (one tile ahead, the unit waited for
+        // memory eight times: one sequence of 4000 tokens 4.0 -> 3.4 us for this kernel, 8000 tokens 5.8 -> 4.7).
+        constexpr int kAhead = 8;
+        uint32_t x[kAhead][2][4];      // [ks][{tokens r, channels lo}, {tokens r, channels hi}, {tokens r + 8, lo}, {tokens r + 8, hi}]
         auto load_tile = [&](int ct) {
 #pragma unroll
           for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-              x[ks][2 * hh] = rowv[2 * ks + hh] ? rowp[2 * ks + hh][8 * ct] : 0u;
-              x[ks][2 * hh + 1] = rowv[2 * ks + hh] ? rowp[2 * ks + hh][8 * ct + 4] : 0u;
+              x[ct][ks][2 * hh] = rowv[2 * ks + hh] ? rowp[2 * ks + hh][8 * ct] : 0u;
+              x[ct][ks][2 * hh + 1] = rowv[2 * ks + hh] ? rowp[2 * ks + hh][8 * ct + 4] : 0u;
             }
         };
-        load_tile(0);
+#pragma unroll
+        for (int ct = 0; ct < kAhead; ++ct) load_tile(ct);
         wait_or_give_up(rfull_u32, rit & 1u);
         const uint32_t rb = ring_u32 + kRBufBase + lane * 32;
         const uint4 s0 = lds128(rb), s1 = lds128(rb + 16);
@@ -789,12 +792,11 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
           uint32_t a[2][4];
 #pragma unroll
           for (int ks = 0; ks < 2; ++ks) {
-            a[ks][0] = movmatrix_trans(x[ks][0]);
-            a[ks][1] = movmatrix_trans(x[ks][1]);
-            a[ks][2] = movmatrix_trans(x[ks][2]);
-            a[ks][3] = movmatrix_trans(x[ks][3]);
+            a[ks][0] = movmatrix_trans(x[ct][ks][0]);
+            a[ks][1] = movmatrix_trans(x[ct][ks][1]);
+            a[ks][2] = movmatrix_trans(x[ct][ks][2]);
+            a[ks][3] = movmatrix_trans(x[ct][ks][3]);
           }
-          if (ct + 1 < 8) load_tile(ct + 1);
 #pragma unroll
           for (int ks = 0; ks < 2; ++ks) {
             mma_bf16(O[ct], a[ks][0], a[ks][1], a[ks][2], a[ks][3], Bh[ks][0], Bh[ks][1]);

@@ -1226,8 +1226,8 @@ int attention_ws_grid(const LayerView& lv, int n_sms) {
   const long long wanted = min((total + 1) / 2, max((long long)n_sms, (total + 3) / 4));
   int grid = (int)min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), wanted);
   // a few positions per team: one CTA per stream, which needs no merge (eight sequences of 333 tokens, 20 positions: 6.6 -> 5.6 us
-  // per layer and a launch less; 40 positions 9.2 -> 9.9; three tiers, 26 positions, 6.7 -> 9.4)
-  if (attention_ws_positions(lv) <= (three_tiers(lv) ? 16 : 28)) grid = min(grid, S);
+  // per layer and a launch less; one sequence of 600, 25 positions, 5.7 -> 6.8; three tiers, 26 positions, 6.7 -> 9.4)
+  if (attention_ws_positions(lv) <= (three_tiers(lv) ? 16 : 20)) grid = min(grid, S);
   if (grid > S) grid = grid / S * S;
   return grid < 1 ? 1 : grid;
 }
