@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libmixkvq.so: argument marshalling only.
+"""Thin binding of libmixkvq.so: argument marshalling only, by ctypes, and in C (_calls) for the calls that a generation
+loop makes per layer and token.
 
 Every step of the path (scoring, quantization, packing, attention) runs in the library's CUDA kernels.
 PyTorch is used for device memory and the current stream.  If the shared library cannot be loaded this
@@ -96,6 +97,19 @@ def lib():
     return _lib
 
 
+_native = None
+
+
+def _calls():
+    """The native form of the per-token calls (csrc/calls.cpp): linked against the library that lib() loads."""
+    global _native
+    if _native is None:
+        lib()
+        from . import _calls as native
+        _native = native
+    return _native
+
+
 def status_string(code: int) -> str:
     return lib().mixkvq_status_string(int(code)).decode()
 
@@ -188,24 +202,26 @@ class Cache:
     def quantize_append(self, layer, k, v, q):
         """k, v [B,Hkv,n,128] bf16; q [B,Hq,n,128] bf16 (n may be 1: a decode step)."""
         n = k.shape[2]
-        _check(lib().mixkvq_quantize_append(self.handle, layer, _ptr(k), _ptr(v), _ptr(q), n, _stream()),
-               "mixkvq_quantize_append")
+        code = (_native or _calls()).quantize_append(self.handle.value, layer, k, v, q, n, _stream())
+        if code:
+            raise MixKVQError(code, "mixkvq_quantize_append")
 
     def decode_attention(self, layer, q, scale, out=None):
         """q [B,Hq,128] bf16 -> out [B,Hq,128] float32."""
         if out is None:
             out = torch.empty(q.shape, dtype=torch.float32, device=q.device)
-        _check(lib().mixkvq_decode_attention(self.handle, layer, _ptr(q), _ptr(out), float(scale),
-                                             *self._ws, _stream()),
-               "mixkvq_decode_attention")
+        code = (_native or _calls()).decode_attention(self.handle.value, layer, q, out, scale, *self._ws, _stream())
+        if code:
+            raise MixKVQError(code, "mixkvq_decode_attention")
         return out
 
     def decode_step(self, layer, k, v, q, scale, out=None):
         """One decode step: k, v [B,Hkv,1,128], q [B,Hq,1,128] bf16 -> out [B,Hq,128] float32 (append + attention)."""
         if out is None:
             out = torch.empty((q.shape[0], q.shape[1], 128), dtype=torch.float32, device=q.device)
-        _check(lib().mixkvq_decode_step(self.handle, layer, _ptr(k), _ptr(v), _ptr(q), _ptr(out), float(scale),
-                                        *self._ws, _stream()), "mixkvq_decode_step")
+        code = (_native or _calls()).decode_step(self.handle.value, layer, k, v, q, out, scale, *self._ws, _stream())
+        if code:
+            raise MixKVQError(code, "mixkvq_decode_step")
         return out
 
     def decode_attention_partial(self, layer, q, scale, out=None, lse=None):
@@ -260,9 +276,10 @@ class Cache:
         """One decode step with the rotation of k and q (in place) in front: see decode_step."""
         if out is None:
             out = torch.empty((q.shape[0], q.shape[1], 128), dtype=torch.float32, device=q.device)
-        _check(lib().mixkvq_rope_decode_step(self.handle, layer, _ptr(k), _ptr(v), _ptr(q), _ptr(cos), _ptr(sin), int(pos),
-                                             _ptr(out), float(scale), *self._ws,
-                                             _stream()), "mixkvq_rope_decode_step")
+        code = (_native or _calls()).rope_decode_step(self.handle.value, layer, k, v, q, cos, sin, int(pos), out, scale,
+                                                      *self._ws, _stream())
+        if code:
+            raise MixKVQError(code, "mixkvq_rope_decode_step")
         return out
 
     def decode_attention_noalloc(self, layer, q, scale, out=None):

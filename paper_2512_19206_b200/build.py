@@ -1,19 +1,21 @@
 """Builds libmixkvq.so (sm_100a) in-tree with nvcc.  Usable as `python -m paper_2512_19206_b200.build`.
 
 Every source file is compiled to an object of its own (in parallel, only when it or a header changed) and the
-objects are linked into the shared library.
+objects are linked into the shared library.  csrc/calls.cpp becomes _calls.so, a CPython module linked against it.
 """
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmixkvq.so")
+CALLS = os.path.join(HERE, "_calls.so")
 SOURCES = ["api.cu", "append.cu", "rope.cu", "prefill.cu", "select.cu", "flush.cu", "combine.cu", "attention_simt.cu", "attention_ws.cu", "attention_single.cu",
            "attention_tc.cu"]
 FLAGS = ["-Xcompiler", "-fPIC", "-O3", "-std=c++17", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
@@ -57,6 +59,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
                              capture_output=True, text=True)
         if res.returncode != 0:
             raise RuntimeError("link failed:\n" + res.stdout + res.stderr)
+    src = os.path.join(CSRC, "calls.cpp")
+    if force or not os.path.exists(CALLS) or max(os.path.getmtime(src), hdr_time) > os.path.getmtime(CALLS):
+        res = subprocess.run(["g++", "-O2", "-std=c++17", "-Wall", "-Wno-cast-function-type", "-fPIC", "-shared",
+                              "-I" + sysconfig.get_paths()["include"], src, "-o", CALLS, "-L" + HERE, "-l:libmixkvq.so",
+                              "-Wl,-rpath,$ORIGIN"], capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError("g++ failed on " + src + ":\n" + res.stdout + res.stderr)
     return LIB
 
 
