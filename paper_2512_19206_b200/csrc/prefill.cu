@@ -10,18 +10,24 @@
 // Per key tile j and row group g:
 //   S_g = Q_g K_j^T   bf16 operands from shared memory, fp32 accumulator in tensor memory;
 //   softmax           the thread reads its row of S (tcgen05.ld), applies scale and causal mask, and writes its row of P as
-//                     fp16 over columns that S occupied (tcgen05.st).  When the maximum of a row of the warp rises, the warp
-//                     rescales its rows of O (after the first tiles that is rare: a third of the 256 tiles at L = 32768);
-//   O_g += P_g V_j    A operand from tensor memory, V from shared memory (MN-major), accumulated in tensor memory.
+//                     fp16 over columns that S occupied (tcgen05.st);
+//   O_g = P_g V_j     A operand from tensor memory, V from shared memory (MN-major).  The thread adds its row of the product to
+//                     an fp32 sum in registers at the start of the next tile; when the maximum of a row of the warp has risen,
+//                     the warp rescales its sums first (after the first tiles that is rare: a third of the 256 tiles at L = 32768).
 // The issue order S_A(j+1) behind P_A V(j), S_B(j+1) behind P_B V(j) keeps the tensor core busy on one row group while
 // the other one is in its softmax; the softmax threads never wait for a P V product (products complete in issue order, so S(j)
 // being there means that P V(j-1) is done).  P and V are fp16 (11 significant bits): bf16 probabilities alone would cost up to
 // 2^-9 of the value range.  Every wait on a barrier is bounded; a wait that runs out sets the status word and the
 // role that saw it stops, after which the others run out too and the CTA finishes.
-// B200, whole call per layer, against the form whose threads kept O in registers and folded every P V into it (us): prompt of
-// 32768 tokens (7b shape) 7990 -> 7206, 8192: 690 -> 566, 333: 102 -> 48; 4 x 777 tokens (8b shape) 176 -> 121.  What went: the
-// wait for P V and the fold (1.6 of 3.9 thousand cycles per tile), 5 of 7 thousand cycles per masked diagonal tile, the Q load
-// one piece after the other (4 of 9 thousand cycles per CTA), the wait for the first K and V behind it.
+// Why the sum over the tiles is not left to the tensor core: its fp32 accumulator truncates, a bias of half a unit in the last
+// place per product, and 8 products per tile add up.  Against fp64, values with a mean (|N(0,1)| + 0.5), relative error at 777 /
+// 8192 / 32768 / 65536 tokens: 3.8e-5 / 3.8e-5 / 10.4e-5 / 17.8e-5 accumulated in tensor memory (bias -1.4e-4 at 32768);
+// 3.8e-5 / 2.8e-5 / 2.8e-5 / 2.8e-5 with the sum in registers, the rounding of P.  Sums over 2, 4, 8 or 16 tiles in tensor memory: 2.83,
+// 2.85, 2.91, 3.09e-5 at 32768, and no faster than 2 % (the registers cost the time, not the additions).
+// B200, whole call per layer (us), sum in tensor memory / in registers: prompt of 32768 tokens (7b shape) 6492 / 6811, 8192: 530 /
+// 558, 333: 29.4 / 29.5; 4 x 777 tokens (8b shape) 100.7 / 103.5.  (Waiting for each product right behind its issue, and with the tensor
+// core idle meanwhile: 7447, 699, 104, 169.)  Register split: 72 for the issuing warps leaves 96 bytes of spills; 56 and 224 spill
+// 212 there.
 #include "common.cuh"
 
 namespace mixkvq {
@@ -84,8 +90,8 @@ __device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a_desc, uint
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// A load of 32 columns of the thread's tensor-memory lane.  The registers are valid only after tmem_wait_ld32 / tmem_wait_ld16 on them (the wait
-// names the registers as operands, so that no use of them is scheduled before it).  tcgen05.wait::ld covers every load
+// A load of 32 columns of the thread's tensor-memory lane.  The registers are valid only after tmem_wait_ld32 on them (the wait names
+//  the registers as operands, so that no use of them is scheduled before it).  tcgen05.wait::ld covers every load
 // the thread has issued, so a load issued before a block of arithmetic and waited for after it runs under that arithmetic.
 __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&u)[32]) {
   asm volatile(
@@ -111,15 +117,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&w)[8])
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(w[0]), "r"(w[1]),
                "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
                : "memory");
-}
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&u)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
-      "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]), "r"(u[8]), "r"(u[9]), "r"(u[10]),
-      "r"(u[11]), "r"(u[12]), "r"(u[13]), "r"(u[14]), "r"(u[15]), "r"(u[16]), "r"(u[17]), "r"(u[18]), "r"(u[19]), "r"(u[20]),
-      "r"(u[21]), "r"(u[22]), "r"(u[23]), "r"(u[24]), "r"(u[25]), "r"(u[26]), "r"(u[27]), "r"(u[28]), "r"(u[29]), "r"(u[30]), "r"(u[31])
-      : "memory");
 }
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -212,12 +209,26 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   return d;
 }
 
+// Adds the row's P V product in tensor memory to the sum kept in registers.
+__device__ __forceinline__ void add_output(uint32_t o_addr, float (&sum_o)[128]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    uint32_t x[32];
+    tmem_ld32_issue(o_addr + 32 * c, x);
+    tmem_wait_ld32(x);
+#pragma unroll
+    for (int k = 0; k < 32; k += 2)
+      unpack2(add2(pack2u(x[k], x[k + 1]), pack2(sum_o[32 * c + k], sum_o[32 * c + k + 1])), sum_o[32 * c + k], sum_o[32 * c + k + 1]);
+  }
+}
+
 // One 128-key tile of one row group's softmax.  The thread owns one row of S (128 fp32 columns of its tensor-memory lane at
-// s_addr) and of O (at o_addr).  Writes P (fp16 pairs) over columns [0, 64) of S.  kDiag: the tile on the diagonal, where row i
+// s_addr) and of the last product P V (at o_addr), which goes to its sum.  Writes P (fp16 pairs) over columns [0, 64) of S.  kDiag: the tile on the diagonal, where row i
 // of the group sees columns <= i: warp w (rows 32 w ..) needs the columns of 32-chunks <= w, and a comparison only in chunk w.
 template <bool kDiag>
 __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, int w, int lane, bool first, float scale_log2e,
-                                             float& m_ref, float& l_run, uint32_t half_bar) {
+                                             float& m_ref, float& l_run, uint32_t half_bar, float (&sum_o)[128]) {
+  if (!first) add_output(o_addr, sum_o);             // the product of the tile before
   // ---- the row's maximum
   float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // four independent chains
   auto reduce = [&](const uint32_t (&u)[32], int last) {
@@ -228,59 +239,22 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, i
       mx4[(i >> 1) & 3] = fmaxf(fmaxf(mx4[(i >> 1) & 3], x0), x1);
     }
   };
-  if constexpr (kDiag) {
 #pragma unroll 1
-    for (int c = 0; c <= w; ++c) {
-      uint32_t a[32];
-      tmem_ld32_issue(s_addr + 32 * c, a);
-      tmem_wait_ld32(a);
-      reduce(a, c == w ? lane : 31);
-    }
-  } else {
-    uint32_t a[32], b[32];                          // chunk c + 1 is in flight while chunk c is reduced
-    tmem_ld32_issue(s_addr, a);
+  for (int c = 0; c < (kDiag ? w + 1 : 4); ++c) {
+    uint32_t a[32];
+    tmem_ld32_issue(s_addr + 32 * c, a);
     tmem_wait_ld32(a);
-    tmem_ld32_issue(s_addr + 32, b);
-    reduce(a, 31);
-    tmem_wait_ld32(b);
-    tmem_ld32_issue(s_addr + 64, a);
-    reduce(b, 31);
-    tmem_wait_ld32(a);
-    tmem_ld32_issue(s_addr + 96, b);
-    reduce(a, 31);
-    tmem_wait_ld32(b);
-    reduce(b, 31);
+    reduce(a, kDiag && c == w ? lane : 31);
   }
   const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale_log2e;
   if (first) {
     m_ref = mx;
   } else if (__any_sync(0xffffffffu, mx > m_ref)) {
-    // raise the reference and rescale what has been accumulated (all products before this S have completed)
+    // raise the reference and rescale the sum of the products before this tile
     const float m_new = fmaxf(m_ref, mx), alpha = ex2(m_ref - m_new);
     const uint64_t alpha2 = pack2(alpha, alpha);
-    uint32_t x[32], y[32];                          // chunk c + 1 is in flight while chunk c is scaled
-    auto rescale = [&](uint32_t (&z)[32], int c) {
 #pragma unroll
-      for (int k = 0; k < 32; k += 2) {
-        float a, b;
-        unpack2(mul2(pack2u(z[k], z[k + 1]), alpha2), a, b);
-        z[k] = __float_as_uint(a);
-        z[k + 1] = __float_as_uint(b);
-      }
-      tmem_st32(o_addr + 32 * c, z);
-    };
-    tmem_ld32_issue(o_addr, x);
-    tmem_wait_ld32(x);
-    tmem_ld32_issue(o_addr + 32, y);
-    rescale(x, 0);
-    tmem_wait_ld32(y);
-    tmem_ld32_issue(o_addr + 64, x);
-    rescale(y, 1);
-    tmem_wait_ld32(x);
-    tmem_ld32_issue(o_addr + 96, y);
-    rescale(x, 2);
-    tmem_wait_ld32(y);
-    rescale(y, 3);
+    for (int d = 0; d < 128; d += 2) unpack2(mul2(pack2(sum_o[d], sum_o[d + 1]), alpha2), sum_o[d], sum_o[d + 1]);
     l_run *= alpha;
     m_ref = m_new;
   }
@@ -431,7 +405,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
   };
 
   if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;" ::: "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;" ::: "memory");
     if (warp == 8 && lane == 0) {
       // ---------------------------------------------------------------- tensor-core issue
       const uint32_t idesc_qk = make_idesc(128, 128, 1, 0), idesc_pv = make_idesc(128, 128, 0, 1);
@@ -442,12 +416,12 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
         for (int ks = 0; ks < 8; ++ks) tc_mma_ss(tbase + 128 * g, qd + (uint64_t)(ks * 16), kd + (uint64_t)(ks * 16), idesc_qk, ks > 0);
         tc_commit(bar(kSFull + g));
       };
-      auto issue_o = [&](int g, int j, int half) {       // O_g += P_g V_j over 64 of the tile's keys
+      auto issue_o = [&](int g, int j, int half) {       // O_g = P_g V_j, 64 of the tile's keys at a time
         const uint64_t vd = make_desc(smem_u32(Vs + (j & 1) * kTileBytes), 128, 2048);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int ks = 4 * half + k;
-          tc_mma_ts(tbase + 256 + 128 * g, tbase + 128 * g + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, j > 0 || ks > 0);
+          tc_mma_ts(tbase + 256 + 128 * g, tbase + 128 * g + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, ks > 0);      // (a product of its own per tile)
         }
       };
       auto both_halves = [&](int g, int j) {             // as soon as each half of P_g is there
@@ -513,7 +487,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
       }
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 224;" ::: "memory");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 216;" ::: "memory");
     // ------------------------------------------------------------------ softmax and output rows
     const int g = warp >> 2, row = tid & 127;
     const uint32_t lane_base = tbase + ((uint32_t)((warp & 3) * 32) << 16);
@@ -521,14 +495,17 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     const int n = g == 0 ? n_a : n_b;
     const int pos = qt * kQRows + g * kTile + row;     // this thread's query position
     float m_ref = -INFINITY, l_run = 0.f;
+    float sum_o[128];
+#pragma unroll
+    for (int d = 0; d < 128; ++d) sum_o[d] = 0.f;
 #pragma unroll 1
     for (int j = 0; j < n; ++j) {
       if (!wait(kSFull + g, (uint32_t)j & 1u)) break;
       tc_fence_after();
       if (j == 2 * qt + g)      // the tile on the diagonal
-        softmax_tile<true>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g));
+        softmax_tile<true>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
       else
-        softmax_tile<false>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g));
+        softmax_tile<false>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
       tc_fence_before();
       mbar_arrive(bar(kPReady + g));
     }
@@ -538,18 +515,16 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     // any more, and leave as one bulk copy each.
     if (wait(g == 0 ? kDoneA : kDone, 0)) {
       tc_fence_after();
+      add_output(o_addr, sum_o);
       const float inv = 1.f / l_run;
       float* dst = out + ((size_t)(b * Hq + h) * L + pos) * kD;
       const bool wide = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
       const uint32_t staged = smem_u32(smem) + (uint32_t)row * 528u;      // (a row's 16-byte pieces on the banks of no other lane)
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        uint32_t x[32];
-        tmem_ld32_issue(o_addr + 32 * c, x);
-        tmem_wait_ld32(x);
         float y[32];
 #pragma unroll
-        for (int d = 0; d < 32; ++d) y[d] = __uint_as_float(x[d]) * inv;
+        for (int d = 0; d < 32; ++d) y[d] = sum_o[32 * c + d] * inv;
         if (g == 1) {
 #pragma unroll
           for (int d = 0; d < 32; d += 4)
