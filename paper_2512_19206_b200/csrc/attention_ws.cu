@@ -11,7 +11,7 @@
 //                     more tile chain per step (rows 0..7 the first unit's group, rows 8..15 the second's); the promoted
 //                     (BF16) channels and the UINT4 high plane are further tiles.  The step's 64 x 8 logits go to the
 //                     partner through shared memory, in the place of the key codes and scales they were made from.
-//   the values warp   keeps the online softmax (lazily raised reference maximum), builds the value-scale tables,
+//   the values warp   keeps the online softmax, builds the value-scale tables,
 //                     folds the value scales into the probabilities and runs P.V with the raw value codes as fp16
 //                     subnormals in the A operand (one logic op per pair of codes); value zero-points and the softmax
 //                     denominator ride on one extra tile.  It owns the output accumulators and refills the ring.
@@ -89,7 +89,6 @@ __host__ __device__ constexpr int smem_bytes(int G, int u4, bool v4) {
 }
 constexpr int kResidualWeight = 3;           // an unquantized 32-token unit counts as this many packed units in the split
 constexpr int kMergeStride = 132;            // floats per head row of a pair's output in the merge
-constexpr float kMaxSlack = 3.0f;            // a packed unit's probabilities are at most 2^kMaxSlack (log2 domain)
 // A wait on a barrier polls at most this many times; a poll suspends the thread for up to about a microsecond, so
 // the wait gives up after about two seconds at the latest (a few milliseconds if the polls return at once).
 constexpr uint32_t kWaitPolls = 1u << 21;
@@ -940,8 +939,10 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         const float zl[2][2] = {{__uint_as_float(zq.x) * scale_log2e, __uint_as_float(zq.y) * scale_log2e},
                                 {__uint_as_float(UPG == 1 ? zq.z : zq.x) * scale_log2e, __uint_as_float(UPG == 1 ? zq.w : zq.y) * scale_log2e}};
         // ---- online softmax (log2 domain); heads 2t, 2t+1; tokens r, r+8 of each m-tile.
-        // The reference maximum only has to keep the probabilities inside the fp16 range: it is raised (to the true
-        // maximum so far, with the accumulators rescaled) when a logit of this step exceeds it by more than kMaxSlack.
+        // The reference is the largest logit so far: a probability is exact in fp16 only where it is the reference, and the
+        // largest matter most.  (Raising it only when it is exceeded by 3 or more keeps the probabilities inside the fp16 range as well
+        // and is 0.5 to 1 % faster; relative error then against now: three tiers, 7b shape, 32768 tokens 1.25e-4 / 0.75e-4, 4-bit base, 8b
+        // shape, 16384 tokens 1.96e-4 / 1.10e-4, two tiers, 32b shape, 8000 tokens 1.83e-4 / 1.10e-4.)
         {
           float uu[2];
 #pragma unroll
@@ -950,7 +951,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
             const float b = fmaf(fmaxf(fmaxf(sx[1][0][h], sx[1][0][2 + h]), fmaxf(sx[1][1][h], sx[1][1][2 + h])), scale_log2e, zl[1][h]);
             uu[h] = fmaxf(a, b);
           }
-          if (__any_sync(0xffffffffu, (uu[0] > m0 + kMaxSlack) || (uu[1] > m1 + kMaxSlack))) raise_reference(uu[0], uu[1]);
+          if (__any_sync(0xffffffffu, uu[0] > m0 || uu[1] > m1)) raise_reference(uu[0], uu[1]);
         }
         // P^T B fragments: [unit][k-step][tokens 2t.. / 2t+8..], head r
         uint32_t Pt[2][2][2];
@@ -1221,6 +1222,10 @@ static bool three_tiers(const LayerView& lv) {
   return !lv.dense_hi && ((lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16);
 }
 
+// A few positions per team: one CTA per stream, which needs no merge (eight sequences of 333 tokens, 20 positions: 6.6 -> 5.6 us
+// per layer and a launch less; one sequence of 600, 25 positions, 5.7 -> 6.8; three tiers, 26 positions, 6.7 -> 9.4).
+static bool one_cta_per_stream(const LayerView& lv) { return attention_ws_positions(lv) <= (three_tiers(lv) ? 16 : 20); }
+
 // Number of CTAs the split kernel runs for this layer state (also the number of partial-slot owners).  When there are
 // fewer streams than CTA slots the grid is a multiple of the stream count, so that no CTA straddles two streams
 // (a second segment costs a pipeline drain, a query load and a second partial).
@@ -1233,9 +1238,7 @@ int attention_ws_grid(const LayerView& lv, int n_sms) {
   // merge: one sequence of 400 tokens 5.6 / 5.5 / 6.0, 4000 tokens 9.6 / 7.1 / 6.3, eight of 333 8.2 / 7.9 / 6.6).
   const long long wanted = min((total + 1) / 2, max((long long)n_sms, (total + 3) / 4));
   int grid = (int)min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), wanted);
-  // a few positions per team: one CTA per stream, which needs no merge (eight sequences of 333 tokens, 20 positions: 6.6 -> 5.6 us
-  // per layer and a launch less; one sequence of 600, 25 positions, 5.7 -> 6.8; three tiers, 26 positions, 6.7 -> 9.4)
-  if (attention_ws_positions(lv) <= (three_tiers(lv) ? 16 : 20)) grid = min(grid, S);
+  if (one_cta_per_stream(lv)) grid = min(grid, S);
   if (grid > S) grid = grid / S * S;
   return grid < 1 ? 1 : grid;
 }
@@ -1250,8 +1253,9 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // shape, batch 8) 8000 tokens, 27 units per CTA, 12.6 / 13.1, 16000 21.5 / 20.5; G = 128 (32b shape, batch 16) 2000 tokens,
   // 31 units, 13.5 / 13.0, 600 tokens, 10 units, 8.3 / 8.15; three tiers (7b shape) 600 tokens, 3 units, 6.4 / 6.7, 2000 tokens,
   // 7 units, 9.3 / 7.8; 4-bit base (8b shape, batch 16) 600 tokens, 12 units, 8.9 / 9.3, 2000 tokens, 31 units, 18.7 / 17.7.
+  // One CTA per stream takes one unit at a time, for the precision: a probability is exact where it is the maximum of its unit.
   const int from_units = three_tiers(lv) ? 6 : lv.dense_hi ? 20 : lv.G == 128 ? 10 : 40;
-  const bool by_two = !(lv.U & 1) && (lv.seq != nullptr ? lv.seq_total : Us * S) >= (long long)from_units * grid;
+  const bool by_two = !(lv.U & 1) && !(lv.seq == nullptr && one_cta_per_stream(lv)) && (lv.seq != nullptr ? lv.seq_total : Us * S) >= (long long)from_units * grid;
   // With one CTA per stream the split kernel writes the output itself (32b shape, 32 sequences of 900 tokens: 17.9 -> 12.4 us per
   // layer).  Merging several partials in the kernel, by the CTA that finds all of a stream's written, was slower than a merge
   // kernel: a fence, a look at the other CTAs' marks and a serial merge against a dependent launch (one sequence of 400

@@ -150,7 +150,7 @@ __device__ __forceinline__ uint32_t hmul2_u(uint32_t a, uint32_t b) {
   asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
 }
-// 2^x by the special-function unit alone (no range fix-up): inputs here are <= kMaxSlack or -inf
+// 2^x by the special-function unit alone (no range fix-up): inputs here are at most about 0, or -inf
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

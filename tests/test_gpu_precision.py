@@ -40,3 +40,39 @@ def test_prefill_sum_over_many_tiles(binding, L):
     assert float(d.norm() / ref.norm()) <= 6e-5
     last = slice(-16, None)
     assert abs(float(d[:, :, last].sum() / ref[:, :, last].sum())) <= 4e-5
+
+
+# Bounds of the relative error in 1e-5, half way between what a reference maximum at the largest probabilities gives (they are
+# then exact) and what one anywhere below them by up to a factor of 8 gives (each then rounded by up to 2^-12, and its product
+# with the value scale once more).
+@pytest.mark.parametrize("name,batch,tokens,preset,v_bits,bound", [
+    ("qwen7b", 1, 130, "P27", 2, 9.7),            # 7.2 / 12.2
+    ("qwen7b", 8, 390, "P24", 2, 7.9),            # 5.7 / 10.1
+    ("qwen7b", 8, 390, "P27", 2, 9.8),            # 6.0 / 13.6
+    ("qwen7b", 8, 390, "P24", 4, 8.5),            # 6.2 / 10.7
+    ("llama8b", 16, 400, "P4BASE", 2, 8.1),       # 5.6 / 10.6
+    ("llama8b", 16, 1200, "P24", 2, 6.6),         # 3.9 / 9.4
+    ("qwen7b", 8, 8000, "P24", 2, 3.9),           # 2.5 / 5.3
+    ("qwen7b", 8, 8000, "P27", 2, 5.1),           # 4.1 / 6.1
+    ("llama8b", 16, 4000, "P4BASE", 2, 10.0),     # 6.9 / 13.0
+    ("llama8b", 16, 4000, "P24", 4, 9.5),         # 6.7 / 12.3
+    ("qwen32b", 64, 700, "P27", 2, 13.6),         # 10.9 / 16.3
+])
+def test_decode_probabilities(binding, name, batch, tokens, preset, v_bits, bound):
+    """Against the plain-ALU kernel, which is fp32 throughout, on the same cache: one CTA per stream, few and many positions per
+    CTA, one and two units per step."""
+    w = W.small(W.CONFIGS[name], n_layers=1, batch=batch, tokens=tokens, **getattr(W, preset))
+    cache = U.make_cache(binding, w, v_bits=v_bits, extras_budget_bytes=(tokens // 128 + 3) * 64 * 128)
+    for t in range(0, tokens, 4096):
+        cache.quantize_append(0, *W.tokens(w, 0, t, min(4096, tokens - t), device="cuda"))
+    num = den = 0.0
+    for step in range(4):
+        q = W.decode_query(w, 0, step, device="cuda")
+        cache.set_attention_kernel(0)
+        out = cache.decode_attention(0, q, W.softmax_scale()).double()
+        cache.set_attention_kernel(1)
+        ref = cache.decode_attention(0, q, W.softmax_scale()).double()
+        num += float((out - ref).square().sum())
+        den += float(ref.square().sum())
+    assert cache.status() == 0
+    assert (num / den) ** 0.5 <= bound * 1e-5
