@@ -11,7 +11,7 @@
 //                     extra tile chain per group) is the initial value of the accumulators; the promoted (BF16)
 //                     channels and the UINT4 high plane are further tiles.  The unit's 32 x 8 logits go to the
 //                     partner through shared memory.
-//   the values warp   keeps the online softmax (its reference follows the units' maxima), builds the unit's value-scale tables,
+//   the values warp   keeps the online softmax, builds the unit's value-scale tables,
 //                     folds the value scales into the probabilities and runs P.V with the raw value codes as fp16
 //                     subnormals in the A operand (one logic op per pair of codes); value zero-points and the softmax
 //                     denominator ride on one extra tile.  It owns the output accumulators and refills the ring.
@@ -58,11 +58,14 @@ constexpr int kMergeStride = 132;            // floats per head row of a pair's 
 // tile does.  (The gathered UINT4 tiles stay with the logits warp in every case: moved, they made the values warp the
 // longer role and the kernel slower.)
 __host__ __device__ constexpr bool promoted_in_values(int u4) { return u4 != 0; }
-// A pair's reference maximum follows every packed unit's maximum, but stays within this (log2 domain) of the largest so far.  A
-// token's probability is exact in fp16 only where it is the reference, and the tokens that matter most are their units' maxima.
-// Relative error (2-norm, against the plain-ALU fp32 kernel) with a reference that is only raised, by 3 or more / with this
-// and the fresh tile of add_products: 7b shape, batch 8, 390 tokens 1.64e-4 / 0.98e-4, 9000 tokens 1.07e-4 / 0.73e-4; 8b shape, batch
-// 16, 400 tokens 1.79e-4 / 1.03e-4.  Cost: nothing below 3000 tokens per sequence, 1 to 2 % above.
+// A token's probability is exact in fp16 only where it is the softmax reference, and the largest matter most.
+//   Short streams (kDirect): a pair's reference follows every packed unit's maximum, but stays within kFollowDrop (log2 domain) of the
+//   largest so far, and a unit's products are added up by themselves (add_products).
+//   Otherwise: the reference is the largest logit so far.
+// Relative error (2-norm, against the plain-ALU fp32 kernel) of a reference that is only raised when exceeded by 3 / of these: 7b
+// shape, batch 8, 390 tokens 1.64e-4 / 0.98e-4, 9000 tokens 1.07e-4 / 0.89e-4; 8b shape, batch 16, 400 tokens 1.79e-4 / 1.03e-4, 1200 tokens
+// 1.52e-4 / 1.03e-4.  Following everywhere would give 0.73e-4 and 0.80e-4 in the second and the last, for 2 to 5 % of the time of long
+// streams; both forms in one kernel, by length, cost 10 to 20 % (registers).
 constexpr float kFollowDrop = 10.0f;
 // A wait on a barrier polls at most this many times; a poll suspends the thread for up to about a microsecond, so
 // the wait gives up after about two seconds at the latest (a few milliseconds if the polls return at once).
@@ -988,11 +991,12 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
         // logit = (sx + q . z) * scale: the zero-point term of the key group is the same for every token of the unit
         const float zl0 = __uint_as_float(zq.x) * scale_log2e, zl1 = __uint_as_float(zq.y) * scale_log2e;
         // ---- online softmax (log2 domain); heads 2t, 2t+1; tokens r, r+8 of each m-tile.
-        // The reference follows the unit's maximum (kFollowDrop).
+        // The reference: see kFollowDrop.
         {
           const float u0 = fmaf(fmaxf(fmaxf(sx[0][0], sx[0][2]), fmaxf(sx[1][0], sx[1][2])), scale_log2e, zl0);
           const float u1 = fmaf(fmaxf(fmaxf(sx[0][1], sx[0][3]), fmaxf(sx[1][1], sx[1][3])), scale_log2e, zl1);
-          follow_reference(u0, u1);
+          if constexpr (kDirect) follow_reference(u0, u1);
+          else if (__any_sync(0xffffffffu, u0 > m0 || u1 > m1)) raise_reference(u0, u1);
         }
         const float c0 = zl0 - m0, c1 = zl1 - m1;
         // P^T B fragments: [k-step][tokens 2t.. / 2t+8..], head r
@@ -1008,13 +1012,13 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
           const uint4 zz = lds128(lane16 + kPrepBase + kZvpOff + ks * 576);
           mma_f16(Zc, zz.x, zz.y, zz.z, zz.w, Pt[ks][0], Pt[ks][1]);
         }
-        // ---- P.V: codes as fp16 subnormals, scales folded into P.  A unit's products start from zero and are added to the output
-        // by fp32 FMAs (which also move it to the new reference): the tensor core aligns its addends by the exponents of the
+        // ---- P.V: codes as fp16 subnormals, scales folded into P.  In short streams a unit's products start from zero and are
+        // added to the output by fp32 FMAs (which also move it to the new reference): the tensor core aligns its addends by the exponents of the
         // operands, and a subnormal operand counts as 2^-14, so an output passed through it loses what lies 2^-17 below a
         // unit's products.
         auto add_products = [&](int ct, uint32_t x0, uint32_t x1, const uint32_t (&Bp)[2][2], bool fresh) {
           constexpr uint32_t k0 = 0x00030003u, k1 = k0 << 2, k2 = k0 << 4, k3 = k0 << 6;
-          if (fresh) {
+          if (kDirect && fresh) {
             float t4[4];
             mma_f16_to(t4, x0 & k0, x1 & k0, x0 & k1, x1 & k1, Bp[0][0], Bp[0][1], 0.f, 0.f, 0.f, 0.f);
             mma_f16(t4, x0 & k2, x1 & k2, x0 & k3, x1 & k3, Bp[1][0], Bp[1][1]);

@@ -1222,9 +1222,16 @@ static bool three_tiers(const LayerView& lv) {
   return !lv.dense_hi && ((lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16);
 }
 
-// A few positions per team: one CTA per stream, which needs no merge (eight sequences of 333 tokens, 20 positions: 6.6 -> 5.6 us
-// per layer and a launch less; one sequence of 600, 25 positions, 5.7 -> 6.8; three tiers, 26 positions, 6.7 -> 9.4).
-static bool one_cta_per_stream(const LayerView& lv) { return attention_ws_positions(lv) <= (three_tiers(lv) ? 16 : 20); }
+// A few positions per team: one CTA per stream, which needs no merge.  With two tiers and 2-bit values it is never slower than the
+// split up to 20 positions (us per layer, one CTA per stream / split, 300 tokens: one sequence 5.4 / 5.3, eight 5.5 / 5.8, 16 of the 8b
+// shape 6.4 / 7.9; 600 tokens, 25 positions, one sequence 6.8 / 5.7).  Otherwise a unit takes longer, and beyond 12 positions
+// the split is faster as long as it gets by with one CTA per SM (three tiers, 300 and 390 tokens, one sequence 6.5 / 5.8, 64 streams
+// 6.9 / 8.8; 4-bit base 6.6 / 5.7, 6.8 / 8.6; 4-bit values 6.2 / 5.5, 6.3 / 7.9; three tiers with 4-bit values 7.1 / 5.9, 7.6 / 9.2).
+static bool one_cta_per_stream(const LayerView& lv, int n_sms) {
+  const long long p = attention_ws_positions(lv);
+  const bool plain = !lv.dense_hi && !three_tiers(lv) && lv.v_bits == 2;
+  return p <= (plain ? 20 : 12) || (p <= 20 && p * lv.B * lv.Hkv > 4 * n_sms);
+}
 
 // Number of CTAs the split kernel runs for this layer state (also the number of partial-slot owners).  When there are
 // fewer streams than CTA slots the grid is a multiple of the stream count, so that no CTA straddles two streams
@@ -1238,7 +1245,7 @@ int attention_ws_grid(const LayerView& lv, int n_sms) {
   // merge: one sequence of 400 tokens 5.6 / 5.5 / 6.0, 4000 tokens 9.6 / 7.1 / 6.3, eight of 333 8.2 / 7.9 / 6.6).
   const long long wanted = min((total + 1) / 2, max((long long)n_sms, (total + 3) / 4));
   int grid = (int)min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), wanted);
-  if (one_cta_per_stream(lv)) grid = min(grid, S);
+  if (one_cta_per_stream(lv, n_sms)) grid = min(grid, S);
   if (grid > S) grid = grid / S * S;
   return grid < 1 ? 1 : grid;
 }
@@ -1252,10 +1259,17 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // coarser split and the longer first step cost more.  us per launch, one unit / two units per step: two tiers, G = 32 (7b
   // shape, batch 8) 8000 tokens, 27 units per CTA, 12.6 / 13.1, 16000 21.5 / 20.5; G = 128 (32b shape, batch 16) 2000 tokens,
   // 31 units, 13.5 / 13.0, 600 tokens, 10 units, 8.3 / 8.15; three tiers (7b shape) 600 tokens, 3 units, 6.4 / 6.7, 2000 tokens,
-  // 7 units, 9.3 / 7.8; 4-bit base (8b shape, batch 16) 600 tokens, 12 units, 8.9 / 9.3, 2000 tokens, 31 units, 18.7 / 17.7.
-  // One CTA per stream takes one unit at a time, for the precision: a probability is exact where it is the maximum of its unit.
-  const int from_units = three_tiers(lv) ? 6 : lv.dense_hi ? 20 : lv.G == 128 ? 10 : 40;
-  const bool by_two = !(lv.U & 1) && !(lv.seq == nullptr && one_cta_per_stream(lv)) && (lv.seq != nullptr ? lv.seq_total : Us * S) >= (long long)from_units * grid;
+  // 7.6 units, 9.3 / 7.8 (8b shape, R = 64, 700 tokens, 6.5 units, 9.3 / 8.5, but an error of 0.86e-4 / 1.12e-4); 4-bit base (8b shape, batch 16) 600 tokens, 12 units, 8.9 / 9.3, 2000 tokens, 31 units, 18.7 / 17.7.
+  const int from_units = three_tiers(lv) ? 7 : lv.dense_hi ? 20 : lv.G == 128 ? 10 : 40;
+  bool by_two = !(lv.U & 1) && (lv.seq != nullptr ? lv.seq_total : Us * S) >= (long long)from_units * grid;
+  // A short stream with a CTA of its own takes one unit at a time, for the precision: a probability is exact where it is the
+  // maximum of its unit.
+  if (lv.seq == nullptr && grid == S && one_cta_per_stream(lv, n_sms)) by_two = false;
+  // 4-bit values: with more streams than CTAs every CTA begins two or three streams, and the longer steps make each beginning longer.
+  // us per launch, one unit / two units per step, 512 streams: three tiers, G = 32 1000 tokens 45 / 49, 1700 58 / 60, 3000 87 / 84,
+  // G = 128 1000 tokens 45 / 46, 1700 57 / 56; 4-bit base, G = 64 1700 tokens 61 / 63, 3000 94 / 91, G = 32 1700 64 / 73, 16000
+  // 422 / 434; two tiers, G = 32 1000 tokens 39 / 44, 3000 75 / 73.
+  if (lv.v_bits == 4 && lv.seq == nullptr && grid < S && (Us < (lv.G == 32 || lv.dense_hi ? 72 : 48) || (lv.dense_hi && lv.G == 32))) by_two = false;
   // With one CTA per stream the split kernel writes the output itself (32b shape, 32 sequences of 900 tokens: 17.9 -> 12.4 us per
   // layer).  Merging several partials in the kernel, by the CTA that finds all of a stream's written, was slower than a merge
   // kernel: a fence, a look at the other CTAs' marks and a serial merge against a dependent launch (one sequence of 400
