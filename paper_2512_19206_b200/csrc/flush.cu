@@ -286,7 +286,7 @@ __device__ inline void keys_role(const LayerView& lv, unsigned char* smem, const
   uint8_t* tierS = reinterpret_cast<uint8_t*>(aS + kD);                               // [128]
   uint8_t* chan16S = tierS + kD;                                                      // [128]
   uint8_t* chan4S = chan16S + kD;                                                     // [128]
-  int* cntS = reinterpret_cast<int*>(chan4S + kD);                                    // [8], then n16, n4, place
+  int* cntS = reinterpret_cast<int*>(chan4S + kD);                                    // [8], then n16, n4, place, whether it has one
   auto key_at = [&](int j, int d) { return reinterpret_cast<const uint16_t*>(kS + j * kKeyRow)[d]; };
 
   char* state = lv.state + (size_t)s * lv.state_stride;
@@ -367,18 +367,20 @@ __device__ inline void keys_role(const LayerView& lv, unsigned char* smem, const
     if (m4 & (1u << lane)) chan4S[b4 + __popc(m4 & below)] = (uint8_t)tid;
   } else if (tid == kD) {
     int n16 = cntS[0] + cntS[1] + cntS[2] + cntS[3], n4 = cntS[4] + cntS[5] + cntS[6] + cntS[7];
+    const uint32_t need = flush_extras_bytes(lv, n16, n4);
     uint32_t off16 = 0;
+    bool placed = true;
     if (bulk) {
       // the tiers role placed the block (and cleared the counts if the arena was full)
-      const uint2 e = *table_entry;
-      off16 = e.x;
-      if ((e.y & 0xFFFFu) == 0u) n16 = n4 = 0;
+      off16 = table_entry->x;
+      placed = (uint64_t)off16 * 16 + need <= lv.extras_budget;
+      if (!placed) n16 = n4 = 0;
     } else {
       uint32_t* used = reinterpret_cast<uint32_t*>(state + 1028);
       off16 = *used;
-      const uint32_t need = flush_extras_bytes(lv, n16, n4);
       if ((uint64_t)off16 * 16 + need > lv.extras_budget) {
         atomicOr(lv.status, (uint32_t)MIXKVQ_DEV_EXTRAS_FULL);
+        placed = false;
         n16 = n4 = 0;      // nothing goes to the arena and the entry records no promoted channel; the status word says so
       } else {
         *used = off16 + need / 16;
@@ -388,6 +390,7 @@ __device__ inline void keys_role(const LayerView& lv, unsigned char* smem, const
     cntS[8] = n16;
     cntS[9] = n4;
     cntS[10] = (int)off16;
+    cntS[11] = placed ? 1 : 0;
   }
   for (int i = tid; i < NG * kD; i += 256) {
     const int kg = i >> 7, d = i & 127;
@@ -551,8 +554,8 @@ __device__ inline void keys_role(const LayerView& lv, unsigned char* smem, const
         }
         reinterpret_cast<uint32_t*>(ex + hdr + (size_t)u * exunit + 128 * n16p)[rem] = w;
       }
-    } else if (n4 == 0 && (n16 > 0)) {
-      // 4-bit base, every channel promoted: the dense plane exists and is zero
+    } else if (n4 == 0 && cntS[11]) {
+      // 4-bit base, no channel in UINT4 (all promoted, or saliences that are NaN): the dense plane exists and is zero
       for (int i = tid; i < U * 64; i += 256)
         reinterpret_cast<uint4*>(ex + hdr + (size_t)(i >> 6) * exunit + 128 * n16p)[i & 63] = make_uint4(0u, 0u, 0u, 0u);
     }

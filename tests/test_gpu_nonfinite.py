@@ -1,0 +1,66 @@
+"""Tokens with NaNs and infinities: the append paths agree with one another and with the definition (the oracle's serial sums)."""
+import numpy as np
+import pytest
+import torch
+
+import gpu_util as U
+from oracle import mixkvq_oracle as O
+from paper_2512_19206_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2512_19206_b200 import build
+    build.build()
+    from paper_2512_19206_b200 import binding as b
+    b.lib()
+    return b
+
+
+def queries(q, kind):
+    q = q.clone()
+    if kind == "nan token":              # nothing else in the append of that token
+        q[:, :, 40] = float("nan")
+    elif kind == "nan window":           # a window of nothing else
+        q[:, :, 32:64] = float("nan")
+    elif kind == "nan among zeros":
+        q[:, :, :64] = 0.0
+        q[:, :, 40, 17] = float("nan")
+    elif kind == "infinity":
+        q[:, :, 40, ::5] = float("-inf")
+    return q
+
+
+def same(got, want):
+    """State of one stream: magnitude sums with NaNs where the oracle has them (their payload is not defined), then the counters."""
+    a, b = np.frombuffer(got[:1024], np.float64), np.frombuffer(want[:1024], np.float64)
+    return np.array_equal(a, b, equal_nan=True) and got[1024:] == want[1024:]
+
+
+@pytest.mark.parametrize("path", ["step"])
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("kind", ["nan token", "nan window", "nan among zeros", "infinity"])
+def test_query_magnitudes(binding, kind, mode, path):
+    T = 2 * 32 + 9
+    w = W.small(W.CONFIGS["qwen7b"], n_layers=1, batch=1, tokens=T, residual_len=32, **W.P4BASE)
+    k, v, q = W.tokens(w, 0, 0, T)
+    q = queries(q, kind)
+    cache = U.make_cache(binding, w, importance_mode=mode, extras_budget_bytes=8 * 64 * 128)
+    cache.mem.fill_(0xA5)                # whatever is not written shows
+    cache.reset()
+    cuda = [x.cuda() for x in (k, v, q)]
+    if path == "bulk":
+        cache.quantize_append(0, *cuda)
+    for t in range(T if path != "bulk" else 0):
+        x = [y[:, :, t:t + 1].contiguous() for y in cuda]
+        if path == "single":
+            cache.quantize_append(0, *x)
+        else:
+            cache.decode_step(0, *x, W.softmax_scale())
+    for (b, hk), st in U.oracle_streams(w, 0, k, v, q, importance_mode=mode).items():
+        got, want = cache.stream_regions(0, b * w.n_kv_heads + hk), O.pack_stream(st)
+        assert same(got["state"], want["state"]), (hk, "state")
+        for key in ("table", "base", "extras", "resK", "resV"):
+            assert got[key] == want[key], (hk, key)
