@@ -498,9 +498,13 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
           // first plane to run is the high plane, which lies with the block's extras in global memory)
           uint4 hw0, hw1;
           if constexpr (kU4 == 2) {
-            const uint4* kplane = reinterpret_cast<const uint4*>(exu + 128 * n16p);
-            hw0 = kplane[lane];
-            hw1 = kplane[32 + lane];
+            // (a block whose extras did not fit the arena has no high plane: nothing of it may be read)
+            hw0 = hw1 = make_uint4(0u, 0u, 0u, 0u);
+            if (n16 + n4 > 0) {
+              const uint4* kplane = reinterpret_cast<const uint4*>(exu + 128 * n16p);
+              hw0 = kplane[lane];
+              hw1 = kplane[32 + lane];
+            }
           } else {
             hw0 = lds128(stg + kUnitOff);
             hw1 = lds128(stg + kUnitOff + 512);

@@ -64,3 +64,21 @@ def test_query_magnitudes(binding, kind, mode, path):
         assert same(got["state"], want["state"]), (hk, "state")
         for key in ("table", "base", "extras", "resK", "resV"):
             assert got[key] == want[key], (hk, key)
+
+
+@pytest.mark.parametrize("tokens", [3 * 128 + 1, 128 * 128])        # one unit per step, two units per step
+def test_blocks_without_a_high_plane(binding, tokens):
+    """4-bit base with an arena that is too small: the blocks that did not fit have no high plane, and the attention takes
+    their codes as the plain-ALU kernel does (the low two bits) without reading behind the arena."""
+    w = W.small(W.CONFIGS["qwen7b"], n_layers=1, batch=4, tokens=tokens, **W.P4BASE)
+    cache = U.make_cache(binding, w, extras_budget_bytes=2 * 4 * 2048)
+    cache.mem.fill_(0xA5)
+    cache.reset()
+    for t in range(0, tokens, 4096):
+        cache.quantize_append(0, *W.tokens(w, 0, t, min(4096, tokens - t), device="cuda"))
+    assert cache.status() == binding.DEV_EXTRAS_FULL
+    q = W.decode_query(w, 0, 0, device="cuda")
+    out = cache.decode_attention(0, q, W.softmax_scale())
+    cache.set_attention_kernel(1)
+    ref = cache.decode_attention(0, q, W.softmax_scale())
+    assert float((out - ref).abs().max()) <= 4e-3          # both kernels are within 2e-3 of the exact result
