@@ -103,22 +103,21 @@ __device__ inline double abs_sum_256(const uint16_t* __restrict__ qw, size_t hea
   double total = a0;
   bool exact = true;
   const uint32_t smallest = *minS;
-  *unit = kAbsSumZero;
-  if (smallest != 0xFFFFu) {
-    const int e = (int)((smallest + 1u) >> 7);                          // biased exponent of the smallest magnitude
-    *unit = e - 134;                                                    // all magnitudes are multiples of 2^unit
-    if (tid < kD) {
-      double s = 0.0;
+  const bool none = smallest == 0xFFFFu;                                // nothing but zeros (and NaNs)
+  const int e = none ? 0 : (int)((smallest + 1u) >> 7);                 // biased exponent of the smallest magnitude
+  *unit = none ? kAbsSumZero : e - 134;                                 // all magnitudes are multiples of 2^unit
+  if (tid < kD) {
+    double s = 0.0;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) s = __dadd_rn(s, redS[w * kD + tid]);
-      s = __dmul_rn(s, kMagnitudeScale);
-      // Zeros went in as 2^-127.  With every other magnitude at least 2^-47 they disappear in the first one they meet (at
-      // most 2^12 of them with the rows past the end, 2^-115 against a half unit of 2^-100), and a channel of zeros alone stays below 2^-100.
-      if (s < 7.888609052210118e-31) s = 0.0;
-      total = __dadd_rn(a0, s);
-      // (a sum of 2^128 or more: possibly infinities)
-      exact = e >= 80 && s < 3.402823669209385e38 && sum_is_exact(a0, total, *unit);
-    }
+    for (int w = 0; w < 8; ++w) s = __dadd_rn(s, redS[w * kD + tid]);
+    s = __dmul_rn(s, kMagnitudeScale);
+    // Zeros went in as 2^-127.  With every other magnitude at least 2^-47 they disappear in the first one they meet (at
+    // most 2^12 of them with the rows past the end, 2^-115 against a half unit of 2^-100), and a channel of zeros alone stays below 2^-100.
+    if (s < 7.888609052210118e-31) s = 0.0;
+    total = __dadd_rn(a0, s);
+    // (a sum of 2^128 or more: possibly infinities, or NaNs, which went in as 2^128 and more and which the search for the
+    // smallest magnitude passes over)
+    exact = s < 3.402823669209385e38 && (none || (e >= 80 && sum_is_exact(a0, total, *unit)));
   }
   if (!__syncthreads_and(exact ? 1 : 0)) {
     *unit = kAbsSumRounded;

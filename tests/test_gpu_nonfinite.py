@@ -39,7 +39,7 @@ def same(got, want):
     return np.array_equal(a, b, equal_nan=True) and got[1024:] == want[1024:]
 
 
-@pytest.mark.parametrize("path", ["step"])
+@pytest.mark.parametrize("path", ["bulk", "single", "step"])
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("kind", ["nan token", "nan window", "nan among zeros", "infinity"])
 def test_query_magnitudes(binding, kind, mode, path):
