@@ -48,24 +48,34 @@ __device__ __forceinline__ float lo_f(uint32_t w) { return __uint_as_float(w << 
 __device__ __forceinline__ float hi_f(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
 // Reciprocal of a stored scale for the code computation; 0 for s = 0 (a constant group, or a channel without codes): every
-// code is then 0.
-__device__ __forceinline__ float code_reciprocal(float s) { return s == 0.0f ? 0.0f : __frcp_rn(s); }
+// code is then 0.  A scale of 2^-128 or less has none in fp32: NaN, which sends every code of the group to the division.
+__device__ __forceinline__ float code_reciprocal(float s) {
+  const float r = __frcp_rn(s);
+  return s == 0.0f ? 0.0f : (fabsf(r) == INFINITY ? __int_as_float(0x7FFFFFFF) : r);
+}
 
 // The code of Eq. 2 (quant_code in common.cuh) without its division: p = t * r with t = x - z rounded as there and
 // r = RN(1 / s) differs from the IEEE quotient by less than 2e-6 (codes are at most 15), so it rounds to the same
 // integer unless it lies within 4e-6 of a half-integer.  Adding 1.5 * 2^23 rounds p to an integer, to nearest even, in
-// the low bits of the sum; `off` collects the largest distance from p to its integer, and the caller settles a batch of
-// codes one by one when it comes that close to one half.  With bf16 data that is mostly an exact tie, x - z = (c + 1/2) s
+// the low bits of the sum; `off` collects the largest distance from p to its integer (NaN if any is: an element that is NaN or
+// infinite, or a scale without a reciprocal), and the caller settles a batch of codes one by one when it comes that close
+// to one half.  With bf16 data that is mostly an exact tie, x - z = (c + 1/2) s
 // (about one code in a thousand, so every third batch of a warp): settled by one FMA, which is zero exactly then; only
 // what is left takes the division (all of them dividing: 44 us for the keys of 992 windows, 34 us so).
 constexpr float kMagic = 12582912.0f, kHalfMargin = 0.5f - 4e-6f;
+__device__ __forceinline__ float max_or_nan(float a, float b) {
+  float y;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+__device__ __forceinline__ bool settled(float off) { return off <= kHalfMargin; }      // (not for a NaN)
 __device__ __forceinline__ uint32_t code_bits(float x, float z, float r, float& off) {
   const float t = __fsub_rn(x, z);
   const float m = __fmaf_rn(t, r, kMagic);
-  off = fmaxf(off, fabsf(__fmaf_rn(t, r, -__fsub_rn(m, kMagic))));
+  off = max_or_nan(off, fabsf(__fmaf_rn(t, r, -__fsub_rn(m, kMagic))));
   return __float_as_uint(m);            // the code in the low four bits
 }
-// a code that came close to one half
+// a code that came close to one half, or whose product is NaN
 __device__ __noinline__ uint32_t close_code(float x, float z, float r, float s, int max_code) {
   const float t = __fsub_rn(x, z);
   const float c = __fsub_rn(__fmaf_rn(t, r, kMagic), kMagic), d = __fmaf_rn(t, r, -c);
@@ -77,7 +87,7 @@ __device__ __noinline__ uint32_t close_code(float x, float z, float r, float s, 
 __device__ __forceinline__ uint32_t settle_code(float x, float z, float r, float s, int max_code) {
   float off = 0.f;
   const uint32_t c = code_bits(x, z, r, off) & 15u;
-  return off <= kHalfMargin ? c : close_code(x, z, r, s, max_code);
+  return settled(off) ? c : close_code(x, z, r, s, max_code);
 }
 // stored metadata word {s, z} -> {r, z}
 __device__ __forceinline__ float2 code_params(uint32_t meta) { return make_float2(code_reciprocal(lo_f(meta)), hi_f(meta)); }
@@ -444,7 +454,7 @@ __device__ inline void keys_role(const LayerView& lv, unsigned char* smem, const
             part |= (code_bits(lo_f(xx[f]), p.y, p.x, off) & 3u) << (2 * (4 * half + f));
             part |= (code_bits(hi_f(xx[f]), p.w, p.z, off) & 3u) << (16 + 2 * (4 * half + f));
           }
-          if (off > kHalfMargin) {
+          if (!settled(off)) {
             part = 0;
             for (int f = 0; f < 4; ++f)
               for (int e = 0; e < 2; ++e)
@@ -499,7 +509,7 @@ __device__ inline void keys_role(const LayerView& lv, unsigned char* smem, const
             c[ch][rh][1] = code_bits(hi_f(x), p.w, p.z, off);
           }
         }
-        if (off > kHalfMargin) {
+        if (!settled(off)) {
 #pragma unroll
           for (int ch = 0; ch < 2; ++ch) {
             const float4 p = prm4[8 * kt + 4 * ch];
@@ -648,7 +658,7 @@ __device__ inline void values_role(const LayerView& lv, unsigned char* smem, con
           part[0] |= (code_bits(lo_f(x), p.y, p.x, off) & 3u) << bit;
           part[1] |= (code_bits(hi_f(x), p.y, p.x, off) & 3u) << bit;
         }
-        if (off > kHalfMargin) {
+        if (!settled(off)) {
           part[0] = part[1] = 0;
           for (int k = 0; k < 8; ++k)
             for (int e = 0; e < 2; ++e)
@@ -685,7 +695,7 @@ __device__ inline void values_role(const LayerView& lv, unsigned char* smem, con
               c[e][rh][1] = code_bits(hi_f(x), p.y, p.x, off);
             }
           }
-          if (off > kHalfMargin) {
+          if (!settled(off)) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               const float2 p = prmS[(j + e) * VG + vg];

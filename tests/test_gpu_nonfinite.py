@@ -82,3 +82,54 @@ def test_blocks_without_a_high_plane(binding, tokens):
     cache.set_attention_kernel(1)
     ref = cache.decode_attention(0, q, W.softmax_scale())
     assert float((out - ref).abs().max()) <= 4e-3          # both kernels are within 2e-3 of the exact result
+
+
+def elements(x, kind, seed):
+    g = torch.Generator().manual_seed(seed)
+    x = x.float()
+    if kind == "subnormal":              # ranges from 0 to a few units of 2^-133, the last bit of a bf16 subnormal
+        scale = torch.pow(2.0, torch.randint(-133, -124, (*x.shape[:2], 1, x.shape[3]), generator=g).float())
+        x = torch.randint(0, 24, x.shape, generator=g).float() * scale
+    elif kind == "huge":                 # ranges that overflow fp32 among them
+        x = x * 2.0 ** 125.5
+    else:
+        value = {"nan": float("nan"), "inf": float("inf"), "-inf": float("-inf")}[kind]
+        x = torch.where(torch.rand(x.shape, generator=g) < 0.002, torch.tensor(value), x)
+    return x.to(torch.bfloat16)
+
+
+def quantize_past_nans(x, bits):
+    """The oracle's quantizer with extrema that pass over NaNs and code 0 for what has no quotient, as the header's contract for
+    finite values extends to them in the kernels."""
+    x = np.asarray(x, np.float32)
+    levels = np.float32((1 << bits) - 1)
+    with np.errstate(all="ignore"):
+        z, mx = np.fmin.reduce(x, axis=-1), np.fmax.reduce(x, axis=-1)
+        s = O.bf16_round_up(((mx - z).astype(np.float32) / levels).astype(np.float32))
+        y = np.rint(((x - z[..., None]).astype(np.float32) / s[..., None]).astype(np.float32))
+    return np.where(np.isnan(y) | (s == 0)[..., None], 0, np.clip(y, 0, float(levels))).astype(np.uint8), s, z
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("preset,v_bits", [("P24", 2), ("P4BASE", 4)])
+@pytest.mark.parametrize("kind", ["subnormal", "huge", "nan", "inf", "-inf"])
+def test_codes(binding, monkeypatch, kind, preset, v_bits, layout):
+    if layout == 1 and v_bits == 4:
+        pytest.skip("the tile layout holds 2-bit values only")
+    w = W.small(W.CONFIGS["qwen7b"], n_layers=1, batch=1, tokens=3 * 128 + 5, **{**getattr(W, preset), "tau_bf16": 1e39})
+    if preset == "P24":
+        w = W.small(w, tau_u4=1e39)
+    k, v, q = W.tokens(w, 0, 0, w.tokens)
+    k, v = elements(k, kind, 1), elements(v, kind, 2)
+    monkeypatch.setattr(O, "quantize_groups", quantize_past_nans)
+    monkeypatch.setattr(O, "salience", lambda acc, cnt, kw, bits: (np.ones(128), np.ones(128), np.ones(128)))     # (one tier: 1e39 is infinite in fp32)
+    caches = [U.make_cache(binding, w, v_bits=v_bits, layout=layout, extras_budget_bytes=4 * 64 * 128) for _ in range(2)]
+    caches[0].quantize_append(0, k.cuda(), v.cuda(), q.cuda())
+    for a in range(0, w.tokens, 100):                      # windows that are flushed from the residual store
+        caches[1].quantize_append(0, *[x[:, :, a:a + 100].contiguous().cuda() for x in (k, v, q)])
+    for cache in caches:
+        assert cache.status() == 0
+        for (b, hk), st in U.oracle_streams(w, 0, k, v, q, v_bits=v_bits).items():
+            got, want = cache.stream_regions(0, hk), O.pack_stream(st, layout=layout)
+            for key in ("table", "base", "extras"):
+                assert got[key] == want[key], (hk, key)
