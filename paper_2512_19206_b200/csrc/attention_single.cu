@@ -241,19 +241,19 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
     // stages the next unit (if there is one left) in ring stage sg; all lanes keep the position
     auto issue = [&](uint32_t sg, bool first) {
       const uint32_t dst = ring_u32 + sg * kStageBytes, bar = bar_u32 + sg * 8u;
-      const uint32_t enabled = issued < n_pack ? 1u : 0u;
+      // Nothing more after a wait that ran out: its stage's barrier is still armed, and what is under way is awaited at the end.
+      // (The lanes may differ in that: the copying lane's own view decides, so it never arms a barrier that it has not seen free.)
+      const uint32_t enabled = issued < n_pack && !gave_up ? 1u : 0u;
       if (UPG == 1) {
         // the group's scales lie directly before the unit: one copy
         stage_copy(dst + kKeyMetaOff, isrc - 512, 512u + kUnitBytes, bar, first ? lv.debug_extra_tx : 0u, enabled);
         isrc += kUnitBytes + 512;
       } else {
-        if (enabled) {
-          if (ig == 0) stage_copy(dst + kKeyMetaOff, isrc - 512, 512u + kUnitBytes, bar, first ? lv.debug_extra_tx : 0u, 1u);
-          else if (first)
-            stage_copy2(dst + kUnitOff, isrc, kUnitBytes, dst + kKeyMetaOff, isrc - (size_t)ig * kUnitBytes - 512, 512u, bar,
-                        lv.debug_extra_tx);
-          else stage_copy(dst + kUnitOff, isrc, kUnitBytes, bar, 0u, 1u);
-        }
+        if (ig == 0) stage_copy(dst + kKeyMetaOff, isrc - 512, 512u + kUnitBytes, bar, first ? lv.debug_extra_tx : 0u, enabled);
+        else if (first)
+          stage_copy2(dst + kUnitOff, isrc, kUnitBytes, dst + kKeyMetaOff, isrc - (size_t)ig * kUnitBytes - 512, 512u, bar,
+                      lv.debug_extra_tx, enabled);
+        else stage_copy(dst + kUnitOff, isrc, kUnitBytes, bar, 0u, enabled);
         isrc += kUnitBytes;
         ig = (ig + 1) & (UPG - 1);
         if (ig == 0) isrc += 512;
@@ -1081,10 +1081,11 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
           }
         }
       }
-      if (gave_up) {
+      if (__any_sync(0xffffffffu, gave_up)) {
+        gave_up = true;
         if (lane == 0) atomicOr(lv.status, (uint32_t)MIXKVQ_DEV_COPY_TIMEOUT);
-        // after the wait that ran out no wait was made, so the last copies may still be on their way, and they write to
-        // the ring: wait for them (bounded) before the ring is reused below or the CTA ends
+        // after the wait that ran out no wait was made and no stage refilled, so the last copies may still be on their way, and
+        // they write to the ring: wait for them (bounded) before the ring is reused below or the CTA ends
         for (int i = max(0, issued - kStages); i < issued; ++i) {
           const uint32_t pos = stage0 + (uint32_t)i;
           mbar_wait_polls(bar_u32 + (pos % kStages) * 8u, parity0 ^ ((pos / kStages) & 1u), lv.wait_polls ? lv.wait_polls : kWaitPolls);

@@ -272,15 +272,16 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     // stages the next step (if there is one left) in ring stage sg; all lanes keep the position
     auto issue = [&](uint32_t sg, bool first) {
       const uint32_t dst = ring_u32 + sg * kStageBytes, bar = bar_u32 + sg * 8u;
-      const uint32_t enabled = issued < n_steps ? 1u : 0u;
+      // Nothing more after a wait that ran out: its stage's barrier is still armed, and what is under way is awaited at the end.
+      // (The lanes may differ in that: the copying lane's own view decides, so it never arms a barrier that it has not seen free.)
+      const uint32_t enabled = issued < n_steps && !gave_up ? 1u : 0u;
       if (UPG != 4 || ihalf == 0u) {
         stage_copy(dst, isrc, (uint32_t)kStageBytes, bar, first ? lv.debug_extra_tx : 0u, enabled);
         isrc += kStageBytes;
       } else {
-        if (enabled) {
-          if (first || kMetaAlways) stage_copy2(dst + 512, isrc, 2 * kUnitBytes, dst, isrc - 2 * kUnitBytes - 512, 512u, bar, first ? lv.debug_extra_tx : 0u);
-          else stage_copy(dst + 512, isrc, 2 * kUnitBytes, bar, 0u, 1u);
-        }
+        if (first || kMetaAlways)
+          stage_copy2(dst + 512, isrc, 2 * kUnitBytes, dst, isrc - 2 * kUnitBytes - 512, 512u, bar, first ? lv.debug_extra_tx : 0u, enabled);
+        else stage_copy(dst + 512, isrc, 2 * kUnitBytes, bar, 0u, enabled);
         isrc += 2 * kUnitBytes;
       }
       if (UPG == 4) ihalf ^= 1u;
@@ -1023,10 +1024,11 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         issue(ring_stage, false);
         advance_stage();
       }
-      if (gave_up) {
+      if (__any_sync(0xffffffffu, gave_up)) {
+        gave_up = true;
         if (lane == 0) atomicOr(lv.status, (uint32_t)MIXKVQ_DEV_COPY_TIMEOUT);
-        // after the wait that ran out no wait was made, so the last copies may still be on their way, and they write to
-        // the ring: wait for them (bounded) before the ring is reused below or the CTA ends
+        // after the wait that ran out no wait was made and no stage refilled, so the last copies may still be on their way, and
+        // they write to the ring: wait for them (bounded) before the ring is reused below or the CTA ends
         for (int i = max(0, issued - kStages); i < issued; ++i) {
           const uint32_t pos = stage0 + (uint32_t)i;
           mbar_wait_polls(bar_u32 + (pos % (uint32_t)kStages) * 8u, parity0 ^ ((pos / (uint32_t)kStages) & 1u), lv.wait_polls ? lv.wait_polls : kWaitPolls);

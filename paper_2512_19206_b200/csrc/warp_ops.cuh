@@ -58,17 +58,19 @@ __device__ __forceinline__ void stage_copy(uint32_t dst, const void* src, uint32
 }
 // the same for a unit whose key-group scales do not lie directly before it: two copies on one barrier
 __device__ __forceinline__ void stage_copy2(uint32_t dst_a, const void* src_a, uint32_t bytes_a, uint32_t dst_b,
-                                            const void* src_b, uint32_t bytes_b, uint32_t bar, uint32_t extra) {
+                                            const void* src_b, uint32_t bytes_b, uint32_t bar, uint32_t extra, uint32_t enabled) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .u32 tx;\n\t"
+      "{\n\t.reg .pred p, e;\n\t.reg .u32 tx;\n\t"
+      "setp.ne.u32 e, %8, 0;\n\t"
       "elect.sync _|p, 0xffffffff;\n\t"
+      "and.pred p, p, e;\n\t"
       "add.u32 tx, %2, %5;\n\t"
       "add.u32 tx, tx, %7;\n\t"
       "@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%6], tx;\n\t"
       "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%6];\n\t"
       "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%3], [%4], %5, [%6];\n\t"
       "}" ::"r"(dst_a),
-      "l"(src_a), "r"(bytes_a), "r"(dst_b), "l"(src_b), "r"(bytes_b), "r"(bar), "r"(extra)
+      "l"(src_a), "r"(bytes_a), "r"(dst_b), "l"(src_b), "r"(bytes_b), "r"(bar), "r"(extra), "r"(enabled)
       : "memory");
 }
 // 16 bytes from global to shared memory, asynchronously (cp.async groups)

@@ -92,3 +92,35 @@ def test_attention_right_after_a_flush_and_after_an_external_write(binding):
     ref = U.oracle_attention(w, oracle, qd.cpu())
     assert U.max_abs_err(w, first, ref) <= ATTN_TOL
     assert cache.status() == 0
+
+
+@pytest.mark.parametrize("name,batch,tokens,preset,v_bits", [
+    ("qwen7b", 16, 6400, "P24", 2),          # two units per step, a logits warp per team
+    ("qwen7b", 16, 6400, "P27", 2),          # two logits warps per team
+    ("qwen7b", 8, 8000, "P24", 2),           # one unit per step
+    ("qwen32b", 64, 700, "P24", 4),          # one unit per step, several streams per CTA
+])
+def test_a_wait_that_runs_out_with_more_steps_than_stages(binding, name, batch, tokens, preset, v_bits):
+    """As above where every team has more units than its ring has stages: after the give-up no stage is refilled, so that every
+    copy under way is awaited before the ring is reused; the call returns, and after a reset the cache works again."""
+    w = W.small(W.CONFIGS[name], n_layers=1, batch=batch, tokens=tokens, **getattr(W, preset))
+    cache = U.make_cache(binding, w, v_bits=v_bits)
+    qd = W.decode_query(w, 0, 0, device="cuda")
+
+    def fill():
+        for t in range(0, tokens, 4096):
+            cache.quantize_append(0, *W.tokens(w, 0, t, min(4096, tokens - t), device="cuda"))
+    fill()
+    want = cache.decode_attention(0, qd, W.softmax_scale())
+    assert cache.status() == 0
+    cache.test_arm_copy_timeout(16, 64)
+    got = cache.decode_attention(0, qd, W.softmax_scale())
+    torch.cuda.synchronize()
+    assert cache.status() & binding.DEV_COPY_TIMEOUT
+    assert torch.isfinite(got).all()
+    cache.test_arm_copy_timeout(0, 0)
+    cache.reset()
+    fill()
+    again = cache.decode_attention(0, qd, W.softmax_scale())
+    assert cache.status() == 0
+    assert torch.equal(again, want)
