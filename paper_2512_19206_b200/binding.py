@@ -20,7 +20,7 @@ EXPORTS = [
     "mixkvq_select_channels", "mixkvq_select_channels_raw", "mixkvq_quantize_append",
     "mixkvq_decode_attention", "mixkvq_decode_attention_noalloc", "mixkvq_decode_step", "mixkvq_set_attention_kernel", "mixkvq_query_status",
     "mixkvq_cache_describe", "mixkvq_launch_count", "mixkvq_status_string",
-    "mixkvq_cache_written_externally", "mixkvq_test_arm_copy_timeout", "mixkvq_rope_append", "mixkvq_rope_decode_step", "mixkvq_prefill", "mixkvq_prefill_scratch_bytes", "mixkvq_quantize_append_ragged", "mixkvq_sequence_fill", "mixkvq_decode_attention_partial", "mixkvq_merge_partials",
+    "mixkvq_cache_written_externally", "mixkvq_test_arm_copy_timeout", "mixkvq_test_arm_value_copy_timeout", "mixkvq_rope_append", "mixkvq_rope_decode_step", "mixkvq_prefill", "mixkvq_prefill_scratch_bytes", "mixkvq_quantize_append_ragged", "mixkvq_sequence_fill", "mixkvq_decode_attention_partial", "mixkvq_merge_partials",
 ]
 
 DEV_EXTRAS_FULL, DEV_COPY_TIMEOUT = 1, 2
@@ -83,7 +83,7 @@ def lib():
         L.mixkvq_rope_append.argtypes = [vp, i32, vp, vp, vp, vp, vp, i32, i32, vp]
         L.mixkvq_rope_decode_step.argtypes = [vp, i32, vp, vp, vp, vp, vp, i32, vp, f32, vp, C.c_size_t, vp]
         L.mixkvq_cache_written_externally.argtypes = [vp]
-        L.mixkvq_test_arm_copy_timeout.argtypes = [vp, C.c_uint32, C.c_uint32]
+        L.mixkvq_test_arm_copy_timeout.argtypes = L.mixkvq_test_arm_value_copy_timeout.argtypes = [vp, C.c_uint32, C.c_uint32]
         L.mixkvq_query_status.argtypes = [vp, C.POINTER(i32), vp]
         L.mixkvq_cache_describe.argtypes = [vp, i32, C.POINTER(LayoutDesc)]
         L.mixkvq_launch_count.argtypes = [vp]
@@ -306,6 +306,9 @@ class Cache:
 
     def test_arm_copy_timeout(self, extra_bytes: int, max_polls: int):
         _check(lib().mixkvq_test_arm_copy_timeout(self.handle, extra_bytes, max_polls), "mixkvq_test_arm_copy_timeout")
+
+    def test_arm_value_copy_timeout(self, extra_bytes: int, max_polls: int):
+        _check(lib().mixkvq_test_arm_value_copy_timeout(self.handle, extra_bytes, max_polls), "mixkvq_test_arm_value_copy_timeout")
 
     def set_attention_kernel(self, kind: int):
         _check(lib().mixkvq_set_attention_kernel(self.handle, kind), "mixkvq_set_attention_kernel")

@@ -28,6 +28,7 @@ struct mixkvq_cache {
   // The next decode attention on such a layer waits for all earlier work before it reads anything.
   int last_packed_writer;
   uint32_t test_extra_tx, test_wait_polls;   // mixkvq_test_arm_copy_timeout
+  uint32_t test_extra_v;                     // mixkvq_test_arm_value_copy_timeout
 };
 
 namespace {
@@ -342,7 +343,7 @@ int mixkvq_cache_init(const mixkvq_config* cfg, void* cache_dev, size_t bytes, v
   h->attn_kind = 0;
   h->launches = 0;
   h->last_packed_writer = kAllPacked;
-  h->test_extra_tx = h->test_wait_polls = 0;
+  h->test_extra_tx = h->test_wait_polls = h->test_extra_v = 0;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -542,7 +543,7 @@ int mixkvq_prefill(mixkvq_cache* cache, int layer, const void* k_dev, const void
     return MIXKVQ_E_CAPACITY;
   if (launch_prefill_attention(q_dev, k_dev, v_dev, out_dev, scratch_dev, cache->cfg.batch, cache->cfg.n_q_heads,
                                cache->cfg.n_kv_heads, n_tokens, softmax_scale, reinterpret_cast<uint32_t*>(cache->mem),
-                               cache->test_wait_polls, cache->test_extra_tx, static_cast<cudaStream_t>(stream)) != cudaSuccess)
+                               cache->test_wait_polls, cache->test_extra_tx, cache->test_extra_v, static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return MIXKVQ_E_CUDA;
   cache->launches += 2;
   cache->last_packed_writer = kNoPackedWrite;
@@ -626,6 +627,13 @@ int mixkvq_cache_written_externally(mixkvq_cache* cache) {
 int mixkvq_test_arm_copy_timeout(mixkvq_cache* cache, uint32_t extra_bytes, uint32_t max_polls) {
   if (!cache || (extra_bytes & 15u)) return MIXKVQ_E_INVALID_ARG;
   cache->test_extra_tx = extra_bytes;
+  cache->test_wait_polls = max_polls;
+  return MIXKVQ_OK;
+}
+
+int mixkvq_test_arm_value_copy_timeout(mixkvq_cache* cache, uint32_t extra_bytes, uint32_t max_polls) {
+  if (!cache || (extra_bytes & 15u)) return MIXKVQ_E_INVALID_ARG;
+  cache->test_extra_v = extra_bytes;
   cache->test_wait_polls = max_polls;
   return MIXKVQ_OK;
 }

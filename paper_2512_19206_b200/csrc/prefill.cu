@@ -38,9 +38,9 @@ constexpr int kTile = 128;                       // query rows and key rows per 
 constexpr int kTileBytes = kTile * kD * 2;       // one 128 x 128 tile of 16-bit elements
 constexpr int kQRows = 2 * kTile;                // query rows per CTA
 constexpr int kThreads = 384;
-constexpr int kBars = 16;
+constexpr int kBars = 17;
 constexpr int kSmem = 6 * kTileBytes + 256;      // two Q tiles, two K and two V stages; barriers and tensor-memory slot
-enum Bar { kKFull = 0, kVFull = 2, kKEmpty = 4, kVEmpty = 6, kSFull = 8, kPHalf = 10, kPReady = 12, kDoneA = 14, kDone = 15 };
+enum Bar { kKFull = 0, kVFull = 2, kKEmpty = 4, kVEmpty = 6, kSFull = 8, kPHalf = 10, kPReady = 12, kDoneA = 14, kDoneB = 15, kDone = 16 };
 constexpr uint32_t kPolls = 1u << 21;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -331,7 +331,7 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, i
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned char* __restrict__ kt,
                          const unsigned char* __restrict__ vt, float* __restrict__ out, int BH, int Hq, int Hkv, int L,
-                         int n_tiles, int n_qtiles, float scale_log2e, uint32_t* status, uint32_t max_polls, uint32_t debug_extra_tx) {
+                         int n_tiles, int n_qtiles, float scale_log2e, uint32_t* status, uint32_t max_polls, uint32_t debug_extra_tx, uint32_t debug_extra_v) {
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* Qs = smem;                              // two tiles
   unsigned char* Ks = smem + 2 * kTileBytes;             // two stages
@@ -356,8 +356,9 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
   int issued = 0;                  // K and V tiles requested (the copying thread)
   auto copy_tile = [&](int j, bool keys) {
     const int st = j & 1, full = (keys ? kKFull : kVFull) + st;
-    // (test hook: the first copy's barrier can be armed for more bytes than arrive, so that it never completes)
-    mbar_expect_tx(bar(full), kTileBytes + (keys && j == 0 ? debug_extra_tx : 0u));
+    // (test hooks: the barrier of the first key tile or of the last value tile can be armed for more bytes than arrive, so that
+    // it never completes)
+    mbar_expect_tx(bar(full), kTileBytes + (keys ? (j == 0 ? debug_extra_tx : 0u) : (j == n_b - 1 ? debug_extra_v : 0u)));
     bulk_copy(smem_u32((keys ? Ks : Vs) + st * kTileBytes), (keys ? ktg : vtg) + (size_t)j * kTileBytes, kTileBytes, bar(full));
   };
   if (tid == 9 * 32) {
@@ -454,6 +455,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
         }
         if (!both_halves(1, j)) break;
         tc_commit(bar(kVEmpty + st));
+        if (j + 1 == n_b) tc_commit(bar(kDoneB));        // (not when a wait ran out: group B must not take an unfinished product)
         if (j + 1 < n_b) {
           if (!wait(kKFull + nx, ph_nx)) break;
           tc_fence_after();
@@ -513,7 +515,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     // 256 rows at once, about half for 128).  Group A is done a tile earlier than group B and stores directly, in 32-byte
     // pieces where the caller's buffer allows, under B's last tile; B's rows go through the shared memory, which nobody needs
     // any more, and leave as one bulk copy each.
-    if (wait(g == 0 ? kDoneA : kDone, 0)) {
+    if (wait(g == 0 ? kDoneA : kDoneB, 0)) {
       tc_fence_after();
       add_output(o_addr, sum_o);
       const float inv = 1.f / l_run;
@@ -570,7 +572,7 @@ size_t prefill_scratch_bytes(int B, int Hkv, int L) {
 
 cudaError_t launch_prefill_attention(const void* q, const void* k, const void* v, float* out, void* scratch, int B, int Hq,
                                      int Hkv, int L, float scale, uint32_t* status, uint32_t max_polls, uint32_t debug_extra_tx,
-                                     cudaStream_t stream) {
+                                     uint32_t debug_extra_v, cudaStream_t stream) {
   const int n_tiles = (L + kTile - 1) / kTile, n_qtiles = (L + kQRows - 1) / kQRows;
   unsigned char* kt = static_cast<unsigned char*>(scratch);
   unsigned char* vt = kt + (size_t)B * Hkv * n_tiles * kTileBytes;
@@ -579,7 +581,7 @@ cudaError_t launch_prefill_attention(const void* q, const void* k, const void* v
   if (e != cudaSuccess) return e;
   return launch_dependent(prefill_attention_kernel, dim3((unsigned)(n_qtiles * B * Hq)), kThreads, kSmem, stream,
                           static_cast<const __nv_bfloat16*>(q), kt, vt, out, B * Hq, Hq, Hkv, L, n_tiles, n_qtiles,
-                          scale * 1.4426950408889634f, status, max_polls ? max_polls : kPolls, debug_extra_tx);
+                          scale * 1.4426950408889634f, status, max_polls ? max_polls : kPolls, debug_extra_tx, debug_extra_v);
 }
 
 }  // namespace mixkvq

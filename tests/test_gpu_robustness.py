@@ -124,3 +124,24 @@ def test_a_wait_that_runs_out_with_more_steps_than_stages(binding, name, batch, 
     again = cache.decode_attention(0, qd, W.softmax_scale())
     assert cache.status() == 0
     assert torch.equal(again, want)
+
+
+def test_a_prefill_wait_for_the_last_values_that_runs_out(binding):
+    """Every CTA's last value tile never arrives: the rows that need its product are left unwritten (those of the second 128 of a
+    CTA's 256, and of a last CTA with one tile more than the one before), all others are right."""
+    w = W.small(W.CONFIGS["qwen7b"], n_layers=1, batch=1, tokens=600, **W.P24)
+    k, v, q = [t.cuda() for t in W.tokens(w, 0, 0, 600)]
+    cache = U.make_cache(binding, w)
+    want = cache.prefill(0, k, v, q, W.softmax_scale())
+    cache.reset()
+    cache.test_arm_value_copy_timeout(16, 2000)
+    out = torch.full_like(want, 7.0)
+    cache.prefill(0, k, v, q, W.softmax_scale(), out=out)
+    torch.cuda.synchronize()
+    assert cache.status() & binding.DEV_COPY_TIMEOUT
+    for a, b, whole in ((0, 128, True), (128, 256, False), (256, 384, True), (384, 512, False), (512, 600, False)):
+        assert torch.equal(out[:, :, a:b], want[:, :, a:b] if whole else torch.full_like(want[:, :, a:b], 7.0)), (a, b)
+    cache.test_arm_value_copy_timeout(0, 0)
+    cache.reset()
+    assert torch.equal(cache.prefill(0, k, v, q, W.softmax_scale()), want)
+    assert cache.status() == 0
