@@ -297,6 +297,16 @@ int mixkvq_query_status(mixkvq_cache* cache, int* device_status, void* stream);
 /* Where one layer's arrays live inside the cache memory, and how full the layer is. */
 int mixkvq_cache_describe(const mixkvq_cache* cache, int layer, mixkvq_layout_desc* out);
 
+/* Which kernel the last decode-attention call on this handle enqueued (diagnostic): the sum of these, 0 before the first. */
+enum {
+  MIXKVQ_ATTN_ONE_UNIT = 1,           /* the tensor-core split kernel, one 32-token unit per step    */
+  MIXKVQ_ATTN_TWO_UNITS = 2,          /* ... two units per step                                      */
+  MIXKVQ_ATTN_DIRECT = 4,             /* one thread block per stream, which wrote the output: no merge */
+  MIXKVQ_ATTN_EARLY = 8,              /* packed blocks were requested before the wait for earlier work */
+  MIXKVQ_ATTN_OTHER = 16              /* the plain-ALU kernel or the tile layout's                   */
+};
+int mixkvq_last_attention(const mixkvq_cache* cache);
+
 /* Number of kernels launched by this handle since it was created (diagnostic). */
 uint64_t mixkvq_launch_count(const mixkvq_cache* cache);
 

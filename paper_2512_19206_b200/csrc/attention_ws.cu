@@ -1253,7 +1253,7 @@ int attention_ws_grid(const LayerView& lv, int n_sms) {
 }
 
 cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, float scale, float* ws, int n_sms,
-                                cudaStream_t stream, int* launches, float* lse_out) {
+                                cudaStream_t stream, int* launches, float* lse_out, int* form) {
   const int S = lv.B * lv.Hkv;
   const long long Us = attention_ws_positions(lv);
   const int grid = attention_ws_grid(lv, n_sms);
@@ -1278,6 +1278,7 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // tokens 7.3 us against 5.6; 7b shape 41.1 against 40.7).
   const bool whole = out != nullptr && lv.seq == nullptr && grid == S;
   float* const kernel_out = whole ? out : nullptr;
+  if (form) *form = (by_two ? MIXKVQ_ATTN_TWO_UNITS : MIXKVQ_ATTN_ONE_UNIT) | (whole ? MIXKVQ_ATTN_DIRECT : 0) | (lv.stage_early ? MIXKVQ_ATTN_EARLY : 0);
   cudaError_t e;
   if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
   else if (lv.G == 32) e = launch_g<32>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
