@@ -157,7 +157,8 @@ int mixkvq_quantize_append(mixkvq_cache* cache, int layer, const void* k_dev, co
  * The kernels are launched with programmatic stream serialization and wait on the device for all earlier work of
  * the stream before they read q_dev or write anything, so stream order holds as for any other launch.  One access comes
  * before that wait: the first packed blocks of the layer are requested early unless the call this library enqueued last
- * on this handle wrote packed blocks of this layer (a flush; initialisation and reset count for all layers).  Cache
+ * on this handle wrote packed blocks of this layer (a flush; initialisation and reset count for all layers) or went to
+ * another stream.  Cache
  * memory is written through this library only; a caller that writes it by other means (restoring saved cache bytes with
  * a kernel of its own, say) calls mixkvq_cache_written_externally before the next attention call.
  * No wait inside the kernels is unbounded: a staged copy or a hand-over between two warps that has not arrived after

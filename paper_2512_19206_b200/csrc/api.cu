@@ -26,8 +26,10 @@ struct mixkvq_cache {
   uint64_t launches;
   // What the library enqueued last on this handle: kNoPackedWrite if it did not write packed blocks, a layer index if
   // it wrote that layer's packed blocks (a flush), kAllPacked after initialisation, a reset or a write from outside.
-  // The next decode attention on such a layer waits for all earlier work before it reads anything.
+  // The next decode attention on such a layer waits for all earlier work before it reads anything, and so does one on another
+  // stream than last_stream: what the library enqueued last there may be a flush of the layer.
   int last_packed_writer;
+  cudaStream_t last_stream;
   uint32_t test_extra_tx, test_wait_polls;   // mixkvq_test_arm_copy_timeout
   uint32_t test_extra_v;                     // mixkvq_test_arm_value_copy_timeout
 };
@@ -161,11 +163,17 @@ LayerView view(const mixkvq_cache* h, int layer, int b0 = 0, int nb = -1) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// every call that enqueues work on the handle notes it
+void note_enqueued(mixkvq_cache* h, cudaStream_t st, int packed_writer) {
+  h->last_packed_writer = packed_writer;
+  h->last_stream = st;
+}
+
 int zero_layer_state(mixkvq_cache* h, int layer, cudaStream_t st) {
   char* L = h->mem + kHeaderBytes + h->layer_stride * (uint64_t)layer;
   if (cudaMemsetAsync(L + h->state_off, 0, h->state_stride * h->S, st) != cudaSuccess) return MIXKVQ_E_CUDA;
   for (int b = 0; b < h->cfg.batch; ++b) h->n_blocks[fi(h, layer, b)] = h->r[fi(h, layer, b)] = h->n_sink[fi(h, layer, b)] = 0;
-  h->last_packed_writer = kAllPacked;
+  note_enqueued(h, st, kAllPacked);
   return MIXKVQ_OK;
 }
 
@@ -181,7 +189,7 @@ int zero_all_layers(mixkvq_cache* h, cudaStream_t st) {
   std::fill(h->n_blocks.begin(), h->n_blocks.end(), 0);
   std::fill(h->r.begin(), h->r.end(), 0);
   std::fill(h->n_sink.begin(), h->n_sink.end(), 0);
-  h->last_packed_writer = kAllPacked;
+  note_enqueued(h, st, kAllPacked);
   return MIXKVQ_OK;
 }
 
@@ -221,9 +229,9 @@ int run_attention(mixkvq_cache* h, int layer, const void* q, float* out, float s
   LayerView lv = view(h, layer);
   lv.new_k = static_cast<const uint16_t*>(new_k);
   lv.new_v = static_cast<const uint16_t*>(new_v);
-  lv.stage_early = (h->last_packed_writer == kNoPackedWrite ||
-                    (h->last_packed_writer >= 0 && h->last_packed_writer != layer)) ? 1 : 0;
-  h->last_packed_writer = kNoPackedWrite;
+  lv.stage_early = (st == h->last_stream && (h->last_packed_writer == kNoPackedWrite ||
+                                             (h->last_packed_writer >= 0 && h->last_packed_writer != layer))) ? 1 : 0;
+  note_enqueued(h, st, kNoPackedWrite);
   if (!uniform(h, layer)) {
     // ragged batch: the split kernel and the merge walk every stream's own positions
     if (h->tile || h->attn_kind == 1) return MIXKVQ_E_UNSUPPORTED;
@@ -264,7 +272,7 @@ int append_run_first(mixkvq_cache* cache, int layer, int b0, int nb, const void*
       LayerView lv = view(cache, layer, b0, nb);
       if (launch_sink_append(lv, k, v, n_stride, t, m, st) != cudaSuccess) return MIXKVQ_E_CUDA;
       cache->launches += 1;
-      cache->last_packed_writer = kNoPackedWrite;
+      note_enqueued(cache, st, kNoPackedWrite);
       sink0 += m;
       t += m;
       continue;
@@ -273,7 +281,7 @@ int append_run_first(mixkvq_cache* cache, int layer, int b0, int nb, const void*
       LayerView lv = view(cache, layer, b0, nb);
       if (launch_flush(lv, st) != cudaSuccess) return MIXKVQ_E_CUDA;
       cache->launches += 1;
-      cache->last_packed_writer = layer;
+      note_enqueued(cache, st, layer);
       nb0 += 1;
       r0 = 0;
     }
@@ -286,7 +294,7 @@ int append_run_first(mixkvq_cache* cache, int layer, int b0, int nb, const void*
       LayerView lv = view(cache, layer, b0, nb);
       if (launch_flush_bulk(lv, k, v, q, n_stride, t, nblk, tail, behind_prefill && t == 0, st) != cudaSuccess) return MIXKVQ_E_CUDA;
       cache->launches += cache->cfg.importance_mode == 1 ? 3 : 2;
-      cache->last_packed_writer = layer;
+      note_enqueued(cache, st, layer);
       nb0 += nblk;
       r0 = tail;
       t += nblk * cache->R + tail;
@@ -296,7 +304,7 @@ int append_run_first(mixkvq_cache* cache, int layer, int b0, int nb, const void*
     LayerView lv = view(cache, layer, b0, nb);
     if (launch_append(lv, k, v, q, n_stride, t, m, st) != cudaSuccess) return MIXKVQ_E_CUDA;
     cache->launches += 1;
-    cache->last_packed_writer = kNoPackedWrite;
+    note_enqueued(cache, st, kNoPackedWrite);
     r0 += m;
     t += m;
   }
@@ -345,7 +353,7 @@ int mixkvq_cache_init(const mixkvq_config* cfg, void* cache_dev, size_t bytes, v
   h->attn_kind = 0;
   h->last_form = 0;
   h->launches = 0;
-  h->last_packed_writer = kAllPacked;
+  note_enqueued(h, static_cast<cudaStream_t>(stream), kAllPacked);
   h->test_extra_tx = h->test_wait_polls = h->test_extra_v = 0;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -380,7 +388,7 @@ int mixkvq_select_channels(mixkvq_cache* cache, int layer, uint8_t* tiers_dev, d
   bool any = false;
   for (int b = 0; b < cache->cfg.batch; ++b) any = any || cache->r[fi(cache, layer, b)] > 0;
   if (!any) return MIXKVQ_E_EMPTY;
-  cache->last_packed_writer = kNoPackedWrite;
+  note_enqueued(cache, static_cast<cudaStream_t>(stream), kNoPackedWrite);
   // one launch per run of sequences with the same fill (one launch for a batch of equal lengths); a sequence whose
   // window is empty has no scores: its rows of the outputs are left as they are
   const int B = cache->cfg.batch, Hkv = cache->cfg.n_kv_heads;
@@ -513,7 +521,7 @@ int mixkvq_decode_step(mixkvq_cache* cache, int layer, const void* k_dev, const 
     }
     if (launch_flush(lv, st) != cudaSuccess) return MIXKVQ_E_CUDA;
     cache->launches += 1;
-    cache->last_packed_writer = layer;
+    note_enqueued(cache, st, layer);
     for (int b = 0; b < B; ++b)
       if (cache->r[fi(cache, layer, b)] == cache->R) {
         cache->n_blocks[fi(cache, layer, b)] += 1;
@@ -549,7 +557,7 @@ int mixkvq_prefill(mixkvq_cache* cache, int layer, const void* k_dev, const void
                                cache->test_wait_polls, cache->test_extra_tx, cache->test_extra_v, static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return MIXKVQ_E_CUDA;
   cache->launches += 2;
-  cache->last_packed_writer = kNoPackedWrite;
+  note_enqueued(cache, static_cast<cudaStream_t>(stream), kNoPackedWrite);
   return append_run(cache, layer, 0, cache->cfg.batch, k_dev, v_dev, q_dev, n_tokens, n_tokens, true, static_cast<cudaStream_t>(stream));
 }
 
@@ -565,7 +573,7 @@ int mixkvq_rope_append(mixkvq_cache* cache, int layer, void* k_dev, const void* 
                   pos0, static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return MIXKVQ_E_CUDA;
   cache->launches += 1;
-  cache->last_packed_writer = kNoPackedWrite;
+  note_enqueued(cache, static_cast<cudaStream_t>(stream), kNoPackedWrite);
   return mixkvq_quantize_append(cache, layer, k_dev, v_dev, q_dev, n_tokens, stream);
 }
 
@@ -584,7 +592,7 @@ int mixkvq_rope_decode_step(mixkvq_cache* cache, int layer, void* k_dev, const v
                   static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return MIXKVQ_E_CUDA;
   cache->launches += 1;
-  cache->last_packed_writer = kNoPackedWrite;
+  note_enqueued(cache, static_cast<cudaStream_t>(stream), kNoPackedWrite);
   return mixkvq_decode_step(cache, layer, k_dev, v_dev, q_dev, out_dev, softmax_scale, workspace_dev, workspace_bytes_given,
                             stream);
 }

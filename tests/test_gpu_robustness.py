@@ -145,3 +145,29 @@ def test_a_prefill_wait_for_the_last_values_that_runs_out(binding):
     cache.reset()
     assert torch.equal(cache.prefill(0, k, v, q, W.softmax_scale()), want)
     assert cache.status() == 0
+
+
+def test_no_early_request_when_the_last_call_went_to_another_stream(binding):
+    """A flush of layer 0 on one stream, a call for layer 1 on another, attention over layer 0 on the first: the flush may still be
+    the last thing on that stream, so the attention waits before its first read.  On one stream throughout it need not."""
+    w = W.small(W.CONFIGS["qwen7b"], n_layers=2, batch=2, tokens=6 * 128, **W.P24)
+    qd = W.decode_query(w, 0, 0, device="cuda")
+    outs = []
+    for streams in ((0, 0), (0, 1)):
+        cache = U.make_cache(binding, w)
+        data = [[t.cuda() for t in W.tokens(w, layer, 0, w.tokens + 1)] for layer in (0, 1)]
+        for layer in (0, 1):
+            cache.quantize_append(layer, *[x[:, :, :-1].contiguous() for x in data[layer]])
+        one = [[x[:, :, -1:].contiguous() for x in data[layer]] for layer in (0, 1)]
+        torch.cuda.synchronize()
+        s = [torch.cuda.Stream(), torch.cuda.Stream()]
+        with torch.cuda.stream(s[streams[0]]):
+            cache.quantize_append(0, *one[0])                  # the window is full: flushed
+        with torch.cuda.stream(s[streams[1]]):
+            cache.quantize_append(1, *one[1])
+        with torch.cuda.stream(s[streams[0]]):
+            outs.append(cache.decode_attention(0, qd, W.softmax_scale()))
+        assert bool(cache.last_attention() & binding.ATTN_EARLY) == (streams[0] == streams[1])
+        torch.cuda.synchronize()
+        assert cache.status() == 0
+    assert torch.equal(*outs)
