@@ -180,11 +180,15 @@ class Cache:
         nbytes, ws_bytes = cache_bytes(cfg)
         self.mem = torch.empty(nbytes, dtype=torch.uint8, device=device)
         self.workspace = torch.empty(ws_bytes, dtype=torch.uint8, device=device)
-        self._ws = (self.workspace.data_ptr(), ws_bytes)
         self.handle = C.c_void_p()
         with torch.cuda.device(self.mem.device):
             _check(lib().mixkvq_cache_init(C.byref(cfg), _ptr(self.mem), nbytes, _stream(), C.byref(self.handle)),
                    "mixkvq_cache_init")
+
+    @property
+    def _ws(self):
+        """(address, bytes) of the workspace; the attribute may be given another tensor at any time."""
+        return _ptr(self.workspace), self.workspace.numel()
 
     def close(self):
         if self.handle:
@@ -211,7 +215,7 @@ class Cache:
         """q [B,Hq,128] bf16 -> out [B,Hq,128] float32."""
         if out is None:
             out = torch.empty(q.shape, dtype=torch.float32, device=q.device)
-        code = (_native or _calls()).decode_attention(self.handle.value, layer, q, out, scale, *self._ws, _stream())
+        code = (_native or _calls()).decode_attention(self.handle.value, layer, q, out, scale, self.workspace, self.workspace.numel(), _stream())
         if code:
             raise MixKVQError(code, "mixkvq_decode_attention")
         return out
@@ -220,7 +224,7 @@ class Cache:
         """One decode step: k, v [B,Hkv,1,128], q [B,Hq,1,128] bf16 -> out [B,Hq,128] float32 (append + attention)."""
         if out is None:
             out = torch.empty((q.shape[0], q.shape[1], 128), dtype=torch.float32, device=q.device)
-        code = (_native or _calls()).decode_step(self.handle.value, layer, k, v, q, out, scale, *self._ws, _stream())
+        code = (_native or _calls()).decode_step(self.handle.value, layer, k, v, q, out, scale, self.workspace, self.workspace.numel(), _stream())
         if code:
             raise MixKVQError(code, "mixkvq_decode_step")
         return out
@@ -278,7 +282,7 @@ class Cache:
         if out is None:
             out = torch.empty((q.shape[0], q.shape[1], 128), dtype=torch.float32, device=q.device)
         code = (_native or _calls()).rope_decode_step(self.handle.value, layer, k, v, q, cos, sin, int(pos), out, scale,
-                                                      *self._ws, _stream())
+                                                      self.workspace, self.workspace.numel(), _stream())
         if code:
             raise MixKVQError(code, "mixkvq_rope_decode_step")
         return out

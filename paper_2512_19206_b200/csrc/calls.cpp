@@ -14,7 +14,7 @@ namespace {
 
 PyObject *s_is_cuda, *s_is_contiguous, *s_data_ptr;
 
-// Handle, workspace and stream: an int, or None for a null pointer.
+// Handle and stream: an int, or None for a null pointer.
 bool raw(PyObject* o, void** p) {
   *p = o == Py_None ? nullptr : PyLong_AsVoidPtr(o);
   return *p || !PyErr_Occurred();
@@ -84,7 +84,7 @@ PyObject* decode_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
   float scale;
   size_t bytes;
   if (!count_is(n, 8) || !raw(a[0], &h) || !integer(a[1], &layer) || !address(a[2], &q) || !address(a[3], &out) ||
-      !real(a[4], &scale) || !raw(a[5], &ws) || !size(a[6], &bytes) || !raw(a[7], &st))
+      !real(a[4], &scale) || !address(a[5], &ws) || !size(a[6], &bytes) || !raw(a[7], &st))
     return nullptr;
   Py_BEGIN_ALLOW_THREADS
   rc = mixkvq_decode_attention(cache_of(h), layer, q, static_cast<float*>(out), scale, ws, bytes, st);
@@ -99,7 +99,7 @@ PyObject* decode_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   float scale;
   size_t bytes;
   if (!count_is(n, 10) || !raw(a[0], &h) || !integer(a[1], &layer) || !address(a[2], &k) || !address(a[3], &v) ||
-      !address(a[4], &q) || !address(a[5], &out) || !real(a[6], &scale) || !raw(a[7], &ws) || !size(a[8], &bytes) ||
+      !address(a[4], &q) || !address(a[5], &out) || !real(a[6], &scale) || !address(a[7], &ws) || !size(a[8], &bytes) ||
       !raw(a[9], &st))
     return nullptr;
   Py_BEGIN_ALLOW_THREADS
@@ -116,7 +116,7 @@ PyObject* rope_decode_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   size_t bytes;
   if (!count_is(n, 13) || !raw(a[0], &h) || !integer(a[1], &layer) || !address(a[2], &k) || !address(a[3], &v) ||
       !address(a[4], &q) || !address(a[5], &cos) || !address(a[6], &sin) || !integer(a[7], &pos) ||
-      !address(a[8], &out) || !real(a[9], &scale) || !raw(a[10], &ws) || !size(a[11], &bytes) ||
+      !address(a[8], &out) || !real(a[9], &scale) || !address(a[10], &ws) || !size(a[11], &bytes) ||
       !raw(a[12], &st))
     return nullptr;
   Py_BEGIN_ALLOW_THREADS
