@@ -106,7 +106,11 @@ def _calls():
     global _native
     if _native is None:
         lib()
-        from . import _calls as native
+        try:
+            from . import _calls as native
+        except ImportError as e:
+            raise RuntimeError(f"{e}: build the native calls for this interpreter first "
+                               "(python -m paper_2512_19206_b200.build); there is no fallback path") from e
         _native = native
     return _native
 

@@ -1,7 +1,8 @@
 """Builds libmixkvq.so (sm_100a) in-tree with nvcc.  Usable as `python -m paper_2512_19206_b200.build`.
 
 Every source file is compiled to an object of its own (in parallel, only when it or a header changed) and the
-objects are linked into the shared library.  csrc/calls.cpp becomes _calls.so, a CPython module linked against it.
+objects are linked into the shared library.  csrc/calls.cpp becomes _calls, a CPython module linked against it (with g++ and
+the headers of the interpreter that builds).
 """
 from __future__ import annotations
 
@@ -15,7 +16,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmixkvq.so")
-CALLS = os.path.join(HERE, "_calls.so")
+# the interpreter's own suffix: another Python version finds no module of its own here and builds one
+CALLS = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["api.cu", "append.cu", "rope.cu", "prefill.cu", "select.cu", "flush.cu", "combine.cu", "attention_simt.cu", "attention_ws.cu", "attention_single.cu",
            "attention_tc.cu"]
 FLAGS = ["-Xcompiler", "-fPIC", "-O3", "-std=c++17", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",

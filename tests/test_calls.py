@@ -7,6 +7,19 @@ import torch
 from paper_2512_19206_b200 import binding, workloads as W
 
 
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2512_19206_b200 import build
+    build.build()
+
+
+def test_the_module_is_built_for_this_interpreter():
+    import sysconfig
+
+    from paper_2512_19206_b200 import build
+    assert build.CALLS.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and binding._calls().__file__ == build.CALLS
+
+
 def test_arguments_are_checked():
     n = binding._calls()
     assert n.decode_step(None, 0, None, None, None, None, 0.1, None, 0, None) == -1
