@@ -92,7 +92,7 @@ def lib():
         L.mixkvq_status_string.argtypes = [i32]
         L.mixkvq_status_string.restype = C.c_char_p
         for name in EXPORTS:
-            if name not in ("mixkvq_launch_count", "mixkvq_status_string"):
+            if name not in ("mixkvq_launch_count", "mixkvq_status_string", "mixkvq_prefill_scratch_bytes"):
                 getattr(L, name).restype = i32
         _lib = L
     return _lib

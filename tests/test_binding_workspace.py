@@ -28,3 +28,12 @@ def test_a_replaced_workspace_is_used(monkeypatch):
         for _, args in native.calls:
             assert args[-3] is cache.workspace and args[-2] == n
         native.calls.clear()
+
+
+def test_scratch_sizes_beyond_32_bits():
+    from paper_2512_19206_b200 import build
+    build.build()
+    cache = object.__new__(binding.Cache)
+    cache.handle = C.c_void_p(None)
+    cache.cfg = binding.make_config(1, 16, 32, 8, 131072)
+    assert cache.prefill_scratch_bytes(131072) == 2 * 16 * 8 * 1024 * 32768          # 8 GiB
