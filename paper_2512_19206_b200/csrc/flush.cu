@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(256, 4) bulk_tiers_values_kernel(LayerView lv,
   if (early) dependency_wait();
 }
 
-// Bulk append, second launch: blockIdx.y < nb: keys of that window, blockIdx.y == nb: the stream's tail.
+// Bulk append, second launch: blockIdx.y < nb: keys of that window, blockIdx.y == nb: the stream's tail (if there is one).
 template <int G, bool kTile>
 __global__ void __launch_bounds__(256, 4) bulk_keys_tail_kernel(LayerView lv, BulkSrc src) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -895,7 +895,7 @@ cudaError_t bulk(const LayerView& lv, const BulkSrc& src, cudaStream_t stream) {
   if (lv.importance_mode == 1) e = launch_dependent(bulk_importance_kernel, dim3(S, src.nb), 256, 0, stream, lv, src);
   if (e == cudaSuccess)
     e = launch_dependent(bulk_tiers_values_kernel<G, kTile>, dim3(S, src.nb, 2), 256, t > b ? t : b, stream, lv, src);
-  if (e == cudaSuccess) e = launch_dependent(bulk_keys_tail_kernel<G, kTile>, dim3(S, src.nb + 1), 256, key_smem(lv), stream, lv, src);
+  if (e == cudaSuccess) e = launch_dependent(bulk_keys_tail_kernel<G, kTile>, dim3(S, src.nb + (src.tail > 0 ? 1 : 0)), 256, key_smem(lv), stream, lv, src);
   return e;
 }
 
