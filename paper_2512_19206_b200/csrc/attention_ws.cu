@@ -69,12 +69,17 @@ constexpr int kRBufBytes = 1024;             // hand-over of an unquantized unit
 // A step's extras (the promoted channels and the UINT4 high plane), copied a step or two ahead by each logits warp for its own steps
 // (three slots, two where two logits warps take turns; the values warp is no place for this although it has more time: it
 // refills the ring, and with the extras its wait for the copies made the 7b shape 38.9 us instead of 35.3):
-// the head of the block's channel lists (64 B, in a step that begins a block) | rows of the first kRowPairs pairs of
-// promoted channels of both units (128 B each) | three tiers: the first kPlanePairs pairs of UINT4 channels of both units
-// (16 B each); 4-bit base: both units' dense planes.  What does not fit is read from global memory (rare).
+// the block's channel lists (in a step that begins a block, and where something does not fit) | where the step's extras lie in
+// the stream's arena (only then) | rows of the first kRowPairs pairs of promoted channels of both units (128 B each) | three tiers:
+// the first kPlanePairs pairs of UINT4 channels of both units (16 B each); 4-bit base: both units' dense planes.  What does not
+// fit is read from global memory in the step itself, requested into the L2 cache with the slot.  (us per launch with the lists and the
+// table entry read in the step and nothing requested / so / one unit at a time: 8b shape, 16384 tokens, 32 promoted channels 133 /
+// 111 / 112, 32 and 32 UINT4 channels 170 / 140 / 140; 32b shape, G = 128, 8192 tokens, 32 promoted 235 / 187 / 188, 12 and 22 221 / 203 / 193;
+// three tiers with 34 and 94 channels, 7b shape 41.6 / 33.2 / 47.6.  8 or 16 pairs in the slots: up to 15 % faster beyond 8 channels,
+// but 4 % slower with the usual 4, the L1 cache being what the slots take.)
 constexpr int kRowPairs = 4, kPlanePairs = 16;
 __host__ __device__ constexpr int slots_of(int u4) { return u4 != 0 ? 2 : 3; }
-constexpr int kRowsOff = 128, kPlaneOff = kRowsOff + 2 * kRowPairs * 128;
+constexpr int kListBytes = 144, kWhereOff = kListBytes, kRowsOff = 160, kPlaneOff = kRowsOff + 2 * kRowPairs * 128;
 __host__ __device__ constexpr int slot_bytes(int u4) { return kPlaneOff + (u4 == 1 ? 2 * kPlanePairs * 16 : u4 == 2 ? 2048 : 0); }
 __host__ __device__ constexpr int team_bytes(int G, int u4, bool v4) {
   return stages_of(u4) * stage_bytes(G, v4) + logits_warps_of(u4) * (slots_of(u4) * slot_bytes(u4) + kRBufBytes) + prep_bytes(u4);
@@ -121,6 +126,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   constexpr int kGroups = UPG == 1 ? 2 : 1;                    // key groups of a step
   constexpr int kTeams = teams_of(kU4, kV4), kL = logits_warps_of(kU4), kThreads = threads_of(kU4, kV4);
   constexpr int kStages = stages_of(kU4), kSlotCount = slots_of(kU4), kSlotBytes = slot_bytes(kU4);
+  static_assert(smem_bytes(G, kU4, kV4) <= 113 * 1024, "two CTAs per SM");
   constexpr int kStageBytes = stage_bytes(G, kV4);
   constexpr int kTeamBytes = team_bytes(G, kU4, kV4);
   // a unit: key codes 1024, value codes 1024, value scales (and the values' high plane 1024)
@@ -130,6 +136,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   constexpr int kPrepBase = kSlotBase + kL * kSlotCount * kSlotBytes;
   constexpr int kRBufBase = kPrepBase + prep_bytes(kU4);
   constexpr int kQBytes = (kU4 == 1 ? 2 : 1) * 8 * kQS * 2;
+  constexpr int kSpillUnroll = kU4 == 0 ? 2 : 4;               // (128 registers / 168)
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, t = lane & 3;
   const int team = kL == 1 ? warp >> 1 : warp / 3;
@@ -331,7 +338,16 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
         const char* ex = extras + (size_t)c_entry.x * 16;
         const char* exu = ex + hdr + (size_t)cu * unit;
         const uint32_t dst = slot0_u32 + slot * kSlotBytes;
-        if (begins && 16u * lane < min(hdr, 64u)) cp_async16(dst + 16 * lane, ex + 16 * lane);
+        const bool spills = n16p > kRowPairs || (kU4 == 1 && n4 > 2 * kPlanePairs);
+        if ((begins || spills) && 16u * lane < hdr) cp_async16(dst + 16 * lane, ex + 16 * lane);          // (hdr <= kListBytes)
+        if (spills) {
+          if (lane == 0) sts32(dst + kWhereOff, c_entry.x + ((hdr + (uint32_t)cu * unit) >> 4));
+          if (kRowPairs + lane < n16p) {
+            prefetch_l2(exu + 128 * (kRowPairs + lane));
+            prefetch_l2(exu + unit + 128 * (kRowPairs + lane));
+          }
+          if (kU4 == 1 && lane < 16 && 16 * (lane & 7) < n4) prefetch_l2(exu + (lane >> 3) * unit + 128 * n16p + 128 * (lane & 7));
+        }
         // rows: lane = (pair, 16-byte piece); the pieces of a row are swizzled by the pair so that the tile's reads fall on
         // different banks
         if ((lane >> 3) < n16p) {
@@ -542,24 +558,19 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
 #pragma unroll
               for (int hp = 0; hp < 2; ++hp) {
                 const int p = 8 * kk + 4 * hp + t;
-                const uint32_t two = p < n4pairs && n16p <= kRowPairs ? lds16(slot_u32 + 2 * n16p + 2 * p) : 0xFFFFu;
+                const uint32_t two = p < n4pairs ? lds16(slot_u32 + 2 * n16p + 2 * p) : 0xFFFFu;
                 u4q[kk][hp] = query_pair(qfrow_u32, two);
                 u4s[kk][hp] = scale_byte(two & 0xFFu) | (scale_byte(two >> 8) << 16);
               }
           }
         }
         // where the step's extras lie in global memory, for what the slot does not hold
-        const bool spill16 = n16p > kRowPairs, spill4 = kU4 == 1 && (n4pairs > kPlanePairs || (n4pairs > 0 && spill16));
-        const char* ex = nullptr;
+        const bool spill16 = n16p > kRowPairs, spill4 = kU4 == 1 && n4pairs > kPlanePairs;
         const char* exu = nullptr;
         uint32_t ex_unit = 0u;
         if (spill16 || spill4) {
-          const int bi = (wb + 2 * i) / U;
-          const uint2 e = table[bi];
-          const int n16 = e.y & 0xFF, n4 = (e.y >> 8) & 0xFF;
-          ex = extras + (size_t)e.x * 16;
-          ex_unit = extras_unit_bytes(n16, n4, kU4 == 2);
-          exu = ex + extras_header_bytes(n16, n4) + (size_t)(wb + 2 * i - bi * U) * ex_unit;
+          ex_unit = extras_unit_bytes(2 * n16p, 2 * n4pairs, kU4 == 2);
+          exu = extras + (size_t)lds32(slot_u32 + kWhereOff) * 16;
         }
         // ---- promoted channels: raw bf16 keys (A fragments with k = 8: lane (r, t) holds channel pair t for tokens r, r + 8 of
         // both m-tiles), a gathered q.  Pairs past the count read the last pair (their query entries are 0).
@@ -571,10 +582,10 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
             for (int mt = 0; mt < 2; ++mt)
               mma_bf16_k8(Sx[un][mt], lds32(row + un * (kRowPairs * 128) + (sw ^ (64 * mt))), lds32(row + un * (kRowPairs * 128) + (sw ^ (64 * mt + 32))), xb);
           if (spill16) {
-#pragma unroll 2
+#pragma unroll kSpillUnroll
             for (int p0 = kRowPairs; p0 < n16p; p0 += 4) {
               const int p = min(p0 + t, n16p - 1);
-              const uint32_t b = p0 + t < n16p ? query_pair(qrow_u32, *reinterpret_cast<const uint16_t*>(ex + 2 * p)) : 0u;
+              const uint32_t b = p0 + t < n16p ? query_pair(qrow_u32, lds16(slot_u32 + 2 * p)) : 0u;
               const char* e = exu + (p * 32 + r) * 4;
 #pragma unroll
               for (int un = 0; un < 2; ++un)
@@ -614,7 +625,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
 #pragma unroll
               for (int mt = 0; mt < 2; ++mt) mma_f16(Sx[un][mt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], qb[0], qb[1]);
             };
-            if (!spill16) {
+            {
               const uint32_t pl = slot_u32 + kPlaneOff + 16 * t + 4 * (r & 3);
 #pragma unroll
               for (int kk = 0; kk < 2; ++kk) {
@@ -629,14 +640,14 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
               }
             }
             if (spill4) {
-              for (int p0 = spill16 ? 0 : kPlanePairs; p0 < n4pairs; p0 += 8) {
+              for (int p0 = kPlanePairs; p0 < n4pairs; p0 += 8) {
                 uint32_t sidx[2], qb[2], words[2][2] = {{0u, 0u}, {0u, 0u}};
 #pragma unroll
                 for (int hp = 0; hp < 2; ++hp) {
                   const int p = p0 + 4 * hp + t;
                   uint32_t two = 0xFFFFu;
                   if (p < n4pairs) {
-                    two = *reinterpret_cast<const uint16_t*>(ex + 2 * n16p + 2 * p);
+                    two = lds16(slot_u32 + 2 * n16p + 2 * p);
 #pragma unroll
                     for (int un = 0; un < 2; ++un)
                       words[un][hp] = reinterpret_cast<const uint32_t*>(exu + un * ex_unit + 128 * n16p)[p * 4 + (r & 3)];
@@ -1264,6 +1275,10 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // 7.6 units, 9.3 / 7.8 (8b shape, R = 64, 700 tokens, 6.5 units, 9.3 / 8.5, but an error of 0.86e-4 / 1.12e-4); 4-bit base (8b shape, batch 16) 600 tokens, 12 units, 8.9 / 9.3, 2000 tokens, 31 units, 18.7 / 17.7.
   const int from_units = three_tiers(lv) ? 7 : lv.dense_hi ? 20 : lv.G == 128 ? 10 : 40;
   bool by_two = !(lv.U & 1) && (lv.seq != nullptr ? lv.seq_total : Us * S) >= (long long)from_units * grid;
+  // A fixed budget of more promoted channels than a step's slot holds: us per launch, one unit / two units per step, 12 channels, 8b
+  // shape, 16384 tokens 83 / 87, 32b shape, G = 128, 8192 tokens 141 / 144; 128 channels, 7b shape, G = 128 48.7 / 53; 32 channels, 8b
+  // shape 112 / 111.  (Three tiers: two units are the faster.)
+  if (lv.budget_bf16 > 2 * kRowPairs && lv.budget_u4 == 0) by_two = false;
   // A short stream with a CTA of its own takes one unit at a time, for the precision: a probability is exact where it is the
   // maximum of its unit.
   if (lv.seq == nullptr && grid == S && one_cta_per_stream(lv, n_sms)) by_two = false;

@@ -77,6 +77,7 @@ __device__ __forceinline__ void stage_copy2(uint32_t dst_a, const void* src_a, u
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // shared-memory accesses by 32-bit shared address (the offsets added at the call sites fold into the instruction)
 __device__ __forceinline__ uint4 lds128(uint32_t a) {
   uint4 v;

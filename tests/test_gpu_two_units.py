@@ -67,3 +67,23 @@ def test_which_kernel(binding, name, batch, tokens, R, preset, v_bits, form):
     cache = filled(binding, w, v_bits=v_bits)
     cache.decode_attention(0, W.decode_query(w, 0, 0, device="cuda"), W.softmax_scale())
     assert cache.last_attention() & 7 == form
+
+
+@pytest.mark.parametrize("name,batch,tokens,tau16,tau4", [
+    ("qwen7b", 16, 6400, 2.5, 1e30), ("qwen32b", 16, 2048, 2.0, 1e30), ("qwen7b", 8, 2560, 2.5, 1.5), ("qwen7b", 8, 2560, 1.0, 0.5),
+    ("llama8b", 16, 2560, 0.5, -1.0),
+])
+def test_more_promoted_channels_than_a_slot_holds(binding, name, batch, tokens, tau16, tau4):
+    w = W.small(W.CONFIGS[name], n_layers=1, batch=batch, tokens=tokens, tau_bf16=tau16, tau_u4=tau4)
+    cache = U.make_cache(binding, w, extras_budget_bytes=(tokens // 128 + 3) * (128 * 260 + 4096))
+    for t in range(0, tokens, 4096):
+        cache.quantize_append(0, *W.tokens(w, 0, t, min(4096, tokens - t), device="cuda"))
+    n16 = cache.stream_regions(0, 0)["table"][4::8]
+    assert max(n16) > 8, n16
+    q = W.decode_query(w, 0, 0, device="cuda")
+    out = cache.decode_attention(0, q, W.softmax_scale())
+    assert cache.last_attention() & 3 == binding.ATTN_TWO_UNITS
+    cache.set_attention_kernel(1)
+    ref = cache.decode_attention(0, q, W.softmax_scale())
+    assert cache.status() == 0
+    assert float((out - ref).abs().max()) <= 4e-3          # both kernels are within 2e-3 of the exact result
