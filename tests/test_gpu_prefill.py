@@ -58,3 +58,27 @@ def test_prefill_large_magnitudes_and_errors(binding):
     with pytest.raises(binding.MixKVQError):                           # the scratch buffer is too small
         cache.prefill(0, k.cuda(), v.cuda(), q.cuda(), W.softmax_scale(), scratch=small)
     assert cache.prefill_scratch_bytes(300) == 2 * w.n_kv_heads * 3 * 32768
+
+
+@pytest.mark.parametrize("sink,mode,v_bits,preset", [(32, 0, 2, "P24"), (0, 1, 2, "P27"), (0, 2, 4, "P24"), (32, 1, 4, "P4BASE")])
+def test_prefill_layer_after_layer_with_options(binding, sink, mode, v_bits, preset):
+    """Prompts of several layers back to back on one scratch buffer, twice over (the second time on a reset cache): the quantization
+    that starts while the attention of its layer still runs leaves the oracle's bytes, with a sink, every importance mode and
+    4-bit values, and the outputs repeat themselves."""
+    T = 3 * 128 + 45
+    w = W.small(W.CONFIGS["qwen7b"], n_layers=3, batch=2, tokens=T, **getattr(W, preset))
+    cache = U.make_cache(binding, w, importance_mode=mode, sink_len=sink, v_bits=v_bits, extras_budget_bytes=8 * 64 * 128)
+    scratch = torch.empty(cache.prefill_scratch_bytes(T), dtype=torch.uint8, device="cuda")
+    data = [W.tokens(w, layer, 0, T) for layer in range(3)]
+    cuda = [[x.cuda() for x in d] for d in data]
+    outs = []
+    for _ in range(2):
+        cache.mem.fill_(0xA5)
+        cache.reset()
+        outs.append([cache.prefill(layer, *cuda[layer], W.softmax_scale(), scratch=scratch) for layer in range(3)])
+        assert cache.status() == 0
+    for layer in range(3):
+        assert torch.equal(outs[0][layer], outs[1][layer])
+        streams = [(0, 0), (1, w.n_kv_heads - 1)]
+        oracle = U.oracle_streams(w, layer, *data[layer], streams=streams, importance_mode=mode, sink_len=sink, v_bits=v_bits)
+        U.compare_regions(cache, layer, w, oracle)
