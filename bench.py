@@ -256,12 +256,13 @@ def algorithmic_bytes_per_layer(w, n16, n4, r, tokens_packed, n_partials, v_bits
 
 
 def n_split_partials(w, d0, dev):
-    """Partials written per launch = CTAs of the split kernel: two per SM, a multiple of the stream count when there
-    are fewer streams than CTA slots (the library's grid rule), each CTA one partial per stream it touches."""
+    """Partials written per launch = CTAs of the split kernel (the library's grid rule: two split positions per CTA while that
+    leaves one CTA per SM, then up to four, then two CTAs per SM; a multiple of the stream count when there are fewer streams
+    than CTAs), each CTA one partial per stream it touches."""
     streams = w.batch * w.n_kv_heads
-    units = (d0.n_blocks * w.residual_len // 32 + (d0.residual_tokens + 31) // 32) * streams
+    units = (d0.n_blocks * w.residual_len // 32 + 3 * ((d0.residual_tokens + 31) // 32)) * streams
     n_sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    n_part = min(2 * n_sms, units)
+    n_part = min(2 * n_sms, (units + 1) // 2, max(n_sms, (units + 3) // 4))
     return n_part // streams * streams if n_part > streams else n_part + streams
 
 
