@@ -1,5 +1,5 @@
-"""The flush kernel's quantizer shortcut, restated in numpy float32: codes from (x - z) * RN(1 / s), with the IEEE division
-only within 1e-4 of a half-integer, equal round-half-even of the IEEE quotient (x - z) / s for every input tried:
+"""The plainest form of the quantizer's shortcut, restated in numpy float32 (the flush kernel's own, with an FMA and a narrower
+margin, is in test_quantizer_fma.py): codes from (x - z) * RN(1 / s), with the IEEE division only within 1e-4 of a half-integer, equal round-half-even of the IEEE quotient (x - z) / s for every input tried:
 random bf16 data over many scales, and inputs placed on and next to the rounding ties."""
 import numpy as np
 
