@@ -283,8 +283,8 @@ int mixkvq_cache_written_externally(mixkvq_cache* cache);
  * hangs: the copies themselves are the normal ones.  (0, 0) restores normal operation. */
 int mixkvq_test_arm_copy_timeout(mixkvq_cache* cache, uint32_t extra_bytes, uint32_t max_polls);
 
-/* The same for the barrier of every CTA's last value tile in the prefill attention: the rows whose last product is
- * missing are left unwritten, the others are as usual. */
+/* The same in the prefill attention for the barrier of a CTA's last value tile where that tile's number is odd or it is the
+ * prompt's last: the rows whose last product is missing are left unwritten, the others are as usual. */
 int mixkvq_test_arm_value_copy_timeout(mixkvq_cache* cache, uint32_t extra_bytes, uint32_t max_polls);
 
 /* Selects the decode-attention kernel: 0 = tensor-core kernel (default), 1 = plain-ALU kernel

@@ -3,7 +3,8 @@
 //
 // Two kernels.  prefill_pack_kernel rewrites K (bf16) and V (converted to fp16) of the prompt into images of 128-token
 // tiles in the tensor core's canonical shared-memory layout, so that a tile reaches shared memory as ONE 32 KB bulk
-// copy.  prefill_attention_kernel runs one CTA of 384 threads per (batch element, query head, 256 query positions):
+// copy.  prefill_attention_kernel runs one CTA of 384 threads per 256 query rows of a stream (batch element and KV head; a token's
+// query heads side by side):
 //   warps 0-3, 4-7   two softmax groups, one per 128 query rows (thread = row = lane of tensor memory);
 //   warp 8           one thread issues every tcgen05.mma;
 //   warp 9           one thread issues the bulk copies of the K and V tiles into two-stage rings.
@@ -26,8 +27,11 @@
 // 2.85, 2.91, 3.09e-5 at 32768, and no faster than 2 % (the registers cost the time, not the additions).
 // B200, whole call per layer (us), sum in tensor memory / in registers: prompt of 32768 tokens (7b shape) 6492 / 6811, 8192: 530 /
 // 558, 333: 29.4 / 29.5; 4 x 777 tokens (8b shape) 100.7 / 103.5.  (Waiting for each product right behind its issue, and with the tensor
-// core idle meanwhile: 7447, 699, 104, 169.)  Register split: 72 for the issuing warps leaves 96 bytes of spills; 56 and 224 spill
-// 212 there.
+// core idle meanwhile: 7447, 699, 104, 169.)  Tensor memory is read 16
+// columns at a time, the next 16 in flight: blocks of 32 registers beside the 128 of the sum spilled 96 to 356 bytes, whatever the split.
+// Rows: with 256 rows of one head per CTA the last row tile of 4 x 777 tokens (8b shape) held 9 rows of 256 and the diagonal tiles were
+// half empty; side by side the heads take 13 row tiles with 49 key tiles per stream instead of 16 with 76: attention 75 -> 54 us,
+// whole call 108 -> 92 us per layer.  32768 tokens (7b shape, no idle rows either way): 7.79 / 7.83 ms.
 #include "common.cuh"
 
 namespace mixkvq {
@@ -90,26 +94,21 @@ __device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a_desc, uint
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// A load of 32 columns of the thread's tensor-memory lane.  The registers are valid only after tmem_wait_ld32 on them (the wait names
+// A load of 16 columns of the thread's tensor-memory lane.  The registers are valid only after tmem_wait_ld16 on them (the wait names
 //  the registers as operands, so that no use of them is scheduled before it).  tcgen05.wait::ld covers every load
 // the thread has issued, so a load issued before a block of arithmetic and waited for after it runs under that arithmetic.
-__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&u)[32]) {
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&u)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]),
-        "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]), "=r"(u[16]),
-        "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]), "=r"(u[22]), "=r"(u[23]), "=r"(u[24]),
-        "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]), "=r"(u[31])
+        "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld32(uint32_t (&u)[32]) {
+__device__ __forceinline__ void tmem_wait_ld16(uint32_t (&u)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]), "+r"(u[7]), "+r"(u[8]),
-                 "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]), "+r"(u[15]), "+r"(u[16]),
-                 "+r"(u[17]), "+r"(u[18]), "+r"(u[19]), "+r"(u[20]), "+r"(u[21]), "+r"(u[22]), "+r"(u[23]), "+r"(u[24]),
-                 "+r"(u[25]), "+r"(u[26]), "+r"(u[27]), "+r"(u[28]), "+r"(u[29]), "+r"(u[30]), "+r"(u[31])
+                 "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]), "+r"(u[15])
                :
                : "memory");
 }
@@ -164,20 +163,23 @@ prefill_pack_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __
   uint4* kd = reinterpret_cast<uint4*>(kt + ((size_t)s * n_tiles + t) * kTileBytes);
   uint4* vd = reinterpret_cast<uint4*>(vt + ((size_t)s * n_tiles + t) * kTileBytes);
   const int rows = min(kTile, L - t * kTile);
-#pragma unroll 2
-  for (int i = threadIdx.x; i < kTile * 16; i += 256) {
-    {  // K: byte offset (r / 8) * 2048 + c * 128 + (r % 8) * 16 of row r, 16-byte chunk c
-      const int r = 8 * (i >> 7) + (i & 7), c = (i >> 3) & 15;
-      uint4 x = make_uint4(0u, 0u, 0u, 0u);
-      if (r < rows) x = *reinterpret_cast<const uint4*>(kg + (size_t)r * kD + 8 * c);
-      kd[i] = x;
-    }
-    {  // V: byte offset c * 2048 + (r / 8) * 128 + (r % 8) * 16
-      const int r = (i & 127), c = i >> 7;
-      uint4 x = make_uint4(0u, 0u, 0u, 0u);
-      if (r < rows) x = *reinterpret_cast<const uint4*>(vg + (size_t)r * kD + 8 * c);
-      vd[i] = make_uint4(bf16x2_to_f16x2(x.x), bf16x2_to_f16x2(x.y), bf16x2_to_f16x2(x.z), bf16x2_to_f16x2(x.w));
-    }
+  // all of a thread's loads are in flight at once
+  constexpr int kEach = kTile * 16 / 256;
+  uint4 x[kEach], y[kEach];
+#pragma unroll
+  for (int n = 0; n < kEach; ++n) {
+    const int i = threadIdx.x + 256 * n;
+    // K: byte offset (r / 8) * 2048 + c * 128 + (r % 8) * 16 of row r, 16-byte chunk c; V: c * 2048 + (r / 8) * 128 + (r % 8) * 16
+    const int kr = 8 * (i >> 7) + (i & 7), kc = (i >> 3) & 15, vr = i & 127, vc = i >> 7;
+    x[n] = y[n] = make_uint4(0u, 0u, 0u, 0u);
+    if (kr < rows) x[n] = *reinterpret_cast<const uint4*>(kg + (size_t)kr * kD + 8 * kc);
+    if (vr < rows) y[n] = *reinterpret_cast<const uint4*>(vg + (size_t)vr * kD + 8 * vc);
+  }
+#pragma unroll
+  for (int n = 0; n < kEach; ++n) {
+    const int i = threadIdx.x + 256 * n;
+    kd[i] = x[n];
+    vd[i] = make_uint4(bf16x2_to_f16x2(y[n].x), bf16x2_to_f16x2(y[n].y), bf16x2_to_f16x2(y[n].z), bf16x2_to_f16x2(y[n].w));
   }
 }
 
@@ -209,43 +211,61 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   return d;
 }
 
-// Adds the row's P V product in tensor memory to the sum kept in registers.
-__device__ __forceinline__ void add_output(uint32_t o_addr, float (&sum_o)[128]) {
+// Calls f(piece, columns) for the pieces of 16 columns below n_pieces of the thread's tensor-memory row, the next piece in flight.
+template <bool kAll, typename F>
+__device__ __forceinline__ void for_pieces(uint32_t taddr, int n_pieces, F f) {
+  if constexpr (kAll) {
+    uint32_t a[16], b[16];
+    tmem_ld16_issue(taddr, a);
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    uint32_t x[32];
-    tmem_ld32_issue(o_addr + 32 * c, x);
-    tmem_wait_ld32(x);
-#pragma unroll
-    for (int k = 0; k < 32; k += 2)
-      unpack2(add2(pack2u(x[k], x[k + 1]), pack2(sum_o[32 * c + k], sum_o[32 * c + k + 1])), sum_o[32 * c + k], sum_o[32 * c + k + 1]);
+    for (int h = 0; h < 8; h += 2) {
+      tmem_wait_ld16(a);
+      tmem_ld16_issue(taddr + 16 * h + 16, b);
+      f(h, a);
+      tmem_wait_ld16(b);
+      if (h < 6) tmem_ld16_issue(taddr + 16 * h + 32, a);
+      f(h + 1, b);
+    }
+  } else {
+#pragma unroll 1
+    for (int h = 0; h < n_pieces; ++h) {
+      uint32_t a[16];
+      tmem_ld16_issue(taddr + 16 * h, a);
+      tmem_wait_ld16(a);
+      f(h, a);
+    }
   }
 }
 
+// Adds the row's P V product in tensor memory to the sum kept in registers.
+__device__ __forceinline__ void add_output(uint32_t o_addr, float (&sum_o)[128]) {
+  for_pieces<true>(o_addr, 8, [&](int h, const uint32_t (&x)[16]) {
+#pragma unroll
+    for (int k = 0; k < 16; k += 2)
+      unpack2(add2(pack2u(x[k], x[k + 1]), pack2(sum_o[16 * h + k], sum_o[16 * h + k + 1])), sum_o[16 * h + k], sum_o[16 * h + k + 1]);
+  });
+}
+
 // One 128-key tile of one row group's softmax.  The thread owns one row of S (128 fp32 columns of its tensor-memory lane at
-// s_addr) and of the last product P V (at o_addr), which goes to its sum.  Writes P (fp16 pairs) over columns [0, 64) of S.  kDiag: the tile on the diagonal, where row i
-// of the group sees columns <= i: warp w (rows 32 w ..) needs the columns of 32-chunks <= w, and a comparison only in chunk w.
+// s_addr) and of the last product P V (at o_addr), which goes to its sum.  Writes P (fp16 pairs) over columns [0, 64) of S.  kDiag: the
+// tile on the diagonal: the thread's row sees the columns <= last, the warp's rows all see those <= warp_first and none those >
+// warp_last; the product takes the pieces of 16 keys below n_write (rows that see none of a piece have zeros there).
 template <bool kDiag>
-__device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, int w, int lane, bool first, float scale_log2e,
+__device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, int warp_first, int warp_last, int last, int n_write, bool first, float scale_log2e,
                                              float& m_ref, float& l_run, uint32_t half_bar, float (&sum_o)[128]) {
   if (!first) add_output(o_addr, sum_o);             // the product of the tile before
   // ---- the row's maximum
   float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // four independent chains
-  auto reduce = [&](const uint32_t (&u)[32], int last) {
+  const int n_seen = kDiag ? (warp_last >> 4) + 1 : 8;              // pieces of 16 columns that some row of the warp sees
+  for_pieces<!kDiag>(s_addr, n_seen, [&](int h, const uint32_t (&u)[16]) {
+    const int lim = last - 16 * h;
 #pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-      const float x0 = kDiag && i > last ? -INFINITY : __uint_as_float(u[i]);
-      const float x1 = kDiag && i + 1 > last ? -INFINITY : __uint_as_float(u[i + 1]);
+    for (int i = 0; i < 16; i += 2) {
+      const float x0 = kDiag && i > lim ? -INFINITY : __uint_as_float(u[i]);
+      const float x1 = kDiag && i + 1 > lim ? -INFINITY : __uint_as_float(u[i + 1]);
       mx4[(i >> 1) & 3] = fmaxf(fmaxf(mx4[(i >> 1) & 3], x0), x1);
     }
-  };
-#pragma unroll 1
-  for (int c = 0; c < (kDiag ? w + 1 : 4); ++c) {
-    uint32_t a[32];
-    tmem_ld32_issue(s_addr + 32 * c, a);
-    tmem_wait_ld32(a);
-    reduce(a, kDiag && c == w ? lane : 31);
-  }
+  });
   const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale_log2e;
   if (first) {
     m_ref = mx;
@@ -264,60 +284,38 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, i
     tc_fence_before();
     mbar_arrive(half_bar);
   };
-  // ---- probabilities in chunks of 32 columns; P chunk c (16 columns of fp16 pairs) lies inside the S columns of chunks
-  // <= c, which are already in registers
+  // ---- probabilities, 16 columns at a time, the next ones in flight; P piece h (8 columns of fp16 pairs) lies inside the S columns of
+  // pieces <= h, which are already in registers
   const uint64_t scale2 = pack2(scale_log2e, scale_log2e), ref2 = pack2(-m_ref, -m_ref);
   uint64_t sum[2] = {0ull, 0ull};
-  auto probs = [&](const uint32_t (&u)[32], int c, int last) {
+  auto probs = [&](const uint32_t (&u)[16], int h) {
+    uint32_t wd[8];
+    const int lim = last - 16 * h;
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      uint32_t wd[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int k = 16 * half + 2 * i;
-        float x0, x1;
-        unpack2(fma2(pack2u(u[k], u[k + 1]), scale2, ref2), x0, x1);
-        float p0 = ex2(x0), p1 = ex2(x1);
-        if constexpr (kDiag) {
-          p0 = k <= last ? p0 : 0.f;
-          p1 = k + 1 <= last ? p1 : 0.f;
-        }
-        sum[i & 1] = add2(sum[i & 1], pack2(p0, p1));
-        wd[i] = pack_half2(p0, p1);
+    for (int i = 0; i < 8; ++i) {
+      float x0, x1;
+      unpack2(fma2(pack2u(u[2 * i], u[2 * i + 1]), scale2, ref2), x0, x1);
+      float p0 = ex2(x0), p1 = ex2(x1);
+      if constexpr (kDiag) {
+        p0 = 2 * i <= lim ? p0 : 0.f;
+        p1 = 2 * i + 1 <= lim ? p1 : 0.f;
       }
-      tmem_st8(s_addr + 16 * c + 8 * half, wd);
+      sum[i & 1] = add2(sum[i & 1], pack2(p0, p1));
+      wd[i] = pack_half2(p0, p1);
     }
+    tmem_st8(s_addr + 8 * h, wd);
   };
+  for_pieces<!kDiag>(s_addr, n_seen, [&](int h, const uint32_t (&u)[16]) {
+    probs(u, h);
+    if (h == 3) half_ready();
+  });
   if constexpr (kDiag) {
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-      if (c <= w) {
-        uint32_t a[32];
-        tmem_ld32_issue(s_addr + 32 * c, a);
-        tmem_wait_ld32(a);
-        probs(a, c, c == w ? lane : 31);
-      } else {
-        const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        tmem_st8(s_addr + 16 * c, zero);
-        tmem_st8(s_addr + 16 * c + 8, zero);
-      }
-      if (c == 1) half_ready();
+    for (int h = n_seen; h < n_write; ++h) {
+      const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+      tmem_st8(s_addr + 8 * h, zero);
+      if (h == 3) half_ready();
     }
-  } else {
-    uint32_t a[32], b[32];                          // the next chunk in flight
-    tmem_ld32_issue(s_addr, a);
-    tmem_wait_ld32(a);
-    tmem_ld32_issue(s_addr + 32, b);
-    probs(a, 0, 31);
-    tmem_wait_ld32(b);
-    tmem_ld32_issue(s_addr + 64, a);
-    probs(b, 1, 31);
-    half_ready();
-    tmem_wait_ld32(a);
-    tmem_ld32_issue(s_addr + 96, b);
-    probs(a, 2, 31);
-    tmem_wait_ld32(b);
-    probs(b, 3, 31);
+    if (max(n_seen, n_write) < 4) half_ready();
   }
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   float s0, s1;
@@ -325,12 +323,15 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, i
   l_run += s0 + s1;
 }
 
-// q [B, Hq, L, 128] bf16; kt, vt the tile images of prefill_pack_kernel; out [B, Hq, L, 128] fp32.  blockIdx.x / BH
-// counts the 256-row query tiles from the last one down (it has the most key tiles: the long CTAs start first),
-// blockIdx.x % BH = b * Hq + h.
+// q [B, Hq, L, 128] bf16; kt, vt the tile images of prefill_pack_kernel; out [B, Hq, L, 128] fp32.  A stream's query rows are numbered
+// token by token, its g heads side by side: row x is head x % g of token x / g.  A CTA takes 256 such rows, two groups of 128.  128
+// tokens are g whole groups, so that a group's tokens lie in one key tile, its last, and a group of 128 / g tokens does less than a
+// group of 128 tokens of one head where it lies at the diagonal, and a prompt that is no multiple of 256 leaves fewer rows idle.
+// blockIdx.x / n_streams counts the row tiles from the last one down (it has the most key tiles: the long CTAs start first),
+// blockIdx.x % n_streams = b * Hkv + hk.
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned char* __restrict__ kt,
-                         const unsigned char* __restrict__ vt, float* __restrict__ out, int BH, int Hq, int Hkv, int L,
+                         const unsigned char* __restrict__ vt, float* __restrict__ out, int n_streams, int g_heads, int L,
                          int n_tiles, int n_qtiles, float scale_log2e, uint32_t* status, uint32_t max_polls, uint32_t debug_extra_tx, uint32_t debug_extra_v) {
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* Qs = smem;                              // two tiles
@@ -340,13 +341,26 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 6 * kTileBytes + 8 * kBars);
   auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int qt = n_qtiles - 1 - (int)blockIdx.x / BH;
-  const int bh = (int)blockIdx.x % BH, b = bh / Hq, h = bh % Hq, hk = h / (Hq / Hkv);
-  const __nv_bfloat16* qg = q + ((size_t)(b * Hq + h) * L) * kD;
-  const unsigned char* ktg = kt + (size_t)(b * Hkv + hk) * n_tiles * kTileBytes;
-  const unsigned char* vtg = vt + (size_t)(b * Hkv + hk) * n_tiles * kTileBytes;
-  // key tiles of the two row groups: rows [256 qt, +128) see tiles 0 .. 2 qt, rows [256 qt + 128, +128) one more
-  const int n_a = 2 * qt + 1, n_b = min(2 * qt + 2, n_tiles);
+  const int qt = n_qtiles - 1 - (int)blockIdx.x / n_streams, s = (int)blockIdx.x % n_streams;
+  const uint32_t g_inv = 65536u / (uint32_t)g_heads + 1u;              // x / g = x * g_inv >> 16 for x < 512
+  struct Rows {          // of a row tile: the first row's token and head
+    int tok0, rem0, L;
+    uint32_t inv;
+    __device__ int token(int row) const { return min(tok0 + (int)((uint32_t)(rem0 + row) * inv >> 16), L - 1); }
+  };
+  auto rows_of = [&](int tile) {
+    const int tok0 = tile * kQRows / g_heads;
+    return Rows{tok0, tile * kQRows - tok0 * g_heads, L, g_inv};
+  };
+  const unsigned char* ktg = kt + (size_t)s * n_tiles * kTileBytes;
+  const unsigned char* vtg = vt + (size_t)s * n_tiles * kTileBytes;
+  // The two groups: the last token (rows past the prompt see what its last token sees and are not stored), its key tiles (n_b = 0: no
+  // row of the prompt in group B; n_a <= n_b otherwise) and the columns of the last of them that some row sees
+  const Rows rows = rows_of(qt);
+  const int tok0 = rows.tok0, rem0 = rows.rem0;
+  const int last_a = rows.token(kTile - 1), last_b = rows.token(kQRows - 1);
+  const int n_a = last_a / kTile + 1, n_b = qt * kQRows + kTile < L * g_heads ? last_b / kTile + 1 : 0, n = max(n_a, n_b);
+  const int seen_a = last_a % kTile + 1, seen_b = last_b % kTile + 1;
 
   if (warp == 8) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512)
@@ -356,9 +370,9 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
   int issued = 0;                  // K and V tiles requested (the copying thread)
   auto copy_tile = [&](int j, bool keys) {
     const int st = j & 1, full = (keys ? kKFull : kVFull) + st;
-    // (test hooks: the barrier of the first key tile or of the last value tile can be armed for more bytes than arrive, so that
-    // it never completes)
-    mbar_expect_tx(bar(full), kTileBytes + (keys ? (j == 0 ? debug_extra_tx : 0u) : (j == n_b - 1 ? debug_extra_v : 0u)));
+    // (test hooks: the barrier of the first key tile, or of the last value tile where that is odd or the prompt's last, can be armed for
+    // more bytes than arrive, so that it never completes)
+    mbar_expect_tx(bar(full), kTileBytes + (keys ? (j == 0 ? debug_extra_tx : 0u) : (j == n - 1 && ((j & 1) || j == n_tiles - 1) ? debug_extra_v : 0u)));
     bulk_copy(smem_u32((keys ? Ks : Vs) + st * kTileBytes), (keys ? ktg : vtg) + (size_t)j * kTileBytes, kTileBytes, bar(full));
   };
   if (tid == 9 * 32) {
@@ -368,7 +382,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     // the first tiles are under way while Q is loaded (Q was written before the kernel that packs the tiles: only the tiles
     // wait for that kernel)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (; issued < min(2, n_b); ++issued) {
+    for (; issued < min(2, n); ++issued) {
       copy_tile(issued, true);
       copy_tile(issued, false);
     }
@@ -380,9 +394,11 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     uint4 x[kEach];
 #pragma unroll
     for (int k = 0; k < kEach; ++k) {
-      const int i = tid + k * kThreads, ii = i & 2047, r = (i >> 11) * kTile + 8 * (ii >> 7) + (ii & 7), c = (ii >> 3) & 15;
+      const int i = tid + k * kThreads, ii = i & 2047, c = (ii >> 3) & 15;
+      const uint32_t r = (uint32_t)(rem0 + (i >> 11) * kTile + 8 * (ii >> 7) + (ii & 7)), tk = r * g_inv >> 16;
       x[k] = make_uint4(0u, 0u, 0u, 0u);
-      if (i < kPieces && qt * kQRows + r < L) x[k] = *reinterpret_cast<const uint4*>(qg + (size_t)(qt * kQRows + r) * kD + 8 * c);
+      if (i < kPieces && tok0 + (int)tk < L)
+        x[k] = *reinterpret_cast<const uint4*>(q + (((size_t)s * g_heads + (r - tk * g_heads)) * L + tok0 + tk) * kD + 8 * c);
     }
 #pragma unroll
     for (int k = 0; k < kEach; ++k)
@@ -410,56 +426,67 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     if (warp == 8 && lane == 0) {
       // ---------------------------------------------------------------- tensor-core issue
       const uint32_t idesc_qk = make_idesc(128, 128, 1, 0), idesc_pv = make_idesc(128, 128, 0, 1);
-      auto issue_s = [&](int g, int j) {                 // S_g = Q_g K_j^T
+      // S_g = Q_g K_j^T; of a group's last key tile only the columns that some row sees
+      auto issue_s = [&](int g, int j, int seen) {
         const uint64_t qd = make_desc(smem_u32(Qs + g * kTileBytes), 128, 2048);
         const uint64_t kd = make_desc(smem_u32(Ks + (j & 1) * kTileBytes), 128, 2048);
+        const uint32_t idesc = seen == kTile ? idesc_qk : make_idesc(128, (seen + 15) & ~15, 1, 0);
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) tc_mma_ss(tbase + 128 * g, qd + (uint64_t)(ks * 16), kd + (uint64_t)(ks * 16), idesc_qk, ks > 0);
+        for (int ks = 0; ks < 8; ++ks) tc_mma_ss(tbase + 128 * g, qd + (uint64_t)(ks * 16), kd + (uint64_t)(ks * 16), idesc, ks > 0);
         tc_commit(bar(kSFull + g));
       };
-      auto issue_o = [&](int g, int j, int half) {       // O_g = P_g V_j, 64 of the tile's keys at a time
+      // O_g = P_g V_j, 64 of the tile's keys at a time, as soon as each half of P_g is there (a product of its own per tile).  Whole tiles
+      // without a decision between the instructions: the issuing thread's own time counts.
+      auto issue_o = [&](int g, int j, int seen) {
         const uint64_t vd = make_desc(smem_u32(Vs + (j & 1) * kTileBytes), 128, 2048);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int ks = 4 * half + k;
-          tc_mma_ts(tbase + 256 + 128 * g, tbase + 128 * g + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, ks > 0);      // (a product of its own per tile)
-        }
-      };
-      auto both_halves = [&](int g, int j) {             // as soon as each half of P_g is there
+        const uint32_t o = tbase + 256 + 128 * g, p = tbase + 128 * g;
         if (!wait(kPHalf + g, (uint32_t)j & 1u)) return false;
         tc_fence_after();
-        issue_o(g, j, 0);
+        if (seen == kTile) {
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) tc_mma_ts(o, p + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, ks > 0);
+        } else {
+          for (int ks = 0; ks < 4 && 16 * ks < seen; ++ks) tc_mma_ts(o, p + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, ks > 0);
+        }
         if (!wait(kPReady + g, (uint32_t)j & 1u)) return false;
         tc_fence_after();
-        issue_o(g, j, 1);
+        if (seen == kTile) {
+#pragma unroll
+          for (int ks = 4; ks < 8; ++ks) tc_mma_ts(o, p + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, 1);
+        } else {
+          for (int ks = 4; 16 * ks < seen; ++ks) tc_mma_ts(o, p + 8 * ks, vd + (uint64_t)(ks * 16), idesc_pv, 1);
+        }
         return true;
       };
       if (wait(kKFull, 0)) {
         tc_fence_after();
-        issue_s(0, 0);
-        issue_s(1, 0);
+        issue_s(0, 0, n_a == 1 ? seen_a : kTile);
+        if (n_b > 0) issue_s(1, 0, n_b == 1 ? seen_b : kTile);
         tc_commit(bar(kKEmpty));
       }
-      for (int j = 0; j < n_b && !dead; ++j) {
+      for (int j = 0; j < n && !dead; ++j) {
         const int st = j & 1, nx = (j + 1) & 1;
         const uint32_t ph = (uint32_t)(j >> 1) & 1u, ph_nx = (uint32_t)((j + 1) >> 1) & 1u;
         if (!wait(kVFull + st, ph)) break;
         if (j < n_a) {
-          if (!both_halves(0, j)) break;
+          if (!issue_o(0, j, j + 1 == n_a ? seen_a : kTile)) break;
+          if (n_b == 0) tc_commit(bar(kVEmpty + st));
           if (j + 1 == n_a) tc_commit(bar(kDoneA));
           if (j + 1 < n_a) {
             if (!wait(kKFull + nx, ph_nx)) break;
             tc_fence_after();
-            issue_s(0, j + 1);
+            issue_s(0, j + 1, j + 2 == n_a ? seen_a : kTile);
+            if (n_b == 0) tc_commit(bar(kKEmpty + nx));
           }
         }
-        if (!both_halves(1, j)) break;
+        if (n_b == 0) continue;
+        if (!issue_o(1, j, j + 1 == n_b ? seen_b : kTile)) break;
         tc_commit(bar(kVEmpty + st));
         if (j + 1 == n_b) tc_commit(bar(kDoneB));        // (not when a wait ran out: group B must not take an unfinished product)
         if (j + 1 < n_b) {
           if (!wait(kKFull + nx, ph_nx)) break;
           tc_fence_after();
-          issue_s(1, j + 1);
+          issue_s(1, j + 1, j + 2 == n_b ? seen_b : kTile);
           tc_commit(bar(kKEmpty + nx));
         }
       }
@@ -468,7 +495,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
       wait(kDone, 0);
     } else if (warp == 9 && lane == 0) {
       // ---------------------------------------------------------------- bulk copies of the K and V tiles
-      for (int j = 2; j < n_b; ++j) {
+      for (int j = 2; j < n; ++j) {
         const int st = j & 1;
         const uint32_t ph_prev = (uint32_t)((j >> 1) - 1) & 1u;
         if (!wait(kKEmpty + st, ph_prev)) break;
@@ -491,49 +518,71 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 216;" ::: "memory");
     // ------------------------------------------------------------------ softmax and output rows
-    const int g = warp >> 2, row = tid & 127;
+    const int g = warp >> 2;
     const uint32_t lane_base = tbase + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t s_addr = lane_base + 128 * g, o_addr = lane_base + 256 + 128 * g;
-    const int n = g == 0 ? n_a : n_b;
-    const int pos = qt * kQRows + g * kTile + row;     // this thread's query position
+    const int n_g = g == 0 ? n_a : n_b;
+    // worked out again where it is needed: the loop has no registers to keep it in
+    auto rows_again = [&]() {
+      int again = qt;
+      asm volatile("" : "+r"(again));
+      return rows_of(again);
+    };
     float m_ref = -INFINITY, l_run = 0.f;
     float sum_o[128];
 #pragma unroll
     for (int d = 0; d < 128; ++d) sum_o[d] = 0.f;
-#pragma unroll 1
-    for (int j = 0; j < n; ++j) {
-      if (!wait(kSFull + g, (uint32_t)j & 1u)) break;
+    int j = 0;
+    auto s_ready = [&]() {
+      if (!wait(kSFull + g, (uint32_t)j & 1u)) return false;
       tc_fence_after();
-      if (j == 2 * qt + g)      // the tile on the diagonal
-        softmax_tile<true>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
-      else
-        softmax_tile<false>(s_addr, o_addr, warp & 3, lane, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
+      return true;
+    };
+    auto p_ready = [&]() {
       tc_fence_before();
       mbar_arrive(bar(kPReady + g));
+    };
+#pragma unroll 1
+    for (; j + 1 < n_g; ++j) {
+      if (!s_ready()) break;
+      softmax_tile<false>(s_addr, o_addr, 0, 0, 0, 8, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
+      p_ready();
     }
-    // Output rows.  The rows of a warp are 512 bytes apart, so direct stores cost a wavefront per lane (10 thousand cycles for
-    // 256 rows at once, about half for 128).  Group A is done a tile earlier than group B and stores directly, in 32-byte
-    // pieces where the caller's buffer allows, under B's last tile; B's rows go through the shared memory, which nobody needs
-    // any more, and leave as one bulk copy each.
-    if (wait(g == 0 ? kDoneA : kDoneB, 0)) {
+    if (n_g > 0 && !dead && s_ready()) {       // the tile on the diagonal
+      const Rows at = rows_again();
+      const int r = g * kTile + (tid & 127), c0 = j * kTile;
+      softmax_tile<true>(s_addr, o_addr, at.token(r & ~31) - c0, at.token(r | 31) - c0, at.token(r) - c0, (at.token(g * kTile + 127) - c0 + 16) >> 4, j == 0,
+                         scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
+      p_ready();
+    }
+    // Output rows.  The rows of a warp are 512 bytes or more apart, so direct stores cost a wavefront per lane (10 thousand cycles for
+    // 256 rows at once, about half for 128).  Where group A is done a tile earlier than group B it stores directly, in 32-byte
+    // pieces where the caller's buffer allows, under B's last tile; otherwise the rows go through the shared memory, which nobody needs
+    // any more once B's last product is there, and leave as one bulk copy each.
+    const bool direct = g == 0 && n_a < n_b;
+    if (n_g > 0 && wait(g == 0 ? kDoneA : kDoneB, 0) && (direct || n_b == 0 || wait(kDoneB, 0))) {
       tc_fence_after();
       add_output(o_addr, sum_o);
       const float inv = 1.f / l_run;
-      float* dst = out + ((size_t)(b * Hq + h) * L + pos) * kD;
+      const Rows at = rows_again();
+      const int row = tid & 127;
+      const uint32_t x = (uint32_t)(at.rem0 + g * kTile + row), tk = x * g_inv >> 16;
+      const bool valid = at.tok0 + (int)tk < L;
+      float* dst = out + (((size_t)s * g_heads + (x - tk * g_heads)) * L + at.tok0 + tk) * kD;
       const bool wide = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
-      const uint32_t staged = smem_u32(smem) + (uint32_t)row * 528u;      // (a row's 16-byte pieces on the banks of no other lane)
+      const uint32_t staged = smem_u32(smem) + (uint32_t)(g * kTile + row) * 528u;      // (a row's 16-byte pieces on the banks of no other lane)
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         float y[32];
 #pragma unroll
         for (int d = 0; d < 32; ++d) y[d] = sum_o[32 * c + d] * inv;
-        if (g == 1) {
+        if (!direct) {
 #pragma unroll
           for (int d = 0; d < 32; d += 4)
             asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(staged + 4 * (32 * c + d)), "f"(y[d]), "f"(y[d + 1]),
                          "f"(y[d + 2]), "f"(y[d + 3])
                          : "memory");
-        } else if (pos < L) {
+        } else if (valid) {
 #pragma unroll
           for (int d = 0; d < 32; d += 8) {
             if (wide) {
@@ -547,7 +596,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
           }
         }
       }
-      if (g == 1 && pos < L) {
+      if (!direct && valid) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(staged), "r"(kD * 4) : "memory");
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -573,14 +622,14 @@ size_t prefill_scratch_bytes(int B, int Hkv, int L) {
 cudaError_t launch_prefill_attention(const void* q, const void* k, const void* v, float* out, void* scratch, int B, int Hq,
                                      int Hkv, int L, float scale, uint32_t* status, uint32_t max_polls, uint32_t debug_extra_tx,
                                      uint32_t debug_extra_v, cudaStream_t stream) {
-  const int n_tiles = (L + kTile - 1) / kTile, n_qtiles = (L + kQRows - 1) / kQRows;
+  const int g = Hq / Hkv, n_tiles = (L + kTile - 1) / kTile, n_qtiles = (int)(((long long)L * g + kQRows - 1) / kQRows);
   unsigned char* kt = static_cast<unsigned char*>(scratch);
   unsigned char* vt = kt + (size_t)B * Hkv * n_tiles * kTileBytes;
   const cudaError_t e = launch_dependent(prefill_pack_kernel, dim3((unsigned)n_tiles, (unsigned)(B * Hkv)), 256, 0, stream,
                                          static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), kt, vt, L, n_tiles);
   if (e != cudaSuccess) return e;
-  return launch_dependent(prefill_attention_kernel, dim3((unsigned)(n_qtiles * B * Hq)), kThreads, kSmem, stream,
-                          static_cast<const __nv_bfloat16*>(q), kt, vt, out, B * Hq, Hq, Hkv, L, n_tiles, n_qtiles,
+  return launch_dependent(prefill_attention_kernel, dim3((unsigned)(n_qtiles * B * Hkv)), kThreads, kSmem, stream,
+                          static_cast<const __nv_bfloat16*>(q), kt, vt, out, B * Hkv, g, L, n_tiles, n_qtiles,
                           scale * 1.4426950408889634f, status, max_polls ? max_polls : kPolls, debug_extra_tx, debug_extra_v);
 }
 

@@ -41,6 +41,23 @@ def test_prefill_attention_and_cache(binding, name, batch, tokens):
     U.compare_regions(cache, 0, w, U.oracle_streams(w, 0, k, v, q, streams=list(set(streams))))
 
 
+@pytest.mark.parametrize("g", [1, 2, 3, 4, 5, 7, 8])
+@pytest.mark.parametrize("tokens", [17, 64, 130, 256, 387])
+def test_prefill_rows_of_every_group_size(binding, g, tokens):
+    """A row tile holds the g heads of neighbouring tokens: groups that end at a key tile's edge or before it, a second group without
+    rows, and rows past the prompt, for every g.  Two streams per batch element, so that a row in the wrong place shows."""
+    gen = torch.Generator().manual_seed(100 * g + tokens)
+    k, v, q = (torch.randn((2, h, tokens, 128), generator=gen).to(torch.bfloat16) for h in (2, 2, 2 * g))
+    cache = binding.Cache(binding.make_config(1, 2, 2 * g, 2, tokens, **W.P24))
+    out = torch.full((2, 2 * g, tokens, 128), 7.0, device="cuda")
+    cache.prefill(0, k.cuda(), v.cuda(), q.cuda(), W.softmax_scale(), out=out)
+    assert cache.status() == 0
+    qf, kf, vf = (t.double() for t in (q, k.repeat_interleave(g, 1), v.repeat_interleave(g, 1)))
+    s = (qf @ kf.transpose(-1, -2)) * W.softmax_scale()
+    s.masked_fill_(torch.ones(tokens, tokens).triu(1).bool(), float("-inf"))
+    assert float((out.cpu() - torch.softmax(s, -1) @ vf).abs().max()) <= ATTN_TOL
+
+
 def test_prefill_large_magnitudes_and_errors(binding):
     w = W.small(W.CONFIGS["qwen7b"], n_layers=1, batch=1, tokens=300)
     k, v, q = W.tokens(w, 0, 0, 300)
