@@ -148,8 +148,8 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
   // running.  Nothing above touches global memory.  dep_wait() waits for that kernel's results and lets the kernel after
   // this one be started early in the same way; every thread calls it before its first access to global memory, with one
   // exception: when the host knows that the kernel before this one did not write this layer's packed blocks
-  // (stage_early), the first staged copies of the packed units go out before the wait.  That is safe because a kernel
-  // of this library triggers its successor only after its own wait, so that everything two launches back is complete.
+  // (stage_early), the first staged copies of the packed units go out before the wait.  That is safe because what may
+  // still be running then besides that kernel is the split kernel before it, if it is a merge (see common.cuh).
   bool dep_waited = false;
   auto dep_wait = [&]() {
     if (!dep_waited) {

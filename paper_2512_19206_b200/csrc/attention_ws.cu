@@ -38,7 +38,7 @@ namespace mixkvq {
 
 cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, int mode, int n,
                            long long units_per_stream, int S, cudaStream_t stream, const int4* seq = nullptr,
-                           const int* seq_prefix = nullptr, float* lse_out = nullptr);
+                           const int* seq_prefix = nullptr, float* lse_out = nullptr, bool early = false);
 // the same split, one unit at a time (attention_single.cu)
 cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse,
                                     cudaStream_t stream);
@@ -181,8 +181,8 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   // running.  Nothing above touches global memory.  dep_wait() waits for that kernel's results and lets the kernel after
   // this one be started early in the same way; every thread calls it before its first access to global memory, with one
   // exception: when the host knows that the kernel before this one did not write this layer's packed blocks
-  // (stage_early), the first staged copies of the packed units go out before the wait.  That is safe because a kernel
-  // of this library triggers its successor only after its own wait, so that everything two launches back is complete.
+  // (stage_early), the first staged copies of the packed units go out before the wait.  That is safe because what may
+  // still be running then besides that kernel is the split kernel before it, if it is a merge (see common.cuh).
   bool dep_waited = false;
   auto dep_wait = [&]() {
     if (!dep_waited) {
@@ -1302,7 +1302,12 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   else e = launch_g<128>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
   *launches = 1;
   if (e != cudaSuccess || out == nullptr || whole) return e;     // out == nullptr: split kernel only (timing)
-  e = launch_combine(ws, out, lv.g, lv.Hkv, lv.Hq, 1, grid, Us, S, stream, lv.seq, lv.seq_prefix, lse_out);
+  // The merge lets the next kernel start early (combine.cu) where the CTAs have enough to do that they finish one by one.  us per layer,
+  // not early / early, 32 streams (288 CTAs), two tiers 1000 tokens 8.0 / 8.2, 6000 (22 positions per CTA) 14.15 / 14.15, 14000 22.8 / 21.8, three
+  // tiers 1000 10.2 / 10.8, 4000 (16) 13.1 / 13.2, 14000 26.6 / 26.2; 64 streams, two tiers 2500 (22) 14.3 / 13.0, 4-bit values 1000 (10) 9.5 / 13.7,
+  // 1500 (14) 12.0 / 13.8, 2500 15.9 / 14.8; 128 streams, 1500 (28) 15.4 / 14.1.
+  const bool early = grid > n_sms && (lv.seq != nullptr ? lv.seq_total : Us * S) >= 20ll * grid;
+  e = launch_combine(ws, out, lv.g, lv.Hkv, lv.Hq, 1, grid, Us, S, stream, lv.seq, lv.seq_prefix, lse_out, early);
   *launches = 2;
   return e;
 }

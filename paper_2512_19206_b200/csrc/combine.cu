@@ -13,15 +13,22 @@ namespace mixkvq {
 // shared memory.  B200, attention + merge per layer from a graph: one sequence of 4000 tokens (74 partials) 17.2 us with
 // one thread per channel walking chunks of 12, 9.6 us so; 8 sequences of 32768 tokens (9 partials) 41.7 and
 // 40.4 us.
+// The kernel behind a merge is let go before the merge waits for its split kernel: the next layer's split kernel then takes the places of
+// this one's CTAs as they finish, and its set-up and first copies run under their tail (28 layers of the 7b shape, 32768 tokens
+// x 8: 1138 -> 1104 us per decode step).  What is still running when that kernel starts are this merge and the split kernel before it, which
+// write partials, outputs, residual windows and accumulators, no packed block; its wait covers both, the merge's own included.  Not with
+// little work per CTA or one CTA per SM (`early` = false; the rule is at the launch): the next CTAs are then placed around those still
+// there, two on some SMs and none on others.
 constexpr int kCombineChunk = 8;
 constexpr int kCombineMaxWarps = 8;
 
 __global__ void __launch_bounds__(kCombineMaxWarps * 32)
 combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int Hkv, int Hq, int mode, int n,
                long long units_per_stream, int S, const int4* __restrict__ seq, const int* __restrict__ seq_prefix,
-               float* __restrict__ lse_out) {
+               float* __restrict__ lse_out, bool early) {
   __shared__ float mlS[kCombineMaxWarps][2];
   __shared__ __align__(16) float oS[kCombineMaxWarps][kD];
+  if (early) let_successor_start();
   const int s = blockIdx.x / g, h = blockIdx.x % g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = blockDim.x >> 5;
   int first, count;
@@ -110,7 +117,8 @@ constexpr int kRowsChunk = 8, kRowsMaxPartials = 8;
 
 __global__ void __launch_bounds__(256)
 combine_rows_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int Hkv, int Hq, int n, long long units_per_stream,
-                    int S, float* __restrict__ lse_out) {
+                    int S, float* __restrict__ lse_out, bool early) {
+  if (early) let_successor_start();
   const int s = blockIdx.x, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long total = units_per_stream * S;
   const long long x0 = units_per_stream * s, x1 = units_per_stream * (s + 1) - 1;
@@ -156,14 +164,14 @@ combine_rows_kernel(const float* __restrict__ ws, float* __restrict__ out, int g
 
 cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, int mode, int n,
                            long long units_per_stream, int S, cudaStream_t stream, const int4* seq, const int* seq_prefix,
-                           float* lse_out) {
+                           float* lse_out, bool early) {
   if (mode == 1 && seq == nullptr && n / S + 2 <= kRowsMaxPartials)
-    return launch_dependent(combine_rows_kernel, dim3((unsigned)S), 32 * g, 0, stream, ws, out, g, Hkv, Hq, n, units_per_stream, S, lse_out);
+    return launch_dependent(combine_rows_kernel, dim3((unsigned)S), 32 * g, 0, stream, ws, out, g, Hkv, Hq, n, units_per_stream, S, lse_out, early);
   // eight warps when four with a chunk each do not cover a stream's partials in one round trip (a ragged batch may give
   // nearly all CTAs to one sequence), four otherwise: more warps only lengthen the last step
   const int partials = mode == 0 ? n : (seq != nullptr ? n : n / S + 1);
   return launch_dependent(combine_kernel, dim3((unsigned)(S * g)), partials > 4 * kCombineChunk ? kCombineMaxWarps * 32 : 128, 0, stream,
-                          ws, out, g, Hkv, Hq, mode, n, units_per_stream, S, seq, seq_prefix, lse_out);
+                          ws, out, g, Hkv, Hq, mode, n, units_per_stream, S, seq, seq_prefix, lse_out, early);
 }
 
 // The table of a ragged batch, from the host's per-sequence fill (kernel arguments: no copy, ordered in the stream).

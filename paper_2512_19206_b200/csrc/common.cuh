@@ -170,12 +170,14 @@ __host__ __device__ inline void hi_plane_pos(int jj, int e, int* word, int* bit)
 
 // ---- Programmatic dependent launch.  A kernel launched with launch_dependent may be started while the kernel before it in
 // the stream is still running: its launch and set-up overlap that kernel's tail.  It calls dependency_wait() before it touches
-// anything an earlier kernel may write or still read, and that call also lets the kernel behind it be started early.  Since no
-// kernel of this library lets its successor start before its own wait, everything two launches back is complete when a
-// kernel starts.
+// anything an earlier kernel may write or still read, and that call also lets the kernel behind it be started early.  Only the merge of
+// split partials lets its successor start before its own wait (let_successor_start); the kernel before a merge is always the split
+// kernel, which does not.  So when a kernel starts, everything is complete but the launch before it and, if that is a merge, the split
+// kernel before the merge.
+__device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dependency_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_successor_start();
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
