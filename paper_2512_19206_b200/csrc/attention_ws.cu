@@ -1247,9 +1247,12 @@ static bool one_cta_per_stream(const LayerView& lv, int n_sms) {
   return p <= (plain ? 20 : 12) || (p <= 20 && p * lv.B * lv.Hkv > 4 * n_sms);
 }
 
-// Number of CTAs the split kernel runs for this layer state (also the number of partial-slot owners).  When there are
-// fewer streams than CTA slots the grid is a multiple of the stream count, so that no CTA straddles two streams
-// (a second segment costs a pipeline drain, a query load and a second partial).
+// Number of CTAs the split kernel runs for this layer state (also the number of partial-slot owners).  With fewer streams than CTA slots
+// a grid that is a multiple of the stream count has no CTA that straddles two streams: a second segment costs a pipeline drain, a
+// query load and a second partial, about 10 positions' time with two tiers and 16 otherwise.  Where that leaves more of the slots idle than
+// the straddling costs, all of them are used.  us per layer, multiple / all slots: 8b shape, batch 16 (128 streams: 256 / 296 CTAs), 4-bit base,
+// 16384 tokens 105.4 / 98.4; 32 streams (288 / 296 CTAs), two tiers, 32768 tokens 39.4 / 40.8, three tiers, 20011 tokens 37.7 / 40.9, 16
+// streams, 120000 tokens 68.5 / 69.0.
 int attention_ws_grid(const LayerView& lv, int n_sms) {
   const int S = lv.B * lv.Hkv;
   if (lv.seq != nullptr) return lv.seq_ctas;
@@ -1260,7 +1263,10 @@ int attention_ws_grid(const LayerView& lv, int n_sms) {
   const long long wanted = min((total + 1) / 2, max((long long)n_sms, (total + 3) / 4));
   int grid = (int)min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), wanted);
   if (one_cta_per_stream(lv, n_sms)) grid = min(grid, S);
-  if (grid > S) grid = grid / S * S;
+  if (grid > S) {
+    const int per_stream = grid / S, straddle = three_tiers(lv) || lv.dense_hi ? 16 : 10;
+    if ((attention_ws_positions(lv) + per_stream - 1) / per_stream <= (total + grid - 1) / grid + straddle) grid = per_stream * S;
+  }
   return grid < 1 ? 1 : grid;
 }
 

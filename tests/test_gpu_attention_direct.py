@@ -40,3 +40,17 @@ def test_direct_output(binding, name, batch, tokens, R, preset):
     ref = cache.decode_attention(0, q, W.softmax_scale())
     assert cache.status() == 0
     assert float((out - ref).abs().max()) <= TOL
+
+
+@pytest.mark.parametrize("batch,tokens,preset", [(9, 3000, "P24"), (12, 4000, "P27"), (16, 4000, "P4BASE"), (18, 2000, "P24")])
+def test_split_that_straddles_streams(binding, batch, tokens, preset):
+    """Stream counts that leave many CTA slots idle at a whole number of CTAs per stream: all slots are used and CTAs straddle streams."""
+    w = W.small(W.CONFIGS["llama8b"], n_layers=1, batch=batch, tokens=tokens, **getattr(W, preset))
+    cache = U.make_cache(binding, w, extras_budget_bytes=(tokens // 128 + 3) * 128 * 64)
+    cache.quantize_append(0, *W.tokens(w, 0, 0, tokens, device="cuda"))
+    q = W.decode_query(w, 0, 0, device="cuda")
+    out = cache.decode_attention(0, q, W.softmax_scale())
+    cache.set_attention_kernel(1)
+    ref = cache.decode_attention(0, q, W.softmax_scale())
+    assert cache.status() == 0
+    assert float((out - ref).abs().max()) <= TOL
