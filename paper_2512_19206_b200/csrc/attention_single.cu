@@ -27,9 +27,9 @@ namespace mixkvq {
 
 namespace {
 
-constexpr int kPairs = 4;                    // warp pairs per CTA
-constexpr int kThreads = kPairs * 64;
-constexpr int kCtasPerSm = 2;
+// Warp pairs per CTA: four, two CTAs per SM; eight and one CTA per SM where a short stream has a CTA of its own and there is an SM for each
+// (the dispatch rule is in attention_ws.cu): every pair's chain of units, one after the other, is then half as long.
+constexpr int kPairsPerSm = 8;
 constexpr int kStages = 4;                   // ring stages per pair (a power of two)
 // one ring stage: a key-meta group (512 B) followed by the unit (<= 2560 B; <= 3584 B with 4-bit values), as in the block
 __host__ __device__ constexpr int stage_bytes(bool v4) { return v4 ? 4096 : 3072; }
@@ -46,10 +46,11 @@ __host__ __device__ constexpr int pair_bytes(bool v4) {
 // mbarriers of a pair: staged copy landed [kStages], logits ready [kStages], then for unquantized units: ready, taken
 constexpr int kBarsPerPair = 2 * kStages + 2;
 constexpr int kQS = 136;                     // halves per row of the query tables (272 bytes: rows fall on different banks)
-constexpr int kBarBytes = ((kPairs * kBarsPerPair * 8 + 127) / 128) * 128;
+__host__ __device__ constexpr int bar_bytes(int pairs) { return ((pairs * kBarsPerPair * 8 + 127) / 128) * 128; }
 constexpr int kPrefixBytes = ((kMaxRaggedBatch + 1) * 4 + 15) / 16 * 16;     // a ragged batch's prefix sums
-constexpr int kSharedTail = kBarBytes + 2 * 8 * kQS * 2 + 2 * kPairs * 32 + kPrefixBytes;
-__host__ __device__ constexpr int smem_bytes(bool v4) { return kPairs * pair_bytes(v4) + kSharedTail; }
+__host__ __device__ constexpr int smem_bytes(bool v4, int pairs) {
+  return pairs * (pair_bytes(v4) + 64) + bar_bytes(pairs) + 2 * 8 * kQS * 2 + kPrefixBytes;
+}
 constexpr int kResidualWeight = 3;           // an unquantized 32-token unit counts as this many packed units in the split
 constexpr int kMergeStride = 132;            // floats per head row of a pair's output in the merge
 // With three tiers and with a 4-bit base the logits warp is by far the longer role (further tiles for the UINT4 high
@@ -89,10 +90,11 @@ __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp
 // per channel pair, gathered), 2 = 4-bit base (dense high plane)
 // kV4: 4-bit values (a second plane of 2-bit value codes per unit, scale 4 s_v)
 // kDirect: one CTA per stream, which writes the output (and the log-denominators) instead of a partial
-template <int G, int kU4, bool kV4, bool kDirect>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+template <int G, int kU4, bool kV4, bool kDirect, int kPairs>
+__global__ void __launch_bounds__(kPairs * 64, kPairsPerSm / kPairs)
 attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float scale_log2e, float* __restrict__ ws,
                     uint32_t four2, float* __restrict__ out, float* __restrict__ lse_out) {
+  constexpr int kThreads = kPairs * 64, kBarBytes = bar_bytes(kPairs);
   constexpr int VG = kD / G;              // value groups per token
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group
   constexpr int kStageBytes = stage_bytes(kV4);
@@ -1168,47 +1170,48 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
   }
 }
 
-template <int G, int kU4, bool kV4, bool kDirect>
+template <int G, int kU4, bool kV4, bool kDirect, int kPairs>
 cudaError_t launch_d(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
-  return launch_dependent(attention_single_kernel<G, kU4, kV4, kDirect>, dim3((unsigned)grid), kThreads, smem_bytes(kV4), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
+  return launch_dependent(attention_single_kernel<G, kU4, kV4, kDirect, kPairs>, dim3((unsigned)grid), kPairs * 64, smem_bytes(kV4, kPairs), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
 }
 template <int G, int kU4, bool kV4>
-cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
-  return out != nullptr ? launch_d<G, kU4, kV4, true>(lv, qb, sl, ws, grid, out, lse, stream)
-                        : launch_d<G, kU4, kV4, false>(lv, qb, sl, ws, grid, out, lse, stream);
+cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, bool wide, cudaStream_t stream) {
+  if (out == nullptr) return launch_d<G, kU4, kV4, false, 4>(lv, qb, sl, ws, grid, out, lse, stream);
+  return wide ? launch_d<G, kU4, kV4, true, 8>(lv, qb, sl, ws, grid, out, lse, stream) : launch_d<G, kU4, kV4, true, 4>(lv, qb, sl, ws, grid, out, lse, stream);
 }
 template <int G, int kU4>
-cudaError_t launch_one(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
-  return lv.v_bits == 4 ? launch_v<G, kU4, true>(lv, qb, sl, ws, grid, out, lse, stream)
-                        : launch_v<G, kU4, false>(lv, qb, sl, ws, grid, out, lse, stream);
+cudaError_t launch_one(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, bool wide, cudaStream_t stream) {
+  return lv.v_bits == 4 ? launch_v<G, kU4, true>(lv, qb, sl, ws, grid, out, lse, wide, stream)
+                        : launch_v<G, kU4, false>(lv, qb, sl, ws, grid, out, lse, wide, stream);
 }
 
 template <int G>
-cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse,
+cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse, bool wide,
                      cudaStream_t stream) {
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   const float sl = scale * 1.4426950408889634f;
-  if (lv.dense_hi) return launch_one<G, 2>(lv, qb, sl, ws, grid, out, lse, stream);
+  if (lv.dense_hi) return launch_one<G, 2>(lv, qb, sl, ws, grid, out, lse, wide, stream);
   const bool uses_u4 = (lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16;
-  if (uses_u4) return launch_one<G, 1>(lv, qb, sl, ws, grid, out, lse, stream);
-  return launch_one<G, 0>(lv, qb, sl, ws, grid, out, lse, stream);
+  if (uses_u4) return launch_one<G, 1>(lv, qb, sl, ws, grid, out, lse, wide, stream);
+  return launch_one<G, 0>(lv, qb, sl, ws, grid, out, lse, wide, stream);
 }
 
 }  // namespace
 
-template <int G, int kU4, bool kV4, bool kDirect>
+template <int G, int kU4, bool kV4, bool kDirect, int kPairs>
 static cudaError_t setup_d() {
-  cudaError_t e = cudaFuncSetAttribute(attention_single_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem_bytes(kV4));
+  cudaError_t e = cudaFuncSetAttribute(attention_single_kernel<G, kU4, kV4, kDirect, kPairs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem_bytes(kV4, kPairs));
   if (e != cudaSuccess) return e;
   // the CTAs of an SM only fit with the largest shared-memory carve-out; ask for it explicitly
-  return cudaFuncSetAttribute(attention_single_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  return cudaFuncSetAttribute(attention_single_kernel<G, kU4, kV4, kDirect, kPairs>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               (int)cudaSharedmemCarveoutMaxShared);
 }
 template <int G, int kU4, bool kV4>
 static cudaError_t setup_v() {
-  cudaError_t e = setup_d<G, kU4, kV4, false>();
-  return e != cudaSuccess ? e : setup_d<G, kU4, kV4, true>();
+  cudaError_t e = setup_d<G, kU4, kV4, false, 4>();
+  if (e == cudaSuccess) e = setup_d<G, kU4, kV4, true, 4>();
+  return e == cudaSuccess ? setup_d<G, kU4, kV4, true, 8>() : e;
 }
 template <int G, int kU4>
 static cudaError_t setup_one() {
@@ -1231,11 +1234,11 @@ cudaError_t attention_single_setup() {
   return setup_g<128>();
 }
 
-cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse,
+cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse, bool wide,
                                     cudaStream_t stream) {
-  if (lv.G == 32) return launch_g<32>(lv, q, scale, ws, grid, out, lse, stream);
-  if (lv.G == 64) return launch_g<64>(lv, q, scale, ws, grid, out, lse, stream);
-  return launch_g<128>(lv, q, scale, ws, grid, out, lse, stream);
+  if (lv.G == 32) return launch_g<32>(lv, q, scale, ws, grid, out, lse, wide, stream);
+  if (lv.G == 64) return launch_g<64>(lv, q, scale, ws, grid, out, lse, wide, stream);
+  return launch_g<128>(lv, q, scale, ws, grid, out, lse, wide, stream);
 }
 
 }  // namespace mixkvq

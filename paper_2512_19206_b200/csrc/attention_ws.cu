@@ -40,7 +40,7 @@ cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, 
                            long long units_per_stream, int S, cudaStream_t stream, const int4* seq = nullptr,
                            const int* seq_prefix = nullptr, float* lse_out = nullptr, bool early = false);
 // the same split, one unit at a time (attention_single.cu)
-cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse,
+cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse, bool wide,
                                     cudaStream_t stream);
 cudaError_t attention_single_setup();
 
@@ -1236,15 +1236,22 @@ static bool three_tiers(const LayerView& lv) {
   return !lv.dense_hi && ((lv.budget_bf16 + lv.budget_u4 > 0) ? lv.budget_u4 > 0 : lv.tau_u4 < lv.tau_bf16);
 }
 
-// A few positions per team: one CTA per stream, which needs no merge.  With two tiers and 2-bit values it is never slower than the
-// split up to 20 positions (us per layer, one CTA per stream / split, 300 tokens: one sequence 5.4 / 5.3, eight 5.5 / 5.8, 16 of the 8b
-// shape 6.4 / 7.9; 600 tokens, 25 positions, one sequence 6.8 / 5.7).  Otherwise a unit takes longer, and beyond 12 positions
-// the split is faster as long as it gets by with one CTA per SM (three tiers, 300 and 390 tokens, one sequence 6.5 / 5.8, 64 streams
-// 6.9 / 8.8; 4-bit base 6.6 / 5.7, 6.8 / 8.6; 4-bit values 6.2 / 5.5, 6.3 / 7.9; three tiers with 4-bit values 7.1 / 5.9, 7.6 / 9.2).
+// A few positions per team: one CTA per stream, which needs no merge.
+// Where every stream has an SM to itself (eight pairs of warps) it is the faster up to a number of positions that grows with the
+// streams, as their split gets the less out of the rest of the SMs.  us per layer, one CTA per stream / split: two tiers, 16 streams, 24 positions
+// 5.96 / 6.02, 28 6.63 / 6.48, 64 streams, 40 8.85 / 9.05, 42 10.3 / 9.6, 128 streams, 42 11.7 / 13.1; three tiers, 4 streams, 14 positions 6.34 / 6.67,
+// 18 7.5 / 6.7, 64 streams, 28 9.25 / 10.8, 32 10.3 / 10.1, 128 streams, 40 14.1 / 14.3, 42 15.8 / 15.5; 4-bit base, 4 streams, 14 5.75 / 5.87, 18 6.8 / 5.9,
+// 128 streams, 40 13.0 / 14.6; 4-bit values, 16 streams, 18 6.1 / 6.7, 32 streams, 28 7.1 / 7.5, 32 8.1 / 7.5.
+// With more streams (four pairs, two CTAs per SM): never slower than the split up to 20 positions with two tiers and 2-bit values
+// (one CTA per stream / split, 16 streams of the 8b shape 6.4 / 7.9); otherwise a unit takes longer, and beyond 12 positions
+// the split is faster as long as it gets by with one CTA per SM (64 streams, 390 tokens, three tiers 6.9 / 8.8; 4-bit base
+// 6.8 / 8.6; 4-bit values 6.3 / 7.9; three tiers with 4-bit values 7.6 / 9.2).
 static bool one_cta_per_stream(const LayerView& lv, int n_sms) {
   const long long p = attention_ws_positions(lv);
+  const int S = lv.B * lv.Hkv;
   const bool plain = !lv.dense_hi && !three_tiers(lv) && lv.v_bits == 2;
-  return p <= (plain ? 20 : 12) || (p <= 20 && p * lv.B * lv.Hkv > 4 * n_sms);
+  if (S <= n_sms) return p <= (plain ? min(20 + S / 5, 42) : min(13 + S / 4, 40));
+  return p <= (plain ? 20 : 12) || (p <= 20 && p * S > 4 * n_sms);
 }
 
 // Number of CTAs the split kernel runs for this layer state (also the number of partial-slot owners).  With fewer streams than CTA slots
@@ -1300,9 +1307,13 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // tokens 7.3 us against 5.6; 7b shape 41.1 against 40.7).
   const bool whole = out != nullptr && lv.seq == nullptr && grid == S;
   float* const kernel_out = whole ? out : nullptr;
+  // ... with eight pairs of warps where every stream has an SM to itself.  us per layer, four / eight pairs: 4 streams of the 7b shape, two
+  // tiers, 300 tokens 5.5 / 5.1; 64 streams, three tiers 7.7 / 6.7, 4-bit base 7.4 / 6.1, 128 streams of the 8b shape, 400 tokens 9.1 / 7.8.  Only
+  // with few positions and most of the SMs in use the larger CTAs cost more: 128 streams, 200 tokens (13 positions) 7.7 / 8.05.
+  const bool wide = whole && grid <= n_sms && (Us > 13 || 2 * grid <= n_sms);
   if (form) *form = (by_two ? MIXKVQ_ATTN_TWO_UNITS : MIXKVQ_ATTN_ONE_UNIT) | (whole ? MIXKVQ_ATTN_DIRECT : 0) | (lv.stage_early ? MIXKVQ_ATTN_EARLY : 0);
   cudaError_t e;
-  if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
+  if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, kernel_out, lse_out, wide, stream);
   else if (lv.G == 32) e = launch_g<32>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
   else if (lv.G == 64) e = launch_g<64>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);
   else e = launch_g<128>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);

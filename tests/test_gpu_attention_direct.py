@@ -42,6 +42,32 @@ def test_direct_output(binding, name, batch, tokens, R, preset):
     assert float((out - ref).abs().max()) <= TOL
 
 
+@pytest.mark.parametrize("name,batch,tokens,preset,v_bits,form", [
+    ("qwen7b", 1, 200, "P27", 4, 1 + 4), ("llama8b", 1, 450, "P24", 2, 1 + 4), ("llama8b", 1, 560, "P24", 2, 1), ("qwen7b", 16, 511, "P4BASE", 2, 1 + 4),
+    ("qwen7b", 16, 1152, "P27", 2, 2), ("llama8b", 16, 1000, "P24", 4, 1 + 4), ("llama8b", 18, 200, "P24", 2, 1 + 4), ("llama8b", 19, 700, "P27", 2, 2 + 4),
+])
+def test_eight_pairs_per_stream(binding, name, batch, tokens, preset, v_bits, form):
+    """One CTA of eight warp pairs per stream while every stream has an SM to itself, on both sides of where that ends (148 SMs: 18
+    sequences of the 8b shape) and of the positions up to which it is chosen: more units than pairs, fewer, pairs without a unit; a fused
+    step across a flush leaves the same bytes as append and attention."""
+    w = W.small(W.CONFIGS[name], n_layers=1, batch=batch, tokens=tokens, **getattr(W, preset))
+    caches = [U.make_cache(binding, w, v_bits=v_bits, sink_len=32 if batch == 18 else 0, extras_budget_bytes=(tokens // 128 + 4) * 128 * 128) for _ in range(2)]
+    for c in caches:
+        c.quantize_append(0, *W.tokens(w, 0, 0, tokens, device="cuda"))
+    k, v, q = [x.contiguous() for x in W.tokens(w, 0, tokens, 1, device="cuda")]
+    out = caches[0].decode_step(0, k, v, q, W.softmax_scale())
+    assert caches[0].last_attention() & 7 == form
+    caches[1].quantize_append(0, k, v, q)
+    plain, lse = caches[1].decode_attention_partial(0, q[:, :, 0].contiguous(), W.softmax_scale())
+    assert torch.equal(out, plain) and bool(torch.isfinite(lse).all())
+    for s in (0, batch * w.n_kv_heads - 1):
+        assert caches[0].stream_regions(0, s) == caches[1].stream_regions(0, s)
+    caches[1].set_attention_kernel(1)
+    ref = caches[1].decode_attention(0, q[:, :, 0].contiguous(), W.softmax_scale())
+    assert caches[0].status() == caches[1].status() == 0
+    assert float((out - ref).abs().max()) <= TOL
+
+
 @pytest.mark.parametrize("batch,tokens,preset", [(9, 3000, "P24"), (12, 4000, "P27"), (16, 4000, "P4BASE"), (18, 2000, "P24")])
 def test_split_that_straddles_streams(binding, batch, tokens, preset):
     """Stream counts that leave many CTA slots idle at a whole number of CTAs per stream: all slots are used and CTAs straddle streams."""
