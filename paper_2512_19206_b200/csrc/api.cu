@@ -225,8 +225,11 @@ int upload_seq_table(mixkvq_cache* h, int layer, cudaStream_t st, LayerView* lv)
 
 // Picks the decode-attention kernel for the layer's layout and the selected kind, enqueues it and counts its launches.
 int run_attention(mixkvq_cache* h, int layer, const void* q, float* out, float scale, float* ws, cudaStream_t st,
-                  const void* new_k = nullptr, const void* new_v = nullptr, float* lse = nullptr) {
+                  const void* new_k = nullptr, const void* new_v = nullptr, float* lse = nullptr, const float* rope_cos = nullptr,
+                  const float* rope_sin = nullptr) {
   LayerView lv = view(h, layer);
+  lv.rope_cos = rope_cos;
+  lv.rope_sin = rope_sin;
   lv.new_k = static_cast<const uint16_t*>(new_k);
   lv.new_v = static_cast<const uint16_t*>(new_v);
   lv.stage_early = (st == h->last_stream && (h->last_packed_writer == kNoPackedWrite ||
@@ -319,6 +322,59 @@ int append_run(mixkvq_cache* cache, int layer, int b0, int nb, const void* k_dev
     cache->r[fi(cache, layer, b)] = cache->r[fi(cache, layer, b0)];
     cache->n_blocks[fi(cache, layer, b)] = cache->n_blocks[fi(cache, layer, b0)];
   }
+  return rc;
+}
+
+// A decode step whose arguments have been checked.  rope_cos / rope_sin: the position's rows of the tables (null: no rotation); the
+// split kernel rotates what it reads and the call's last kernel leaves the rotated rows in the caller's tensors, so that the rotation is
+// no launch in front of the step.
+int run_decode_step(mixkvq_cache* cache, int layer, const void* k_dev, const void* v_dev, const void* q_dev, float* out_dev, float softmax_scale,
+                    void* workspace_dev, cudaStream_t st, const float* rope_cos = nullptr, const float* rope_sin = nullptr) {
+  const int B = cache->cfg.batch;
+  bool sink_room = false;
+  for (int b = 0; b < B; ++b) sink_room = sink_room || cache->n_sink[fi(cache, layer, b)] < cache->cfg.sink_len;
+  const bool apart = cache->attn_kind != 0 || sink_room;
+  if (rope_cos != nullptr && (apart || cache->tile)) {
+    // the rotation is a launch of its own (its tables' rows are those of the position, and there is one token)
+    if (launch_rope(const_cast<void*>(k_dev), const_cast<void*>(q_dev), rope_cos, rope_sin, B, cache->cfg.n_kv_heads, cache->cfg.n_q_heads, 1, 0, st) !=
+        cudaSuccess)
+      return MIXKVQ_E_CUDA;
+    cache->launches += 1;
+    note_enqueued(cache, st, kNoPackedWrite);
+    rope_cos = rope_sin = nullptr;
+  }
+  if (apart) {
+    // the comparison kernels do not take the new token themselves, and a sink token is not a residual token:
+    // plain append, then attention
+    int rc = mixkvq_quantize_append(cache, layer, k_dev, v_dev, q_dev, 1, st);
+    if (rc != MIXKVQ_OK) return rc;
+    return run_attention(cache, layer, q_dev, out_dev, softmax_scale, static_cast<float*>(workspace_dev), st);
+  }
+  // full windows are flushed first: one launch; in a ragged batch the kernel reads the fills from the layer's table and
+  // only the sequences whose window is full take part
+  bool any_full = false;
+  for (int b = 0; b < B; ++b) any_full = any_full || cache->r[fi(cache, layer, b)] == cache->R;
+  if (any_full) {
+    LayerView lv = view(cache, layer);
+    if (!uniform(cache, layer)) {
+      if (cache->tile) return MIXKVQ_E_UNSUPPORTED;
+      const int rc = upload_seq_table(cache, layer, st, &lv);
+      if (rc != MIXKVQ_OK) return rc;
+    }
+    if (launch_flush(lv, st) != cudaSuccess) return MIXKVQ_E_CUDA;
+    cache->launches += 1;
+    note_enqueued(cache, st, layer);
+    for (int b = 0; b < B; ++b)
+      if (cache->r[fi(cache, layer, b)] == cache->R) {
+        cache->n_blocks[fi(cache, layer, b)] += 1;
+        cache->r[fi(cache, layer, b)] = 0;
+      }
+  }
+  for (int b = 0; b < B; ++b) cache->r[fi(cache, layer, b)] += 1;   // the attention kernel stores the token at slot r - 1 and accumulates |q|
+  const int rc = run_attention(cache, layer, q_dev, out_dev, softmax_scale, static_cast<float*>(workspace_dev), st, k_dev, v_dev, nullptr,
+                               rope_cos, rope_sin);
+  if (rc != MIXKVQ_OK)
+    for (int b = 0; b < B; ++b) cache->r[fi(cache, layer, b)] -= 1;   // nothing was enqueued: the token is not part of the layer
   return rc;
 }
 
@@ -497,42 +553,7 @@ int mixkvq_decode_step(mixkvq_cache* cache, int layer, const void* k_dev, const 
     return MIXKVQ_E_ALIGNMENT;
   if (workspace_bytes_given < workspace_bytes(cache->S)) return MIXKVQ_E_BUFFER_TOO_SMALL;
   if (max_tokens_held(cache, layer) + 1 > cache->cfg.max_tokens) return MIXKVQ_E_CAPACITY;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int B = cache->cfg.batch;
-  bool sink_room = false;
-  for (int b = 0; b < B; ++b) sink_room = sink_room || cache->n_sink[fi(cache, layer, b)] < cache->cfg.sink_len;
-  if (cache->attn_kind != 0 || sink_room) {
-    // the comparison kernels do not take the new token themselves, and a sink token is not a residual token:
-    // plain append, then attention
-    int rc = mixkvq_quantize_append(cache, layer, k_dev, v_dev, q_dev, 1, stream);
-    if (rc != MIXKVQ_OK) return rc;
-    return run_attention(cache, layer, q_dev, out_dev, softmax_scale, static_cast<float*>(workspace_dev), st);
-  }
-  // full windows are flushed first: one launch; in a ragged batch the kernel reads the fills from the layer's table and
-  // only the sequences whose window is full take part
-  bool any_full = false;
-  for (int b = 0; b < B; ++b) any_full = any_full || cache->r[fi(cache, layer, b)] == cache->R;
-  if (any_full) {
-    LayerView lv = view(cache, layer);
-    if (!uniform(cache, layer)) {
-      if (cache->tile) return MIXKVQ_E_UNSUPPORTED;
-      const int rc = upload_seq_table(cache, layer, st, &lv);
-      if (rc != MIXKVQ_OK) return rc;
-    }
-    if (launch_flush(lv, st) != cudaSuccess) return MIXKVQ_E_CUDA;
-    cache->launches += 1;
-    note_enqueued(cache, st, layer);
-    for (int b = 0; b < B; ++b)
-      if (cache->r[fi(cache, layer, b)] == cache->R) {
-        cache->n_blocks[fi(cache, layer, b)] += 1;
-        cache->r[fi(cache, layer, b)] = 0;
-      }
-  }
-  for (int b = 0; b < B; ++b) cache->r[fi(cache, layer, b)] += 1;   // the attention kernel stores the token at slot r - 1 and accumulates |q|
-  const int rc = run_attention(cache, layer, q_dev, out_dev, softmax_scale, static_cast<float*>(workspace_dev), st, k_dev, v_dev);
-  if (rc != MIXKVQ_OK)
-    for (int b = 0; b < B; ++b) cache->r[fi(cache, layer, b)] -= 1;   // nothing was enqueued: the token is not part of the layer
-  return rc;
+  return run_decode_step(cache, layer, k_dev, v_dev, q_dev, out_dev, softmax_scale, workspace_dev, static_cast<cudaStream_t>(stream));
 }
 
 size_t mixkvq_prefill_scratch_bytes(const mixkvq_config* cfg, int n_tokens) {
@@ -588,13 +609,8 @@ int mixkvq_rope_decode_step(mixkvq_cache* cache, int layer, void* k_dev, const v
     return MIXKVQ_E_ALIGNMENT;
   if (workspace_bytes_given < workspace_bytes(cache->S)) return MIXKVQ_E_BUFFER_TOO_SMALL;
   if (max_tokens_held(cache, layer) + 1 > cache->cfg.max_tokens) return MIXKVQ_E_CAPACITY;
-  if (launch_rope(k_dev, q_dev, cos_dev, sin_dev, cache->cfg.batch, cache->cfg.n_kv_heads, cache->cfg.n_q_heads, 1, pos,
-                  static_cast<cudaStream_t>(stream)) != cudaSuccess)
-    return MIXKVQ_E_CUDA;
-  cache->launches += 1;
-  note_enqueued(cache, static_cast<cudaStream_t>(stream), kNoPackedWrite);
-  return mixkvq_decode_step(cache, layer, k_dev, v_dev, q_dev, out_dev, softmax_scale, workspace_dev, workspace_bytes_given,
-                            stream);
+  return run_decode_step(cache, layer, k_dev, v_dev, q_dev, out_dev, softmax_scale, workspace_dev, static_cast<cudaStream_t>(stream),
+                         cos_dev + (size_t)pos * 64, sin_dev + (size_t)pos * 64);
 }
 
 // ---- decode attention with the split partials in storage compiled into the library (no allocation)

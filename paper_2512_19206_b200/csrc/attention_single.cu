@@ -297,12 +297,24 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
     }
     dep_wait();
 
+    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the CTA with its unit stores its key there first,
+    // and the warps that take the unit read its value from the step's tensors, store it and update the importance accumulator
+    const int jn = f_r - 1;
     // ---- query of this stream: bf16 and fp16 tables (heads >= g are zero rows)
     {
-      uint4 q_regs = make_uint4(0u, 0u, 0u, 0u);      // thread (h, c) of the first 128: head h, channels 8c .. 8c+7
+      // thread (h, c) of the first 128: head h, channels 8c .. 8c+7; the next 16 (h = 8): the step's new key
+      uint4 q_regs = make_uint4(0u, 0u, 0u, 0u);
       const int b = s / lv.Hkv, hk = s % lv.Hkv, h = threadIdx.x >> 4, c = threadIdx.x & 15;
-      if (h < g) q_regs = *reinterpret_cast<const uint4*>(q + ((size_t)b * lv.Hq + hk * g + h) * kD + 8 * c);
-      __syncthreads();          // the previous segment's readers of the tables are done
+      const uint4* row = h < g ? reinterpret_cast<const uint4*>(q + ((size_t)b * lv.Hq + hk * g + h) * kD)
+                               : (h == 8 && lv.new_k != nullptr ? reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD) : nullptr);
+      if (row != nullptr) {
+        q_regs = row[c];
+        if (lv.rope_cos != nullptr) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
+      }
+      __syncthreads();          // the previous segment's readers of the tables are done, and so are the rotation's reads
+      if (kDirect && row != nullptr && lv.rope_cos != nullptr) const_cast<uint4*>(row)[c] = q_regs;      // (no other CTA reads them)
+      if (h == 8 && row != nullptr && jn >= 32 * res_b && jn < 32 * res_e)      // this CTA has the new key's unit: it reads the key from the store
+        reinterpret_cast<uint4*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[c] = q_regs;
       if (h < 8) {
         sts128(qb16_u32 + (h * kQS + 8 * c) * 2, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
         if (kU4 == 1)      // the fp16 table is for the gathered UINT4 channels
@@ -314,9 +326,6 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
 
     // unquantized units of this pair: first_res, first_res + kPairs, ... < n_res
     const int first_res = kPairs - 1 - pair;
-    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the pair whose unit holds it
-    // takes its rows from the step's tensors, stores them and updates the importance accumulator
-    const int jn = f_r - 1;
 
     if (logits_role) {
       // =====================================================================================================
@@ -341,8 +350,6 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
           const int ta = j0 + mt * 16 + r, tb = ta + 8;
           const uint4* rowa = reinterpret_cast<const uint4*>(resk + (size_t)ta * 256);
           const uint4* rowb = reinterpret_cast<const uint4*>(resk + (size_t)tb * 256);
-          if (holds_new && ta == jn) rowa = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
-          if (holds_new && tb == jn) rowb = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
           uint4 ka[4], kb[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -679,10 +686,7 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
       // Four channels' sums run side by side.  One sequence of 333 to 433 tokens, decode steps of 8 layers: 7.2 us per step and
       // layer with it before the residual unit's hand-over, a channel after the other; 6.2 here.
       if (takes_new) {
-        // store the new key row and add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads
-        // ascending: the order of the plain append)
-        const uint2 kn = reinterpret_cast<const uint2*>(lv.new_k + (size_t)s * kD)[lane];
-        reinterpret_cast<uint2*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[lane] = kn;
+        // add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads ascending: the order of the plain append)
         double2* acc = reinterpret_cast<double2*>(lv.state + (size_t)s * lv.state_stride) + 2 * lane;
         double2 a0 = acc[0], a1 = acc[1];
         for (int h = 0; h < g; ++h) {

@@ -38,7 +38,8 @@ namespace mixkvq {
 
 cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, int mode, int n,
                            long long units_per_stream, int S, cudaStream_t stream, const int4* seq = nullptr,
-                           const int* seq_prefix = nullptr, float* lse_out = nullptr, bool early = false);
+                           const int* seq_prefix = nullptr, float* lse_out = nullptr, bool early = false, void* rope_q = nullptr, void* rope_k = nullptr,
+                           const float* rope_cos = nullptr, const float* rope_sin = nullptr);
 // the same split, one unit at a time (attention_single.cu)
 cudaError_t launch_attention_single(const LayerView& lv, const void* q, float scale, float* ws, int grid, float* out, float* lse, bool wide,
                                     cudaStream_t stream);
@@ -397,12 +398,24 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     dep_wait();
     if (to_request > 0 && !lv.stage_early) request_first();
 
+    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the CTA with its unit stores its key there first,
+    // and the warps that take the unit read its value from the step's tensors, store it and update the importance accumulator
+    const int jn = f_r - 1;
     // ---- query of this stream: bf16 and fp16 tables (heads >= g are zero rows)
     {
-      uint4 q_regs = make_uint4(0u, 0u, 0u, 0u);      // thread (h, c) of the first 128: head h, channels 8c .. 8c+7
+      // thread (h, c) of the first 128: head h, channels 8c .. 8c+7; the next 16 (h = 8): the step's new key
+      uint4 q_regs = make_uint4(0u, 0u, 0u, 0u);
       const int b = s / lv.Hkv, hk = s % lv.Hkv, h = threadIdx.x >> 4, c = threadIdx.x & 15;
-      if (h < g) q_regs = *reinterpret_cast<const uint4*>(q + ((size_t)b * lv.Hq + hk * g + h) * kD + 8 * c);
-      __syncthreads();          // the previous segment's readers of the tables are done
+      const uint4* row = h < g ? reinterpret_cast<const uint4*>(q + ((size_t)b * lv.Hq + hk * g + h) * kD)
+                               : (h == 8 && lv.new_k != nullptr ? reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD) : nullptr);
+      if (row != nullptr) {
+        q_regs = row[c];
+        if (lv.rope_cos != nullptr) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
+      }
+      __syncthreads();          // the previous segment's readers of the tables are done, and so are the rotation's reads
+      if (kDirect && row != nullptr && lv.rope_cos != nullptr) const_cast<uint4*>(row)[c] = q_regs;      // (no other CTA reads them)
+      if (h == 8 && row != nullptr && jn >= 32 * res_b && jn < 32 * res_e)      // this CTA has the new key's unit: it reads the key from the store
+        reinterpret_cast<uint4*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[c] = q_regs;
       if (h < 8) {
         sts128(qb16_u32 + (h * kQS + 8 * c) * 2, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
         if (kU4 == 1)      // the fp16 table is for the gathered UINT4 channels
@@ -414,9 +427,6 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
 
     // unquantized units of this team: first_res, first_res + kTeams, ... < n_res
     const int first_res = kTeams - 1 - team;
-    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the team whose unit holds it
-    // takes its rows from the step's tensors, stores them and updates the importance accumulator
-    const int jn = f_r - 1;
 
     const uint32_t qrow_u32 = qb16_u32 + r * (kQS * 2), qfrow_u32 = qf16_u32 + r * (kQS * 2);
 
@@ -442,8 +452,6 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
           const int ta = j0 + mt * 16 + r, tb = ta + 8;
           const uint4* rowa = reinterpret_cast<const uint4*>(resk + (size_t)ta * 256);
           const uint4* rowb = reinterpret_cast<const uint4*>(resk + (size_t)tb * 256);
-          if (holds_new && ta == jn) rowa = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
-          if (holds_new && tb == jn) rowb = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
           uint4 ka[4], kb[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -735,10 +743,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       // Four channels' sums run side by side.  Decode steps, 7b shape, batch 8: 32768 tokens, 28 layers 1134.6 -> 1126.0 us;
       // three tiers, 20011 tokens, 14 layers 524.3 -> 517.7.
       if (takes_new) {
-        // store the new key row and add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads
-        // ascending: the order of the plain append)
-        const uint2 kn = reinterpret_cast<const uint2*>(lv.new_k + (size_t)s * kD)[lane];
-        reinterpret_cast<uint2*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[lane] = kn;
+        // add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads ascending: the order of the plain append)
         double2* acc = reinterpret_cast<double2*>(lv.state + (size_t)s * lv.state_stride) + 2 * lane;
         double2 a0 = acc[0], a1 = acc[1];
         for (int h = 0; h < g; ++h) {
@@ -1324,7 +1329,8 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // tiers 1000 10.2 / 10.8, 4000 (16) 13.1 / 13.2, 14000 26.6 / 26.2; 64 streams, two tiers 2500 (22) 14.3 / 13.0, 4-bit values 1000 (10) 9.5 / 13.7,
   // 1500 (14) 12.0 / 13.8, 2500 15.9 / 14.8; 128 streams, 1500 (28) 15.4 / 14.1.
   const bool early = grid > n_sms && (lv.seq != nullptr ? lv.seq_total : Us * S) >= 20ll * grid;
-  e = launch_combine(ws, out, lv.g, lv.Hkv, lv.Hq, 1, grid, Us, S, stream, lv.seq, lv.seq_prefix, lse_out, early);
+  e = launch_combine(ws, out, lv.g, lv.Hkv, lv.Hq, 1, grid, Us, S, stream, lv.seq, lv.seq_prefix, lse_out, early,
+                     lv.rope_cos != nullptr ? const_cast<void*>(q) : nullptr, const_cast<uint16_t*>(lv.new_k), lv.rope_cos, lv.rope_sin);
   *launches = 2;
   return e;
 }

@@ -50,6 +50,10 @@ struct LayerView {
   // The attention kernel then stores them at residual slot r - 1 and adds |q| to the importance accumulator itself.
   const uint16_t* new_k;
   const uint16_t* new_v;
+  // ... with the rotation in front: rows of the position in the caller's cos and sin tables ([64] fp32; null: no rotation).  The split kernel
+  // rotates the query and the new key as it reads them; the last kernel of the call (the merge, or the split kernel where a CTA has a
+  // whole stream) leaves the rotated rows in the caller's tensors.
+  const float *rope_cos, *rope_sin;
   // decode attention may stage its first packed units before it waits for the kernel launched before it: set by the
   // host when that kernel did not write this layer's packed blocks
   int stage_early;
@@ -109,6 +113,35 @@ __device__ inline float stored_scale(float mx, float mn, float levels) {
   uint32_t b = __float_as_uint(q);
   if (b & 0xFFFFu) b = (b + 0x10000u) & 0xFFFF0000u;
   return __uint_as_float(b);
+}
+
+// Rotary embedding of 8 channels of a row (Appendix D: importance scores and keys are taken after the rotation): channel pairing
+// (i, i + 64) ("rotate-half"), with c = cos[p][i], s = sin[p][i] from the caller's tables
+//   y[i] = x[i] c - x[i + 64] s,   y[i + 64] = x[i + 64] c + x[i] s
+// Every product and the sum are single fp32 operations rounded to nearest (no fused multiply-add), and the result is rounded to bf16
+// (nearest, ties to even): the rotated bits are a defined function of the inputs and the tables.  `own` holds channels 8 chunk ..
+// 8 chunk + 7, `other` those 64 away.
+__device__ inline uint4 rotate_chunk(uint4 own, uint4 other, const float* cos_row, const float* sin_row, int chunk) {
+  const float4* cp = reinterpret_cast<const float4*>(cos_row + 8 * (chunk & 7));
+  const float4* sp = reinterpret_cast<const float4*>(sin_row + 8 * (chunk & 7));
+  const float4 c0 = cp[0], c1 = cp[1], s0 = sp[0], s1 = sp[1];
+  const float cs[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+  const float sn[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+  const uint32_t a[4] = {own.x, own.y, own.z, own.w}, b[4] = {other.x, other.y, other.z, other.w};
+  uint32_t y[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float r[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float p = __fmul_rn(bf16_bits_to_float(e ? a[j] >> 16 : a[j] & 0xFFFFu), cs[2 * j + e]);
+      const float m = __fmul_rn(bf16_bits_to_float(e ? b[j] >> 16 : b[j] & 0xFFFFu), sn[2 * j + e]);
+      r[e] = chunk < 8 ? __fsub_rn(p, m) : __fadd_rn(p, m);
+    }
+    const __nv_bfloat162 h = __floats2bfloat162_rn(r[0], r[1]);
+    y[j] = *reinterpret_cast<const uint32_t*>(&h);
+  }
+  return make_uint4(y[0], y[1], y[2], y[3]);
 }
 
 // Code of Eq. 2: round-half-even of the IEEE fp32 quotient (x - z) / s, clamped; 0 when s == 0.

@@ -71,6 +71,34 @@ def test_bulk_then_decode_steps_with_rotation(binding, layout):
     assert cache.status() == 0
 
 
+@pytest.mark.parametrize("name,batch,tokens,preset,lens,sink", [
+    ("qwen7b", 1, 20, "P24", None, 0),                  # the split kernel writes the output itself, eight pairs
+    ("llama8b", 20, 300, "P24", None, 0),               # the same with four pairs
+    ("qwen32b", 32, 1500, "P27", None, 0),              # the same, two units per step
+    ("qwen7b", 1, 1000, "P27", None, 0),                # merge: a CTA per head
+    ("qwen7b", 8, 6000, "P4BASE", None, 0),             # the same, two logits warps
+    ("llama8b", 16, 1700, "P24", None, 0),              # merge: a CTA per stream
+    ("qwen7b", 3, 700, "P24", [700, 128, 5], 0),        # ragged, one window full
+    ("qwen7b", 1, 40, "P24", None, 64),                 # room in the sink: append and attention by themselves
+])
+def test_step_that_rotates_equals_rotation_append_and_attention(binding, name, batch, tokens, preset, lens, sink):
+    w = W.small(W.CONFIGS[name], n_layers=1, batch=batch, tokens=tokens, group_size=32, **getattr(W, preset))
+    cos, sin = [torch.from_numpy(x).cuda() for x in tables(tokens + 8)]
+    caches = [U.make_cache(binding, w, sink_len=sink, extras_budget_bytes=(tokens // 128 + 4) * 128 * 128) for _ in range(2)]
+    kvq = W.tokens(w, 0, 0, tokens, device="cuda")
+    for c in caches:
+        c.quantize_append_ragged(0, *kvq, lens or [tokens] * batch)
+    for step in range(2):
+        a, b = [[x.contiguous().clone() for x in W.tokens(w, 0, tokens + step, 1, device="cuda")] for _ in range(2)]
+        out = caches[0].rope_decode_step(0, *a, cos, sin, tokens + step, W.softmax_scale())
+        caches[1].rope_append(0, *b, cos, sin, tokens + step)
+        assert torch.equal(out, caches[1].decode_attention(0, b[2].view(batch, w.n_q_heads, 128), W.softmax_scale()))
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
+    for s in (0, batch * w.n_kv_heads - 1):
+        assert caches[0].stream_regions(0, s) == caches[1].stream_regions(0, s)
+    assert caches[0].status() == caches[1].status() == 0
+
+
 def test_rotation_errors(binding):
     w = W.small(W.CONFIGS["qwen7b"], n_layers=1, batch=1, tokens=40)
     cos, sin = tables(64)
