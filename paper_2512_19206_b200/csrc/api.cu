@@ -219,7 +219,7 @@ int upload_seq_table(mixkvq_cache* h, int layer, cudaStream_t st, LayerView* lv)
   h->launches += 1;
   lv->seq = seq;
   lv->seq_prefix = prefix;
-  lv->seq_total = total;
+  lv->seq_total = (int)total;
   return MIXKVQ_OK;
 }
 

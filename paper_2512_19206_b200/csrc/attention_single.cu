@@ -49,7 +49,7 @@ constexpr int kQS = 136;                     // halves per row of the query tabl
 __host__ __device__ constexpr int bar_bytes(int pairs) { return ((pairs * kBarsPerPair * 8 + 127) / 128) * 128; }
 constexpr int kPrefixBytes = ((kMaxRaggedBatch + 1) * 4 + 15) / 16 * 16;     // a ragged batch's prefix sums
 __host__ __device__ constexpr int smem_bytes(bool v4, int pairs) {
-  return pairs * (pair_bytes(v4) + 64) + bar_bytes(pairs) + 2 * 8 * kQS * 2 + kPrefixBytes;
+  return pairs * (pair_bytes(v4) + 64) + bar_bytes(pairs) + 2 * 8 * kQS * 2 + kPrefixBytes + 2 * kD;
 }
 constexpr int kResidualWeight = 3;           // an unquantized 32-token unit counts as this many packed units in the split
 constexpr int kMergeStride = 132;            // floats per head row of a pair's output in the merge
@@ -118,6 +118,7 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
   float* mS = reinterpret_cast<float*>(smem + kPairs * kPairBytes + kBarBytes + 2 * 8 * kQS * 2);    // [kPairs][8]
   float* lS = mS + kPairs * 8;                                                                       // [kPairs][8]
   int* prefS = reinterpret_cast<int*>(lS + kPairs * 8);                     // ragged batch: seq_prefix[0 .. B]
+  const uint32_t knew_u32 = smem_u32(prefS) + kPrefixBytes;                 // the step's new key [128], rotated if the step rotates
 
   if (threadIdx.x < kPairs * kBarsPerPair) {
     mbar_init(tail_u32 + 8 * threadIdx.x, 1);
@@ -297,8 +298,8 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
     }
     dep_wait();
 
-    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the CTA with its unit stores its key there first,
-    // and the warps that take the unit read its value from the step's tensors, store it and update the importance accumulator
+    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the warps that take its unit read it from
+    // the step's tensors, store its rows and update the importance accumulator
     const int jn = f_r - 1;
     // ---- query of this stream: bf16 and fp16 tables (heads >= g are zero rows)
     {
@@ -309,12 +310,11 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
                                : (h == 8 && lv.new_k != nullptr ? reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD) : nullptr);
       if (row != nullptr) {
         q_regs = row[c];
-        if (lv.rope_cos != nullptr) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
+        if (__builtin_expect(lv.rope_cos != nullptr, 0)) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
       }
       __syncthreads();          // the previous segment's readers of the tables are done, and so are the rotation's reads
       if (kDirect && row != nullptr && lv.rope_cos != nullptr) const_cast<uint4*>(row)[c] = q_regs;      // (no other CTA reads them)
-      if (h == 8 && row != nullptr && jn >= 32 * res_b && jn < 32 * res_e)      // this CTA has the new key's unit: it reads the key from the store
-        reinterpret_cast<uint4*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[c] = q_regs;
+      if (h == 8) sts128(knew_u32 + 16 * c, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
       if (h < 8) {
         sts128(qb16_u32 + (h * kQS + 8 * c) * 2, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
         if (kU4 == 1)      // the fp16 table is for the gathered UINT4 channels
@@ -355,6 +355,13 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
           for (int j = 0; j < 4; ++j) {
             ka[j] = ta < rt ? rowa[4 * j + t] : make_uint4(0u, 0u, 0u, 0u);
             kb[j] = tb < rt ? rowb[4 * j + t] : make_uint4(0u, 0u, 0u, 0u);
+          }
+          if (holds_new) {          // (what lies in the store at the newest token's place is not its key yet)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              if (ta == jn) ka[j] = lds128(knew_u32 + 16 * (4 * j + t));
+              if (tb == jn) kb[j] = lds128(knew_u32 + 16 * (4 * j + t));
+            }
           }
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -686,7 +693,9 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float
       // Four channels' sums run side by side.  One sequence of 333 to 433 tokens, decode steps of 8 layers: 7.2 us per step and
       // layer with it before the residual unit's hand-over, a channel after the other; 6.2 here.
       if (takes_new) {
-        // add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads ascending: the order of the plain append)
+        // store the new key row and add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads
+        // ascending: the order of the plain append)
+        reinterpret_cast<uint2*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[lane] = lds64(knew_u32 + 8 * lane);
         double2* acc = reinterpret_cast<double2*>(lv.state + (size_t)s * lv.state_stride) + 2 * lane;
         double2 a0 = acc[0], a1 = acc[1];
         for (int h = 0; h < g; ++h) {

@@ -92,7 +92,7 @@ constexpr int kQS = 136;                     // halves per row of the query tabl
 constexpr int kPrefixBytes = ((kMaxRaggedBatch + 1) * 4 + 15) / 16 * 16;     // a ragged batch's prefix sums
 __host__ __device__ constexpr int bar_bytes(int teams) { return (teams * kBarsPerTeam * 8 + 127) / 128 * 128; }
 __host__ __device__ constexpr int smem_bytes(int G, int u4, bool v4) {
-  return teams_of(u4, v4) * (team_bytes(G, u4, v4) + 64) + bar_bytes(teams_of(u4, v4)) + (u4 == 1 ? 2 : 1) * 8 * kQS * 2 + kPrefixBytes;
+  return teams_of(u4, v4) * (team_bytes(G, u4, v4) + 64) + bar_bytes(teams_of(u4, v4)) + (u4 == 1 ? 2 : 1) * 8 * kQS * 2 + kPrefixBytes + 2 * kD;
 }
 constexpr int kResidualWeight = 3;           // an unquantized 32-token unit counts as this many packed units in the split
 constexpr int kMergeStride = 132;            // floats per head row of a pair's output in the merge
@@ -126,6 +126,10 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group
   constexpr int UPG = G / 32;             // units per key group
   constexpr int kGroups = UPG == 1 ? 2 : 1;                    // key groups of a step
+  // The step's new key reaches the warp that has its unit through shared memory, or through its place in the residual window, which costs a
+  // round trip to L2 but no registers: us per decode step, shared / window: two tiers, 7b shape, 8 x 32768 tokens, 28 layers 1094 / 1103, 4 x
+  // 120000, 8 layers 512 / 521; three tiers, 8 x 20011, 14 layers 519 / 498, 4-bit base, 8b shape, 16 x 16384, 8 layers 803 / 792.
+  constexpr bool kKeyInShared = kU4 == 0;
   constexpr int kTeams = teams_of(kU4, kV4), kL = logits_warps_of(kU4), kThreads = threads_of(kU4, kV4);
   constexpr int kStages = stages_of(kU4), kSlotCount = slots_of(kU4), kSlotBytes = slot_bytes(kU4);
   static_assert(smem_bytes(G, kU4, kV4) <= 113 * 1024, "two CTAs per SM");
@@ -156,6 +160,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   float* mS = reinterpret_cast<float*>(smem + kTeams * kTeamBytes + bar_bytes(kTeams) + kQBytes);    // [kTeams][8]
   float* lS = mS + kTeams * 8;                                                                       // [kTeams][8]
   int* prefS = reinterpret_cast<int*>(lS + kTeams * 8);                     // ragged batch: seq_prefix[0 .. B]
+  const uint32_t knew_u32 = smem_u32(prefS) + kPrefixBytes;                 // the step's new key [128], rotated if the step rotates
 
   if (threadIdx.x < kTeams * kBarsPerTeam) {
     mbar_init(tail_u32 + 8 * threadIdx.x, 1);
@@ -398,8 +403,8 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     dep_wait();
     if (to_request > 0 && !lv.stage_early) request_first();
 
-    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the CTA with its unit stores its key there first,
-    // and the warps that take the unit read its value from the step's tensors, store it and update the importance accumulator
+    // fused decode step: the newest token (slot r - 1) is not in the residual store yet; the warps that take its unit read it from
+    // the step's tensors, store its rows and update the importance accumulator
     const int jn = f_r - 1;
     // ---- query of this stream: bf16 and fp16 tables (heads >= g are zero rows)
     {
@@ -410,12 +415,15 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
                                : (h == 8 && lv.new_k != nullptr ? reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD) : nullptr);
       if (row != nullptr) {
         q_regs = row[c];
-        if (lv.rope_cos != nullptr) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
+        if (__builtin_expect(lv.rope_cos != nullptr, 0)) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
       }
       __syncthreads();          // the previous segment's readers of the tables are done, and so are the rotation's reads
       if (kDirect && row != nullptr && lv.rope_cos != nullptr) const_cast<uint4*>(row)[c] = q_regs;      // (no other CTA reads them)
-      if (h == 8 && row != nullptr && jn >= 32 * res_b && jn < 32 * res_e)      // this CTA has the new key's unit: it reads the key from the store
-        reinterpret_cast<uint4*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[c] = q_regs;
+      if (h == 8 && row != nullptr) {
+        if (kKeyInShared) sts128(knew_u32 + 16 * c, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
+        else if (jn >= 32 * res_b && jn < 32 * res_e)      // this CTA has the new key's unit
+          reinterpret_cast<uint4*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[c] = q_regs;
+      }
       if (h < 8) {
         sts128(qb16_u32 + (h * kQS + 8 * c) * 2, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
         if (kU4 == 1)      // the fp16 table is for the gathered UINT4 channels
@@ -457,6 +465,13 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
           for (int j = 0; j < 4; ++j) {
             ka[j] = ta < rt ? rowa[4 * j + t] : make_uint4(0u, 0u, 0u, 0u);
             kb[j] = tb < rt ? rowb[4 * j + t] : make_uint4(0u, 0u, 0u, 0u);
+          }
+          if (kKeyInShared && holds_new) {          // (what lies in the store at the newest token's place is not its key yet)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              if (ta == jn) ka[j] = lds128(knew_u32 + 16 * (4 * j + t));
+              if (tb == jn) kb[j] = lds128(knew_u32 + 16 * (4 * j + t));
+            }
           }
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -743,7 +758,9 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       // Four channels' sums run side by side.  Decode steps, 7b shape, batch 8: 32768 tokens, 28 layers 1134.6 -> 1126.0 us;
       // three tiers, 20011 tokens, 14 layers 524.3 -> 517.7.
       if (takes_new) {
-        // add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads ascending: the order of the plain append)
+        // store the new key row and add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads
+        // ascending: the order of the plain append)
+        if (kKeyInShared) reinterpret_cast<uint2*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[lane] = lds64(knew_u32 + 8 * lane);
         double2* acc = reinterpret_cast<double2*>(lv.state + (size_t)s * lv.state_stride) + 2 * lane;
         double2 a0 = acc[0], a1 = acc[1];
         for (int h = 0; h < g; ++h) {
@@ -1313,9 +1330,9 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   const bool whole = out != nullptr && lv.seq == nullptr && grid == S;
   float* const kernel_out = whole ? out : nullptr;
   // ... with eight pairs of warps where every stream has an SM to itself.  us per layer, four / eight pairs: 4 streams of the 7b shape, two
-  // tiers, 300 tokens 5.5 / 5.1; 64 streams, three tiers 7.7 / 6.7, 4-bit base 7.4 / 6.1, 128 streams of the 8b shape, 400 tokens 9.1 / 7.8.  Only
-  // with few positions and most of the SMs in use the larger CTAs cost more: 128 streams, 200 tokens (13 positions) 7.7 / 8.05.
-  const bool wide = whole && grid <= n_sms && (Us > 13 || 2 * grid <= n_sms);
+  // tiers, 300 tokens 5.5 / 5.1; 64 streams, three tiers 7.7 / 6.7, 4-bit base 7.4 / 6.1, 128 streams of the 8b shape, 400 tokens 9.1 / 7.8.  With
+  // fewer positions the larger CTAs cost more: 128 streams, 200 tokens (13 positions) 7.7 / 8.05; requests of 27 and of 54 tokens 5 to 9 % slower.
+  const bool wide = whole && grid <= n_sms && (Us > 13 || (Us == 13 && 2 * grid <= n_sms));
   if (form) *form = (by_two ? MIXKVQ_ATTN_TWO_UNITS : MIXKVQ_ATTN_ONE_UNIT) | (whole ? MIXKVQ_ATTN_DIRECT : 0) | (lv.stage_early ? MIXKVQ_ATTN_EARLY : 0);
   cudaError_t e;
   if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, kernel_out, lse_out, wide, stream);

@@ -26,7 +26,7 @@ constexpr int kCombineMaxWarps = 8;
 // part: lanes 0 .. 15 the query row `row`, lanes 16 .. 31 (with the stream's head 0) its new key row.  Requested before the merge
 // (rope_load) and stored behind it.
 struct RopeRows {
-  uint16_t *q, *k;                       // [B Hq][128], [S][128]; q is null without a rotation
+  uint16_t *q, *k;                       // [B Hq][128], [S][128]
   const float *cos_row, *sin_row;
 };
 struct RopeWork {
@@ -35,7 +35,7 @@ struct RopeWork {
 __device__ __forceinline__ RopeWork rope_load(const RopeRows& r, size_t row, int s, int h, int lane) {
   RopeWork w;
   w.at = nullptr;
-  if (r.q != nullptr && (lane < 16 || h == 0)) {
+  if (lane < 16 || h == 0) {
     uint4* base = reinterpret_cast<uint4*>(lane < 16 ? r.q + row * kD : r.k + (size_t)s * kD);
     const int c = lane & 15;
     w.at = base + c;
@@ -49,6 +49,7 @@ __device__ __forceinline__ void rope_store(const RopeWork& w) {
   if (w.at != nullptr) *w.at = w.y;
 }
 
+template <bool kRope>
 __global__ void __launch_bounds__(kCombineMaxWarps * 32)
 combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int Hkv, int Hq, int mode, int n,
                long long units_per_stream, int S, const int4* __restrict__ seq, const int* __restrict__ seq_prefix,
@@ -79,7 +80,7 @@ combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int
   }
   dependency_wait();
   RopeWork rotated{};
-  if (warp == W - 1) rotated = rope_load(rope, ((size_t)(s / Hkv) * Hq + (s % Hkv) * g + h), s, h, lane);
+  if (kRope && warp == W - 1) rotated = rope_load(rope, ((size_t)(s / Hkv) * Hq + (s % Hkv) * g + h), s, h, lane);
   // ---- this warp's partials: one pass with a running maximum; a lane has channels 2 lane, 2 lane + 1 and 64 more
   const float* base = ws + (size_t)first * kPartialFloats + h * 130;
   float M = -INFINITY, l = 0.f;
@@ -113,7 +114,7 @@ combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int
     }
     M = Mn;
   }
-  if (warp == W - 1) rope_store(rotated);
+  if (kRope && warp == W - 1) rope_store(rotated);
   // ---- the warps' results
   if (lane == 0) {
     mlS[warp][0] = M;
@@ -145,6 +146,7 @@ combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int
 // 231.6 us; 32 streams with nine partials 15.7 / 15.9; 16 streams with 18, 37.4 / 37.9).
 constexpr int kRowsChunk = 8, kRowsMaxPartials = 8;
 
+template <bool kRope>
 __global__ void __launch_bounds__(256)
 combine_rows_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int Hkv, int Hq, int n, long long units_per_stream,
                     int S, float* __restrict__ lse_out, bool early, RopeRows rope) {
@@ -155,7 +157,8 @@ combine_rows_kernel(const float* __restrict__ ws, float* __restrict__ out, int g
   const int c0 = (int)(((x0 + 1) * n - 1) / total), c1 = (int)(((x1 + 1) * n - 1) / total), count = c1 - c0 + 1;
   const float* base = ws + (size_t)(c0 + s) * kPartialFloats + h * 130;
   dependency_wait();
-  const RopeWork rotated = rope_load(rope, (size_t)s * g + h, s, h, lane);
+  RopeWork rotated{};
+  if (kRope) rotated = rope_load(rope, (size_t)s * g + h, s, h, lane);
   float M = -INFINITY, l = 0.f;
   float2 oa = make_float2(0.f, 0.f), ob = make_float2(0.f, 0.f);
   for (int i0 = 0; i0 < count; i0 += kRowsChunk) {
@@ -186,7 +189,7 @@ combine_rows_kernel(const float* __restrict__ ws, float* __restrict__ out, int g
     }
     M = Mn;
   }
-  rope_store(rotated);
+  if (kRope) rope_store(rotated);
   const size_t row = (size_t)s * g + h;             // (b Hkv + hk) g + h = b Hq + hk g + h
   float2* dst = reinterpret_cast<float2*>(out + row * kD);
   dst[lane] = l > 0.f ? make_float2(oa.x / l, oa.y / l) : make_float2(0.f, 0.f);
@@ -199,12 +202,14 @@ cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, 
                            float* lse_out, bool early, void* rope_q, void* rope_k, const float* rope_cos, const float* rope_sin) {
   const RopeRows rope{static_cast<uint16_t*>(rope_q), static_cast<uint16_t*>(rope_k), rope_cos, rope_sin};
   if (mode == 1 && seq == nullptr && n / S + 2 <= kRowsMaxPartials)
-    return launch_dependent(combine_rows_kernel, dim3((unsigned)S), 32 * g, 0, stream, ws, out, g, Hkv, Hq, n, units_per_stream, S, lse_out, early, rope);
+    return launch_dependent(rope_q != nullptr ? combine_rows_kernel<true> : combine_rows_kernel<false>, dim3((unsigned)S), 32 * g, 0, stream, ws, out, g, Hkv, Hq,
+                            n, units_per_stream, S, lse_out, early, rope);
   // eight warps when four with a chunk each do not cover a stream's partials in one round trip (a ragged batch may give
   // nearly all CTAs to one sequence), four otherwise: more warps only lengthen the last step
   const int partials = mode == 0 ? n : (seq != nullptr ? n : n / S + 1);
-  return launch_dependent(combine_kernel, dim3((unsigned)(S * g)), partials > 4 * kCombineChunk ? kCombineMaxWarps * 32 : 128, 0, stream,
-                          ws, out, g, Hkv, Hq, mode, n, units_per_stream, S, seq, seq_prefix, lse_out, early, rope);
+  return launch_dependent(rope_q != nullptr ? combine_kernel<true> : combine_kernel<false>, dim3((unsigned)(S * g)),
+                          partials > 4 * kCombineChunk ? kCombineMaxWarps * 32 : 128, 0, stream, ws, out, g, Hkv, Hq, mode, n, units_per_stream, S, seq,
+                          seq_prefix, lse_out, early, rope);
 }
 
 // The table of a ragged batch, from the host's per-sequence fill (kernel arguments: no copy, ordered in the stream).
