@@ -92,7 +92,7 @@ constexpr int kQS = 136;                     // halves per row of the query tabl
 constexpr int kPrefixBytes = ((kMaxRaggedBatch + 1) * 4 + 15) / 16 * 16;     // a ragged batch's prefix sums
 __host__ __device__ constexpr int bar_bytes(int teams) { return (teams * kBarsPerTeam * 8 + 127) / 128 * 128; }
 __host__ __device__ constexpr int smem_bytes(int G, int u4, bool v4) {
-  return teams_of(u4, v4) * (team_bytes(G, u4, v4) + 64) + bar_bytes(teams_of(u4, v4)) + (u4 == 1 ? 2 : 1) * 8 * kQS * 2 + kPrefixBytes + 2 * kD;
+  return teams_of(u4, v4) * (team_bytes(G, u4, v4) + 64) + bar_bytes(teams_of(u4, v4)) + (u4 == 1 ? 2 : 1) * 8 * kQS * 2 + kPrefixBytes;
 }
 constexpr int kResidualWeight = 3;           // an unquantized 32-token unit counts as this many packed units in the split
 constexpr int kMergeStride = 132;            // floats per head row of a pair's output in the merge
@@ -118,7 +118,8 @@ __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp
 // per channel pair, gathered), 2 = 4-bit base (dense high plane)
 // kV4: 4-bit values (a second plane of 2-bit value codes per unit, scale 4 s_v)
 // kDirect: one CTA per stream, which writes the output (and the log-denominators) instead of a partial
-template <int G, int kU4, bool kV4, bool kDirect>
+// kRope: the step rotates (kernels of their own: the others have no registers to spare for it)
+template <int G, int kU4, bool kV4, bool kDirect, bool kRope>
 __global__ void __launch_bounds__(threads_of(kU4, kV4), kCtasPerSm)
 attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float scale_log2e, float* __restrict__ ws,
                     uint32_t four2, float* __restrict__ out, float* __restrict__ lse_out) {
@@ -126,10 +127,6 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group
   constexpr int UPG = G / 32;             // units per key group
   constexpr int kGroups = UPG == 1 ? 2 : 1;                    // key groups of a step
-  // The step's new key reaches the warp that has its unit through shared memory, or through its place in the residual window, which costs a
-  // round trip to L2 but no registers: us per decode step, shared / window: two tiers, 7b shape, 8 x 32768 tokens, 28 layers 1094 / 1103, 4 x
-  // 120000, 8 layers 512 / 521; three tiers, 8 x 20011, 14 layers 519 / 498, 4-bit base, 8b shape, 16 x 16384, 8 layers 803 / 792.
-  constexpr bool kKeyInShared = kU4 == 0;
   constexpr int kTeams = teams_of(kU4, kV4), kL = logits_warps_of(kU4), kThreads = threads_of(kU4, kV4);
   constexpr int kStages = stages_of(kU4), kSlotCount = slots_of(kU4), kSlotBytes = slot_bytes(kU4);
   static_assert(smem_bytes(G, kU4, kV4) <= 113 * 1024, "two CTAs per SM");
@@ -160,7 +157,6 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   float* mS = reinterpret_cast<float*>(smem + kTeams * kTeamBytes + bar_bytes(kTeams) + kQBytes);    // [kTeams][8]
   float* lS = mS + kTeams * 8;                                                                       // [kTeams][8]
   int* prefS = reinterpret_cast<int*>(lS + kTeams * 8);                     // ragged batch: seq_prefix[0 .. B]
-  const uint32_t knew_u32 = smem_u32(prefS) + kPrefixBytes;                 // the step's new key [128], rotated if the step rotates
 
   if (threadIdx.x < kTeams * kBarsPerTeam) {
     mbar_init(tail_u32 + 8 * threadIdx.x, 1);
@@ -403,8 +399,9 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     // The query rows, the step's token and the segment's unquantized units are requested into the L2 cache before the wait (a request has no
     // other effect, whatever the kernel before this one still writes): of a model's many layers they have left it since the step before.
     // us per decode step without / with: 7b shape, 8 x 32768 tokens, 28 layers 1103 / 1075, 4 x 120000, 8 layers 521 / 509, ragged 826 / 814;
-    // three tiers, 8 x 20011, 14 layers 498 / 504.  (By the values warps alone, which refill the rings: no gain.)
-    {
+    // three tiers, 8 x 20011, 14 layers 498 / 504.  (By the values warps alone, which refill the rings: no gain.)  Only for a CTA's first
+    // segment: the others come long behind the wait.
+    if (lv.seq != nullptr || !dep_waited) {
       const int b = s / lv.Hkv, hk = s % lv.Hkv, h = threadIdx.x >> 1;
       if (h < g) prefetch_l2(reinterpret_cast<const char*>(q + ((size_t)b * lv.Hq + hk * g + h) * kD) + 128 * (threadIdx.x & 1));
       else if (lv.new_k != nullptr && h < g + 2) prefetch_l2(reinterpret_cast<const char*>((h == g ? lv.new_k : lv.new_v) + (size_t)s * kD) + 128 * (threadIdx.x & 1));
@@ -424,22 +421,19 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
     const int jn = f_r - 1;
     // ---- query of this stream: bf16 and fp16 tables (heads >= g are zero rows)
     {
-      // thread (h, c) of the first 128: head h, channels 8c .. 8c+7; the next 16 (h = 8): the step's new key
+      // thread (h, c) of the first 128: head h, channels 8c .. 8c+7; the next 16 (h = 8): the new key of a step that rotates
       uint4 q_regs = make_uint4(0u, 0u, 0u, 0u);
       const int b = s / lv.Hkv, hk = s % lv.Hkv, h = threadIdx.x >> 4, c = threadIdx.x & 15;
       const uint4* row = h < g ? reinterpret_cast<const uint4*>(q + ((size_t)b * lv.Hq + hk * g + h) * kD)
-                               : (h == 8 && lv.new_k != nullptr ? reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD) : nullptr);
+                               : (kRope && h == 8 ? reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD) : nullptr);
       if (row != nullptr) {
         q_regs = row[c];
-        if (__builtin_expect(lv.rope_cos != nullptr, 0)) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
+        if (kRope) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
       }
       __syncthreads();          // the previous segment's readers of the tables are done, and so are the rotation's reads
-      if (kDirect && row != nullptr && lv.rope_cos != nullptr) const_cast<uint4*>(row)[c] = q_regs;      // (no other CTA reads them)
-      if (h == 8 && row != nullptr) {
-        if (kKeyInShared) sts128(knew_u32 + 16 * c, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
-        else if (jn >= 32 * res_b && jn < 32 * res_e)      // this CTA has the new key's unit
-          reinterpret_cast<uint4*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[c] = q_regs;
-      }
+      if (kRope && kDirect && row != nullptr) const_cast<uint4*>(row)[c] = q_regs;      // (no other CTA reads them)
+      if (kRope && h == 8 && jn >= 32 * res_b && jn < 32 * res_e)      // this CTA has the new key's unit and reads it from the window
+        reinterpret_cast<uint4*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[c] = q_regs;
       if (h < 8) {
         sts128(qb16_u32 + (h * kQS + 8 * c) * 2, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
         if (kU4 == 1)      // the fp16 table is for the gathered UINT4 channels
@@ -476,18 +470,13 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
           const int ta = j0 + mt * 16 + r, tb = ta + 8;
           const uint4* rowa = reinterpret_cast<const uint4*>(resk + (size_t)ta * 256);
           const uint4* rowb = reinterpret_cast<const uint4*>(resk + (size_t)tb * 256);
+          if (!kRope && holds_new && ta == jn) rowa = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
+          if (!kRope && holds_new && tb == jn) rowb = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
           uint4 ka[4], kb[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             ka[j] = ta < rt ? rowa[4 * j + t] : make_uint4(0u, 0u, 0u, 0u);
             kb[j] = tb < rt ? rowb[4 * j + t] : make_uint4(0u, 0u, 0u, 0u);
-          }
-          if (kKeyInShared && holds_new) {          // (what lies in the store at the newest token's place is not its key yet)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              if (ta == jn) ka[j] = lds128(knew_u32 + 16 * (4 * j + t));
-              if (tb == jn) kb[j] = lds128(knew_u32 + 16 * (4 * j + t));
-            }
           }
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -776,7 +765,10 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
       if (takes_new) {
         // store the new key row and add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads
         // ascending: the order of the plain append)
-        if (kKeyInShared) reinterpret_cast<uint2*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[lane] = lds64(knew_u32 + 8 * lane);
+        if (!kRope) {
+          const uint2 kn = reinterpret_cast<const uint2*>(lv.new_k + (size_t)s * kD)[lane];
+          reinterpret_cast<uint2*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[lane] = kn;
+        }
         double2* acc = reinterpret_cast<double2*>(lv.state + (size_t)s * lv.state_stride) + 2 * lane;
         double2 a0 = acc[0], a1 = acc[1];
         for (int h = 0; h < g; ++h) {
@@ -1167,9 +1159,14 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float sca
   }
 }
 
+template <int G, int kU4, bool kV4, bool kDirect, bool kRope>
+cudaError_t launch_r(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
+  return launch_dependent(attention_ws_kernel<G, kU4, kV4, kDirect, kRope>, dim3((unsigned)grid), threads_of(kU4, kV4), smem_bytes(G, kU4, kV4), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
+}
 template <int G, int kU4, bool kV4, bool kDirect>
 cudaError_t launch_d(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
-  return launch_dependent(attention_ws_kernel<G, kU4, kV4, kDirect>, dim3((unsigned)grid), threads_of(kU4, kV4), smem_bytes(G, kU4, kV4), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
+  return lv.rope_cos != nullptr ? launch_r<G, kU4, kV4, kDirect, true>(lv, qb, sl, ws, grid, out, lse, stream)
+                                : launch_r<G, kU4, kV4, kDirect, false>(lv, qb, sl, ws, grid, out, lse, stream);
 }
 template <int G, int kU4, bool kV4>
 cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
@@ -1195,14 +1192,17 @@ cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws,
 
 }  // namespace
 
-template <int G, int kU4, bool kV4, bool kDirect>
-static cudaError_t setup_d() {
-  cudaError_t e = cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem_bytes(G, kU4, kV4));
+template <int G, int kU4, bool kV4, bool kDirect, bool kRope>
+static cudaError_t setup_r() {
+  cudaError_t e = cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect, kRope>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(G, kU4, kV4));
   if (e != cudaSuccess) return e;
   // the CTAs of an SM only fit with the largest shared-memory carve-out; ask for it explicitly
-  return cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                              (int)cudaSharedmemCarveoutMaxShared);
+  return cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect, kRope>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+}
+template <int G, int kU4, bool kV4, bool kDirect>
+static cudaError_t setup_d() {
+  const cudaError_t e = setup_r<G, kU4, kV4, kDirect, false>();
+  return e == cudaSuccess ? setup_r<G, kU4, kV4, kDirect, true>() : e;
 }
 template <int G, int kU4, bool kV4>
 static cudaError_t setup_v() {
