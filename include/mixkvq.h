@@ -304,9 +304,13 @@ enum {
   MIXKVQ_ATTN_TWO_UNITS = 2,          /* ... two units per step                                      */
   MIXKVQ_ATTN_DIRECT = 4,             /* one thread block per stream, which wrote the output: no merge */
   MIXKVQ_ATTN_EARLY = 8,              /* packed blocks were requested before the wait for earlier work */
-  MIXKVQ_ATTN_OTHER = 16              /* the plain-ALU kernel or the tile layout's                   */
+  MIXKVQ_ATTN_OTHER = 16,             /* the plain-ALU kernel or the tile layout's                   */
+  MIXKVQ_ATTN_EIGHT_PAIRS = 32        /* ONE_UNIT | DIRECT with eight instead of four pairs of warps per thread block */
 };
 int mixkvq_last_attention(const mixkvq_cache* cache);
+/* Thread blocks of that call's split kernel (0: none, or MIXKVQ_ATTN_OTHER).  With fewer streams than thread blocks a number that
+ * is no multiple of batch * n_kv_heads means that thread blocks straddle two streams. */
+int mixkvq_last_attention_ctas(const mixkvq_cache* cache);
 
 /* Number of kernels launched by this handle since it was created (diagnostic). */
 uint64_t mixkvq_launch_count(const mixkvq_cache* cache);

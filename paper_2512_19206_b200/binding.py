@@ -19,12 +19,12 @@ EXPORTS = [
     "mixkvq_cache_bytes", "mixkvq_cache_init", "mixkvq_cache_destroy", "mixkvq_cache_reset",
     "mixkvq_select_channels", "mixkvq_select_channels_raw", "mixkvq_quantize_append",
     "mixkvq_decode_attention", "mixkvq_decode_attention_noalloc", "mixkvq_decode_step", "mixkvq_set_attention_kernel", "mixkvq_query_status",
-    "mixkvq_cache_describe", "mixkvq_last_attention", "mixkvq_launch_count", "mixkvq_status_string",
+    "mixkvq_cache_describe", "mixkvq_last_attention", "mixkvq_last_attention_ctas", "mixkvq_launch_count", "mixkvq_status_string",
     "mixkvq_cache_written_externally", "mixkvq_test_arm_copy_timeout", "mixkvq_test_arm_value_copy_timeout", "mixkvq_rope_append", "mixkvq_rope_decode_step", "mixkvq_prefill", "mixkvq_prefill_scratch_bytes", "mixkvq_quantize_append_ragged", "mixkvq_sequence_fill", "mixkvq_decode_attention_partial", "mixkvq_merge_partials",
 ]
 
 DEV_EXTRAS_FULL, DEV_COPY_TIMEOUT = 1, 2
-ATTN_ONE_UNIT, ATTN_TWO_UNITS, ATTN_DIRECT, ATTN_EARLY, ATTN_OTHER = 1, 2, 4, 8, 16
+ATTN_ONE_UNIT, ATTN_TWO_UNITS, ATTN_DIRECT, ATTN_EARLY, ATTN_OTHER, ATTN_EIGHT_PAIRS = 1, 2, 4, 8, 16, 32
 
 
 class Config(C.Structure):
@@ -87,7 +87,7 @@ def lib():
         L.mixkvq_test_arm_copy_timeout.argtypes = L.mixkvq_test_arm_value_copy_timeout.argtypes = [vp, C.c_uint32, C.c_uint32]
         L.mixkvq_query_status.argtypes = [vp, C.POINTER(i32), vp]
         L.mixkvq_cache_describe.argtypes = [vp, i32, C.POINTER(LayoutDesc)]
-        L.mixkvq_launch_count.argtypes = L.mixkvq_last_attention.argtypes = [vp]
+        L.mixkvq_launch_count.argtypes = L.mixkvq_last_attention.argtypes = L.mixkvq_last_attention_ctas.argtypes = [vp]
         L.mixkvq_launch_count.restype = u64
         L.mixkvq_status_string.argtypes = [i32]
         L.mixkvq_status_string.restype = C.c_char_p
@@ -335,6 +335,10 @@ class Cache:
     def last_attention(self) -> int:
         """ATTN_* bits of the last decode-attention call: which kernel, which output form."""
         return int(lib().mixkvq_last_attention(self.handle))
+
+    def last_attention_ctas(self) -> int:
+        """Thread blocks of that call's split kernel (0: it had none)."""
+        return int(lib().mixkvq_last_attention_ctas(self.handle))
 
     def launch_count(self) -> int:
         return int(lib().mixkvq_launch_count(self.handle))

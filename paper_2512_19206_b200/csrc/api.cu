@@ -22,7 +22,7 @@ struct mixkvq_cache {
   std::vector<int> n_blocks, r, n_sink;
   int n_sms;
   int attn_kind;
-  int last_form;                             // mixkvq_last_attention
+  int last_form, last_ctas;                  // mixkvq_last_attention, mixkvq_last_attention_ctas
   uint64_t launches;
   // What the library enqueued last on this handle: kNoPackedWrite if it did not write packed blocks, a layer index if
   // it wrote that layer's packed blocks (a flush), kAllPacked after initialisation, a reset or a write from outside.
@@ -245,12 +245,13 @@ int run_attention(mixkvq_cache* h, int layer, const void* q, float* out, float s
   int launches = 0;
   cudaError_t e;
   h->last_form = MIXKVQ_ATTN_OTHER;
+  h->last_ctas = 0;
   if (h->attn_kind == 1)
     e = launch_attention_simt(lv, q, out, scale, ws, h->n_sms, st, &launches);
   else if (h->tile)
     e = launch_attention_tc(lv, q, h->attn_kind == 2 ? nullptr : out, scale, ws, h->n_sms, st, &launches);
   else
-    e = launch_attention_ws(lv, q, h->attn_kind == 2 ? nullptr : out, scale, ws, h->n_sms, st, &launches, lse, &h->last_form);
+    e = launch_attention_ws(lv, q, h->attn_kind == 2 ? nullptr : out, scale, ws, h->n_sms, st, &launches, lse, &h->last_form, &h->last_ctas);
   h->launches += launches;
   return e == cudaSuccess ? MIXKVQ_OK : MIXKVQ_E_CUDA;
 }
@@ -407,7 +408,7 @@ int mixkvq_cache_init(const mixkvq_config* cfg, void* cache_dev, size_t bytes, v
   h->r.assign((size_t)cfg->n_layers * cfg->batch, 0);
   h->n_sink.assign((size_t)cfg->n_layers * cfg->batch, 0);
   h->attn_kind = 0;
-  h->last_form = 0;
+  h->last_form = h->last_ctas = 0;
   h->launches = 0;
   note_enqueued(h, static_cast<cudaStream_t>(stream), kAllPacked);
   h->test_extra_tx = h->test_wait_polls = h->test_extra_v = 0;
@@ -711,6 +712,8 @@ int mixkvq_sequence_fill(const mixkvq_cache* cache, int layer, int b, uint32_t* 
 }
 
 int mixkvq_last_attention(const mixkvq_cache* cache) { return cache ? cache->last_form : 0; }
+
+int mixkvq_last_attention_ctas(const mixkvq_cache* cache) { return cache ? cache->last_ctas : 0; }
 
 uint64_t mixkvq_launch_count(const mixkvq_cache* cache) { return cache ? cache->launches : 0; }
 

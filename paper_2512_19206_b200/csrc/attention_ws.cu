@@ -1316,7 +1316,7 @@ int attention_ws_grid(const LayerView& lv, int n_sms) {
 }
 
 cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, float scale, float* ws, int n_sms,
-                                cudaStream_t stream, int* launches, float* lse_out, int* form) {
+                                cudaStream_t stream, int* launches, float* lse_out, int* form, int* ctas) {
   const int S = lv.B * lv.Hkv;
   const long long Us = attention_ws_positions(lv);
   const int grid = attention_ws_grid(lv, n_sms);
@@ -1349,7 +1349,10 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // tiers, 300 tokens 5.5 / 5.1; 64 streams, three tiers 7.7 / 6.7, 4-bit base 7.4 / 6.1, 128 streams of the 8b shape, 400 tokens 9.1 / 7.8.  With
   // fewer positions the larger CTAs cost more: 128 streams, 200 tokens (13 positions) 7.7 / 8.05; requests of 27 and of 54 tokens 5 to 9 % slower.
   const bool wide = whole && grid <= n_sms && (Us > 13 || (Us == 13 && 2 * grid <= n_sms));
-  if (form) *form = (by_two ? MIXKVQ_ATTN_TWO_UNITS : MIXKVQ_ATTN_ONE_UNIT) | (whole ? MIXKVQ_ATTN_DIRECT : 0) | (lv.stage_early ? MIXKVQ_ATTN_EARLY : 0);
+  if (form)
+    *form = (by_two ? MIXKVQ_ATTN_TWO_UNITS : MIXKVQ_ATTN_ONE_UNIT) | (whole ? MIXKVQ_ATTN_DIRECT : 0) | (lv.stage_early ? MIXKVQ_ATTN_EARLY : 0) |
+            (wide && !by_two ? MIXKVQ_ATTN_EIGHT_PAIRS : 0);
+  if (ctas) *ctas = grid;
   cudaError_t e;
   if (!by_two) e = launch_attention_single(lv, q, scale, ws, grid, kernel_out, lse_out, wide, stream);
   else if (lv.G == 32) e = launch_g<32>(lv, q, scale, ws, grid, kernel_out, lse_out, stream);

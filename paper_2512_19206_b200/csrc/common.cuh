@@ -269,7 +269,8 @@ cudaError_t launch_select_raw(const void* q, const void* k, int B, int Hq, int H
 cudaError_t launch_attention_simt(const LayerView& lv, const void* q, float* out, float scale, float* ws,
                                   int n_sms, cudaStream_t stream, int* launches);
 cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, float scale, float* ws,
-                                int n_sms, cudaStream_t stream, int* launches, float* lse_out = nullptr, int* form = nullptr);
+                                int n_sms, cudaStream_t stream, int* launches, float* lse_out = nullptr, int* form = nullptr,
+                                int* ctas = nullptr);
 cudaError_t attention_ws_setup();
 // tile layout (R == 128): tcgen05 kernel
 cudaError_t launch_attention_tc(const LayerView& lv, const void* q, float* out, float scale, float* ws,

@@ -43,8 +43,8 @@ def test_direct_output(binding, name, batch, tokens, R, preset):
 
 
 @pytest.mark.parametrize("name,batch,tokens,preset,v_bits,form", [
-    ("qwen7b", 1, 200, "P27", 4, 1 + 4), ("llama8b", 1, 450, "P24", 2, 1 + 4), ("llama8b", 1, 560, "P24", 2, 1), ("qwen7b", 16, 511, "P4BASE", 2, 1 + 4),
-    ("qwen7b", 16, 1152, "P27", 2, 2), ("llama8b", 16, 1000, "P24", 4, 1 + 4), ("llama8b", 18, 200, "P24", 2, 1 + 4), ("llama8b", 19, 700, "P27", 2, 2 + 4),
+    ("qwen7b", 1, 200, "P27", 4, 1 + 4 + 32), ("llama8b", 1, 450, "P24", 2, 1 + 4 + 32), ("llama8b", 1, 560, "P24", 2, 1), ("qwen7b", 16, 511, "P4BASE", 2, 1 + 4 + 32),
+    ("qwen7b", 16, 1152, "P27", 2, 2), ("llama8b", 16, 1000, "P24", 4, 1 + 4 + 32), ("llama8b", 18, 200, "P24", 2, 1 + 4), ("llama8b", 19, 700, "P27", 2, 2 + 4),
 ])
 def test_eight_pairs_per_stream(binding, name, batch, tokens, preset, v_bits, form):
     """One CTA of eight warp pairs per stream while every stream has an SM to itself, on both sides of where that ends (148 SMs: 18
@@ -56,7 +56,7 @@ def test_eight_pairs_per_stream(binding, name, batch, tokens, preset, v_bits, fo
         c.quantize_append(0, *W.tokens(w, 0, 0, tokens, device="cuda"))
     k, v, q = [x.contiguous() for x in W.tokens(w, 0, tokens, 1, device="cuda")]
     out = caches[0].decode_step(0, k, v, q, W.softmax_scale())
-    assert caches[0].last_attention() & 7 == form
+    assert caches[0].last_attention() & ~binding.ATTN_EARLY == form
     caches[1].quantize_append(0, k, v, q)
     plain, lse = caches[1].decode_attention_partial(0, q[:, :, 0].contiguous(), W.softmax_scale())
     assert torch.equal(out, plain) and bool(torch.isfinite(lse).all())
@@ -68,14 +68,21 @@ def test_eight_pairs_per_stream(binding, name, batch, tokens, preset, v_bits, fo
     assert float((out - ref).abs().max()) <= TOL
 
 
-@pytest.mark.parametrize("batch,tokens,preset", [(9, 3000, "P24"), (12, 4000, "P27"), (16, 4000, "P4BASE"), (18, 2000, "P24")])
-def test_split_that_straddles_streams(binding, batch, tokens, preset):
-    """Stream counts that leave many CTA slots idle at a whole number of CTAs per stream: all slots are used and CTAs straddle streams."""
-    w = W.small(W.CONFIGS["llama8b"], n_layers=1, batch=batch, tokens=tokens, **getattr(W, preset))
-    cache = U.make_cache(binding, w, extras_budget_bytes=(tokens // 128 + 3) * 128 * 64)
-    cache.quantize_append(0, *W.tokens(w, 0, 0, tokens, device="cuda"))
+@pytest.mark.parametrize("name,batch,tokens,preset,v_bits,straddles", [
+    ("llama8b", 9, 3000, "P24", 2, False), ("llama8b", 12, 4000, "P27", 2, False), ("llama8b", 16, 2000, "P4BASE", 2, False), ("llama8b", 18, 2000, "P24", 2, False),
+    ("llama8b", 20, 3000, "P24", 2, True), ("llama8b", 14, 10000, "P24", 2, True), ("llama8b", 14, 6000, "P24", 4, True), ("qwen7b", 19, 12000, "P27", 2, True),
+    ("llama8b", 16, 10000, "P4BASE", 2, True),
+])
+def test_split_that_straddles_streams(binding, name, batch, tokens, preset, v_bits, straddles):
+    """Stream counts that leave many CTA slots idle at a whole number of CTAs per stream: all slots are used and CTAs straddle streams where
+    the streams are long enough for it; shorter ones keep a whole number."""
+    w = W.small(W.CONFIGS[name], n_layers=1, batch=batch, tokens=tokens, **getattr(W, preset))
+    cache = U.make_cache(binding, w, v_bits=v_bits, extras_budget_bytes=(tokens // 128 + 3) * 128 * 64)
+    for t in range(0, tokens, 4096):
+        cache.quantize_append(0, *W.tokens(w, 0, t, min(4096, tokens - t), device="cuda"))
     q = W.decode_query(w, 0, 0, device="cuda")
     out = cache.decode_attention(0, q, W.softmax_scale())
+    assert (cache.last_attention_ctas() % (batch * w.n_kv_heads) != 0) == straddles
     cache.set_attention_kernel(1)
     ref = cache.decode_attention(0, q, W.softmax_scale())
     assert cache.status() == 0
