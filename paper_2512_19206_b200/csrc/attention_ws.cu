@@ -118,10 +118,11 @@ __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp
 // per channel pair, gathered), 2 = 4-bit base (dense high plane)
 // kV4: 4-bit values (a second plane of 2-bit value codes per unit, scale 4 s_v)
 // kDirect: one CTA per stream, which writes the output (and the log-denominators) instead of a partial
+// (q without __restrict__: a direct call that rotates writes the rows that it reads)
 // kRope: the step rotates (kernels of their own: the others have no registers to spare for it)
 template <int G, int kU4, bool kV4, bool kDirect, bool kRope>
 __global__ void __launch_bounds__(threads_of(kU4, kV4), kCtasPerSm)
-attention_ws_kernel(LayerView lv, const __nv_bfloat16* __restrict__ q, float scale_log2e, float* __restrict__ ws,
+attention_ws_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, float* __restrict__ ws,
                     uint32_t four2, float* __restrict__ out, float* __restrict__ lse_out) {
   constexpr int VG = kD / G;              // value groups per token
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group

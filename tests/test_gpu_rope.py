@@ -72,8 +72,8 @@ def test_bulk_then_decode_steps_with_rotation(binding, layout):
 
 
 @pytest.mark.parametrize("name,batch,tokens,preset,lens,sink", [
-    ("qwen7b", 1, 20, "P24", None, 0),                  # the split kernel writes the output itself, eight pairs
-    ("llama8b", 20, 300, "P24", None, 0),               # the same with four pairs
+    ("qwen7b", 1, 20, "P24", None, 0),                  # the split kernel writes the output itself, four pairs
+    ("llama8b", 20, 300, "P24", None, 0),               # the same with more streams than SMs
     ("qwen32b", 32, 1500, "P27", None, 0),              # the same, two units per step
     ("qwen7b", 1, 1000, "P27", None, 0),                # merge: a CTA per head
     ("qwen7b", 8, 6000, "P4BASE", None, 0),             # the same, two logits warps
@@ -95,6 +95,42 @@ def test_step_that_rotates_equals_rotation_append_and_attention(binding, name, b
         assert torch.equal(out, caches[1].decode_attention(0, b[2].view(batch, w.n_q_heads, 128), W.softmax_scale()))
         assert all(torch.equal(x, y) for x, y in zip(a, b))
     for s in (0, batch * w.n_kv_heads - 1):
+        assert caches[0].stream_regions(0, s) == caches[1].stream_regions(0, s)
+    assert caches[0].status() == caches[1].status() == 0
+
+
+@pytest.mark.parametrize("name,batch,tokens,preset,R,G,v_bits,sink,form,straddles", [
+    ("qwen7b", 1, 300, "P24", 128, 32, 2, 0, 1 + 4 + 32, False),       # eight pairs of warps
+    ("qwen7b", 16, 511, "P4BASE", 128, 64, 4, 0, 1 + 4 + 32, False),
+    ("qwen7b", 8, 300, "P27", 128, 128, 2, 32, 1 + 4 + 32, False),
+    ("llama8b", 3, 1000, "P27", 32, 32, 4, 0, 1, False),               # one unit per step, blocks of one unit
+    ("qwen7b", 2, 700, "P24", 128, 32, 2, 64, 1, False),               # a filled sink
+    ("qwen7b", 4, 1000, "P4BASE", 128, 128, 2, 0, 1, False),
+    ("llama8b", 20, 3000, "P24", 128, 32, 2, 0, 2, True),              # CTAs that straddle two streams
+    ("llama8b", 14, 6000, "P24", 128, 64, 4, 0, 2, True),
+    ("llama8b", 40, 700, "P27", 128, 32, 2, 0, 2, True),               # CTAs with several streams
+    ("llama8b", 40, 700, "P24", 64, 32, 4, 0, 1, True),
+    ("qwen7b", 8, 6000, "P27", 128, 128, 4, 0, 2, False),              # two units per step
+    ("qwen32b", 32, 1500, "P4BASE", 256, 128, 2, 32, 2 + 4, False),    # the same, output written by the split kernel
+])
+def test_step_that_rotates_in_every_form_of_the_split_kernel(binding, name, batch, tokens, preset, R, G, v_bits, sink, form, straddles):
+    """Bit for bit the rotation, the append and the attention as calls of their own; a second step rotates again from the caller's rows."""
+    w = W.small(W.CONFIGS[name], n_layers=1, batch=batch, tokens=tokens, residual_len=R, group_size=G, **getattr(W, preset))
+    cos, sin = [torch.from_numpy(x).cuda() for x in tables(tokens + 8)]
+    caches = [U.make_cache(binding, w, sink_len=sink, v_bits=v_bits, extras_budget_bytes=(tokens // R + 4) * R * 128) for _ in range(2)]
+    for t in range(0, tokens, 2048):
+        kvq = W.tokens(w, 0, t, min(2048, tokens - t), device="cuda")
+        for c in caches:
+            c.quantize_append(0, *kvq)
+    for step in range(2):
+        a, b = [[x.contiguous().clone() for x in W.tokens(w, 0, tokens + step, 1, device="cuda")] for _ in range(2)]
+        out = caches[0].rope_decode_step(0, *a, cos, sin, tokens + step, W.softmax_scale())
+        assert caches[0].last_attention() & ~binding.ATTN_EARLY == form
+        assert (caches[0].last_attention_ctas() % (batch * w.n_kv_heads) != 0) == straddles
+        caches[1].rope_append(0, *b, cos, sin, tokens + step)
+        assert torch.equal(out, caches[1].decode_attention(0, b[2].view(batch, w.n_q_heads, 128), W.softmax_scale()))
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
+    for s in (0, batch * w.n_kv_heads // 2, batch * w.n_kv_heads - 1):
         assert caches[0].stream_regions(0, s) == caches[1].stream_regions(0, s)
     assert caches[0].status() == caches[1].status() == 0
 
