@@ -119,8 +119,7 @@ __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp
 // kV4: 4-bit values (a second plane of 2-bit value codes per unit, scale 4 s_v)
 // kDirect: one CTA per stream, which writes the output (and the log-denominators) instead of a partial
 // (q without __restrict__: a direct call that rotates writes the rows that it reads)
-// kRope: the step rotates (kernels of their own: the others have no registers to spare for it)
-template <int G, int kU4, bool kV4, bool kDirect, bool kRope>
+template <int G, int kU4, bool kV4, bool kDirect>
 __global__ void __launch_bounds__(threads_of(kU4, kV4), kCtasPerSm)
 attention_ws_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, float* __restrict__ ws,
                     uint32_t four2, float* __restrict__ out, float* __restrict__ lse_out) {
@@ -422,24 +421,27 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, flo
     const int jn = f_r - 1;
     // ---- query of this stream: bf16 and fp16 tables (heads >= g are zero rows)
     {
-      // thread (h, c) of the first 128: head h, channels 8c .. 8c+7; the next 16 (h = 8): the new key of a step that rotates
-      uint4 q_regs = make_uint4(0u, 0u, 0u, 0u);
-      const int b = s / lv.Hkv, hk = s % lv.Hkv, h = threadIdx.x >> 4, c = threadIdx.x & 15;
-      const uint4* row = h < g ? reinterpret_cast<const uint4*>(q + ((size_t)b * lv.Hq + hk * g + h) * kD)
-                               : (kRope && h == 8 ? reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD) : nullptr);
-      if (row != nullptr) {
-        q_regs = row[c];
-        if (kRope) q_regs = rotate_chunk(q_regs, row[c ^ 8], lv.rope_cos, lv.rope_sin, c);
-      }
-      __syncthreads();          // the previous segment's readers of the tables are done, and so are the rotation's reads
-      if (kRope && kDirect && row != nullptr) const_cast<uint4*>(row)[c] = q_regs;      // (no other CTA reads them)
-      if (kRope && h == 8 && jn >= 32 * res_b && jn < 32 * res_e)      // this CTA has the new key's unit and reads it from the window
-        reinterpret_cast<uint4*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[c] = q_regs;
+      uint4 q_regs = make_uint4(0u, 0u, 0u, 0u);      // thread (h, c) of the first 128: head h, channels 8c .. 8c+7
+      const size_t row0 = (size_t)s * g;              // (b Hkv + hk) g = b Hq + hk g
+      const int h = threadIdx.x >> 4, c = threadIdx.x & 15;
+      if (h < g) q_regs = reinterpret_cast<const uint4*>(q + (row0 + h) * kD)[c];
+      RopeInput rope_in{};
+      if (lv.rope_cos != nullptr) rope_in = rope_request<kThreads>(lv, s);
+      __syncthreads();          // the previous segment's readers of the tables are done
       if (h < 8) {
         sts128(qb16_u32 + (h * kQS + 8 * c) * 2, q_regs.x, q_regs.y, q_regs.z, q_regs.w);
         if (kU4 == 1)      // the fp16 table is for the gathered UINT4 channels
           sts128(qf16_u32 + (h * kQS + 8 * c) * 2, bf16x2_to_f16x2(q_regs.x), bf16x2_to_f16x2(q_regs.y),
                  bf16x2_to_f16x2(q_regs.z), bf16x2_to_f16x2(q_regs.w));
+      }
+      if (lv.rope_cos != nullptr) {
+        __syncthreads();
+        // the CTA with the new key's unit reads the rotated key from the window; where the CTA has the whole stream nobody else reads
+        // the caller's rows, and it leaves them rotated
+        rope_rotate<kThreads, kQS, kU4 == 1>(
+            lv, s, g, rope_in, qb16_u32, qf16_u32,
+            jn >= 32 * res_b && jn < 32 * res_e ? reinterpret_cast<uint16_t*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256) : nullptr,
+            kDirect ? reinterpret_cast<uint16_t*>(const_cast<__nv_bfloat16*>(q)) + row0 * kD : nullptr);
       }
       __syncthreads();
     }
@@ -471,8 +473,8 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, flo
           const int ta = j0 + mt * 16 + r, tb = ta + 8;
           const uint4* rowa = reinterpret_cast<const uint4*>(resk + (size_t)ta * 256);
           const uint4* rowb = reinterpret_cast<const uint4*>(resk + (size_t)tb * 256);
-          if (!kRope && holds_new && ta == jn) rowa = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
-          if (!kRope && holds_new && tb == jn) rowb = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
+          if (holds_new && lv.rope_cos == nullptr && ta == jn) rowa = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
+          if (holds_new && lv.rope_cos == nullptr && tb == jn) rowb = reinterpret_cast<const uint4*>(lv.new_k + (size_t)s * kD);
           uint4 ka[4], kb[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
@@ -766,7 +768,7 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, flo
       if (takes_new) {
         // store the new key row and add |q| to the importance accumulator (channels 4*lane .. 4*lane+3, heads
         // ascending: the order of the plain append)
-        if (!kRope) {
+        if (lv.rope_cos == nullptr) {
           const uint2 kn = reinterpret_cast<const uint2*>(lv.new_k + (size_t)s * kD)[lane];
           reinterpret_cast<uint2*>(lv.resk + (size_t)s * lv.resk_stride + (size_t)jn * 256)[lane] = kn;
         }
@@ -1160,14 +1162,9 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, flo
   }
 }
 
-template <int G, int kU4, bool kV4, bool kDirect, bool kRope>
-cudaError_t launch_r(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
-  return launch_dependent(attention_ws_kernel<G, kU4, kV4, kDirect, kRope>, dim3((unsigned)grid), threads_of(kU4, kV4), smem_bytes(G, kU4, kV4), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
-}
 template <int G, int kU4, bool kV4, bool kDirect>
 cudaError_t launch_d(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
-  return lv.rope_cos != nullptr ? launch_r<G, kU4, kV4, kDirect, true>(lv, qb, sl, ws, grid, out, lse, stream)
-                                : launch_r<G, kU4, kV4, kDirect, false>(lv, qb, sl, ws, grid, out, lse, stream);
+  return launch_dependent(attention_ws_kernel<G, kU4, kV4, kDirect>, dim3((unsigned)grid), threads_of(kU4, kV4), smem_bytes(G, kU4, kV4), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
 }
 template <int G, int kU4, bool kV4>
 cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
@@ -1193,17 +1190,14 @@ cudaError_t launch_g(const LayerView& lv, const void* q, float scale, float* ws,
 
 }  // namespace
 
-template <int G, int kU4, bool kV4, bool kDirect, bool kRope>
-static cudaError_t setup_r() {
-  cudaError_t e = cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect, kRope>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(G, kU4, kV4));
-  if (e != cudaSuccess) return e;
-  // the CTAs of an SM only fit with the largest shared-memory carve-out; ask for it explicitly
-  return cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect, kRope>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-}
 template <int G, int kU4, bool kV4, bool kDirect>
 static cudaError_t setup_d() {
-  const cudaError_t e = setup_r<G, kU4, kV4, kDirect, false>();
-  return e == cudaSuccess ? setup_r<G, kU4, kV4, kDirect, true>() : e;
+  cudaError_t e = cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem_bytes(G, kU4, kV4));
+  if (e != cudaSuccess) return e;
+  // the CTAs of an SM only fit with the largest shared-memory carve-out; ask for it explicitly
+  return cudaFuncSetAttribute(attention_ws_kernel<G, kU4, kV4, kDirect>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                              (int)cudaSharedmemCarveoutMaxShared);
 }
 template <int G, int kU4, bool kV4>
 static cudaError_t setup_v() {

@@ -115,12 +115,16 @@ __device__ inline float stored_scale(float mx, float mn, float levels) {
   return __uint_as_float(b);
 }
 
-// Rotary embedding of 8 channels of a row (Appendix D: importance scores and keys are taken after the rotation): channel pairing
-// (i, i + 64) ("rotate-half"), with c = cos[p][i], s = sin[p][i] from the caller's tables
+// Rotary embedding (Appendix D: importance scores and keys are taken after the rotation): channel pairing (i, i + 64)
+// ("rotate-half"), with c = cos[p][i], s = sin[p][i] from the caller's tables
 //   y[i] = x[i] c - x[i + 64] s,   y[i + 64] = x[i + 64] c + x[i] s
 // Every product and the sum are single fp32 operations rounded to nearest (no fused multiply-add), and the result is rounded to bf16
-// (nearest, ties to even): the rotated bits are a defined function of the inputs and the tables.  `own` holds channels 8 chunk ..
-// 8 chunk + 7, `other` those 64 away.
+// (nearest, ties to even): the rotated bits are a defined function of the inputs and the tables.
+__device__ inline float rotate_one(float own, float other, float c, float s, bool first_half) {
+  const float p = __fmul_rn(own, c), m = __fmul_rn(other, s);
+  return first_half ? __fsub_rn(p, m) : __fadd_rn(p, m);
+}
+// 8 channels of a row: `own` holds channels 8 chunk .. 8 chunk + 7, `other` those 64 away.
 __device__ inline uint4 rotate_chunk(uint4 own, uint4 other, const float* cos_row, const float* sin_row, int chunk) {
   const float4* cp = reinterpret_cast<const float4*>(cos_row + 8 * (chunk & 7));
   const float4* sp = reinterpret_cast<const float4*>(sin_row + 8 * (chunk & 7));
@@ -133,11 +137,9 @@ __device__ inline uint4 rotate_chunk(uint4 own, uint4 other, const float* cos_ro
   for (int j = 0; j < 4; ++j) {
     float r[2];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const float p = __fmul_rn(bf16_bits_to_float(e ? a[j] >> 16 : a[j] & 0xFFFFu), cs[2 * j + e]);
-      const float m = __fmul_rn(bf16_bits_to_float(e ? b[j] >> 16 : b[j] & 0xFFFFu), sn[2 * j + e]);
-      r[e] = chunk < 8 ? __fsub_rn(p, m) : __fadd_rn(p, m);
-    }
+    for (int e = 0; e < 2; ++e)
+      r[e] = rotate_one(bf16_bits_to_float(e ? a[j] >> 16 : a[j] & 0xFFFFu), bf16_bits_to_float(e ? b[j] >> 16 : b[j] & 0xFFFFu), cs[2 * j + e],
+                        sn[2 * j + e], chunk < 8);
     const __nv_bfloat162 h = __floats2bfloat162_rn(r[0], r[1]);
     y[j] = *reinterpret_cast<const uint32_t*>(&h);
   }

@@ -172,5 +172,68 @@ __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 
 // two bf16 in one word -> two fp16 in one word (exact inside the fp16 range)
 __device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t w) { return pack_half2(bf_lo(w), bf_hi(w)); }
 
+// ---- The rotation of a fused decode step, on the query rows in shared memory.  A thread has one channel pair (i, i + 64) of every
+// kThreads / 64-th row, one row behind another, so that it needs hardly any registers: rotated 16 bytes at a time on the way from global
+// memory to the table, the main loops of a third of the kernels spilled, and the step without rotation needed kernels of its own.
+// us per decode step, so / here: three tiers, 7b shape, 8 x 20011 tokens, 14 layers, rotating 497 / 487; 8 x 32768, not rotating 730 / 710;
+// two tiers, 28 layers, not rotating 1056 / 1045; one sequence of 1024 tokens, 28 layers, rotating 177 / 174, not 159 / 155.
+struct RopeInput {
+  float c, s;               // of the thread's channel pair
+  uint32_t k0, k1;          // the pair of the new key (the last 64 threads)
+};
+template <int kThreads>
+__device__ __forceinline__ RopeInput rope_request(const LayerView& lv, int s) {
+  static_assert(kThreads % 64 == 0, "a thread keeps its channel pair");
+  const int i = threadIdx.x & 63;
+  RopeInput in{lv.rope_cos[i], lv.rope_sin[i], 0u, 0u};
+  if ((int)threadIdx.x >= kThreads - 64) {
+    in.k0 = lv.new_k[(size_t)s * kD + i];
+    in.k1 = lv.new_k[(size_t)s * kD + i + 64];
+  }
+  return in;
+}
+// Rotates the g rows of the table at qb16 (kStride halves apart; their fp16 copies at qf16 if kHalf) and the new key, which goes to
+// key_row, its place in the residual window, unless that is null.  out_q: the rows in the caller's tensor, to be left rotated as the
+// key there is (null: the merge does that).
+template <int kThreads, int kStride, bool kHalf>
+__device__ __forceinline__ void rope_rotate(const LayerView& lv, int s, int g, const RopeInput& in, uint32_t qb16, uint32_t qf16, uint16_t* key_row,
+                                            uint16_t* out_q) {
+  const int i = threadIdx.x & 63;
+  auto pair = [&](uint32_t& lo, uint32_t& hi) {
+    const float x0 = bf16_bits_to_float(lo), x1 = bf16_bits_to_float(hi);
+    lo = pack_bf162(rotate_one(x0, x1, in.c, in.s, true), 0.f) & 0xFFFFu;
+    hi = pack_bf162(rotate_one(x1, x0, in.c, in.s, false), 0.f) & 0xFFFFu;
+  };
+#pragma unroll 1
+  for (int h = threadIdx.x >> 6; h < g; h += kThreads / 64) {
+    const uint32_t at = qb16 + (h * kStride + i) * 2;
+    uint32_t lo = lds16(at), hi = lds16(at + 128);
+    pair(lo, hi);
+    sts16(at, lo);
+    sts16(at + 128, hi);
+    if (kHalf) {
+      sts16(qf16 + (h * kStride + i) * 2, bf16x2_to_f16x2(lo));
+      sts16(qf16 + (h * kStride + i) * 2 + 128, bf16x2_to_f16x2(hi));
+    }
+    if (out_q != nullptr) {
+      out_q[h * kD + i] = (uint16_t)lo;
+      out_q[h * kD + i + 64] = (uint16_t)hi;
+    }
+  }
+  if ((int)threadIdx.x >= kThreads - 64) {
+    uint32_t lo = in.k0, hi = in.k1;
+    pair(lo, hi);
+    if (key_row != nullptr) {
+      key_row[i] = (uint16_t)lo;
+      key_row[i + 64] = (uint16_t)hi;
+    }
+    if (out_q != nullptr) {
+      uint16_t* out_k = const_cast<uint16_t*>(lv.new_k) + (size_t)s * kD;
+      out_k[i] = (uint16_t)lo;
+      out_k[i + 64] = (uint16_t)hi;
+    }
+  }
+}
+
 }  // namespace
 }  // namespace mixkvq
