@@ -21,7 +21,6 @@ enum Tier : uint8_t { kU2 = 0, kU4 = 1, kBF16 = 2 };
 // Geometry + pointers of one layer, passed by value to every kernel.
 constexpr int kMaxRaggedBatch = 128;   // sequences of a batch whose fills may differ
 
-// (Its size is host time of every launch: one sequence of 1024 tokens, attention alone, 5.1 us of the host per call with 296 bytes, 5.5 with 312.)
 struct LayerView {
   // geometry
   int B, Hq, Hkv, g;          // batch, query heads, KV heads, GQA group size
@@ -33,8 +32,9 @@ struct LayerView {
   int8_t score_bits, importance_mode;
   int8_t v_bits;              // 2, or 4: a second plane of 2-bit value codes follows the value scales in every unit
   // decode attention may stage its first packed units before it waits for the kernel launched before it: set by the
-  // host when that kernel did not write this layer's packed blocks
-  int8_t stage_early;
+  // host when that kernel did not write this layer's packed blocks.  (A whole word: as a byte it is widened into a register that the
+  // split kernels keep, and most instantiations of the one-unit kernel spilled 8 to 12 bytes more: 5 x 1668 tokens, 4-bit base, 302.6 / 296.5 us.)
+  int stage_early;
   uint32_t base_bytes, unit_bytes;
   uint64_t extras_budget;     // bytes per stream
   // method parameters
