@@ -49,11 +49,13 @@ __device__ __forceinline__ void rope_store(const RopeWork& w) {
   if (w.at != nullptr) *w.at = w.y;
 }
 
-template <bool kRope>
+// (Rope: nothing, or the RopeRows of a step that rotates: the other merges do not carry its parameters)
+template <typename... Rope>
 __global__ void __launch_bounds__(kCombineMaxWarps * 32)
 combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int Hkv, int Hq, int mode, int n,
                long long units_per_stream, int S, const int4* __restrict__ seq, const int* __restrict__ seq_prefix,
-               float* __restrict__ lse_out, bool early, RopeRows rope) {
+               float* __restrict__ lse_out, bool early, Rope... rope) {
+  constexpr bool kRope = sizeof...(Rope) > 0;
   __shared__ float mlS[kCombineMaxWarps][2];
   __shared__ __align__(16) float oS[kCombineMaxWarps][kD];
   if (early) let_successor_start();
@@ -80,7 +82,9 @@ combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int
   }
   dependency_wait();
   RopeWork rotated{};
-  if (kRope && warp == W - 1) rotated = rope_load(rope, ((size_t)(s / Hkv) * Hq + (s % Hkv) * g + h), s, h, lane);
+  if constexpr (kRope) {
+    if (warp == W - 1) rotated = rope_load(rope..., ((size_t)(s / Hkv) * Hq + (s % Hkv) * g + h), s, h, lane);
+  }
   // ---- this warp's partials: one pass with a running maximum; a lane has channels 2 lane, 2 lane + 1 and 64 more
   const float* base = ws + (size_t)first * kPartialFloats + h * 130;
   float M = -INFINITY, l = 0.f;
@@ -146,10 +150,11 @@ combine_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int
 // 231.6 us; 32 streams with nine partials 15.7 / 15.9; 16 streams with 18, 37.4 / 37.9).
 constexpr int kRowsChunk = 8, kRowsMaxPartials = 8;
 
-template <bool kRope>
+template <typename... Rope>
 __global__ void __launch_bounds__(256)
 combine_rows_kernel(const float* __restrict__ ws, float* __restrict__ out, int g, int Hkv, int Hq, int n, long long units_per_stream,
-                    int S, float* __restrict__ lse_out, bool early, RopeRows rope) {
+                    int S, float* __restrict__ lse_out, bool early, Rope... rope) {
+  constexpr bool kRope = sizeof...(Rope) > 0;
   if (early) let_successor_start();
   const int s = blockIdx.x, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long total = units_per_stream * S;
@@ -158,7 +163,7 @@ combine_rows_kernel(const float* __restrict__ ws, float* __restrict__ out, int g
   const float* base = ws + (size_t)(c0 + s) * kPartialFloats + h * 130;
   dependency_wait();
   RopeWork rotated{};
-  if (kRope) rotated = rope_load(rope, (size_t)s * g + h, s, h, lane);
+  if constexpr (kRope) rotated = rope_load(rope..., (size_t)s * g + h, s, h, lane);
   float M = -INFINITY, l = 0.f;
   float2 oa = make_float2(0.f, 0.f), ob = make_float2(0.f, 0.f);
   for (int i0 = 0; i0 < count; i0 += kRowsChunk) {
@@ -200,16 +205,19 @@ combine_rows_kernel(const float* __restrict__ ws, float* __restrict__ out, int g
 cudaError_t launch_combine(const float* ws, float* out, int g, int Hkv, int Hq, int mode, int n,
                            long long units_per_stream, int S, cudaStream_t stream, const int4* seq, const int* seq_prefix,
                            float* lse_out, bool early, void* rope_q, void* rope_k, const float* rope_cos, const float* rope_sin) {
-  const RopeRows rope{static_cast<uint16_t*>(rope_q), static_cast<uint16_t*>(rope_k), rope_cos, rope_sin};
-  if (mode == 1 && seq == nullptr && n / S + 2 <= kRowsMaxPartials)
-    return launch_dependent(rope_q != nullptr ? combine_rows_kernel<true> : combine_rows_kernel<false>, dim3((unsigned)S), 32 * g, 0, stream, ws, out, g, Hkv, Hq,
-                            n, units_per_stream, S, lse_out, early, rope);
+  const bool rows = mode == 1 && seq == nullptr && n / S + 2 <= kRowsMaxPartials;
   // eight warps when four with a chunk each do not cover a stream's partials in one round trip (a ragged batch may give
   // nearly all CTAs to one sequence), four otherwise: more warps only lengthen the last step
   const int partials = mode == 0 ? n : (seq != nullptr ? n : n / S + 1);
-  return launch_dependent(rope_q != nullptr ? combine_kernel<true> : combine_kernel<false>, dim3((unsigned)(S * g)),
-                          partials > 4 * kCombineChunk ? kCombineMaxWarps * 32 : 128, 0, stream, ws, out, g, Hkv, Hq, mode, n, units_per_stream, S, seq,
-                          seq_prefix, lse_out, early, rope);
+  auto launch = [&](auto... rope) {
+    if (rows)
+      return launch_dependent(combine_rows_kernel<decltype(rope)...>, dim3((unsigned)S), 32 * g, 0, stream, ws, out, g, Hkv, Hq, n, units_per_stream, S, lse_out,
+                              early, rope...);
+    return launch_dependent(combine_kernel<decltype(rope)...>, dim3((unsigned)(S * g)), partials > 4 * kCombineChunk ? kCombineMaxWarps * 32 : 128, 0, stream, ws,
+                            out, g, Hkv, Hq, mode, n, units_per_stream, S, seq, seq_prefix, lse_out, early, rope...);
+  };
+  if (rope_q != nullptr) return launch(RopeRows{static_cast<uint16_t*>(rope_q), static_cast<uint16_t*>(rope_k), rope_cos, rope_sin});
+  return launch();
 }
 
 // The table of a ragged batch, from the host's per-sequence fill (kernel arguments: no copy, ordered in the stream).
