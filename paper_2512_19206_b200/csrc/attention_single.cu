@@ -93,8 +93,8 @@ __device__ __forceinline__ bool is_logits_warp(int warp) { return ((warp ^ (warp
 // (q without __restrict__: a direct call that rotates writes the rows that it reads)
 template <int G, int kU4, bool kV4, bool kDirect, int kPairs>
 __global__ void __launch_bounds__(kPairs * 64, kPairsPerSm / kPairs)
-attention_single_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, float* __restrict__ ws,
-                    uint32_t four2, float* __restrict__ out, float* __restrict__ lse_out) {
+attention_single_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, uint32_t four2, float* __restrict__ ws,
+                    float* __restrict__ out, float* __restrict__ lse_out) {
   constexpr int kThreads = kPairs * 64, kBarBytes = bar_bytes(kPairs);
   constexpr int VG = kD / G;              // value groups per token
   constexpr int TPG = 8 / VG;             // 16-channel tiles per value group
@@ -1203,7 +1203,7 @@ attention_single_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e,
 
 template <int G, int kU4, bool kV4, bool kDirect, int kPairs>
 cudaError_t launch_d(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, cudaStream_t stream) {
-  return launch_dependent(attention_single_kernel<G, kU4, kV4, kDirect, kPairs>, dim3((unsigned)grid), kPairs * 64, smem_bytes(kV4, kPairs), stream, lv, qb, sl, ws, 0x44004400u, out, lse);
+  return launch_dependent(attention_single_kernel<G, kU4, kV4, kDirect, kPairs>, dim3((unsigned)grid), kPairs * 64, smem_bytes(kV4, kPairs), stream, lv, qb, sl, 0x44004400u, ws, out, lse);
 }
 template <int G, int kU4, bool kV4>
 cudaError_t launch_v(const LayerView& lv, const __nv_bfloat16* qb, float sl, float* ws, int grid, float* out, float* lse, bool wide, cudaStream_t stream) {

@@ -21,6 +21,8 @@ enum Tier : uint8_t { kU2 = 0, kU4 = 1, kBF16 = 2 };
 // Geometry + pointers of one layer, passed by value to every kernel.
 constexpr int kMaxRaggedBatch = 128;   // sequences of a batch whose fills may differ
 
+// (A launch's parameters are host time: attention alone in one launch, 3.7 us of the host per call with 336 or 344 bytes, 3.4 with the 328 that
+// it, the query, scale, constant, workspace and outputs take in this order of the kernel's parameters.)
 struct LayerView {
   // geometry
   int B, Hq, Hkv, g;          // batch, query heads, KV heads, GQA group size
