@@ -396,12 +396,16 @@ attention_ws_kernel(LayerView lv, const __nv_bfloat16* q, float scale_log2e, uin
       for (uint32_t i = 0, sg = ring_stage; i < (uint32_t)kStages; ++i, sg = next_stage(sg)) issue(sg, i == 0);
     }
     if (to_request > 0 && lv.stage_early) request_first();
-    // The query rows, the step's token and the segment's unquantized units are requested into the L2 cache before the wait (a request has no
-    // other effect, whatever the kernel before this one still writes): of a model's many layers they have left it since the step before.
-    // us per decode step without / with: 7b shape, 8 x 32768 tokens, 28 layers 1103 / 1075, 4 x 120000, 8 layers 521 / 509, ragged 826 / 814;
-    // three tiers, 8 x 20011, 14 layers 498 / 504.  (By the values warps alone, which refill the rings: no gain.)  Only for a CTA's first
-    // segment: the others come long behind the wait.
-    if (lv.seq != nullptr || !dep_waited) {
+    // Two tiers, G = 32, split streams: the query rows, the step's token and the segment's unquantized units are requested into the L2 cache
+    // before the wait (a request has no other effect, whatever the kernel before this one still writes): of a model's many layers they have
+    // left it since the step before.  Only ahead of a wait: not for a CTA's later segments, nor in a ragged batch, whose table is read behind it.
+    // us per decode step, without / with: 7b shape, 8 x 32768 tokens, 28 layers 1062 / 1047, 4 x 120000, 8 layers 503 / 493, 32b shape, 64 x
+    // 8000, 6 layers 779 / 771, 64 x 1500 250 / 253.  (Not all of it is the requests': a ragged batch, which makes none, takes 799 / 791 in the
+    // two builds of the kernel.)  Elsewhere it delays what goes out first or gives nothing: three tiers, 7b shape, 8 x 32768, 14 layers 700 / 709; 4-bit
+    // base, G = 128, 8 x 38643, 4 layers 220.6 / 221.4; two tiers, G = 128, 32b shape, 64 x 32768, 3 layers 1266 / 1287, G = 64, 7b shape, 16 x 12000,
+    // 14 layers 427 / 430; one CTA per stream, 32b shape, 32 x 2000, 8 layers 176 / 180; one unit per step, 4-bit values, 24 x 1147, 28 layers 364 /
+    // 370, 4 x 6001, 16 layers 251.2 / 250.1.
+    if (kU4 == 0 && G == 32 && !kDirect && !dep_waited) {
       const int b = s / lv.Hkv, hk = s % lv.Hkv, h = threadIdx.x >> 1;
       if (h < g) prefetch_l2(reinterpret_cast<const char*>(q + ((size_t)b * lv.Hq + hk * g + h) * kD) + 128 * (threadIdx.x & 1));
       else if (lv.new_k != nullptr && h < g + 2) prefetch_l2(reinterpret_cast<const char*>((h == g ? lv.new_k : lv.new_v) + (size_t)s * kD) + 128 * (threadIdx.x & 1));
