@@ -1299,11 +1299,14 @@ static bool one_cta_per_stream(const LayerView& lv, int n_sms) {
 }
 
 // Number of CTAs the split kernel runs for this layer state (also the number of partial-slot owners).  With fewer streams than CTA slots
-// a grid that is a multiple of the stream count has no CTA that straddles two streams: a second segment costs a pipeline drain, a
-// query load and a second partial, about 10 positions' time with two tiers and 16 otherwise.  Where that leaves more of the slots idle than
-// the straddling costs, all of them are used.  us per layer, multiple / all slots: 8b shape, batch 16 (128 streams: 256 / 296 CTAs), 4-bit base,
-// 16384 tokens 105.4 / 98.4; 32 streams (288 / 296 CTAs), two tiers, 32768 tokens 39.4 / 40.8, three tiers, 20011 tokens 37.7 / 40.9, 16
-// streams, 120000 tokens 68.5 / 69.0.
+// a grid that is a multiple of the stream count has no CTA that straddles two streams (a second segment costs a pipeline drain, a
+// query load and a second partial), and with one CTA per stream no merge.  All slots are used where that leaves a CTA fewer positions by more
+// than the straddling costs: 26 positions against one CTA per stream, 17 against several, 10 with two tiers and 4-bit values, whose
+// positions take longer.  Time with a multiple over time with all slots, behind the positions saved.  One CTA per stream: two tiers, 160
+// streams 19 .89, 26 1.01, 32 1.03, 224 streams 16 .89, 23 .99, 27 1.015, 37 1.08; three tiers, 224 streams 23 .993, 27 1.05; 4-bit base 23 .973, 27
+// 1.04; 4-bit values 23 .993, 27 1.045.  Two to four per stream: two tiers, 112 streams 11 .92, 15 .95, 19 1.01, 64 streams 9 .91, 17 .998, 60
+// streams 24 1.045; three tiers 15 .97 to .98, 19 1.01 to 1.02; 4-bit base 15 .985, 19 1.014, 36 (128 streams, 16384 tokens) 105.4 / 98.4 us; two tiers
+// with 4-bit values 8 .996, 11 1.01, 19 1.07.
 int attention_ws_grid(const LayerView& lv, int n_sms) {
   const int S = lv.B * lv.Hkv;
   if (lv.seq != nullptr) return lv.seq_ctas;
@@ -1315,7 +1318,8 @@ int attention_ws_grid(const LayerView& lv, int n_sms) {
   int grid = (int)min((long long)min(n_sms * kCtasPerSm, kMaxCtas / 2), wanted);
   if (one_cta_per_stream(lv, n_sms)) grid = min(grid, S);
   if (grid > S) {
-    const int per_stream = grid / S, straddle = three_tiers(lv) || lv.dense_hi ? 16 : 10;
+    const int per_stream = grid / S;
+    const int straddle = per_stream == 1 ? 26 : (lv.v_bits == 4 && !three_tiers(lv) && !lv.dense_hi ? 10 : 17);
     if ((attention_ws_positions(lv) + per_stream - 1) / per_stream <= (total + grid - 1) / grid + straddle) grid = per_stream * S;
   }
   return grid < 1 ? 1 : grid;
