@@ -1355,10 +1355,13 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // tokens 7.3 us against 5.6; 7b shape 41.1 against 40.7).
   const bool whole = out != nullptr && lv.seq == nullptr && grid == S;
   float* const kernel_out = whole ? out : nullptr;
-  // ... with eight pairs of warps where every stream has an SM to itself.  us per layer, four / eight pairs: 4 streams of the 7b shape, two
-  // tiers, 300 tokens 5.5 / 5.1; 64 streams, three tiers 7.7 / 6.7, 4-bit base 7.4 / 6.1, 128 streams of the 8b shape, 400 tokens 9.1 / 7.8.  With
-  // fewer positions the larger CTAs cost more: 128 streams, 200 tokens (13 positions) 7.7 / 8.05; requests of 27 and of 54 tokens 5 to 9 % slower.
-  const bool wide = whole && grid <= n_sms && (Us > 13 || (Us == 13 && 2 * grid <= n_sms));
+  // ... with eight pairs of warps where every stream has an SM to itself and four pairs would take several units each.  us per layer, four /
+  // eight pairs: 4 streams of the 7b shape, 13 positions (4 packed, 3 unquantized units) 4.6 / 4.3, three tiers 5.7 / 4.6, 20 positions 6.0 / 5.5; 144 streams
+  // of the 8b shape, 13 6.4 / 6.3, three tiers 9.2 / 7.4, 4-bit base 7.9 / 6.9, 20 8.2 / 8.2, 10.1 / 9.5, 10.0 / 9.1.  At most 12 positions are at most one unit per pair
+  // beside the unquantized ones, and the larger CTA costs more: 9 positions, 4 streams 3.9 / 4.2, 144 streams 5.0 / 5.9.  So it is with most SMs in use
+  // and two tiers up to one packed and one unquantized unit per pair (144 streams, 16 positions 7.2 / 7.7; 64 streams 5.5 / 5.3).
+  const bool one_each = lv.n_blocks * lv.U <= 4 && Us <= 16;
+  const bool wide = whole && grid <= n_sms && Us > 12 && !(one_each && 2 * grid > n_sms && !lv.dense_hi && !three_tiers(lv));
   if (form)
     *form = (by_two ? MIXKVQ_ATTN_TWO_UNITS : MIXKVQ_ATTN_ONE_UNIT) | (whole ? MIXKVQ_ATTN_DIRECT : 0) | (lv.stage_early ? MIXKVQ_ATTN_EARLY : 0) |
             (wide && !by_two ? MIXKVQ_ATTN_EIGHT_PAIRS : 0);

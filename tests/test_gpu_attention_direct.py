@@ -45,6 +45,8 @@ def test_direct_output(binding, name, batch, tokens, R, preset):
 @pytest.mark.parametrize("name,batch,tokens,preset,v_bits,form", [
     ("qwen7b", 1, 200, "P27", 4, 1 + 4 + 32), ("llama8b", 1, 450, "P24", 2, 1 + 4 + 32), ("llama8b", 1, 560, "P24", 2, 1), ("qwen7b", 16, 511, "P4BASE", 2, 1 + 4 + 32),
     ("qwen7b", 16, 1152, "P27", 2, 2), ("llama8b", 16, 1000, "P24", 4, 1 + 4 + 32), ("llama8b", 18, 200, "P24", 2, 1 + 4), ("llama8b", 19, 700, "P27", 2, 2 + 4),
+    ("llama8b", 18, 249, "P24", 2, 1 + 4), ("llama8b", 16, 249, "P27", 2, 1 + 4 + 32), ("qwen7b", 1, 383, "P24", 2, 1 + 4 + 32), ("llama8b", 16, 639, "P4BASE", 4, 1 + 4 + 32),
+    ("qwen7b", 8, 249, "P24", 4, 1 + 4 + 32),
 ])
 def test_eight_pairs_per_stream(binding, name, batch, tokens, preset, v_bits, form):
     """One CTA of eight warp pairs per stream while every stream has an SM to itself, on both sides of where that ends (148 SMs: 18
