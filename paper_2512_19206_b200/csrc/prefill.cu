@@ -248,10 +248,10 @@ __device__ __forceinline__ void add_output(uint32_t o_addr, float (&sum_o)[128])
 
 // One 128-key tile of one row group's softmax.  The thread owns one row of S (128 fp32 columns of its tensor-memory lane at
 // s_addr) and of the last product P V (at o_addr), which goes to its sum.  Writes P (fp16 pairs) over columns [0, 64) of S.  kDiag: the
-// tile on the diagonal: the thread's row sees the columns <= last, the warp's rows all see those <= warp_first and none those >
-// warp_last; the product takes the pieces of 16 keys below n_write (rows that see none of a piece have zeros there).
+// tile on the diagonal: the thread's row sees the columns <= last, none of the warp's rows sees those > warp_last; the product takes the
+// pieces of 16 keys below n_write (rows that see none of a piece have zeros there).
 template <bool kDiag>
-__device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, int warp_first, int warp_last, int last, int n_write, bool first, float scale_log2e,
+__device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, int warp_last, int last, int n_write, bool first, float scale_log2e,
                                              float& m_ref, float& l_run, uint32_t half_bar, float (&sum_o)[128]) {
   if (!first) add_output(o_addr, sum_o);             // the product of the tile before
   // ---- the row's maximum
@@ -368,11 +368,12 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   int issued = 0;                  // K and V tiles requested (the copying thread)
+  // (test hooks: the barrier of the first key tile, or of the last value tile where that is odd or the prompt's last, can be armed for
+  // more bytes than arrive, so that it never completes.  Not of every last value tile: some CTAs end as usual beside those that give up.)
+  const int armed_v = (n & 1) == 0 || n == n_tiles ? n - 1 : -1;
   auto copy_tile = [&](int j, bool keys) {
     const int st = j & 1, full = (keys ? kKFull : kVFull) + st;
-    // (test hooks: the barrier of the first key tile, or of the last value tile where that is odd or the prompt's last, can be armed for
-    // more bytes than arrive, so that it never completes)
-    mbar_expect_tx(bar(full), kTileBytes + (keys ? (j == 0 ? debug_extra_tx : 0u) : (j == n - 1 && ((j & 1) || j == n_tiles - 1) ? debug_extra_v : 0u)));
+    mbar_expect_tx(bar(full), kTileBytes + (keys ? (j == 0 ? debug_extra_tx : 0u) : (j == armed_v ? debug_extra_v : 0u)));
     bulk_copy(smem_u32((keys ? Ks : Vs) + st * kTileBytes), (keys ? ktg : vtg) + (size_t)j * kTileBytes, kTileBytes, bar(full));
   };
   if (tid == 9 * 32) {
@@ -545,13 +546,13 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
 #pragma unroll 1
     for (; j + 1 < n_g; ++j) {
       if (!s_ready()) break;
-      softmax_tile<false>(s_addr, o_addr, 0, 0, 0, 8, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
+      softmax_tile<false>(s_addr, o_addr, 0, 0, 8, j == 0, scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
       p_ready();
     }
     if (n_g > 0 && !dead && s_ready()) {       // the tile on the diagonal
       const Rows at = rows_again();
       const int r = g * kTile + (tid & 127), c0 = j * kTile;
-      softmax_tile<true>(s_addr, o_addr, at.token(r & ~31) - c0, at.token(r | 31) - c0, at.token(r) - c0, (at.token(g * kTile + 127) - c0 + 16) >> 4, j == 0,
+      softmax_tile<true>(s_addr, o_addr, at.token(r | 31) - c0, at.token(r) - c0, (at.token(g * kTile + 127) - c0 + 16) >> 4, j == 0,
                          scale_log2e, m_ref, l_run, bar(kPHalf + g), sum_o);
       p_ready();
     }

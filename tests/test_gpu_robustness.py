@@ -127,8 +127,9 @@ def test_a_wait_that_runs_out_with_more_steps_than_stages(binding, name, batch, 
 
 
 def test_a_prefill_wait_for_the_last_values_that_runs_out(binding):
-    """Every CTA's last value tile never arrives: the rows that need its product are left unwritten (those of the second 128 of a
-    CTA's 256, and of a last CTA with one tile more than the one before), all others are right."""
+    """A CTA's last value tile never arrives where its number is odd or it is the prompt's last: tiles 1, 3 and 4 of the five.  A row tile
+    holds the heads of neighbouring tokens, whose last key tile is the one that they lie in: the rows of the tokens in those tiles need
+    the missing product and are left unwritten, all others are right."""
     w = W.small(W.CONFIGS["qwen7b"], n_layers=1, batch=1, tokens=600, **W.P24)
     k, v, q = [t.cuda() for t in W.tokens(w, 0, 0, 600)]
     cache = U.make_cache(binding, w)
