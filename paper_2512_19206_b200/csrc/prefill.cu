@@ -25,13 +25,15 @@
 // 8192 / 32768 / 65536 tokens: 3.8e-5 / 3.8e-5 / 10.4e-5 / 17.8e-5 accumulated in tensor memory (bias -1.4e-4 at 32768);
 // 3.8e-5 / 2.8e-5 / 2.8e-5 / 2.8e-5 with the sum in registers, the rounding of P.  Sums over 2, 4, 8 or 16 tiles in tensor memory: 2.83,
 // 2.85, 2.91, 3.09e-5 at 32768, and no faster than 2 % (the registers cost the time, not the additions).
-// B200, whole call per layer (us), sum in tensor memory / in registers: prompt of 32768 tokens (7b shape) 6492 / 6811, 8192: 530 /
-// 558, 333: 29.4 / 29.5; 4 x 777 tokens (8b shape) 100.7 / 103.5.  (Waiting for each product right behind its issue, and with the tensor
-// core idle meanwhile: 7447, 699, 104, 169.)  Tensor memory is read 16
-// columns at a time, the next 16 in flight: blocks of 32 registers beside the 128 of the sum spilled 96 to 356 bytes, whatever the split.
+// B200, whole call per layer (us), sum in tensor memory / in registers, both with 256 rows of one head per CTA: prompt of 32768 tokens (7b
+// shape) 6492 / 6811, 8192: 530 / 558, 333: 29.4 / 29.5; 4 x 777 tokens (8b shape) 100.7 / 103.5.  (Waiting for each product right behind its
+// issue, and with the tensor core idle meanwhile: 7447, 699, 104, 169.)
+// Tensor memory is read 16 columns at a time, the next 16 in flight, on the diagonal too: blocks of 32 registers beside the 128 of the sum
+// spilled 96 to 356 bytes, whatever the split.  By 32 columns / by 16, on the diagonal one after another / in flight everywhere, 32768 tokens 6782 /
+// 6919 / 6757, 8192 542 / 547 / 539.
 // Rows: with 256 rows of one head per CTA the last row tile of 4 x 777 tokens (8b shape) held 9 rows of 256 and the diagonal tiles were
 // half empty; side by side the heads take 13 row tiles with 49 key tiles per stream instead of 16 with 76: attention 75 -> 54 us,
-// whole call 108 -> 92 us per layer.  32768 tokens (7b shape, no idle rows either way): 7.79 / 7.83 ms.
+// whole call 108 -> 93 us per layer.
 #include "common.cuh"
 
 namespace mixkvq {
@@ -227,12 +229,18 @@ __device__ __forceinline__ void for_pieces(uint32_t taddr, int n_pieces, F f) {
       f(h + 1, b);
     }
   } else {
+    uint32_t a[16], b[16];
+    tmem_ld16_issue(taddr, a);
 #pragma unroll 1
-    for (int h = 0; h < n_pieces; ++h) {
-      uint32_t a[16];
-      tmem_ld16_issue(taddr + 16 * h, a);
+    for (int h = 0; h < n_pieces; h += 2) {
       tmem_wait_ld16(a);
+      if (h + 1 < n_pieces) tmem_ld16_issue(taddr + 16 * h + 16, b);
       f(h, a);
+      if (h + 1 < n_pieces) {
+        tmem_wait_ld16(b);
+        if (h + 2 < n_pieces) tmem_ld16_issue(taddr + 16 * h + 32, a);
+        f(h + 1, b);
+      }
     }
   }
 }
