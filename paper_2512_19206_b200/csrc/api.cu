@@ -576,7 +576,8 @@ int mixkvq_prefill(mixkvq_cache* cache, int layer, const void* k_dev, const void
     return MIXKVQ_E_CAPACITY;
   if (launch_prefill_attention(q_dev, k_dev, v_dev, out_dev, scratch_dev, cache->cfg.batch, cache->cfg.n_q_heads,
                                cache->cfg.n_kv_heads, n_tokens, softmax_scale, reinterpret_cast<uint32_t*>(cache->mem),
-                               cache->test_wait_polls, cache->test_extra_tx, cache->test_extra_v, static_cast<cudaStream_t>(stream)) != cudaSuccess)
+                               cache->test_wait_polls, cache->test_extra_tx, cache->test_extra_v, cache->n_sms, static_cast<cudaStream_t>(stream)) !=
+      cudaSuccess)
     return MIXKVQ_E_CUDA;
   cache->launches += 2;
   note_enqueued(cache, static_cast<cudaStream_t>(stream), kNoPackedWrite);

@@ -3,7 +3,7 @@
 //
 // Two kernels.  prefill_pack_kernel rewrites K (bf16) and V (converted to fp16) of the prompt into images of 128-token
 // tiles in the tensor core's canonical shared-memory layout, so that a tile reaches shared memory as ONE 32 KB bulk
-// copy.  prefill_attention_kernel runs one CTA of 384 threads per 256 query rows of a stream (batch element and KV head; a token's
+// copy.  prefill_attention_kernel runs one CTA of 384 threads per 256 (short prompts: 128) query rows of a stream (batch element and KV head; a token's
 // query heads side by side):
 //   warps 0-3, 4-7   two softmax groups, one per 128 query rows (thread = row = lane of tensor memory);
 //   warp 8           one thread issues every tcgen05.mma;
@@ -42,7 +42,7 @@ namespace {
 
 constexpr int kTile = 128;                       // query rows and key rows per tile
 constexpr int kTileBytes = kTile * kD * 2;       // one 128 x 128 tile of 16-bit elements
-constexpr int kQRows = 2 * kTile;                // query rows per CTA
+constexpr int kQRows = 2 * kTile;                // query rows per CTA, or kTile (the rule is at the launch)
 constexpr int kThreads = 384;
 constexpr int kBars = 17;
 constexpr int kSmem = 6 * kTileBytes + 256;      // two Q tiles, two K and two V stages; barriers and tensor-memory slot
@@ -340,7 +340,8 @@ __device__ __forceinline__ void softmax_tile(uint32_t s_addr, uint32_t o_addr, i
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned char* __restrict__ kt,
                          const unsigned char* __restrict__ vt, float* __restrict__ out, int n_streams, int g_heads, int L,
-                         int n_tiles, int n_qtiles, float scale_log2e, uint32_t* status, uint32_t max_polls, uint32_t debug_extra_tx, uint32_t debug_extra_v) {
+                         int n_tiles, int n_qtiles, int q_rows, float scale_log2e, uint32_t* status, uint32_t max_polls, uint32_t debug_extra_tx,
+                         uint32_t debug_extra_v) {
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* Qs = smem;                              // two tiles
   unsigned char* Ks = smem + 2 * kTileBytes;             // two stages
@@ -357,8 +358,8 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
     __device__ int token(int row) const { return min(tok0 + (int)((uint32_t)(rem0 + row) * inv >> 16), L - 1); }
   };
   auto rows_of = [&](int tile) {
-    const int tok0 = tile * kQRows / g_heads;
-    return Rows{tok0, tile * kQRows - tok0 * g_heads, L, g_inv};
+    const int tok0 = tile * q_rows / g_heads;
+    return Rows{tok0, tile * q_rows - tok0 * g_heads, L, g_inv};
   };
   const unsigned char* ktg = kt + (size_t)s * n_tiles * kTileBytes;
   const unsigned char* vtg = vt + (size_t)s * n_tiles * kTileBytes;
@@ -367,7 +368,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
   const Rows rows = rows_of(qt);
   const int tok0 = rows.tok0, rem0 = rows.rem0;
   const int last_a = rows.token(kTile - 1), last_b = rows.token(kQRows - 1);
-  const int n_a = last_a / kTile + 1, n_b = qt * kQRows + kTile < L * g_heads ? last_b / kTile + 1 : 0, n = max(n_a, n_b);
+  const int n_a = last_a / kTile + 1, n_b = q_rows == kQRows && qt * kQRows + kTile < L * g_heads ? last_b / kTile + 1 : 0, n = max(n_a, n_b);
   const int seen_a = last_a % kTile + 1, seen_b = last_b % kTile + 1;
 
   if (warp == 8) {
@@ -406,7 +407,7 @@ prefill_attention_kernel(const __nv_bfloat16* __restrict__ q, const unsigned cha
       const int i = tid + k * kThreads, ii = i & 2047, c = (ii >> 3) & 15;
       const uint32_t r = (uint32_t)(rem0 + (i >> 11) * kTile + 8 * (ii >> 7) + (ii & 7)), tk = r * g_inv >> 16;
       x[k] = make_uint4(0u, 0u, 0u, 0u);
-      if (i < kPieces && tok0 + (int)tk < L)
+      if (i < q_rows * 16 && tok0 + (int)tk < L)
         x[k] = *reinterpret_cast<const uint4*>(q + (((size_t)s * g_heads + (r - tk * g_heads)) * L + tok0 + tk) * kD + 8 * c);
     }
 #pragma unroll
@@ -630,15 +631,21 @@ size_t prefill_scratch_bytes(int B, int Hkv, int L) {
 
 cudaError_t launch_prefill_attention(const void* q, const void* k, const void* v, float* out, void* scratch, int B, int Hq,
                                      int Hkv, int L, float scale, uint32_t* status, uint32_t max_polls, uint32_t debug_extra_tx,
-                                     uint32_t debug_extra_v, cudaStream_t stream) {
-  const int g = Hq / Hkv, n_tiles = (L + kTile - 1) / kTile, n_qtiles = (int)(((long long)L * g + kQRows - 1) / kQRows);
+                                     uint32_t debug_extra_v, int n_sms, cudaStream_t stream) {
+  const int g = Hq / Hkv, n_tiles = (L + kTile - 1) / kTile;
+  // A short prompt's row tiles leave most SMs idle: 128 rows per CTA as long as every CTA has an SM to itself and a sixth of the SMs is left
+  // for the append, which runs beside the attention (no SM has the registers for both).  us per layer of the whole call, 256 / 128 rows: one prompt
+  // of the 7b shape, 60 tokens (16 CTAs with 128 rows) 19.2 / 17.3, 333 (76) 27.2 / 25.5, 550 (124) 31.3 / 28.6, 621 (136) 37.3 / 38.9, 655 (144)
+  // 33.7 / 46.7; 8b shape 450 (120) 29.6 / 26.9, 540 (136) 30.9 / 32.8; 4 prompts of the 7b shape, 100 (96) 29.4 / 27.0, 130 (128) 26.3 / 27.8.
+  const int q_rows = ((long long)L * g + kTile - 1) / kTile * B * Hkv <= n_sms * 5 / 6 ? kTile : kQRows;
+  const int n_qtiles = (int)(((long long)L * g + q_rows - 1) / q_rows);
   unsigned char* kt = static_cast<unsigned char*>(scratch);
   unsigned char* vt = kt + (size_t)B * Hkv * n_tiles * kTileBytes;
   const cudaError_t e = launch_dependent(prefill_pack_kernel, dim3((unsigned)n_tiles, (unsigned)(B * Hkv)), 256, 0, stream,
                                          static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), kt, vt, L, n_tiles);
   if (e != cudaSuccess) return e;
   return launch_dependent(prefill_attention_kernel, dim3((unsigned)(n_qtiles * B * Hkv)), kThreads, kSmem, stream,
-                          static_cast<const __nv_bfloat16*>(q), kt, vt, out, B * Hkv, g, L, n_tiles, n_qtiles,
+                          static_cast<const __nv_bfloat16*>(q), kt, vt, out, B * Hkv, g, L, n_tiles, n_qtiles, q_rows,
                           scale * 1.4426950408889634f, status, max_polls ? max_polls : kPolls, debug_extra_tx, debug_extra_v);
 }
 

@@ -58,6 +58,23 @@ def test_prefill_rows_of_every_group_size(binding, g, tokens):
     assert float((out.cpu() - torch.softmax(s, -1) @ vf).abs().max()) <= ATTN_TOL
 
 
+@pytest.mark.parametrize("g,tokens,batch", [(1, 17, 80), (1, 256, 40), (3, 130, 80), (5, 387, 16), (7, 64, 40), (7, 387, 16), (8, 300, 16),
+                                            (4, 128, 15), (4, 128, 16), (8, 1, 61), (8, 1, 62)])
+def test_prefill_row_tiles_of_256(binding, g, tokens, batch):
+    """With more than 123 row tiles (on 148 SMs) a CTA takes 256 rows instead of 128: from 16 sequences of two streams with four tiles on, or from
+    62 with one."""
+    gen = torch.Generator(device="cuda").manual_seed(100 * g + tokens)
+    k, v, q = (torch.randn((batch, h, tokens, 128), generator=gen, device="cuda").to(torch.bfloat16) for h in (2, 2, 2 * g))
+    cache = binding.Cache(binding.make_config(1, batch, 2 * g, 2, tokens, **W.P24))
+    out = torch.full((batch, 2 * g, tokens, 128), 7.0, device="cuda")
+    cache.prefill(0, k, v, q, W.softmax_scale(), out=out)
+    assert cache.status() == 0
+    qf, kf, vf = (t.double() for t in (q, k.repeat_interleave(g, 1), v.repeat_interleave(g, 1)))
+    s = (qf @ kf.transpose(-1, -2)) * W.softmax_scale()
+    s.masked_fill_(torch.ones(tokens, tokens, device="cuda").triu(1).bool(), float("-inf"))
+    assert float((out - torch.softmax(s, -1) @ vf).abs().max()) <= ATTN_TOL
+
+
 def test_prefill_large_magnitudes_and_errors(binding):
     w = W.small(W.CONFIGS["qwen7b"], n_layers=1, batch=1, tokens=300)
     k, v, q = W.tokens(w, 0, 0, 300)
