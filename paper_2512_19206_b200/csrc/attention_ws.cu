@@ -1377,11 +1377,13 @@ cudaError_t launch_attention_ws(const LayerView& lv, const void* q, float* out, 
   // not early / early, 32 streams (288 CTAs), two tiers 1000 tokens 8.0 / 8.2, 6000 (22 positions per CTA) 14.15 / 14.15, 12000 21.0 / 20.0, three
   // tiers 1000 10.2 / 10.8, 4000 (16) 13.1 / 13.2, 14000 26.6 / 26.2; 64 streams, two tiers 2500 (21) 13.7 / 12.7, three tiers 16.5 / 15.0, 4-bit values 1000
   // (10) 9.5 / 13.7, 1500 (14) 12.0 / 13.8, 2500 15.9 / 14.8; 128 streams, 2500 20.7 / 18.1, three tiers 25.2 / 24.0.  With three tiers or a 4-bit base
-  // not where a stream is split over many CTAs or a CTA takes several streams: 8 streams, 28000 tokens 16.9 / 17.4, 17.3 / 18.0 (two tiers 14.9 /
-  // 14.8, G = 128 14.2 / 13.8), 16 streams, 13000 16.7 / 17.2, 17.0 / 17.6; 320 streams, 900 28.7 / 28.9, 27.6 / 28.0.  Two tiers with several streams per CTA: 320
+  // later where a stream is split over many CTAs, and not where a CTA takes several streams: 8 streams, 28000 tokens (25) 16.9 / 17.4, 4-bit base
+  // 17.3 / 18.0 (two tiers 14.9 / 14.8), 16 streams, 13000 (23) 16.7 / 17.2, 17.0 / 17.6, 20000 (36) 21.2 / 21.4, 21.5 / 21.65, 24 streams, 20000 (53) 27.95 / 27.6,
+  // 28.4 / 27.9, 8 streams, 70000 (61) 30.1 / 29.9, 30.7 / 30.1; 320 streams, 900 28.7 / 28.9, 27.6 / 28.0.  Two tiers with several streams per CTA: 320
   // streams, 700 tokens (26 positions per stream) 19.9 / 20.1, G = 128 20.7 / 21.2, 1100 (41) 27.4 / 26.6, 25.9 / 25.8.
-  const bool gains = three_tiers(lv) || lv.dense_hi ? S >= 32 && S <= grid : S <= grid || lv.seq != nullptr || Us >= 32;
-  const bool early = grid > n_sms && gains && (lv.seq != nullptr ? lv.seq_total : Us * S) >= 20ll * grid;
+  const bool two_tiers = !three_tiers(lv) && !lv.dense_hi, may = two_tiers ? S <= grid || lv.seq != nullptr || Us >= 32 : S <= grid;
+  const int from_positions = two_tiers || S >= 32 ? 20 : 50;
+  const bool early = grid > n_sms && may && (lv.seq != nullptr ? lv.seq_total : Us * S) >= (long long)from_positions * grid;
   e = launch_combine(ws, out, lv.g, lv.Hkv, lv.Hq, 1, grid, Us, S, stream, lv.seq, lv.seq_prefix, lse_out, early,
                      lv.rope_cos != nullptr ? const_cast<void*>(q) : nullptr, const_cast<uint16_t*>(lv.new_k), lv.rope_cos, lv.rope_sin);
   *launches = 2;
