@@ -19,6 +19,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -255,15 +256,13 @@ def algorithmic_bytes_per_layer(w, n16, n4, r, tokens_packed, n_partials, v_bits
     return streams * per_stream + 2 * n_partials * g * (D + 2) * 4
 
 
-def n_split_partials(w, d0, dev):
-    """Partials written per launch = CTAs of the split kernel (the library's grid rule: two split positions per CTA while that
-    leaves one CTA per SM, then up to four, then two CTAs per SM; a multiple of the stream count when there are fewer streams
-    than CTAs), each CTA one partial per stream it touches."""
+def n_split_partials(cache, w, dev):
+    """Partials written by the last attention call: one per CTA of the split kernel and stream that it touches.  The CTAs share the
+    streams' positions evenly, so that CTAs and streams begin together gcd times.  (The tile layout's kernel does not report its CTAs:
+    one per SM.)"""
     streams = w.batch * w.n_kv_heads
-    units = (d0.n_blocks * w.residual_len // 32 + 3 * ((d0.residual_tokens + 31) // 32)) * streams
-    n_sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    n_part = min(2 * n_sms, (units + 1) // 2, max(n_sms, (units + 3) // 4))
-    return n_part // streams * streams if n_part > streams else n_part + streams
+    ctas = cache.last_attention_ctas() or torch.cuda.get_device_properties(dev).multi_processor_count
+    return ctas + streams - math.gcd(ctas, streams)
 
 
 def time_loop(fn, reps):
@@ -278,7 +277,7 @@ def time_loop(fn, reps):
 
 
 def attention_timings(cache, w, qs, out, scale):
-    """(split kernel ms per launch, attention + combine us per layer) at the cache's current state."""
+    """(split kernel ms per launch, attention + combine us per layer, partials per split kernel) at the cache's current state."""
     def all_layers():
         for layer in range(w.n_layers):
             cache.decode_attention(layer, qs[layer], scale, out=out[layer])
@@ -286,17 +285,18 @@ def attention_timings(cache, w, qs, out, scale):
     cache.set_attention_kernel(2)
     all_layers()
     kern_ms = time_loop(all_layers, reps) / w.n_layers
+    partials = n_split_partials(cache, w, out.device)
     cache.set_attention_kernel(0)
     all_layers()
     attn_us = time_loop(all_layers, reps) / w.n_layers * 1e3
-    return kern_ms, attn_us
+    return kern_ms, attn_us, partials
 
 
-def roofline_entry(cache, w, dev, args, kern_ms):
+def roofline_entry(cache, w, args, kern_ms, partials):
     d0 = cache.describe(0)
     n16, n4 = tier_mix(cache, w)
     tokens_packed = d0.n_blocks * w.residual_len
-    alg = algorithmic_bytes_per_layer(w, n16, n4, d0.residual_tokens, tokens_packed, n_split_partials(w, d0, dev), args.v_bits)
+    alg = algorithmic_bytes_per_layer(w, n16, n4, d0.residual_tokens, tokens_packed, partials, args.v_bits)
     peak, peak_src = measured_peaks()
     achieved = alg / (kern_ms * 1e-3) / 1e9
     return n16, n4, tokens_packed, alg, achieved, peak, peak_src
@@ -314,8 +314,8 @@ def other_config(binding, dev, args, name, w, label, contexts=None):
         prefill(cache, w, dev, done, T)
         done = T
         qs = [W.decode_query(w, layer, 0, device=dev) for layer in range(w.n_layers)]
-        kern_ms, attn_us = attention_timings(cache, w, qs, out, scale)
-        n16, n4, tokens_packed, alg, achieved, peak, _ = roofline_entry(cache, w, dev, args, kern_ms)
+        kern_ms, attn_us, partials = attention_timings(cache, w, qs, out, scale)
+        n16, n4, tokens_packed, alg, achieved, peak, _ = roofline_entry(cache, w, args, kern_ms, partials)
         entries.append({
             "workload": label, "shape": f"B={w.batch} Hq={w.n_q_heads} Hkv={w.n_kv_heads} T={T} G={w.group_size}",
             "layers_measured": w.n_layers, "layers_of_model": W.CONFIGS[name].n_layers,
@@ -344,7 +344,7 @@ def ragged_config(binding, dev, args):
     scale = W.softmax_scale()
     out = torch.empty((w.n_layers, w.batch, w.n_q_heads, 128), dtype=torch.float32, device=dev)
     qs = [W.decode_query(w, layer, 0, device=dev) for layer in range(w.n_layers)]
-    kern_ms, attn_us = attention_timings(cache, w, qs, out, scale)
+    kern_ms, attn_us, _ = attention_timings(cache, w, qs, out, scale)
     n16, n4 = tier_mix(cache, w)             # of sequence 0, the longest
     one = W.small(w, batch=1)
     alg, units = 0.0, 0
@@ -484,7 +484,7 @@ def run_gpu(args, w):
     # ---- dominant kernel alone (split kernel, no combine), and attention + combine, same state
     nxt = Wm + K                                    # next unused decode-step input
     qs = [steps_in[layer][nxt][2].view(w.batch, w.n_q_heads, 128) for layer in range(w.n_layers)]
-    kern_ms, attn_us_layer = attention_timings(cache, w, qs, out, scale)
+    kern_ms, attn_us_layer, partials = attention_timings(cache, w, qs, out, scale)
     reps = max(3, min(20, int(200 / max(1, w.n_layers))))
     # ---- attention + combine for all layers from one CUDA graph (fixed state): launch gaps removed
     g = torch.cuda.CUDAGraph()
@@ -501,7 +501,7 @@ def run_gpu(args, w):
     g.replay()
     graph_us = time_loop(g.replay, reps) * 1e3
     clocks = sampler.stop() if rank == 0 else None
-    n16, n4, tokens_packed, alg, achieved, peak, peak_src = roofline_entry(cache, w, dev, args, kern_ms)
+    n16, n4, tokens_packed, alg, achieved, peak, peak_src = roofline_entry(cache, w, args, kern_ms, partials)
 
     # ---- the parts of the step on their own: the plain append of one token (no flush), and the step on which the
     # residual window is full, so that the append first scores, quantizes and packs it (once every R steps)
