@@ -31,7 +31,7 @@
 // per values warp there.  us per launch, one unit / two units per step / with two logits warps: 7b shape (B = 8, T = 32768) 36.7 /
 // 35.3; three tiers 54.4 / 48.7 / 46.2; 4-bit base (8b shape, B = 16, T = 16384) 110.7 / 109.5 / 101.7; 4-bit values 88.4 / 82;
 // 32b shape (B = 64, T = 32768, G = 128) 463 / 433 = 3.1 TB/s.  (Those five were taken side by side with a reference maximum raised only
-// by factors of 8; as the kernel is now: 35.7, 46.1, 101.3, 83, 425.)
+// by factors of 8; as the kernel is now: 34.3, 46.4, 95.5, 80.6, 421.)
 #include "warp_ops.cuh"
 
 namespace mixkvq {
@@ -1285,7 +1285,8 @@ static bool three_tiers(const LayerView& lv) {
 // streams, as their split gets the less out of the rest of the SMs.  us per layer, one CTA per stream / split: two tiers, 16 streams, 24 positions
 // 5.96 / 6.02, 28 6.63 / 6.48, 64 streams, 40 8.85 / 9.05, 42 10.3 / 9.6, 128 streams, 42 11.7 / 13.1; three tiers, 4 streams, 14 positions 6.34 / 6.67,
 // 18 7.5 / 6.7, 64 streams, 28 9.25 / 10.8, 32 10.3 / 10.1, 128 streams, 40 14.1 / 14.3, 42 15.8 / 15.5; 4-bit base, 4 streams, 14 5.75 / 5.87, 18 6.8 / 5.9,
-// 128 streams, 40 13.0 / 14.6; 4-bit values, 16 streams, 18 6.1 / 6.7, 32 streams, 28 7.1 / 7.5, 32 8.1 / 7.5.
+// 128 streams, 40 13.0 / 14.6; 4-bit values, 16 streams, 18 6.1 / 6.7, 32 streams, 28 7.1 / 7.5, 32 8.1 / 7.5.  With few streams it is the launch
+// saved that counts: 4 streams, two tiers, as calls / from a graph, 17 positions 4.7 / 6.3, 4.9 / 5.0, 20 5.75 / 6.3, 5.5 / 5.1, 26 6.6 / 6.3, 6.6 / 5.0.
 // With more streams (four pairs, two CTAs per SM): never slower than the split up to 20 positions with two tiers and 2-bit values
 // (one CTA per stream / split, 16 streams of the 8b shape 6.4 / 7.9); otherwise a unit takes longer, and beyond 12 positions
 // the split is faster as long as it gets by with one CTA per SM (64 streams, 390 tokens, three tiers 6.9 / 8.8; 4-bit base
